@@ -130,13 +130,16 @@ static size_t carve(Plan& pl, void* ws) {
     off += up256(bytes);
     return p;
   };
-  const size_t vol = pl.n3 * pl.esize, dat = pl.nd * pl.esize, wvol = pl.nw3 * pl.esize;
+  const size_t vol = pl.n3 * pl.esize, wvol = pl.nw3 * pl.esize;
+  // the wave input doubles as the z-innermost operand of P, the data scratch as
+  // that of P^T (rows padded to 16 bytes)
+  const size_t zvol = zvolume_bytes(pl.nw, pl.esize), dat = zdata_bytes(pl.nw, pl.nth, pl.esize);
   pl.kap = take(vol);
   pl.kapw = pl.pad ? take(wvol) : pl.kap;
   for (int i = 0; i < 6; ++i) pl.s[i] = i < nstate(pl) ? take(wvol) : nullptr;
-  pl.x = take(vol);
+  pl.x = take(pl.pad ? vol : zvol);
   pl.v = take(vol);
-  pl.xw = pl.pad ? take(wvol) : nullptr;
+  pl.xw = pl.pad ? take(zvol) : nullptr;
   pl.xo = pl.pad ? take(vol) : nullptr;
   pl.xg = pl.pad ? take(wvol) : nullptr;
   pl.r = take(dat);
@@ -555,7 +558,7 @@ static int wave_back(const Plan& pl, const void* x, const void** w, cudaStream_t
 // h = E^T W^T P^T g  ->  x = K P^T g ; w = E^T W x ; h = w / K
 static int apply_adjoint(const Plan& pl, const void* g, void* h, cudaStream_t st) {
   const Plan wp = wave_plan(pl);
-  TRY(launch_backproject(wp, g, wave_in(pl), wp.kap, st));
+  TRY(launch_backproject(wp, g, wave_in(pl), wp.kap, st, pl.r));
   const void* w = nullptr;
   TRY(wave_back(pl, wave_in(pl), &w, st));
   TRY(launch_kscale(pl, w, h, false, st));
@@ -579,7 +582,7 @@ static int data_gradient(const Plan& pl, const void* v, const void* g, const voi
       lr = pl.r2;
     }
     if (dots) TRY(launch_dot(pl, pl.nd, lr, pl.r, dots, st));
-    TRY(launch_backproject(wp, lr, wave_in(pl), wp.kap, st));
+    TRY(launch_backproject(wp, lr, wave_in(pl), wp.kap, st, lr == pl.r ? pl.r2 : pl.r));
   }
   TRY(wave_back(pl, wave_in(pl), w, st));
   return FFPAT_OK;
@@ -777,42 +780,37 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
   return FFPAT_OK;
 }
 
-int ffpat_project(const ffpat_problem* problem, const void* p, void* g, void* stream) {
-  Trace trace_("ffpat_project");
-  cudaStream_t st = (cudaStream_t)stream;
+// P or P^T alone: the angle tables and the z-innermost operand in one
+// stream-ordered allocation.
+static int project_alone(const ffpat_problem* problem, const void* in, void* out, bool transpose,
+                         cudaStream_t st) {
   Plan pl;
   g_err[0] = 0;
   TRY(validate(problem, pl));
-  if (!p || !g) return fail(FFPAT_EINVAL, "p or g is NULL");
-  void* tabs = nullptr;
-  void* tr = nullptr;
-  const size_t trb = project_scratch_bytes(wave_plan(pl));
-  CK(cudaMallocAsync(&tabs, table_bytes(pl.nth), st));
-  if (trb) CK(cudaMallocAsync(&tr, trb, st));
-  int rc = upload_tables(pl, tabs, st);
-  if (rc == FFPAT_OK) rc = launch_project(wave_plan(pl), p, g, nullptr, st, nullptr, tr);
-  if (tr) CK(cudaFreeAsync(tr, st));
-  CK(cudaFreeAsync(tabs, st));
+  if (!in || !out) return fail(FFPAT_EINVAL, transpose ? "g or h is NULL" : "p or g is NULL");
+  const size_t tb = up256(table_bytes(pl.nth));
+  const size_t zb = transpose ? zdata_bytes(pl.nw, pl.nth, pl.esize) : zvolume_bytes(pl.nw, pl.esize);
+  char* mem = nullptr;
+  CK(cudaMallocAsync((void**)&mem, tb + zb, st));
+  int rc = upload_tables(pl, mem, st);
+  const Plan wp = wave_plan(pl);
+  if (rc == FFPAT_OK)
+    rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb)
+                   : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb);
+  CK(cudaFreeAsync(mem, st));
   TRY(rc);
   CK(cudaStreamSynchronize(st));
   return FFPAT_OK;
 }
 
+int ffpat_project(const ffpat_problem* problem, const void* p, void* g, void* stream) {
+  Trace trace_("ffpat_project");
+  return project_alone(problem, p, g, false, (cudaStream_t)stream);
+}
+
 int ffpat_backproject(const ffpat_problem* problem, const void* g, void* h, void* stream) {
   Trace trace_("ffpat_backproject");
-  cudaStream_t st = (cudaStream_t)stream;
-  Plan pl;
-  g_err[0] = 0;
-  TRY(validate(problem, pl));
-  if (!h || !g) return fail(FFPAT_EINVAL, "g or h is NULL");
-  void* tabs = nullptr;
-  CK(cudaMallocAsync(&tabs, table_bytes(pl.nth), st));
-  int rc = upload_tables(pl, tabs, st);
-  if (rc == FFPAT_OK) rc = launch_backproject(wave_plan(pl), g, h, nullptr, st);
-  CK(cudaFreeAsync(tabs, st));
-  TRY(rc);
-  CK(cudaStreamSynchronize(st));
-  return FFPAT_OK;
+  return project_alone(problem, g, h, true, (cudaStream_t)stream);
 }
 
 int ffpat_ramp(const ffpat_problem* problem, const void* r, void* out, void* stream) {
@@ -919,7 +917,7 @@ int ffpat_fbp(const ffpat_problem* problem, const void* G, void* out, void* ws, 
   TRY(upload_tables(pl, pl.tab, st));
   const Plan wp = wave_plan(pl);
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(wp, pl.r2, out, nullptr, st, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(wp, pl.r2, out, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
   return FFPAT_OK;
 }
 
@@ -978,7 +976,7 @@ int ffpat_fb_two_step_ex(const ffpat_problem* problem, const void* c, const void
   const Plan wp = wave_plan(pl);
   void* gt = pl.pad ? pl.xg : pl.v;
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(wp, pl.r2, gt, nullptr, st, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(wp, pl.r2, gt, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
   int k = 0;
   for (; k < max_iters; ++k) {
     Trace trace_it("FB iteration (Algorithm 9)");

@@ -142,7 +142,7 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   void* B[4] = {pl.x, pl.s[0], pl.s[1], pl.s[2]};
   const bool two_t = two_step_three_term(pl, tma) && pl.s[1] && pl.s[2];
   int u = 0, v = 1;
-  int rc = launch_backproject(pl, grad_g, B[u], pl.kap, st);
+  int rc = launch_backproject(pl, grad_g, B[u], pl.kap, st, pl.r);
   if (rc != FFPAT_OK) return rc;
   if (cudaMemsetAsync(B[v], 0, vb, st) != cudaSuccess ||
       cudaMemsetAsync(ck.acc(), 0, vb, st) != cudaSuccess)

@@ -176,17 +176,17 @@ int read_device_status(unsigned* out, bool clear);
 int launch_wait_timeout(long long cycles, cudaStream_t st);
 
 // xray.cu
+// bytes of a volume / of the data (n detectors, nth angles) with z innermost
+size_t zvolume_bytes(int n, size_t esize);
+size_t zdata_bytes(int n, int nth, size_t esize);
 // g = mask .* (P p - sub)  (sub, mask nullable)
-// scratch (nullable): a volume of the plan's grid that aliases neither p nor
-// g; when the planes are too large for shared memory it receives a transposed
-// copy of p, from which the steep angles read (same result, coalesced loads).
+// scratch: zvolume_bytes that alias neither p nor g; receives p with z innermost
 int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
-                   const void* mask = nullptr, void* scratch = nullptr);
-// bytes of that scratch (0 when the shared-memory kernel is used)
-size_t project_scratch_bytes(const Plan& pl);
+                   const void* mask, void* scratch);
 // h = mult * scale .* P^T g  (scale nullable)
+// scratch: zdata_bytes that alias neither g nor h; receives g with z innermost
 int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       double mult = 1.0);
+                       void* scratch, double mult = 1.0);
 // out = mask .* (Lambda r)  (mask nullable)
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st,
                 const void* mask = nullptr);

@@ -225,7 +225,7 @@ int after_wave(ffpat_server* S, Req& r) {
       lr = pl.r2;
     }
     if (!power && launch_dot(pl, pl.nd, lr, pl.r, pl.hist, st) != FFPAT_OK) return FFPAT_ECUDA;
-    if (launch_backproject(pl, lr, pl.x, pl.kap, st) != FFPAT_OK) return FFPAT_ECUDA;
+    if (launch_backproject(pl, lr, pl.x, pl.kap, st, lr == pl.r ? pl.r2 : pl.r) != FFPAT_OK) return FFPAT_ECUDA;
     r.phase = kAdj;
     r.wstep = 0;
     r.w_in = (const float*)pl.x;

@@ -8,20 +8,25 @@
 // sqrt 2) ray samples, both spaced dx.  The index geometry depends on n only;
 // dx enters as the sample length and the detector spacing of Lambda.
 //
-// P (ray-driven, no atomics): one thread per detector xi_k of one (theta_j,
-// z_l) row; it walks the ray samples s_m that can touch the grid and
-// accumulates the zero-extended bilinear samples in order, reading the plane
-// through the read-only cache.  For FP64 problems the sample arithmetic is
-// done in round-to-nearest multiply/add with no contraction, in the same
-// order as the plain definition, so that indices and weights are reproducible
-// bit for bit.
+// The geometry is the same in every plane, so both kernels run along z: the
+// operand is first copied to a layout with z innermost (k_zlast), the bilinear
+// weights of one angle are worked out once into shared-memory lists, and the
+// lanes of a warp then apply each weight to 32, 64 or 128 planes at a time.
+// What bounds them is thus the multiply-adds and the loads of the operand
+// (through L1), no longer the index arithmetic.  Fixed order, no atomics:
+// deterministic.
 //
-// P^T (voxel-driven gather, no atomics): one thread per voxel.  For every
-// angle the samples whose bilinear footprint covers the voxel lie within
-// sqrt(2) grid units of it in the rotated (xi, s) frame, i.e. at most 3 x 3
-// candidates; each contributes hat(dx) hat(dy) times its row value, which is
-// exactly the bilinear weight P gives that voxel.  Deterministic: fixed order.
-// P stages the plane in shared memory when it fits (N <= 220 in FP32).
+// P (ray-driven).  FP32: a ray is walked along its major axis (y where |cos|
+// >= |sin|, else x); the weights of all its samples in one row of cells are
+// merged into at most four taps.  FP64: sample by sample, with the
+// interpolation done in round-to-nearest multiply/add with no contraction, in
+// the order of the plain definition, so that indices, weights and sums are
+// reproducible bit for bit.
+//
+// P^T (voxel-driven).  For every angle the samples whose bilinear footprint
+// covers a voxel lie within sqrt(2) grid units of it in the rotated (xi, s)
+// frame, i.e. at most 3 x 3 candidates; each contributes hat(dx) hat(dy) times
+// its row value, which is exactly the bilinear weight P gives that voxel.
 //
 // Lambda: one CTA per detector row, the row staged in shared memory, the odd
 // taps t_d = -1/(2 pi^2 d^2 dxi) and t_0 = 1/(8 dxi) applied as a linear
@@ -29,9 +34,10 @@
 #include <limits.h>
 #include <math.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <mutex>
-#include <vector>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -58,19 +64,6 @@ __device__ __forceinline__ void sample64(double cs, double sn, int k, int m, int
   j0 = (int)fly;
   fx = __dsub_rn(gx, flx);
   fy = __dsub_rn(gy, fly);
-}
-
-// fraction (bits 0..30 of a scale-2^31 fixed-point value) as a float in
-// [0, 1): the top 23 fraction bits become the mantissa of a number in [1, 2)
-// (integer and logic ops only; no int-to-float conversion)
-__device__ __forceinline__ float frac31(long long v) {
-  const unsigned f = (unsigned)v & 0x7fffffffu;
-  return __uint_as_float(0x3f800000u | (f >> 8)) - 1.0f;
-}
-
-template <typename T>
-__device__ __forceinline__ T pix(const T* __restrict__ sl, int n, int iy, int ix) {
-  return (ix >= 0 && iy >= 0 && ix < n && iy < n) ? __ldg(sl + (size_t)iy * n + ix) : T(0);
 }
 
 // Range [mlo, mhi) of ray samples that can touch the grid (conservative).
@@ -110,890 +103,660 @@ __device__ __forceinline__ void ray_range(float cs, float sn, int k, int n, int 
   if (mhi < mlo) mhi = mlo;
 }
 
-// Plane value at (row iy, column ix); `tr`: the plane is stored transposed
-// (column-major), so element (iy, ix) sits at ix * n + iy.
-template <typename T>
-__device__ __forceinline__ T pix2(const T* __restrict__ sl, int n, int iy, int ix, bool tr) {
-  return (ix >= 0 && iy >= 0 && ix < n && iy < n)
-             ? __ldg(sl + (tr ? (size_t)ix * n + iy : (size_t)iy * n + ix))
-             : T(0);
-}
-
-// P from global memory (planes too large for shared memory).  The threads of
-// a block are neighbouring detectors of one angle: at a given sample index
-// they sit one cell apart along (cos, sin).  For steep angles (|sin| > |cos|)
-// that is mostly along y, so their loads would touch one row each; given the
-// transposed planes `pt` the block reads those instead and the same loads run
-// along memory.  Same values, weights and summation order either way.
-template <typename T>
-__global__ void __launch_bounds__(128)
-    k_project(const T* __restrict__ p, const T* __restrict__ pt, T* __restrict__ g,
-              const T* __restrict__ sub, const T* __restrict__ mask,
-              const double* __restrict__ tab, const float* __restrict__ tabf,
-              const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int l = blockIdx.y;
-  const int j = blockIdx.z;
-  const float csf = tabf[j], snf = tabf[nth + j];
-  const bool tr = pt != nullptr && fabsf(snf) > fabsf(csf);
-  const T* __restrict__ sl = (tr ? pt : p) + (size_t)l * n * n;
-  int mlo = 0, mhi = 0;
-  if (k < n) ray_range(csf, snf, k, n, ns, mlo, mhi);
-  T acc = T(0);
-  if constexpr (sizeof(T) == 8) {
-    const double cs = tab[j], sn = tab[nth + j];
-    const double dx = 2.0 / nimg, half = nimg / 2.0, L = (double)n / nimg;
-    for (int m = mlo; m < mhi; ++m) {
-      int i0, j0;
-      double fx, fy;
-      sample64(cs, sn, k, m, ns, dx, half, L, i0, j0, fx, fy);
-      const double ofx = __dsub_rn(1.0, fx), ofy = __dsub_rn(1.0, fy);
-      double b = __dmul_rn(__dmul_rn(ofx, ofy), pix2(sl, n, j0, i0, tr));
-      b = __dadd_rn(b, __dmul_rn(__dmul_rn(fx, ofy), pix2(sl, n, j0, i0 + 1, tr)));
-      b = __dadd_rn(b, __dmul_rn(__dmul_rn(ofx, fy), pix2(sl, n, j0 + 1, i0, tr)));
-      b = __dadd_rn(b, __dmul_rn(__dmul_rn(fx, fy), pix2(sl, n, j0 + 1, i0 + 1, tr)));
-      acc = __dadd_rn(acc, b);
-    }
-    if (k < n) {
-      double out = __dmul_rn(dx, acc);
-      const size_t o = ((size_t)j * n + l) * n + k;
-      if (sub) out = out - sub[o];
-      if (mask) out = out * mask[o];
-      g[o] = out;
-    }
-  } else {
-    // fixed point, scale 2^31 grid units: the coordinates of the samples of one
-    // ray advance by exact integer steps, so fx, fy carry ~1e-9 absolute error
-    // at any grid size (a float coordinate near 384 would carry 3e-5)
-    const long long CS = tabi[j], SN = tabi[nth + j];
-    const long long u2 = 2LL * k + 1 - n, v2 = 2LL * mlo + 1 - ns;
-    const long long c2 = (long long)(n - 1) << 30;
-    long long GX = c2 + u2 * CS - v2 * SN;
-    long long GY = c2 + u2 * SN + v2 * CS;
-    const long long dGX = -2 * SN, dGY = 2 * CS;
-    for (int m = mlo; m < mhi; ++m) {
-      const int i0 = (int)(GX >> 31), j0 = (int)(GY >> 31);
-      const float fx = frac31(GX), fy = frac31(GY);
-      GX += dGX;
-      GY += dGY;
-      const float v00 = pix2(sl, n, j0, i0, tr), v10 = pix2(sl, n, j0, i0 + 1, tr);
-      const float v01 = pix2(sl, n, j0 + 1, i0, tr), v11 = pix2(sl, n, j0 + 1, i0 + 1, tr);
-      const float r0 = fmaf(fx, v10 - v00, v00);
-      const float r1 = fmaf(fx, v11 - v01, v01);
-      acc += fmaf(fy, r1 - r0, r0);
-    }
-    if (k < n) {
-      float out = (2.0f / (float)nimg) * acc;
-      const size_t o = ((size_t)j * n + l) * n + k;
-      if (sub) out = out - sub[o];
-      if (mask) out = out * mask[o];
-      g[o] = out;
-    }
-  }
-}
-
-// P with the whole plane staged in shared memory behind a zero border of
-// kPad points, so the bilinear corner loads need no bounds tests (used when
-// the padded plane fits; one CTA per (plane, group of angles), threads over
-// (angle, detector) pairs).  Same per-sample arithmetic as k_project.
-constexpr int kPad = 3;
-constexpr int kProjThreads = 1024;  // threads of the whole-plane kernel (8 angles x N rays)
-
-// row pitch of the staged plane: at least n + 2 kPad, and 1 mod 32 so that the
-// 32 rays of a warp, which cross the plane along one direction, fall on
-// different shared-memory banks when they run along y
-__host__ __device__ inline int plane_pitch(int n) {
-  const int w = n + 2 * kPad;
-  return w + ((33 - w % 32) % 32);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kProjThreads)
-    k_project_smem(const T* __restrict__ p, T* __restrict__ g, const T* __restrict__ sub,
-                   const T* __restrict__ mask, const double* __restrict__ tab,
-                   const float* __restrict__ tabf, const int32_t* __restrict__ tabi, int n,
-                   int nth, int ns, int nimg, int group) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* s = reinterpret_cast<T*>(smem_raw);
-  const int W = plane_pitch(n);  // row pitch; rows = n + 2 kPad
-  const int l = blockIdx.x;
-  const int ja = blockIdx.y * group, jb = min(nth, ja + group);
-  const T* __restrict__ sl = p + (size_t)l * n * n;
-  const int H = n + 2 * kPad;
-  for (int yy = threadIdx.x / 32; yy < H; yy += blockDim.x / 32) {
-    const int y = yy - kPad;
-    for (int xx = threadIdx.x % 32; xx < W; xx += 32) {
-      const int x = xx - kPad;
-      s[yy * W + xx] = (x >= 0 && y >= 0 && x < n && y < n) ? __ldg(sl + (size_t)y * n + x) : T(0);
-    }
-  }
-  __syncthreads();
-  // corner (i0, j0) of the padded plane, clamped so that no load leaves it
-  auto at = [&](int j0, int i0) -> int {
-    const int jj = min(max(j0 + kPad, 0), H - 2), ii = min(max(i0 + kPad, 0), H - 2);
-    return jj * W + ii;
-  };
-  const int work = (jb - ja) * n;
-  for (int w = threadIdx.x; w < work; w += blockDim.x) {
-    const int j = ja + w / n, k = w % n;
-    int mlo, mhi;
-    ray_range(tabf[j], tabf[nth + j], k, n, ns, mlo, mhi);
-    T acc = T(0);
-    if constexpr (sizeof(T) == 8) {
-      const double cs = tab[j], sn = tab[nth + j];
-      const double dx = 2.0 / nimg, half = nimg / 2.0, L = (double)n / nimg;
-      for (int m = mlo; m < mhi; ++m) {
-        int i0, j0;
-        double fx, fy;
-        sample64(cs, sn, k, m, ns, dx, half, L, i0, j0, fx, fy);
-        const int o = at(j0, i0);
-        const double ofx = __dsub_rn(1.0, fx), ofy = __dsub_rn(1.0, fy);
-        double b = __dmul_rn(__dmul_rn(ofx, ofy), s[o]);
-        b = __dadd_rn(b, __dmul_rn(__dmul_rn(fx, ofy), s[o + 1]));
-        b = __dadd_rn(b, __dmul_rn(__dmul_rn(ofx, fy), s[o + W]));
-        b = __dadd_rn(b, __dmul_rn(__dmul_rn(fx, fy), s[o + W + 1]));
-        acc = __dadd_rn(acc, b);
-      }
-      double out = __dmul_rn(dx, acc);
-      const size_t oo = ((size_t)j * n + l) * n + k;
-      if (sub) out = out - sub[oo];
-      if (mask) out = out * mask[oo];
-      g[oo] = out;
-    } else {
-      const long long CS = tabi[j], SN = tabi[nth + j];
-      const long long u2 = 2LL * k + 1 - n, v2 = 2LL * mlo + 1 - ns;
-      const long long c2 = (long long)(n - 1) << 30;
-      long long GX = c2 + u2 * CS - v2 * SN;
-      long long GY = c2 + u2 * SN + v2 * CS;
-      const long long dGX = -2 * SN, dGY = 2 * CS;
-      for (int m = mlo; m < mhi; ++m) {
-        const int i0 = (int)(GX >> 31), j0 = (int)(GY >> 31);
-        const float fx = frac31(GX), fy = frac31(GY);
-        GX += dGX;
-        GY += dGY;
-        const int o = at(j0, i0);
-        const float v00 = s[o], v10 = s[o + 1], v01 = s[o + W], v11 = s[o + W + 1];
-        const float r0 = fmaf(fx, v10 - v00, v00);
-        const float r1 = fmaf(fx, v11 - v01, v01);
-        acc += fmaf(fy, r1 - r0, r0);
-      }
-      float out = (2.0f / (float)nimg) * acc;
-      const size_t oo = ((size_t)j * n + l) * n + k;
-      if (sub) out = out - sub[oo];
-      if (mask) out = out * mask[oo];
-      g[oo] = out;
-    }
-  }
-}
-
-// FP32 P for planes too large for shared memory, band by band.  A CTA owns
-// one plane and a group of angles whose rays all run the same way in y (cos
-// >= 0, or cos < 0): it stages the plane in bands of bh rows (plus the zero
-// border) and visits the bands in the order its rays cross them, so every ray
-// still adds its samples in increasing m, the order of k_project.  Between
-// bands each ray's next sample, end of range and running sum live in shared
-// memory.  A sample belongs to the band of its lower row j0 (the first and
-// last bands take the rows beyond), whose buffer also holds row j0 + 1.
-__global__ void __launch_bounds__(1024)
-    k_project_band(const float* __restrict__ p, float* __restrict__ g,
-                   const float* __restrict__ sub, const float* __restrict__ mask,
-                   const float* __restrict__ tabf, const int32_t* __restrict__ tabi, int n,
-                   int nth, int ns, int nimg, int group, int jsplit, int bh, int nb) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int W = plane_pitch(n);
-  const int HB = bh + 2 * kPad;  // rows of the band buffer
-  float* s = reinterpret_cast<float*>(smem_raw);
-  float* racc = s + (size_t)HB * W;
-  int* rm = reinterpret_cast<int*>(racc + (size_t)group * n);  // next sample of each ray
-  int* rend = rm + (size_t)group * n;                          // end of its sample range
-  // angle groups vary fastest, so the CTAs resident together read the same
-  // planes and the plane traffic hits L2
-  const int l = blockIdx.y;
-  const int g1 = (jsplit + group - 1) / group;
-  int ja, jb;
-  if ((int)blockIdx.x < g1) {
-    ja = blockIdx.x * group;
-    jb = min(jsplit, ja + group);
-  } else {
-    ja = jsplit + (blockIdx.x - g1) * group;
-    jb = min(nth, ja + group);
-  }
-  const bool asc = ja < jsplit;
-  const float* __restrict__ sl = p + (size_t)l * n * n;
-  const int work = (jb - ja) * n;
-  for (int w = threadIdx.x; w < work; w += blockDim.x) {
-    const int j = ja + w / n, k = w % n;
-    int mlo, mhi;
-    ray_range(tabf[j], tabf[nth + j], k, n, ns, mlo, mhi);
-    racc[w] = 0.0f;
-    rm[w] = mlo;
-    rend[w] = mhi;
-  }
-  for (int bi = 0; bi < nb; ++bi) {
-    const int b = asc ? bi : nb - 1 - bi;
-    const int y_lo = b * bh;  // first row of the band
-    __syncthreads();
-    for (int yy = threadIdx.x / 32; yy < HB; yy += blockDim.x / 32) {
-      const int y = y_lo - kPad + yy;
-      for (int xx = threadIdx.x % 32; xx < W; xx += 32) {
-        const int x = xx - kPad;
-        s[yy * W + xx] =
-            (x >= 0 && y >= 0 && x < n && y < n) ? __ldg(sl + (size_t)y * n + x) : 0.0f;
-      }
-    }
-    __syncthreads();
-    // rows j0 of this band (the first and last bands take everything beyond)
-    const int jlo = b == 0 ? INT_MIN : y_lo;
-    const int jhi = b == nb - 1 ? INT_MAX : y_lo + bh;
-    for (int w = threadIdx.x; w < work; w += blockDim.x) {
-      const int j = ja + w / n, k = w % n;
-      int m = rm[w];
-      const int mhi = rend[w];
-      if (m >= mhi) continue;
-      float acc = racc[w];
-      const long long CS = tabi[j], SN = tabi[nth + j];
-      const long long u2 = 2LL * k + 1 - n, v2 = 2LL * m + 1 - ns;
-      const long long c2 = (long long)(n - 1) << 30;
-      long long GX = c2 + u2 * CS - v2 * SN;
-      long long GY = c2 + u2 * SN + v2 * CS;
-      const long long dGX = -2 * SN, dGY = 2 * CS;
-      for (; m < mhi; ++m) {
-        const int i0 = (int)(GX >> 31), j0 = (int)(GY >> 31);
-        if (j0 < jlo || j0 >= jhi) break;
-        const float fx = frac31(GX), fy = frac31(GY);
-        GX += dGX;
-        GY += dGY;
-        // buffer offset of corner (i0, j0), clamped into the buffer
-        const int jj = min(max(j0 - y_lo + kPad, 0), HB - 2);
-        const int ii = min(max(i0 + kPad, 0), n + 2 * kPad - 2);
-        const int o = jj * W + ii;
-        const float v00 = s[o], v10 = s[o + 1], v01 = s[o + W], v11 = s[o + W + 1];
-        const float r0 = fmaf(fx, v10 - v00, v00);
-        const float r1 = fmaf(fx, v11 - v01, v01);
-        acc += fmaf(fy, r1 - r0, r0);
-      }
-      racc[w] = acc;
-      rm[w] = m;
-    }
-  }
-  __syncthreads();
-  for (int w = threadIdx.x; w < work; w += blockDim.x) {
-    const int j = ja + w / n, k = w % n;
-    const size_t oo = ((size_t)j * n + l) * n + k;
-    float out = (2.0f / (float)nimg) * racc[w];
-    if (sub) out = out - sub[oo];
-    if (mask) out = out * mask[oo];
-    g[oo] = out;
-  }
-}
-
-// FP32 P by angle classes (even N, even n_angles = 2h), the forward
-// counterpart of k_backproject_quad.  The bilinear samples of theta's
-// lattice serve four angles: (1) theta's ray k is the sum over its samples m
-// ("row" k); (2) theta + 90 deg's ray k' is the sum of "column" m = k' + koff
-// (koff = (Ns - N)/2) over the lattice points k = -koff .. N + koff - 1 (its
-// samples m' = (N + Ns)/2 - 1 - k); (3) pi - theta's ray k sums the mirror
-// image x -> N-1-x of theta's row k (its sample m' is theta's Ns-1-m', so
-// only the order of the terms differs); (4) pi/2 - theta's ray k' sums that
-// mirror image's column k' + koff, by (2) applied to the pair (pi/2 - theta,
-// pi - theta).  So the lattice spans Ns x Ns points, both indices shifted to
-// 0 .. Ns-1 (kidx = k + koff): rows kidx in [koff, koff + N) and columns m in
-// [koff, koff + N) are rays.  The mirror image of a sample uses the same
-// corner row, fractions and weights, read at the mirrored columns.  Classes
-// j = 0 and 2j = h have only the pair (1), (2).
-// A CTA takes one plane and one class (several classes, one after the
-// other, when the plane fits one band and is staged once).  Warp (kg, mg)
-// owns the tiles of 32 lattice rows (lane = row) x 16 samples whose k-tile
-// is kg mod KG and m-tile mg mod MG; tiles whose samples miss the plane (or the band) are skipped, and tiles
-// whose samples all lie on it take a path without per-sample tests.  A lane's
-// running sum over a tile is its row's partial sum; the column partials of an
-// m-tile accumulate per lane over the warp's k-tiles, then one transposed
-// butterfly over the lanes gives the 16 column sums.  The owner adds both to
-// its partial sums in shared memory (rows per m-group, columns per k-group),
-// and the groups are summed at the end.  The plane is staged band by band
-// (one band when it fits) behind a zero border of 4 points, with rows of a
-// pitch = 16 mod 32 words: the 32 lanes of a load lie along theta (direct
-// image) or along its mirror, and this pitch keeps both near two wavefronts
-// per load.  A sample belongs to the band of its lower corner row j0, the
-// first and last bands taking the rows beyond.  Fixed order everywhere:
-// deterministic, no atomics.
-constexpr int kQuadMaxWarps = 16;
-constexpr int kQPad = 4;  // zero border of the staged plane (keeps rows 16-byte aligned)
-
-__host__ __device__ inline int quad_pitch(int n) {
-  const int w = n + 2 * kQPad;
-  return w + ((48 - w % 32) % 32);
-}
-
-constexpr int kQuadTM = 16;  // samples of a lattice tile (its rows: the 32 lanes)
-
-// kQuadTM samples of one lattice row per lane (the lanes: 32 consecutive rows),
-// both images; CHECK: skip the samples that do not exist or miss the plane
-// or band (else every sample is known to touch it)
-template <bool CHECK>
-__device__ __forceinline__ void quad_tile(const float* __restrict__ sb, int W, int n,
-                                          long long GX, long long GY, long long dGX,
-                                          long long dGY, bool kin, int mlim, int jmin,
-                                          unsigned jspan, float (&cv)[kQuadTM],
-                                          float (&cm)[kQuadTM], float& rt, float& rm) {
-  const int nm1 = n - 1;
-#pragma unroll
-  for (int i = 0; i < kQuadTM; ++i) {
-    const int i0 = (int)(GX >> 32), j0 = (int)(GY >> 32);
-    const unsigned lx = (unsigned)GX, ly = (unsigned)GY;
-    GX += dGX;
-    GY += dGY;
-    if (!CHECK ||
-        (kin && i < mlim && (unsigned)(j0 - jmin) <= jspan && (unsigned)(i0 + 1) <= (unsigned)n)) {
-      const float fx = __uint_as_float(0x3f800000u | (lx >> 9)) - 1.0f;
-      const float fy = __uint_as_float(0x3f800000u | (ly >> 9)) - 1.0f;
-      const float* q = sb + j0 * W;
-      const float v00 = q[i0], v10 = q[i0 + 1], v01 = q[i0 + W], v11 = q[i0 + W + 1];
-      const int im = nm1 - i0;  // the mirror column N - 1 - i0
-      const float a0 = q[im], b0 = q[im - 1], a1 = q[im + W], b1 = q[im + W - 1];
-      const float r0 = fmaf(fx, v10 - v00, v00), r1 = fmaf(fx, v11 - v01, v01);
-      const float q0 = fmaf(fx, b0 - a0, a0), q1 = fmaf(fx, b1 - a1, a1);
-      const float v = fmaf(fy, r1 - r0, r0), vm = fmaf(fy, q1 - q0, q0);
-      rt += v;
-      rm += vm;
-      cv[i] += v;
-      cm[i] += vm;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kQuadMaxWarps * 32, 1)
-    k_project_quad(const float* __restrict__ p, float* __restrict__ g,
-                   const float* __restrict__ sub, const float* __restrict__ mask,
-                   const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg, int tiles,
-                   int kg_n, int mg_n, int bh, int nb, int cpb) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int W = quad_pitch(n);
-  const int HB = bh + 2 * kQPad;  // rows of the band buffer
-  const int TW = tiles * 32;      // lattice rows (and samples) rounded up to tiles
-  float* s = reinterpret_cast<float*>(smem_raw);
-  float* rowp = s + (size_t)HB * W;             // [mg][2][TW]: row sums of both images
-  float* colp = rowp + (size_t)mg_n * 2 * TW;   // [kg][2][TW]: column sums of both images
-  const int hh = nth / 2;
-  const int ncls = nth / 4 + 1;
-  const int l = blockIdx.y;  // plane
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nthreads = blockDim.x, nwarps = nthreads / 32;
-  const int kg = warp % kg_n, mg = warp / kg_n;
-  const float* __restrict__ sl = p + (size_t)l * n * n;
-  const int koff = (ns - n) / 2;
-
-  // stage rows y_lo - 4 .. y_lo + bh + 3 of the plane (zero outside it)
-  auto stage = [&](int y_lo) {
-    if ((n & 3) == 0 && ((uintptr_t)p & 15) == 0) {
-      // rows of W / 4 float4: column 4q .. 4q+3 holds the plane's 4q-4 .. 4q-1
-      const int W4 = W / 4, n4 = n / 4;
-      for (int yy = warp; yy < HB; yy += nwarps) {
-        const int y = y_lo - kQPad + yy;
-        float4* dst = reinterpret_cast<float4*>(s + (size_t)yy * W);
-        if (y >= 0 && y < n) {
-          const float4* src = reinterpret_cast<const float4*>(sl + (size_t)y * n);
-          for (int q = lane; q < W4; q += 32)
-            dst[q] = (q >= 1 && q <= n4) ? __ldg(src + q - 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-        } else {
-          for (int q = lane; q < W4; q += 32) dst[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
-    } else {
-      for (int yy = warp; yy < HB; yy += nwarps) {
-        const int y = y_lo - kQPad + yy;
-        for (int xx = lane; xx < W; xx += 32) {
-          const int x = xx - kQPad;
-          s[yy * W + xx] =
-              (x >= 0 && y >= 0 && x < n && y < n) ? __ldg(sl + (size_t)y * n + x) : 0.0f;
-        }
-      }
-    }
-  };
-  if (nb == 1) stage(0);  // one band: staged once for all classes of the CTA
-
-  const int c1 = min(ncls, (int)(blockIdx.x + 1) * cpb);
-  for (int j = blockIdx.x * cpb; j < c1; ++j) {  // angle class: theta_j in [0, 45] degrees
-    const bool four = j != 0 && 2 * j != hh;
-    __syncthreads();  // the previous class's sums are read
-    for (int i = tid; i < (mg_n + kg_n) * 2 * TW; i += nthreads) rowp[i] = 0.0f;
-    // fixed-point coordinates at twice the scale of the other FP32 kernels
-    // (2^32 per cell): the corner index is the high word and the fraction the
-    // low word, the same corners and fraction bits as frac31 of the 2^31 form.
-    // cos, sin >= 0: x grows along the rows and falls along the samples, y
-    // grows along both, so a tile's extremes sit at known corners
-    const long long CS = 2LL * tabi[j], SN = 2LL * tabi[nth + j];
-    const long long c2 = (long long)(n - 1) << 31;
-    const long long dGX = -2 * SN, dGY = 2 * CS;
-    for (int b = 0; b < nb; ++b) {
-      const int y_lo = b * bh;
-      if (nb > 1) {
-        __syncthreads();  // the previous band's readers are done
-        stage(y_lo);
-      }
-      __syncthreads();
-      // corner rows whose samples can be nonzero and belong to this band
-      const int jmin = b == 0 ? -1 : y_lo;
-      const int jmax = b == nb - 1 ? n - 1 : min(y_lo + bh, n) - 1;
-      const unsigned jspan = (unsigned)(jmax - jmin);
-      const float* sb = s + (kQPad - y_lo) * W + kQPad;  // element (row j0, column i0)
-      const int mtiles = (ns + kQuadTM - 1) / kQuadTM;
-      for (int mt = mg; mt < mtiles; mt += mg_n) {
-        const int m0 = mt * kQuadTM;
-        const long long v2 = 2LL * m0 + 1 - ns, vb = v2 + 2 * (kQuadTM - 1);
-        const long long xa = c2 - vb * SN, xb = c2 - v2 * SN;  // x at the low / high samples
-        const long long ya = c2 + v2 * CS, yb = c2 + vb * CS;  // y at them
-        const int mlim = ns - m0;  // samples m0 + i with i < mlim exist
-        float cv[kQuadTM], cm[kQuadTM];
-#pragma unroll
-        for (int i = 0; i < kQuadTM; ++i) cv[i] = cm[i] = 0.0f;
-        bool any = false;
-        for (int kt = kg; kt < tiles; kt += kg_n) {
-          const int r0i = kt * 32;  // first lattice row of the tile
-          const long long ua = 2LL * (r0i - koff) + 1 - n, ub = ua + 62;
-          const long long xlo = (xa + ua * CS) >> 32, xhi = (xb + ub * CS) >> 32;
-          const long long ylo = (ya + ua * SN) >> 32, yhi = (yb + ub * SN) >> 32;
-          // no sample of the tile touches the plane within this band
-          if (xhi < -1 || xlo > n - 1 || yhi < jmin || ylo > jmax) continue;
-          any = true;
-          const int kidx = r0i + lane;
-          const long long u2 = ua + 2 * lane;
-          const long long GX = c2 + u2 * CS - v2 * SN;
-          const long long GY = c2 + u2 * SN + v2 * CS;
-          float rt = 0.0f, rm = 0.0f;
-          if (xlo >= -1 && xhi <= n - 1 && ylo >= jmin && yhi <= jmax && r0i + 31 < ns &&
-              mlim >= kQuadTM)
-            quad_tile<false>(sb, W, n, GX, GY, dGX, dGY, true, kQuadTM, jmin, jspan, cv, cm, rt,
-                             rm);
-          else
-            quad_tile<true>(sb, W, n, GX, GY, dGX, dGY, kidx < ns, mlim, jmin, jspan, cv, cm, rt,
-                            rm);
-          float* rp = rowp + (size_t)mg * 2 * TW + kidx;
-          rp[0] += rt;
-          rp[TW] += rm;
-        }
-        if (!any) continue;
-        // column sums over the 32 lanes: fold the lane groups above the tile
-        // length, then a transposed butterfly over the kQuadTM lanes of each
-        // group leaves the sum of sample t mod kQuadTM in lane t
-#pragma unroll
-        for (int sh = 16; sh >= kQuadTM; sh >>= 1) {
-#pragma unroll
-          for (int i = 0; i < kQuadTM; ++i) {
-            cv[i] += __shfl_xor_sync(0xffffffffu, cv[i], sh);
-            cm[i] += __shfl_xor_sync(0xffffffffu, cm[i], sh);
-          }
-        }
-#pragma unroll
-        for (int sh = kQuadTM / 2; sh >= 1; sh >>= 1) {
-          const bool up = (lane & sh) != 0;
-#pragma unroll
-          for (int i = 0; i < sh; ++i) {
-            const float sv = up ? cv[i] : cv[i + sh], kv = up ? cv[i + sh] : cv[i];
-            const float sm = up ? cm[i] : cm[i + sh], km = up ? cm[i + sh] : cm[i];
-            cv[i] = kv + __shfl_xor_sync(0xffffffffu, sv, sh);
-            cm[i] = km + __shfl_xor_sync(0xffffffffu, sm, sh);
-          }
-        }
-        if (lane < kQuadTM) {
-          float* cp = colp + (size_t)kg * 2 * TW + m0 + lane;
-          cp[0] += cv[0];
-          cp[TW] += cm[0];
-        }
-      }
-    }
-    __syncthreads();
-    const float scale = 2.0f / (float)nimg;
-    const int nout = four ? 4 : 2;
-    for (int w = tid; w < nout * n; w += nthreads) {
-      const int which = w / n, kk = w % n;
-      // row sums of theta and pi - theta; column sums of theta + 90 and pi/2 - theta
-      const bool row = which == 0 || which == 2;
-      const float* src = (row ? rowp : colp) + (which >= 2 ? TW : 0) + koff + kk;
-      const int groups = row ? mg_n : kg_n;
-      float acc = 0.0f;
-      for (int q = 0; q < groups; ++q) acc += src[(size_t)q * 2 * TW];
-      const int ang = which == 0 ? j : which == 1 ? j + hh : which == 2 ? nth - j : hh - j;
-      const size_t oo = ((size_t)ang * n + l) * n + kk;
-      float out = scale * acc;
-      if (sub) out = out - sub[oo];
-      if (mask) out = out * mask[oo];
-      g[oo] = out;
-    }
-  }
-}
-
-// P^T, voxel-driven gather (deterministic, no atomics).  For each angle the
-// voxel's position in the rotated frame, kk (detector units) and mm (sample
-// units), is split into integer and fractional parts; the samples that can
-// reach the voxel are the 3 x 3 candidates k = kb .. kb + 2, m = mb .. mb + 2
-// around it (|k - kk|, |m - mm| < sqrt 2).  Each contributes hat(a) hat(b) of
-// its offset (a, b) in the grid frame, the bilinear weight P gives the voxel;
-// a and b step by (cos, sin) and (-sin, cos) between candidates.
-template <typename T>
-__device__ __forceinline__ T hat1(T a) {
-  const T v = T(1) - fabs(a);
-  return v > T(0) ? v : T(0);
-}
-
-// FP32 hat: 1 - |a| <= 1 always, so clamping to [0, 1] is max(0, .); one
-// saturating add on the FMA pipe instead of an add and a min/max on the ALU
-__device__ __forceinline__ float hat1f(float a) { return __saturatef(1.0f - fabsf(a)); }
-template <>
-__device__ __forceinline__ float hat1<float>(float a) {
-  return hat1f(a);
-}
-
-constexpr int kAngleChunk = 1024;
-
+// ------------------------------------------------- z-innermost operands --
+// out[slab][o][i][rl] = in[o so + z sz + i], z = slab rl + r: the volume (o = y,
+// i = x) or the data (o = theta, i = xi) with z innermost, in slabs of rl planes
+// (zero past the last plane), so that the lanes of a warp read planes side by
+// side with aligned vector loads.  32 x 32 tiles through shared memory.
 template <typename T>
 __global__ void __launch_bounds__(256)
-    k_backproject2(const T* __restrict__ g, T* __restrict__ h, const T* __restrict__ scale,
-                   const double* __restrict__ tab, const float* __restrict__ tabf,
-                   const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg, T mult) {
-  __shared__ T s_cs[kAngleChunk], s_sn[kAngleChunk];
-  __shared__ int s_CS[kAngleChunk], s_SN[kAngleChunk];
-  const int ix = blockIdx.x * 32 + threadIdx.x;
-  const int iy = blockIdx.y * 8 + threadIdx.y;
-  const int l = blockIdx.z;
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  const bool in = ix < n && iy < n;
-  T acc = T(0);
-  for (int ja = 0; ja < nth; ja += kAngleChunk) {
-    const int jn = min(kAngleChunk, nth - ja);
-    __syncthreads();
-    for (int t = tid; t < jn; t += 256) {
-      if constexpr (sizeof(T) == 8) {
-        s_cs[t] = tab[ja + t];
-        s_sn[t] = tab[nth + ja + t];
-      } else {
-        s_cs[t] = tabf[ja + t];
-        s_sn[t] = tabf[nth + ja + t];
-      }
-      s_CS[t] = tabi[ja + t];
-      s_SN[t] = tabi[nth + ja + t];
-    }
-    __syncthreads();
-    if (!in) continue;
-    for (int t = 0; t < jn; ++t) {
-      const T cs = s_cs[t], sn = s_sn[t];
-      int KI, MI;
-      T fk, fm;
-      if constexpr (sizeof(T) == 8) {
-        const double X = ix - 0.5 * (n - 1), Y = iy - 0.5 * (n - 1);
-        const double kk = fma(X, cs, Y * sn) + 0.5 * (n - 1);
-        const double mm = fma(Y, cs, -X * sn) + 0.5 * (ns - 1);
-        const double fkk = floor(kk), fmm = floor(mm);
-        KI = (int)fkk;
-        MI = (int)fmm;
-        fk = kk - fkk;
-        fm = mm - fmm;
-      } else {
-        // fixed point, scale 2^31: exact integer parts, fractions to ~1e-9
-        const int X2 = 2 * ix - (n - 1), Y2 = 2 * iy - (n - 1);
-        const int CS = s_CS[t], SN = s_SN[t];
-        const long long KK = (long long)X2 * CS + (long long)Y2 * SN + ((long long)(n - 1) << 30);
-        const long long MM = (long long)Y2 * CS - (long long)X2 * SN + ((long long)(ns - 1) << 30);
-        KI = (int)(KK >> 31);
-        MI = (int)(MM >> 31);
-        fk = frac31(KK);
-        fm = frac31(MM);
-      }
-      const int hk = fk >= T(0.5) ? 1 : 0, hm = fm >= T(0.5) ? 1 : 0;
-      const int kb = KI - 1 + hk, mb = MI - 1 + hm;
-      const T du0 = T(hk - 1) - fk, dv0 = T(hm - 1) - fm;  // offsets of candidate (kb, mb)
-      const T a0 = du0 * cs - dv0 * sn, b0 = du0 * sn + dv0 * cs;
-      const bool m0 = mb >= 0 && mb < ns, m1 = mb + 1 >= 0 && mb + 1 < ns,
-                 m2 = mb + 2 >= 0 && mb + 2 < ns;
-      const T* __restrict__ row = g + ((size_t)(ja + t) * n + l) * n;
+    k_zlast(const T* __restrict__ in, T* __restrict__ out, int nz, int ni, size_t so, size_t sz,
+            int rl) {
+  __shared__ T t[32][33];
+  const size_t o = blockIdx.z;
+  const int i0 = blockIdx.x * 32, z0 = blockIdx.y * 32;
+  for (int r = threadIdx.y; r < 32; r += 8) {
+    const int z = z0 + r, i = i0 + threadIdx.x;
+    t[r][threadIdx.x] = (z < nz && i < ni) ? in[o * so + (size_t)z * sz + i] : T(0);
+  }
+  __syncthreads();
+  const int z = z0 + threadIdx.x, slab = z / rl;
+  const size_t row = ((size_t)slab * gridDim.z + o) * ni;
+  if (z >= (nz + rl - 1) / rl * rl) return;
+  for (int r = threadIdx.y; r < 32; r += 8) {
+    const int i = i0 + r;
+    if (i < ni) out[(row + i) * rl + z % rl] = t[threadIdx.x][r];
+  }
+}
+
+// The planes of one lane in a slab of 32 V C planes: C vectors of V neighbours,
+// 32 V apart.  Sums go through the packed two-lane FMA of sm_100+ in pairs.
+template <int V, int C>
+struct ZRow {
+  static constexpr int N = V * C, RL = 32 * N;
+  float v[N];
+  __device__ __forceinline__ void load(const float* q) {  // q: the lane's first plane
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int k = kb + i;
-        if (k < 0 || k >= n) continue;
-        const T ai = a0 + T(i) * cs, bi = b0 + T(i) * sn;
-        T w = T(0);
-        if (m0) w += hat1(ai) * hat1(bi);
-        if (m1) w += hat1(ai - sn) * hat1(bi + cs);
-        if (m2) w += hat1(ai - T(2) * sn) * hat1(bi + T(2) * cs);
-        acc += w * __ldg(row + k);
+    for (int c = 0; c < C; ++c) {
+      if constexpr (V == 4) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(q + c * 32 * V));
+        v[4 * c] = t.x;
+        v[4 * c + 1] = t.y;
+        v[4 * c + 2] = t.z;
+        v[4 * c + 3] = t.w;
+      } else if constexpr (V == 2) {
+        const float2 t = __ldg(reinterpret_cast<const float2*>(q + c * 32 * V));
+        v[2 * c] = t.x;
+        v[2 * c + 1] = t.y;
+      } else {
+        v[c] = __ldg(q + c * 32);
       }
     }
   }
-  if (!in) return;
-  const size_t o = ((size_t)l * n + iy) * n + ix;
-  T out = (T(2) / T(nimg)) * acc;
-  if (scale) out *= scale[o];
-  if (mult != T(1)) out *= mult;
-  h[o] = out;
-}
-
-// FP32 P^T with the angles paired as theta_j and theta_j + 90 degrees (even
-// n_angles, even N).  With equal detector and sample spacing the rays of
-// theta + 90 degrees sample exactly the points of theta's lattice: detector
-// k' = m - (Ns - N)/2 and sample m' = (N + Ns)/2 - 1 - k of the rotated angle
-// is the point (k, m) of theta, in the fixed-point coordinates of P as well
-// (the tables hold cos(theta + 90) = -sin(theta), sin(theta + 90) = cos(theta)
-// to the rounding of the angle itself).  So the 3 x 3 candidate weights w_ij
-// that a voxel gets from theta's samples serve both angles: theta's detector
-// kb + i takes the row sum over valid samples, the rotated angle's detector
-// k'(mb + j) the column sum.  Half the weight evaluations of k_backproject2.
-__global__ void __launch_bounds__(256)
-    k_backproject_pair(const float* __restrict__ g, float* __restrict__ h,
-                       const float* __restrict__ scale, const float* __restrict__ tabf,
-                       const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg,
-                       float mult) {
-  __shared__ float s_cs[kAngleChunk], s_sn[kAngleChunk];
-  __shared__ int s_CS[kAngleChunk], s_SN[kAngleChunk];
-  const int ix = blockIdx.x * 32 + threadIdx.x;
-  const int iy = blockIdx.y * 8 + threadIdx.y;
-  const int l = blockIdx.z;
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  const bool in = ix < n && iy < n;
-  const int half = nth / 2;
-  const int koff = (ns - n) / 2;       // k' = m - koff
-  const int mrot = (n + ns) / 2 - 1;   // m' = mrot - k
-  const int X2 = 2 * ix - (n - 1), Y2 = 2 * iy - (n - 1);
-  float acc = 0.0f;
-  for (int ja = 0; ja < half; ja += kAngleChunk) {
-    const int jn = min(kAngleChunk, half - ja);
-    __syncthreads();
-    for (int t = tid; t < jn; t += 256) {
-      s_cs[t] = tabf[ja + t];
-      s_sn[t] = tabf[nth + ja + t];
-      s_CS[t] = tabi[ja + t];
-      s_SN[t] = tabi[nth + ja + t];
-    }
-    __syncthreads();
-    if (!in) continue;
-    for (int t = 0; t < jn; ++t) {
-      const float cs = s_cs[t], sn = s_sn[t];
-      const int CS = s_CS[t], SN = s_SN[t];
-      const long long KK = (long long)X2 * CS + (long long)Y2 * SN + ((long long)(n - 1) << 30);
-      const long long MM = (long long)Y2 * CS - (long long)X2 * SN + ((long long)(ns - 1) << 30);
-      const int KI = (int)(KK >> 31), MI = (int)(MM >> 31);
-      const float fk = frac31(KK), fm = frac31(MM);
-      const int hk = fk >= 0.5f ? 1 : 0, hm = fm >= 0.5f ? 1 : 0;
-      const int kb = KI - 1 + hk, mb = MI - 1 + hm;
-      const float du0 = (float)(hk - 1) - fk, dv0 = (float)(hm - 1) - fm;
-      const float a0 = du0 * cs - dv0 * sn, b0 = du0 * sn + dv0 * cs;
-      // validity of theta's samples mb + jj and of the rotated angle's
-      // samples (its m' = mrot - k) as 0/1 factors
-      float mv[3], mv2[3];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        mv[q] = (unsigned)(mb + q) < (unsigned)ns ? 1.0f : 0.0f;
-        mv2[q] = (unsigned)(mrot - (kb + q)) < (unsigned)ns ? 1.0f : 0.0f;
-      }
-      float r[3] = {0.0f, 0.0f, 0.0f}, cc[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 3; ++jj) {
-          const float a = a0 + (float)i * cs - (float)jj * sn;
-          const float b = b0 + (float)i * sn + (float)jj * cs;
-          const float w = hat1f(a) * hat1f(b);
-          r[i] = fmaf(w, mv[jj], r[i]);
-          cc[jj] = fmaf(w, mv2[i], cc[jj]);
-        }
-      const float* __restrict__ row = g + ((size_t)(ja + t) * n + l) * n;
-      const float* __restrict__ row2 = g + ((size_t)(ja + t + half) * n + l) * n;
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int k = kb + i;
-        if ((unsigned)k < (unsigned)n) acc = fmaf(r[i], __ldg(row + k), acc);
-      }
-#pragma unroll
-      for (int jj = 0; jj < 3; ++jj) {
-        const int k2 = mb + jj - koff;
-        if ((unsigned)k2 < (unsigned)n) acc = fmaf(cc[jj], __ldg(row2 + k2), acc);
-      }
-    }
+  // the plane of element i within the slab
+  static __device__ __forceinline__ int plane(int lane, int i) {
+    return i / V * 32 * V + lane * V + i % V;
   }
-  if (!in) return;
-  const size_t o = ((size_t)l * n + iy) * n + ix;
-  float out = (2.0f / (float)nimg) * acc;
-  if (scale) out *= scale[o];
-  if (mult != 1.0f) out *= mult;
-  h[o] = out;
-}
-
-// The 3 x 3 candidate weights of one voxel for angle theta (fixed-point
-// frame KK, MM), reduced to row sums over theta's valid samples (r) and
-// column sums over the rotated angle's valid samples (c), with the first
-// candidate detector kb and sample mb (see k_backproject_pair).
-struct Sums3 {
-  float r[3], c[3];
-  int kb, mb;
 };
 
-// IN: the voxel lies within (N - 6) / 2 grid units of the plane's centre,
-// where every candidate detector and sample of every angle exists (its
-// rotated coordinates stay within (N - 5) / 2), so no validity factors.
-template <bool IN>
-__device__ __forceinline__ Sums3 candidate_sums(long long KK, long long MM, float cs, float sn,
-                                                int ns, int mrot) {
-  Sums3 o;
-  const int KI = (int)(KK >> 31), MI = (int)(MM >> 31);
-  const float fk = frac31(KK), fm = frac31(MM);
-  const int hk = fk >= 0.5f ? 1 : 0, hm = fm >= 0.5f ? 1 : 0;
-  o.kb = KI - 1 + hk;
-  o.mb = MI - 1 + hm;
-  const float du0 = (float)(hk - 1) - fk, dv0 = (float)(hm - 1) - fm;
-  const float a0 = du0 * cs - dv0 * sn, b0 = du0 * sn + dv0 * cs;
-  float mv[3], mv2[3];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    if (!IN) {
-      mv[q] = (unsigned)(o.mb + q) < (unsigned)ns ? 1.0f : 0.0f;
-      mv2[q] = (unsigned)(mrot - (o.kb + q)) < (unsigned)ns ? 1.0f : 0.0f;
-    }
-    o.r[q] = 0.0f;
-    o.c[q] = 0.0f;
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 3; ++jj) {
-      const float a = a0 + (float)i * cs - (float)jj * sn;
-      const float b = b0 + (float)i * sn + (float)jj * cs;
-      const float w = hat1f(a) * hat1f(b);
-      if (IN) {
-        o.r[i] += w;
-        o.c[jj] += w;
-      } else {
-        o.r[i] = fmaf(w, mv[jj], o.r[i]);
-        o.c[jj] = fmaf(w, mv2[i], o.c[jj]);
-      }
-    }
+__device__ __forceinline__ float2 ffma2(float w, float2 x, float2 a) {
+  unsigned long long r, u, p, q;
+  const float2 ww = make_float2(w, w);
+  memcpy(&u, &ww, 8);
+  memcpy(&p, &x, 8);
+  memcpy(&q, &a, 8);
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(u), "l"(p), "l"(q));
+  float2 o;
+  memcpy(&o, &r, 8);
   return o;
 }
 
-// acc += sum_i r_i row[kb + i] + sum_j c_j row2[mb + j - koff] (valid detectors)
-template <bool IN>
-__device__ __forceinline__ float apply_sums(const Sums3& s, const float* __restrict__ row,
-                                            const float* __restrict__ row2, int n, int koff,
-                                            float acc) {
+template <int N>
+struct ZAcc {
+  float2 a[N / 2 + 1];  // pairs; the last one's first lane is the odd plane
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const int k = s.kb + i;
-    if (IN || (unsigned)k < (unsigned)n) acc = fmaf(s.r[i], __ldg(row + k), acc);
+    for (int i = 0; i <= N / 2; ++i) a[i] = make_float2(0.0f, 0.0f);
   }
+  __device__ __forceinline__ void fma(float w, const float* v) {
 #pragma unroll
-  for (int jj = 0; jj < 3; ++jj) {
-    const int k2 = s.mb + jj - koff;
-    if (IN || (unsigned)k2 < (unsigned)n) acc = fmaf(s.c[jj], __ldg(row2 + k2), acc);
+    for (int i = 0; i < N / 2; ++i) a[i] = ffma2(w, make_float2(v[2 * i], v[2 * i + 1]), a[i]);
+    if constexpr (N % 2) a[N / 2].x = fmaf(w, v[N - 1], a[N / 2].x);
   }
-  return acc;
+  __device__ __forceinline__ void add(const ZAcc& o) {
+#pragma unroll
+    for (int i = 0; i <= N / 2; ++i) {
+      a[i].x += o.a[i].x;
+      a[i].y += o.a[i].y;
+    }
+  }
+  __device__ __forceinline__ float get(int i) const { return i & 1 ? a[i / 2].y : a[i / 2].x; }
+};
+
+// fraction (bits 0 .. 30 of a scale-2^31 fixed-point value) as a float
+__device__ __forceinline__ float frac31(long long v) {
+  return __uint2float_rn((unsigned)v & 0x7fffffffu) * 0x1p-31f;
 }
 
-// The angle classes of k_backproject_quad for one voxel pair (u, u').
-template <bool IN>
-__device__ __forceinline__ void bp_quad_classes(const float* __restrict__ gl, size_t rows, int n,
-                                                int nth, int ns, int hh, int nclass, int koff,
-                                                int mrot, long long X2, long long Y2,
-                                                long long ck, long long cm, bool in, int tid,
-                                                const float* __restrict__ tabf,
-                                                const int32_t* __restrict__ tabi, float* s_cs,
-                                                float* s_sn, int* s_CS, int* s_SN, float& acc_u,
-                                                float& acc_m) {
-  for (int ja = 0; ja < nclass; ja += kAngleChunk) {
-    const int jn = min(kAngleChunk, nclass - ja);
+// --------------------------------------------------------------- P, FP32 --
+// The taps of ray k (angle cs, sn in fixed point, 2^30) in row `a` of the
+// ray's major axis: weight w[t] = sum over the ray's samples of hat(major
+// distance) hat(minor distance) for the cells base .. base + 3 of the minor
+// axis.  Samples advance by at least 1/sqrt 2 along the major and at most that
+// much along the minor axis, so at most three samples touch the row and their
+// corners span at most four cells.  Coordinates are 64-bit fixed point (2^31
+// per cell; the steps along a ray are exact), inv = 1 / (major step).
+struct RowTaps {
+  float w[4];
+  int base, count;  // the nonzero taps are among base .. base + count - 1, inside the plane
+};
+__device__ __forceinline__ RowTaps row_taps(int a, int k, long long CS, long long SN, bool ymajor,
+                                            float inv, int n, int ns) {
+  const long long u2 = 2LL * k + 1 - n, v0 = 1LL - ns, c2 = (long long)(n - 1) << 30;
+  const long long X0 = c2 + u2 * CS - v0 * SN, Y0 = c2 + u2 * SN + v0 * CS;
+  const long long A0 = ymajor ? Y0 : X0, B0 = ymajor ? X0 : Y0;
+  const long long dA = ymajor ? 2 * CS : -2 * SN, dB = ymajor ? -2 * SN : 2 * CS;
+  const long long D0 = ((long long)a << 31) - A0;
+  // samples within sqrt 2 of the row's crossing (0.01 covers the float rounding
+  // of the crossing; three integers always cover the interval)
+  const int m0 = (int)ceilf(__ll2float_rn(D0) * inv - 1.4243f);
+  const long long Bm = B0 + m0 * dB;
+  RowTaps r;
+  r.base = min((int)(Bm >> 31), (int)((Bm + 2 * dB) >> 31));
+#pragma unroll
+  for (int t = 0; t < 4; ++t) r.w[t] = 0.0f;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const long long D = D0 - (m0 + s) * dA, B = Bm + s * dB;
+    float ha = __saturatef(1.0f - fabsf(__int2float_rn((int)(D >> 2)) * 0x1p-29f));
+    if ((unsigned)(m0 + s) >= (unsigned)ns) ha = 0.0f;
+    const int p = (int)(B >> 31) - r.base;
+    const float fb = frac31(B), hi = ha * fb, lo = ha * (1.0f - fb);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) r.w[t] += p == t ? lo : (p + 1 == t ? hi : 0.0f);
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    if ((unsigned)(r.base + t) >= (unsigned)n) r.w[t] = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (r.w[0] == 0.0f) {  // the first tap kept is a nonzero one
+      r.w[0] = r.w[1];
+      r.w[1] = r.w[2];
+      r.w[2] = r.w[3];
+      r.w[3] = 0.0f;
+      r.base += 1;
+    }
+  }
+  r.count = r.w[3] != 0.0f ? 4 : (r.w[2] != 0.0f ? 3 : (r.w[1] != 0.0f ? 2 : (r.w[0] != 0.0f ? 1 : 0)));
+  return r;
+}
+
+// P for all planes of a slab at once.  A CTA takes one angle, as many
+// neighbouring rays as it has warps and one slab; a warp owns a ray, a lane V C
+// planes.  Row by row of the major axis, the taps of every ray are worked out
+// into shared memory (kPRows rows at a time) and applied to all planes: two
+// broadcast shared loads, then two to four taps of C vector loads and V C / 2
+// packed FMAs.  The loads hit L1 (neighbouring rays share their cells), whose
+// 128 B a cycle are the bound for long rows, instruction issue for short ones.
+// 64 registers and 32 warps an SM: half of the loads miss L1 (every cell is new
+// to the CTA once), and more warps hid that better than fetching a row ahead
+// (192^3, 90 angles: 0.36 ms, against 0.54 with 16 warps and two rows in
+// flight).  Per standalone call, 384^3 and 180 angles: 13.0 -> 5.2 ms against
+// the plane-by-plane kernel it replaces, 256^3 and 180: 3.7 -> 1.7 ms.
+// Sums: per kPSum rows, then over those.
+constexpr int kPRows = 32;
+constexpr int kPSum = 8;
+constexpr int kPWarps = 16;
+
+template <int T, int V, int C>
+__device__ __forceinline__ void ray_taps(const float* q, long long sb, float4 w,
+                                         ZAcc<V * C>& c) {
+  ZRow<V, C> x[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t) x[t].load(q + t * sb);
+  c.fma(w.x, x[0].v);
+  if constexpr (T > 1) c.fma(w.y, x[1].v);
+  if constexpr (T > 2) c.fma(w.z, x[2].v);
+  if constexpr (T > 3) c.fma(w.w, x[3].v);
+}
+
+template <int V, int C>
+__global__ void __launch_bounds__(kPWarps * 32, 2)
+    k_project_z(const float* __restrict__ pt, float* __restrict__ g,
+                const float* __restrict__ sub, const float* __restrict__ mask,
+                const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg) {
+  constexpr int RL = ZRow<V, C>::RL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rg = blockDim.x / 32;
+  float4* w4 = reinterpret_cast<float4*>(smem_raw);            // [kPRows][rg]
+  int* xb = reinterpret_cast<int*>(w4 + (size_t)kPRows * rg);  // [kPRows][rg]: 8 base + count
+  float* stage = reinterpret_cast<float*>(smem_raw);           // [RL][rg + 1], afterwards
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int j = blockIdx.y, k0 = blockIdx.x * rg;
+  const int zbase = blockIdx.z * RL;
+  const float* __restrict__ pz = pt + (size_t)blockIdx.z * n * n * RL + lane * V;
+  const int CSi = tabi[j], SNi = tabi[nth + j];
+  const long long CS = CSi, SN = SNi;
+  const bool ymajor = abs(CSi) >= abs(SNi);
+  const float inv = 1.0f / (float)(ymajor ? 2 * CS : -2 * SN);
+  const long long sa = (long long)(ymajor ? n : 1) * RL, sb = (long long)(ymajor ? 1 : n) * RL;
+  ZAcc<V * C> total;
+  total.zero();
+  for (int a0 = 0; a0 < n; a0 += kPRows) {
+    const int rows = min(kPRows, n - a0);
     __syncthreads();
-    for (int t = tid; t < jn; t += 256) {
-      s_cs[t] = tabf[ja + t];
-      s_sn[t] = tabf[nth + ja + t];
-      s_CS[t] = tabi[ja + t];
-      s_SN[t] = tabi[nth + ja + t];
+    for (int e = tid; e < rows * rg; e += blockDim.x) {
+      const int k = k0 + e % rg;
+      RowTaps t{{0.0f, 0.0f, 0.0f, 0.0f}, 0, 0};
+      if (k < n) t = row_taps(a0 + e / rg, k, CS, SN, ymajor, inv, n, ns);
+      w4[e] = make_float4(t.w[0], t.w[1], t.w[2], t.w[3]);
+      xb[e] = t.base * 8 + t.count;
     }
     __syncthreads();
-    if (!in) continue;
+    const float* prow = pz + a0 * sa;
+#pragma unroll 1
+    for (int rs = 0; rs < rows; rs += kPSum) {
+      ZAcc<V * C> c;
+      c.zero();
+      const int re = min(rs + kPSum, rows);
+#pragma unroll 1
+      for (int r = rs; r < re; ++r, prow += sa) {
+        const int code = xb[r * rg + warp], cnt = code & 7;
+        const float4 w = w4[r * rg + warp];
+        const float* q = prow + (code >> 3) * sb;
+        if (cnt == 3)
+          ray_taps<3, V, C>(q, sb, w, c);
+        else if (cnt == 2)
+          ray_taps<2, V, C>(q, sb, w, c);
+        else if (cnt == 4)
+          ray_taps<4, V, C>(q, sb, w, c);
+        else if (cnt == 1)
+          ray_taps<1, V, C>(q, sb, w, c);
+      }
+      total.add(c);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < V * C; ++i)
+    stage[ZRow<V, C>::plane(lane, i) * (rg + 1) + warp] = total.get(i);
+  __syncthreads();
+  const float scale = 2.0f / (float)nimg;
+  for (int e = tid; e < RL * rg; e += blockDim.x) {
+    const int r = e % rg, zl = e / rg;
+    if (k0 + r >= n || zbase + zl >= n) continue;
+    const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
+    float out = scale * stage[zl * (rg + 1) + r];
+    if (sub) out = out - sub[o];
+    if (mask) out = out * mask[o];
+    g[o] = out;
+  }
+}
+
+// --------------------------------------------------------------- P, FP64 --
+// The same organisation sample by sample: per sample of a ray the four corner
+// weights, the corner cell and which corners lie in the plane go to shared
+// memory; every plane then takes four multiplications and four additions in
+// the order of the plain definition (corners outside count as zero), bit for
+// bit.  Bound by the FP64 pipe: 8 instructions a sample and plane (128^3, 90
+// angles: 14.1 -> 3.3 ms; 2.9 ms at the measured FP64 rate).
+constexpr int kP64Samples = 32;
+
+template <int V>
+__global__ void __launch_bounds__(384)
+    k_project_z64(const double* __restrict__ pt, double* __restrict__ g,
+                  const double* __restrict__ sub, const double* __restrict__ mask,
+                  const double* __restrict__ tab, const float* __restrict__ tabf, int n, int nth,
+                  int ns, int nimg, int zp, int nslab, int rg) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* wlo = reinterpret_cast<double2*>(smem_raw);               // row j0: (x0, x0 + 1)
+  double2* whi = wlo + (size_t)kP64Samples * rg;                      // row j0 + 1
+  int* at = reinterpret_cast<int*>(whi + (size_t)kP64Samples * rg);   // 16 (j0 n + i0) + corners
+  double* stage = reinterpret_cast<double*>(smem_raw);
+  __shared__ int s_lo, s_hi;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slab = warp % nslab, r0 = 2 * (warp / nslab);
+  const int j = blockIdx.y, k0 = blockIdx.x * rg;
+  const int zbase = blockIdx.z * nslab * 32 * V;
+  const int z = zbase + (slab * 32 + lane) * V;
+  const double* __restrict__ pz = pt + min(z, zp - V);
+  const double cs = tab[j], sn = tab[nth + j];
+  const double dx = 2.0 / nimg, half = nimg / 2.0, L = (double)n / nimg;
+  if (tid == 0) {
+    s_lo = INT_MAX;
+    s_hi = 0;
+  }
+  __syncthreads();
+  if (tid < rg && k0 + tid < n) {
+    int mlo, mhi;
+    ray_range(tabf[j], tabf[nth + j], k0 + tid, n, ns, mlo, mhi);
+    if (mlo < mhi) {
+      atomicMin(&s_lo, mlo);
+      atomicMax(&s_hi, mhi);
+    }
+  }
+  __syncthreads();
+  const int lo = s_lo, hi = s_hi;
+  double acc0[V], acc1[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) acc0[v] = acc1[v] = 0.0;
+  for (int ma = lo; ma < hi; ma += kP64Samples) {
+    const int ms = min(kP64Samples, hi - ma);
+    __syncthreads();
+    for (int e = tid; e < ms * rg; e += blockDim.x) {
+      const int k = k0 + e % rg;
+      int code = 0;
+      if (k < n) {
+        int i0, j0;
+        double fx, fy;
+        sample64(cs, sn, k, ma + e / rg, ns, dx, half, L, i0, j0, fx, fy);
+        const double ofx = __dsub_rn(1.0, fx), ofy = __dsub_rn(1.0, fy);
+        wlo[e] = make_double2(__dmul_rn(ofx, ofy), __dmul_rn(fx, ofy));
+        whi[e] = make_double2(__dmul_rn(ofx, fy), __dmul_rn(fx, fy));
+        const bool x0 = (unsigned)i0 < (unsigned)n, x1 = (unsigned)(i0 + 1) < (unsigned)n;
+        const bool y0 = (unsigned)j0 < (unsigned)n, y1 = (unsigned)(j0 + 1) < (unsigned)n;
+        const int in = (x0 && y0 ? 1 : 0) | (x1 && y0 ? 2 : 0) | (x0 && y1 ? 4 : 0) |
+                       (x1 && y1 ? 8 : 0);
+        if (in) code = (j0 * n + i0) * 16 + in;
+      }
+      at[e] = code;
+    }
+    __syncthreads();
+    auto sample = [&](int e, double (&acc)[V]) {
+      const int code = at[e];
+      if ((code & 15) == 0) return;  // adds an exact zero
+      const double2 wl = wlo[e], wh = whi[e];
+      const double* q = pz + (long long)(code >> 4) * zp;
+      const double* qh = q + (long long)n * zp;
+      double v[4][V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) v[0][i] = v[1][i] = v[2][i] = v[3][i] = 0.0;
+      auto load = [&](const double* p, double (&d)[V]) {
+        if constexpr (V == 1) {
+          d[0] = __ldg(p);
+        } else {
+          const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+          d[0] = t.x;
+          d[1] = t.y;
+        }
+      };
+      if (code & 1) load(q, v[0]);
+      if (code & 2) load(q + zp, v[1]);
+      if (code & 4) load(qh, v[2]);
+      if (code & 8) load(qh + zp, v[3]);
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        double b = __dmul_rn(wl.x, v[0][i]);
+        b = __dadd_rn(b, __dmul_rn(wl.y, v[1][i]));
+        b = __dadd_rn(b, __dmul_rn(wh.x, v[2][i]));
+        b = __dadd_rn(b, __dmul_rn(wh.y, v[3][i]));
+        acc[i] = __dadd_rn(acc[i], b);
+      }
+    };
+    for (int m = 0; m < ms; ++m) {
+      sample(m * rg + r0, acc0);
+      sample(m * rg + r0 + 1, acc1);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    double* s = stage + ((slab * 32 + lane) * V + v) * (rg + 1) + r0;
+    s[0] = acc0[v];
+    s[1] = acc1[v];
+  }
+  __syncthreads();
+  for (int e = tid; e < nslab * 32 * V * rg; e += blockDim.x) {
+    const int r = e % rg, zl = e / rg;
+    if (k0 + r >= n || zbase + zl >= n) continue;
+    const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
+    double out = __dmul_rn(dx, stage[zl * (rg + 1) + r]);
+    if (sub) out = out - sub[o];
+    if (mask) out = out * mask[o];
+    g[o] = out;
+  }
+}
+
+// ------------------------------------------------------------- P^T, FP32 --
+// FP32 hat: 1 - |a| <= 1 always, so clamping to [0, 1] is max(0, .); one
+// saturating add on the FMA pipe instead of an add and a min/max on the ALU
+__device__ __forceinline__ float hat1f(float a) { return __saturatef(1.0f - fabsf(a)); }
+
+// The weights a voxel gets from angle (cs, sn): its position in the rotated
+// frame, kk (detector units) and mm (sample units), in fixed point (2^31; exact
+// integer parts, fractions to ~1e-9); the candidate samples are k = kb .. kb + 2
+// and m = mb .. mb + 2 around it (|k - kk|, |m - mm| < sqrt 2), each weighted by
+// hat(a) hat(b) of its offset in the grid frame.  r[i]: the sum over the samples
+// of detector kb + i.
+__device__ __forceinline__ int voxel_sums(long long KK, long long MM, float cs, float sn, int ns,
+                                          float (&r)[3]) {
+  const int KI = (int)(KK >> 31), MI = (int)(MM >> 31);
+  const float fk = frac31(KK), fm = frac31(MM);
+  const int hk = fk >= 0.5f ? 1 : 0, hm = fm >= 0.5f ? 1 : 0;
+  const int mb = MI - 1 + hm;
+  const float du0 = (float)(hk - 1) - fk, dv0 = (float)(hm - 1) - fm;
+  const float a0 = du0 * cs - dv0 * sn, b0 = du0 * sn + dv0 * cs;
+  float mv[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) mv[q] = (unsigned)(mb + q) < (unsigned)ns ? 1.0f : 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    r[i] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float a = a0 + (float)i * cs - (float)q * sn;
+      const float b = b0 + (float)i * sn + (float)q * cs;
+      r[i] = fmaf(hat1f(a) * hat1f(b), mv[q], r[i]);
+    }
+  }
+  return KI - 1 + hk;
+}
+
+// P^T for all planes of a slab at once.  A warp owns a block of 2 x 2 voxels
+// and the slab's planes, V C a lane.  Its lanes work out the weights of eight
+// angles at a time (a lane: one voxel and angle) into the warp's part of shared
+// memory; then, angle by angle, the (at most five) detectors any of the four
+// voxels sees are loaded once and applied to all four: C vector loads and 2 V C
+// packed FMAs per detector, which balances L1 and the FMA pipe (a voxel alone
+// would load three detectors for as many multiply-adds each).  kk of the block
+// spans |cos| + |sin| =: s <= sqrt 2 and a voxel's detectors lie within s of its
+// kk: 3 s < 4.25 holds at most five.  Per standalone call, 384^3 and 180 angles:
+// 14.5 -> 2.6 ms against the plane-by-plane gather it replaces, 192^3 and 90:
+// 1.18 -> 0.38 ms.
+constexpr int kBAngles = 8;
+constexpr int kBDet = 5;
+constexpr int kBTileX = 4, kBTileY = 2;  // blocks of a CTA (8 x 4 voxels), one a warp
+constexpr size_t kBWarpBytes = kBAngles * (kBDet * 16 + 4);
+
+template <int T, int V, int C>
+__device__ __forceinline__ void block_taps(const float* q, const float4* w,
+                                           ZAcc<V * C> (&acc)[4]) {
+  ZRow<V, C> x[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t) x[t].load(q + t * ZRow<V, C>::RL);
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const float4 u = w[t];
+    acc[0].fma(u.x, x[t].v);
+    acc[1].fma(u.y, x[t].v);
+    acc[2].fma(u.z, x[t].v);
+    acc[3].fma(u.w, x[t].v);
+  }
+}
+
+template <int V, int C>
+__global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
+    k_backproject_z(const float* __restrict__ gt, float* __restrict__ h,
+                    const float* __restrict__ scale, const float* __restrict__ tabf,
+                    const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg, int tx,
+                    float mult) {
+  constexpr int RL = ZRow<V, C>::RL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x / 32;
+  float4* W = reinterpret_cast<float4*>(smem_raw) + (size_t)warp * kBAngles * kBDet;
+  int* info = reinterpret_cast<int*>(smem_raw + (size_t)warps * kBAngles * kBDet * 16) +
+              warp * kBAngles;
+  const int ty = warps / tx;  // tx x ty blocks in this CTA
+  const int x0 = 2 * (blockIdx.x * tx + warp % tx), y0 = 2 * (blockIdx.y * ty + warp / tx);
+  const int zbase = blockIdx.z * RL;
+  const float* __restrict__ gz = gt + (size_t)blockIdx.z * nth * n * RL + lane * V;
+  const long long ck = (long long)(n - 1) << 30, cm = (long long)(ns - 1) << 30;
+  // this lane's voxel and angle in the weight pass
+  const int vox = lane & 3, al = lane >> 2;
+  const long long X2 = 2 * x0 - (n - 1), Y2 = 2 * y0 - (n - 1);
+  const long long dx = 2 * (vox & 1), dy = vox & 2;
+  ZAcc<V * C> acc[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) acc[v].zero();
+  for (int ja = 0; ja < nth; ja += kBAngles) {
+    const int j = min(ja + al, nth - 1);
+    const float cs = tabf[j], sn = tabf[nth + j];
+    const long long CS = tabi[j], SN = tabi[nth + j];
+    const long long KK = X2 * CS + Y2 * SN + ck, MM = Y2 * CS - X2 * SN + cm;
+    // the first detector closer than s to the block (SN >= 0)
+    int kd = (int)((KK + min(2 * CS, 0LL) - 2 * (llabs(CS) + SN)) >> 31) + 1;
+    float r[3], w[kBDet];
+    const int p = voxel_sums(KK + dx * CS + dy * SN, MM + dy * CS - dx * SN, cs, sn, ns, r) - kd;
+    unsigned on = 0;
+#pragma unroll
+    for (int d = 0; d < kBDet; ++d) {
+      w[d] = p == d ? r[0] : (p + 1 == d ? r[1] : (p + 2 == d ? r[2] : 0.0f));
+      if ((unsigned)(kd + d) >= (unsigned)n) w[d] = 0.0f;
+      if (w[d] != 0.0f) on |= 1u << d;
+    }
+    on |= __shfl_xor_sync(0xffffffffu, on, 1);
+    on |= __shfl_xor_sync(0xffffffffu, on, 2);
+    // the detectors from the first to the last that any voxel sees
+    const int first = on ? __ffs(on) - 1 : 0, count = on ? 32 - __clz(on) - first : 0;
+    __syncwarp();
+    float* wl = reinterpret_cast<float*>(W + al * kBDet) + vox;
+#pragma unroll
+    for (int d = 0; d < kBDet; ++d)
+      if (d >= first) wl[4 * (d - first)] = w[d];
+    if (vox == 0) info[al] = (kd + first) * 8 + count;
+    __syncwarp();
+    const int jn = min(kBAngles, nth - ja);
+    const float* row = gz + (size_t)ja * n * RL;
+#pragma unroll 1
+    for (int t = 0; t < jn; ++t, row += (size_t)n * RL) {
+      const int code = info[t], cnt = code & 7;
+      const float* q = row + (long long)(code >> 3) * RL;
+      const float4* u = W + t * kBDet;
+      if (cnt == 4)
+        block_taps<4, V, C>(q, u, acc);
+      else if (cnt == 3)
+        block_taps<3, V, C>(q, u, acc);
+      else if (cnt == 5) {
+        block_taps<3, V, C>(q, u, acc);
+        block_taps<2, V, C>(q + 3 * RL, u + 3, acc);
+      } else if (cnt == 2)
+        block_taps<2, V, C>(q, u, acc);
+      else if (cnt == 1)
+        block_taps<1, V, C>(q, u, acc);
+    }
+  }
+  // through shared memory to the planes' rows, 32 planes at a time
+  const int sx = 2 * tx, nv = 4 * warps;
+  const float f = 2.0f / (float)nimg;
+  float* stage = reinterpret_cast<float*>(smem_raw);  // [32 V planes][nv + 1]
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int at = (2 * (warp / tx) + (v >> 1)) * sx + 2 * (warp % tx) + (v & 1);
+#pragma unroll
+      for (int i = 0; i < V; ++i) stage[(lane * V + i) * (nv + 1) + at] = acc[v].get(c * V + i);
+    }
+    __syncthreads();
+    for (int e = tid; e < nv * 32 * V; e += blockDim.x) {
+      const int v = e % nv, zl = e / nv;
+      const int x = blockIdx.x * sx + v % sx, y = blockIdx.y * 2 * ty + v / sx;
+      const int z = zbase + c * 32 * V + zl;
+      if (x >= n || y >= n || z >= n) continue;
+      const size_t o = ((size_t)z * n + y) * n + x;
+      float out = f * stage[zl * (nv + 1) + v];
+      if (scale) out *= scale[o];
+      if (mult != 1.0f) out *= mult;
+      h[o] = out;
+    }
+  }
+}
+
+// ------------------------------------------------------------- P^T, FP64 --
+// The same, each voxel of the block with its own three detectors: here the
+// FP64 pipe is the bound, so only nonzero weights are applied (2.3 of them a
+// voxel and angle on average) and the loads do not matter (128^3, 90 angles:
+// 32.9 -> 1.1 ms; 0.8 ms at the measured FP64 rate).
+__device__ __forceinline__ double hat1d(double a) {
+  const double v = 1.0 - fabs(a);
+  return v > 0.0 ? v : 0.0;
+}
+
+constexpr int kB64Angles = 32;
+constexpr size_t kB64WarpBytes = kB64Angles * (4 * 3 * 8 + 4 * 4);
+
+template <int V>
+__global__ void __launch_bounds__(128)
+    k_backproject_z64(const double* __restrict__ gt, double* __restrict__ h,
+                      const double* __restrict__ scale, const double* __restrict__ tab, int n,
+                      int nth, int ns, int nimg, int zp, int tb, double mult) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* W = reinterpret_cast<double*>(smem_raw) + (size_t)warp * kB64Angles * 12;
+  int* info = reinterpret_cast<int*>(smem_raw + (size_t)(blockDim.x / 32) * kB64Angles * 96) +
+              warp * kB64Angles * 4;
+  const int x0 = 2 * (blockIdx.x * tb + warp % tb), y0 = 2 * (blockIdx.y * tb + warp / tb);
+  const int zbase = blockIdx.z * 32 * V;
+  const double* __restrict__ gz = gt + min(zbase + lane * V, zp - (V < 2 ? 1 : 2));
+  const bool hi_ok = V < 4 || zbase + lane * V + 2 < zp;
+  double acc[4][V];
+#pragma unroll
+  for (int v = 0; v < 4; ++v)
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc[v][i] = 0.0;
+  for (int ja = 0; ja < nth; ja += kB64Angles) {
+    __syncwarp();
+    if (ja + lane < nth) {
+      const double cs = tab[ja + lane], sn = tab[nth + ja + lane];
+#pragma unroll 1
+      for (int v = 0; v < 4; ++v) {
+        const double X = (x0 + (v & 1)) - 0.5 * (n - 1), Y = (y0 + (v >> 1)) - 0.5 * (n - 1);
+        const double kk = fma(X, cs, Y * sn) + 0.5 * (n - 1);
+        const double mm = fma(Y, cs, -X * sn) + 0.5 * (ns - 1);
+        const double fkk = floor(kk), fmm = floor(mm);
+        const double fk = kk - fkk, fm = mm - fmm;
+        const int hk = fk >= 0.5 ? 1 : 0, hm = fm >= 0.5 ? 1 : 0;
+        const int kb = (int)fkk - 1 + hk, mb = (int)fmm - 1 + hm;
+        const double du0 = (double)(hk - 1) - fk, dv0 = (double)(hm - 1) - fm;
+        const double a0 = du0 * cs - dv0 * sn, b0 = du0 * sn + dv0 * cs;
+        int on = 0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const double ai = a0 + i * cs, bi = b0 + i * sn;
+          double w = 0.0;
+          if ((unsigned)mb < (unsigned)ns) w += hat1d(ai) * hat1d(bi);
+          if ((unsigned)(mb + 1) < (unsigned)ns) w += hat1d(ai - sn) * hat1d(bi + cs);
+          if ((unsigned)(mb + 2) < (unsigned)ns) w += hat1d(ai - 2.0 * sn) * hat1d(bi + 2.0 * cs);
+          W[(lane * 4 + v) * 3 + i] = w;
+          if (w != 0.0 && (unsigned)(kb + i) < (unsigned)n) on |= 1 << i;
+        }
+        info[lane * 4 + v] = kb * 8 + on;
+      }
+    }
+    __syncwarp();
+    const int jn = min(kB64Angles, nth - ja);
     for (int t = 0; t < jn; ++t) {
-      const int j = ja + t;
-      const float cs = s_cs[t], sn = s_sn[t];
-      const long long CS = s_CS[t], SN = s_SN[t];
-      const long long A = X2 * CS, B = Y2 * SN, C = Y2 * CS, D = X2 * SN;
-      const Sums3 su = candidate_sums<IN>(A + B + ck, C - D + cm, cs, sn, ns, mrot);
-      const Sums3 sm = candidate_sums<IN>(-A + B + ck, C + D + cm, cs, sn, ns, mrot);
-      const float* __restrict__ r0 = gl + (size_t)j * rows;         // theta_j
-      const float* __restrict__ r1 = gl + (size_t)(j + hh) * rows;  // theta_j + 90
-      acc_u = apply_sums<IN>(su, r0, r1, n, koff, acc_u);
-      acc_m = apply_sums<IN>(sm, r0, r1, n, koff, acc_m);
-      if (j != 0 && 2 * j != hh) {
-        const float* __restrict__ r2 = gl + (size_t)(nth - j) * rows;  // pi - theta_j
-        const float* __restrict__ r3 = gl + (size_t)(hh - j) * rows;   // pi/2 - theta_j
-        acc_m = apply_sums<IN>(su, r2, r3, n, koff, acc_m);
-        acc_u = apply_sums<IN>(sm, r2, r3, n, koff, acc_u);
+      const double* row = gz + (long long)(ja + t) * n * zp;
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int on = info[t * 4 + v];
+        const double* q = row + (long long)(on >> 3) * zp;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          if (on & (1 << i)) {
+            const double w = W[(t * 4 + v) * 3 + i];
+            if constexpr (V == 1) {
+              acc[v][0] = fma(w, __ldg(q + i * zp), acc[v][0]);
+            } else {
+              const double2 d = __ldg(reinterpret_cast<const double2*>(q + i * zp));
+              acc[v][0] = fma(w, d.x, acc[v][0]);
+              acc[v][1] = fma(w, d.y, acc[v][1]);
+              if constexpr (V == 4) {
+                if (hi_ok) {
+                  const double2 e = __ldg(reinterpret_cast<const double2*>(q + i * zp + 2));
+                  acc[v][2] = fma(w, e.x, acc[v][2]);
+                  acc[v][3] = fma(w, e.y, acc[v][3]);
+                }
+              }
+            }
+          }
+        }
       }
     }
   }
-}
-
-// FP32 P^T using two exact symmetries of the sample lattices (even N, even
-// n_angles = 2h).  (1) theta + 90 deg samples theta's lattice points (see
-// k_backproject_pair).  (2) pi - theta samples the mirror image x -> N-1-x of
-// theta's lattice with the sample index reversed (m -> Ns-1-m), which keeps
-// the detector index and the row sums; so the weight sums a voxel u gets at
-// theta are those its mirror u' gets at pi - theta, and (through (1) for the
-// pair pi/2 - theta, pi - theta) at pi/2 - theta with the same column sums and
-// detectors.  A thread owns u and u': for each angle class j = 1 .. h/2 with
-// 2j != h it evaluates the weights of u and u' at theta_j once and applies
-// each set to four angles {j, j + h, 2h - j, h - j}; j = 0 and j = h/2 (0 and
-// 45 degrees) have only the pair (j, j + h).  A quarter of the weight
-// evaluations of k_backproject2.  In fixed point the mirror frame is exact
-// (KK' = -X2 CS + Y2 SN + c, MM' = Y2 CS + X2 SN + c); the tables of
-// pi - theta and pi/2 - theta agree with -cos, sin and sin, cos of theta to the
-// rounding of the angles themselves.
-__global__ void __launch_bounds__(256)
-    k_backproject_quad(const float* __restrict__ g, float* __restrict__ h,
-                       const float* __restrict__ scale, const float* __restrict__ tabf,
-                       const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg,
-                       float mult) {
-  __shared__ float s_cs[kAngleChunk], s_sn[kAngleChunk];
-  __shared__ int s_CS[kAngleChunk], s_SN[kAngleChunk];
-  const int ix = blockIdx.x * 32 + threadIdx.x;  // voxel u; its mirror is n - 1 - ix
-  const int iy = blockIdx.y * 8 + threadIdx.y;
-  const int l = blockIdx.z;
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  const int nh = n / 2;
-  const bool in = ix < nh && iy < n;
-  const int hh = nth / 2;
-  const int nclass = hh / 2 + 1;        // classes j = 0 .. hh/2
-  const int koff = (ns - n) / 2;
-  const int mrot = (n + ns) / 2 - 1;
-  const long long X2 = 2 * ix - (n - 1), Y2 = 2 * iy - (n - 1);
-  const long long ck = (long long)(n - 1) << 30, cm = (long long)(ns - 1) << 30;
-  const size_t rows = (size_t)n * n;    // stride between the angles' data
-  const float* __restrict__ gl = g + (size_t)l * n;
-  // the CTA's voxels (and their mirrors) all within (N - 6) / 2 of the centre:
-  // the loop without validity tests
-  const float cc = 0.5f * (float)(n - 1);
-  const float x0 = (float)(blockIdx.x * 32), x1 = (float)min((int)blockIdx.x * 32 + 31, nh - 1);
-  const float y0 = (float)(blockIdx.y * 8), y1 = (float)min((int)blockIdx.y * 8 + 7, n - 1);
-  const float dxm = fmaxf(fabsf(x0 - cc), fabsf(x1 - cc)), dym = fmaxf(fabsf(y0 - cc), fabsf(y1 - cc));
-  const float rin = 0.5f * (float)(n - 6);
-  const bool inner = n > 6 && dxm * dxm + dym * dym <= rin * rin;
-  float acc_u = 0.0f, acc_m = 0.0f;
-  if (inner)
-    bp_quad_classes<true>(gl, rows, n, nth, ns, hh, nclass, koff, mrot, X2, Y2, ck, cm, in, tid,
-                          tabf, tabi, s_cs, s_sn, s_CS, s_SN, acc_u, acc_m);
-  else
-    bp_quad_classes<false>(gl, rows, n, nth, ns, hh, nclass, koff, mrot, X2, Y2, ck, cm, in, tid,
-                           tabf, tabi, s_cs, s_sn, s_CS, s_SN, acc_u, acc_m);
-  if (!in) return;
-  const float f = 2.0f / (float)nimg;
-  const size_t ou = ((size_t)l * n + iy) * n + ix;
-  const size_t om = ((size_t)l * n + iy) * n + (n - 1 - ix);
-  float out_u = f * acc_u, out_m = f * acc_m;
-  if (scale) {
-    out_u *= scale[ou];
-    out_m *= scale[om];
+  __syncthreads();
+  double* stage = reinterpret_cast<double*>(smem_raw);
+  const int side = 2 * tb;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const int vx = 2 * (warp % tb) + (v & 1), vy = 2 * (warp / tb) + (v >> 1);
+#pragma unroll
+    for (int i = 0; i < V; ++i) stage[(vy * side + vx) * 32 * V + lane * V + i] = acc[v][i];
   }
-  if (mult != 1.0f) {
-    out_u *= mult;
-    out_m *= mult;
+  __syncthreads();
+  for (int e = tid; e < side * side * 32 * V; e += blockDim.x) {
+    const int v = e % (side * side), zl = e / (side * side);
+    const int x = blockIdx.x * side + v % side, y = blockIdx.y * side + v / side;
+    const int z = zbase + zl;
+    if (x >= n || y >= n || z >= n) continue;
+    const size_t o = ((size_t)z * n + y) * n + x;
+    double out = (2.0 / nimg) * stage[v * 32 * V + zl];
+    if (scale) out *= scale[o];
+    if (mult != 1.0) out *= mult;
+    h[o] = out;
   }
-  h[ou] = out_u;
-  h[om] = out_m;
 }
 
 // Lambda on rows of n detectors.  A CTA computes the taps once (FP64, then
@@ -1035,24 +798,6 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// out[l][x][y] = in[l][y][x] for every plane l (32 x 32 tiles through shared memory)
-template <typename T>
-__global__ void __launch_bounds__(256) k_transpose_planes(const T* __restrict__ in,
-                                                          T* __restrict__ out, int n) {
-  __shared__ T t[32][33];
-  const size_t off = (size_t)blockIdx.z * n * n;
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int y = y0 + r, x = x0 + threadIdx.x;
-    if (x < n && y < n) t[r][threadIdx.x] = in[off + (size_t)y * n + x];
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int x = x0 + r, y = y0 + threadIdx.x;
-    if (x < n && y < n) out[off + (size_t)x * n + y] = t[threadIdx.x][r];
-  }
-}
-
 __global__ void k_debug_samples(int count, const int32_t* __restrict__ jkm, int32_t* __restrict__ ij,
                                 double* __restrict__ f, const double* __restrict__ tab, int n,
                                 int nth, int ns, int nimg) {
@@ -1072,253 +817,162 @@ __global__ void k_debug_samples(int count, const int32_t* __restrict__ jkm, int3
 
 }  // namespace
 
-static size_t project_smem_bytes(const Plan& pl) {
-  return (size_t)plane_pitch(pl.n) * (pl.n + 2 * kPad) * pl.esize;
-}
-
-// FFPAT_BACKPROJECT_QUAD=0 turns the four-angle transpose off (a comparison knob)
-static bool backproject_quad_off() {
-  static const bool off = [] {
-    const char* e = getenv("FFPAT_BACKPROJECT_QUAD");
-    return e && e[0] == '0';
-  }();
-  return off;
-}
-
-// FFPAT_BACKPROJECT_PAIR=0 turns both multi-angle transposes off: the per-angle gather runs
-static bool backproject_pair_off() {
-  static const bool off = [] {
-    const char* e = getenv("FFPAT_BACKPROJECT_PAIR");
-    return e && e[0] == '0';
-  }();
-  return off;
-}
-
-// FFPAT_PROJECT_BAND=0 turns the banded projection off (a comparison knob)
-static bool project_band_off() {
-  static const bool off = [] {
-    const char* e = getenv("FFPAT_PROJECT_BAND");
-    return e && e[0] == '0';
-  }();
-  return off;
-}
-
-// The banded projection's shape: a group of angles whose per-ray state (sum
-// and sample range) takes <= 48 KB, and bands of bh >= 16 rows, so that one
-// CTA stays within ~110 KB of shared memory (two per SM).  False if the whole
-// plane fits (the one-pass kernel) or no such band fits (global memory).
-static bool band_plan(const Plan& pl, int* group, int* bh, int* nb, size_t* sm) {
-  // FP64 projections are bound by the FP64 pipes, not by loads: measured on
-  // GB300 the banded kernel gains nothing there (656 ms either way at 384^3, 180
-  // angles) and loses at 256^3, so FP64 keeps the global-memory kernel
-  if (pl.esize != 4 || project_smem_bytes(pl) <= 200 * 1024 || project_band_off()) return false;
-  const int W = plane_pitch(pl.n);
-  int gr = 8;
-  while (gr > 1 && (size_t)gr * pl.n * (pl.esize + 8) > 48 * 1024) gr /= 2;
-  const size_t state = (size_t)gr * pl.n * (pl.esize + 8);
-  const size_t budget = 110 * 1024;
-  const long long rows =
-      state < budget ? (long long)((budget - state) / ((size_t)W * pl.esize)) - 2 * kPad : 0;
-  if (rows < 16) return false;
-  *group = gr;
-  *nb = (int)((pl.n + rows - 1) / rows);
-  *bh = (pl.n + *nb - 1) / *nb;
-  *sm = (size_t)(*bh + 2 * kPad) * W * pl.esize + state;
-  return true;
-}
-
-// FFPAT_PROJECT_QUAD=0 turns the angle-class projection off (a comparison knob)
-static bool project_quad_off() {
-  static const bool off = [] {
-    const char* e = getenv("FFPAT_PROJECT_QUAD");
-    return e && e[0] == '0';
-  }();
-  return off;
-}
-
-// Shape of the angle-class projection (FP32, even N, even angle count): a
-// lattice of `tiles` x `tiles` tiles of 32 x 32, warps kg x mg, and the plane
-// in nb bands of bh rows.  When the plane fits with the partial sums in half
-// the shared memory of an SM, one band and 2 x 4 warps (two CTAs per SM);
-// else 4 x 4 warps and bands as tall as the rest of 220 KB allows.
-constexpr size_t kQuadSmem = 220 * 1024;
-
-static bool quad_plan(const Plan& pl, int* tiles, int* kg, int* mg, int* bh, int* nb,
-                      size_t* sm, int* cpb) {
-  if (pl.esize != 4 || pl.n % 2 != 0 || pl.nth % 2 != 0 || project_quad_off()) return false;
-  const int T = (pl.ns + 31) / 32;
-  const size_t W = (size_t)quad_pitch(pl.n);
-  auto state = [&](int g1, int g2) { return (size_t)(g1 + g2) * 2 * T * 32 * 4; };
-  int KG = 2, MG = 4, rows_b = pl.n, nbands = 1;
-  size_t need = (size_t)(pl.n + 2 * kQPad) * W * 4 + state(KG, MG);
-  if (need > 110 * 1024) {
-    KG = 4;
-    MG = 4;
-    const size_t st = state(KG, MG);
-    need = (size_t)(pl.n + 2 * kQPad) * W * 4 + st;
-    if (need > kQuadSmem) {
-      const long long rows = st < kQuadSmem ? (long long)((kQuadSmem - st) / (W * 4)) - 2 * kQPad : 0;
-      if (rows < 16) return false;
-      nbands = (int)((pl.n + rows - 1) / rows);
-      rows_b = (pl.n + nbands - 1) / nbands;
-      need = (size_t)(rows_b + 2 * kQPad) * W * 4 + st;
+// Planes in a slab of a z-innermost operand.  FP64: all of them in one slab,
+// rounded up to 16 bytes.  FP32: 32 V C for one of the instantiated (V, C), the
+// one of least time for n planes, slabs x the measured cost of a slab (P + P^T
+// at 128^3, 192^3 and 384^3 with every width, in units of the 64-plane slab):
+// wider slabs share the weights and addresses among more planes, until the last
+// one is mostly idle lanes.
+static int slab_planes(int n, size_t esize) {
+  if (esize == 8) return (n + 1) / 2 * 2;
+  static const int rl[] = {32, 64, 96, 128, 160, 192, 256, 320, 384};
+  static const float cost[] = {0.85f, 1.0f, 1.14f, 1.25f, 1.4f, 1.5f, 1.85f, 2.3f, 2.7f};
+  int best = 0;
+  float best_cost = 1e30f;
+  for (int i = 0; i < 9; ++i) {
+    const float c = cost[i] * (float)((n + rl[i] - 1) / rl[i]);
+    if (c < best_cost) {
+      best = rl[i];
+      best_cost = c;
     }
   }
-  *tiles = T;
-  *kg = KG;
-  *mg = MG;
-  *bh = rows_b;
-  *nb = nbands;
-  *sm = need;
-  // one band: several classes per CTA share the staged plane, as long as the
-  // grid keeps about four CTAs per SM
-  const int ncls = pl.nth / 4 + 1;
-  int c = 1;
-  if (nbands == 1)
-    while (c < ncls && (long long)((ncls + 2 * c - 1) / (2 * c)) * pl.n >= 4LL * kNumSMs) c *= 2;
-  *cpb = c;
-  return true;
+  return best;
 }
 
-size_t project_scratch_bytes(const Plan& pl) {
-  int group, bh, nb, tl, kg, mg, cpb;
-  size_t sm;
-  if (quad_plan(pl, &tl, &kg, &mg, &bh, &nb, &sm, &cpb) || project_smem_bytes(pl) <= 200 * 1024 ||
-      band_plan(pl, &group, &bh, &nb, &sm))
-    return 0;
-  return (size_t)pl.n * pl.n * pl.n * pl.esize;
+size_t zvolume_bytes(int n, size_t esize) {
+  const size_t rl = slab_planes(n, esize);
+  return (size_t)n * n * ((n + rl - 1) / rl * rl) * esize;
+}
+size_t zdata_bytes(int n, int nth, size_t esize) {
+  const size_t rl = slab_planes(n, esize);
+  return (size_t)nth * n * ((n + rl - 1) / rl * rl) * esize;
+}
+
+template <typename T>
+static int launch_zlast(const void* in, void* out, int nz, int ni, int no, size_t so, size_t sz,
+                        int rl, cudaStream_t st) {
+  const int zn = (nz + rl - 1) / rl * rl;
+  const dim3 grid((ni + 31) / 32, (zn + 31) / 32, no);
+  k_zlast<T><<<grid, dim3(32, 8), 0, st>>>((const T*)in, (T*)out, nz, ni, so, sz, rl);
+  count_launch();
+  return check_launch("k_zlast");
+}
+
+// f(V, C) as compile-time constants for a slab of rl planes
+template <class Fn>
+static void with_slab(int rl, Fn f) {
+  switch (rl) {
+    case 32: f(std::integral_constant<int, 1>(), std::integral_constant<int, 1>()); break;
+    case 64: f(std::integral_constant<int, 2>(), std::integral_constant<int, 1>()); break;
+    case 96: f(std::integral_constant<int, 1>(), std::integral_constant<int, 3>()); break;
+    case 128: f(std::integral_constant<int, 4>(), std::integral_constant<int, 1>()); break;
+    case 160: f(std::integral_constant<int, 1>(), std::integral_constant<int, 5>()); break;
+    case 192: f(std::integral_constant<int, 2>(), std::integral_constant<int, 3>()); break;
+    case 256: f(std::integral_constant<int, 4>(), std::integral_constant<int, 2>()); break;
+    case 320: f(std::integral_constant<int, 2>(), std::integral_constant<int, 5>()); break;
+    default: f(std::integral_constant<int, 4>(), std::integral_constant<int, 3>()); break;
+  }
+}
+
+// FP64: planes per lane, of the widths 1, 2 and 4 up to vmax the one of least
+// cost (FP64 instructions, idle lanes included, plus a little per slab); the
+// wider on ties
+static int choose_v64(int n, int vmax) {
+  int best = 1;
+  float best_cost = 1e30f;
+  for (int v = 1; v <= vmax; v *= 2) {
+    const float c = ((float)v + 0.3f) * (float)((n + 32 * v - 1) / (32 * v));
+    if (c <= best_cost) {
+      best = v;
+      best_cost = c;
+    }
+  }
+  return best;
 }
 
 int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
                    const void* mask, void* scratch) {
-  {
-    // FP32, even N and angle count: one weight evaluation per four angles
-    int tl, kg, mg, bh, nb, cpb;
-    size_t sm;
-    if (quad_plan(pl, &tl, &kg, &mg, &bh, &nb, &sm, &cpb)) {
-      static std::once_flag once;
-      static cudaError_t attr = cudaSuccess;
-      std::call_once(once, [] {
-        attr = cudaFuncSetAttribute(k_project_quad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kQuadSmem);
-      });
-      if (attr != cudaSuccess) {
-        cudaGetLastError();
-        return report(FFPAT_ECUDA, "k_project_quad: %zu bytes of shared memory refused", sm);
-      }
-      const dim3 grid((pl.nth / 4 + cpb) / cpb, pl.n);
-      k_project_quad<<<grid, kg * mg * 32, sm, st>>>((const float*)p, (float*)g,
-                                                     (const float*)sub, (const float*)mask,
-                                                     pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg, tl,
-                                                     kg, mg, bh, nb, cpb);
-      count_launch();
-      return check_launch("k_project_quad");
-    }
-  }
-  const size_t smem = project_smem_bytes(pl);
-  if (smem <= 200 * 1024) {
-    // one CTA per (plane, group of 8 angles); the padded plane is read once per CTA
-    const int group = 8;
-    const dim3 grid(pl.n, (pl.nth + group - 1) / group);
-    if (pl.prec == FFPAT_FP64) {
-      static bool attr = false;
-      if (!attr) {
-        cudaFuncSetAttribute(k_project_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024);
-        attr = true;
-      }
-      k_project_smem<double><<<grid, kProjThreads, smem, st>>>((const double*)p, (double*)g,
-                                                      (const double*)sub, (const double*)mask,
-                                                      pl.tab, pl.tabf, pl.tabi, pl.n, pl.nth,
-                                                      pl.ns, pl.nimg, group);
-    } else {
-      static bool attr = false;
-      if (!attr) {
-        cudaFuncSetAttribute(k_project_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024);
-        attr = true;
-      }
-      k_project_smem<float><<<grid, kProjThreads, smem, st>>>((const float*)p, (float*)g, (const float*)sub,
-                                                     (const float*)mask, pl.tab, pl.tabf, pl.tabi,
-                                                     pl.n, pl.nth, pl.ns, pl.nimg, group);
-    }
+  const int n = pl.n, rl = slab_planes(n, pl.esize), slabs = (n + rl - 1) / rl;
+  if (!scratch) return report(FFPAT_EINVAL, "launch_project: no scratch volume");
+  const size_t nn = (size_t)n * n;
+  if (pl.prec == FFPAT_FP64) {
+    const int rc = launch_zlast<double>(p, scratch, n, n, n, (size_t)n, nn, rl, st);
+    if (rc != FFPAT_OK) return rc;
+    const int V = choose_v64(n, 2);
+    // slabs of 32 V planes, up to four of them in a CTA (they share the sample
+    // lists), two rays a warp and at most 12 warps; fewer rays a CTA while the
+    // grid would not give every SM two
+    const int vs = (n + 32 * V - 1) / (32 * V), nslab = vs < 4 ? vs : 4;
+    int rg = nslab == 1 ? 16 : (nslab == 2 ? 12 : (nslab == 3 ? 8 : 6));
+    const int zg = (vs + nslab - 1) / nslab;
+    while (rg > 4 && (n + rg - 1) / rg * (long long)pl.nth * zg < 2 * kNumSMs) rg -= 4;
+    const size_t list = (size_t)kP64Samples * rg * 36, stage = (size_t)nslab * 32 * V * (rg + 1) * 8;
+    auto kern = V == 2 ? k_project_z64<2> : k_project_z64<1>;
+    kern<<<dim3((n + rg - 1) / rg, pl.nth, zg), 32 * nslab * (rg / 2), list > stage ? list : stage,
+           st>>>((const double*)scratch, (double*)g, (const double*)sub, (const double*)mask, pl.tab,
+                 pl.tabf, n, pl.nth, pl.ns, pl.nimg, rl, nslab, rg);
     count_launch();
-    return check_launch(__func__);
+    return check_launch("k_project_z64");
   }
-  // FP32 planes too large for shared memory: band by band ...
-  int group, bh, nb;
-  size_t sm;
-  if (band_plan(pl, &group, &bh, &nb, &sm)) {
-    // angles with cos >= 0 first (the table is in increasing theta)
-    int jsplit = 0;
-    for (int j = 0; j < pl.nth; ++j)
-      if (cos((M_PI * j) / pl.nth) >= 0.0) jsplit = j + 1;
-    const int groups = (jsplit + group - 1) / group + (pl.nth - jsplit + group - 1) / group;
-    const dim3 grid(groups, pl.n);
-    cudaFuncSetAttribute(k_project_band, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_project_band<<<grid, 1024, sm, st>>>((const float*)p, (float*)g, (const float*)sub,
-                                          (const float*)mask, pl.tabf, pl.tabi, pl.n, pl.nth,
-                                          pl.ns, pl.nimg, group, jsplit, bh, nb);
-    count_launch();
-    return check_launch("k_project_band");
-  }
-  // ... else from global memory; with scratch, the steep angles read a
-  // transposed copy of the volume
-  if (scratch) {
-    const dim3 tg((pl.n + 31) / 32, (pl.n + 31) / 32, pl.n);
-    if (pl.prec == FFPAT_FP64)
-      k_transpose_planes<double><<<tg, dim3(32, 8), 0, st>>>((const double*)p, (double*)scratch,
-                                                            pl.n);
-    else
-      k_transpose_planes<float><<<tg, dim3(32, 8), 0, st>>>((const float*)p, (float*)scratch,
-                                                           pl.n);
-    count_launch();
-    if (check_launch("transpose planes") != FFPAT_OK) return FFPAT_ECUDA;
-  }
-  const dim3 block(128);
-  const dim3 grid((pl.n + 127) / 128, pl.n, pl.nth);
-  if (pl.prec == FFPAT_FP64)
-    k_project<double><<<grid, block, 0, st>>>((const double*)p, (const double*)scratch, (double*)g,
-                                              (const double*)sub, (const double*)mask, pl.tab,
-                                              pl.tabf, pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg);
-  else
-    k_project<float><<<grid, block, 0, st>>>((const float*)p, (const float*)scratch, (float*)g,
-                                             (const float*)sub, (const float*)mask, pl.tab,
-                                             pl.tabf, pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg);
+  const int rc = launch_zlast<float>(p, scratch, n, n, n, (size_t)n, nn, rl, st);
+  if (rc != FFPAT_OK) return rc;
+  // rays (warps) a CTA: fewer while the grid would not give every SM two CTAs
+  int rg = kPWarps;
+  while (rg > 4 && (n + rg - 1) / rg * (long long)pl.nth * slabs < 2 * kNumSMs) rg -= 4;
+  const size_t list = (size_t)kPRows * rg * 20, stage = (size_t)rl * (rg + 1) * 4;
+  with_slab(rl, [&](auto V, auto C) {
+    k_project_z<V.value, C.value>
+        <<<dim3((n + rg - 1) / rg, pl.nth, slabs), 32 * rg, list > stage ? list : stage, st>>>(
+            (const float*)scratch, (float*)g, (const float*)sub, (const float*)mask, pl.tabi, n,
+            pl.nth, pl.ns, pl.nimg);
+  });
   count_launch();
-  return check_launch(__func__);
+  return check_launch("k_project_z");
 }
 
 int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       double mult) {
-  const dim3 block(32, 8);
-  const dim3 grid((pl.n + 31) / 32, (pl.n + 7) / 8, pl.n);
-  if (pl.prec != FFPAT_FP64 && pl.nth % 2 == 0 && pl.n % 2 == 0 && !backproject_quad_off() &&
-      !backproject_pair_off()) {
-    const dim3 gq((pl.n / 2 + 31) / 32, (pl.n + 7) / 8, pl.n);
-    k_backproject_quad<<<gq, block, 0, st>>>((const float*)g, (float*)h, (const float*)scale,
-                                             pl.tabf, pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg,
-                                             (float)mult);
+                       void* scratch, double mult) {
+  const int n = pl.n, rl = slab_planes(n, pl.esize), slabs = (n + rl - 1) / rl;
+  if (!scratch) return report(FFPAT_EINVAL, "launch_backproject: no data scratch");
+  const size_t nn = (size_t)n * n;
+  if (pl.prec == FFPAT_FP64) {
+    const int rc = launch_zlast<double>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
+    if (rc != FFPAT_OK) return rc;
+    const int V = choose_v64(n, 4), vs = (n + 32 * V - 1) / (32 * V);
+    int tb = 2;  // tb x tb blocks of 2 x 2 voxels a CTA
+    if ((long long)((n + 3) / 4) * ((n + 3) / 4) * vs < 2 * kNumSMs) tb = 1;
+    const int side = 2 * tb, tiles = (n + side - 1) / side;
+    const size_t list = (size_t)tb * tb * kB64WarpBytes, stage = (size_t)side * side * 32 * V * 8;
+    auto kern =
+        V == 4 ? k_backproject_z64<4> : (V == 2 ? k_backproject_z64<2> : k_backproject_z64<1>);
+    kern<<<dim3(tiles, tiles, vs), 32 * tb * tb, list > stage ? list : stage, st>>>(
+        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.nth, pl.ns, pl.nimg,
+        rl, tb, mult);
     count_launch();
-    return check_launch("k_backproject_quad");
+    return check_launch("k_backproject_z64");
   }
-  if (pl.prec != FFPAT_FP64 && pl.nth % 2 == 0 && pl.n % 2 == 0 && !backproject_pair_off()) {
-    k_backproject_pair<<<grid, block, 0, st>>>((const float*)g, (float*)h, (const float*)scale,
-                                               pl.tabf, pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg,
-                                               (float)mult);
-    count_launch();
-    return check_launch("k_backproject_pair");
-  }
-  if (pl.prec == FFPAT_FP64)
-    k_backproject2<double><<<grid, block, 0, st>>>((const double*)g, (double*)h,
-                                                  (const double*)scale, pl.tab, pl.tabf,
-                                                  pl.tabi, pl.n, pl.nth, pl.ns, pl.nimg, mult);
-  else
-    k_backproject2<float><<<grid, block, 0, st>>>((const float*)g, (float*)h, (const float*)scale,
-                                                 pl.tab, pl.tabf, pl.tabi, pl.n, pl.nth, pl.ns,
-                                                 pl.nimg, (float)mult);
+  const int rc = launch_zlast<float>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
+  if (rc != FFPAT_OK) return rc;
+  // blocks of 2 x 2 voxels a CTA: neighbouring blocks share detectors in L1;
+  // fewer while the grid would not give every SM two CTAs
+  int tx = kBTileX, ty = kBTileY;
+  auto ctas = [&] {
+    return (long long)((n + 2 * tx - 1) / (2 * tx)) * ((n + 2 * ty - 1) / (2 * ty)) * slabs;
+  };
+  if (ctas() < 2 * kNumSMs) tx = 2;
+  if (ctas() < 2 * kNumSMs) ty = 1;
+  if (ctas() < 2 * kNumSMs) tx = 1;
+  const size_t list = (size_t)tx * ty * kBWarpBytes;
+  with_slab(rl, [&](auto V, auto C) {
+    const size_t stage = (size_t)32 * V.value * (4 * tx * ty + 1) * 4;
+    k_backproject_z<V.value, C.value>
+        <<<dim3((n + 2 * tx - 1) / (2 * tx), (n + 2 * ty - 1) / (2 * ty), slabs), 32 * tx * ty,
+           list > stage ? list : stage, st>>>((const float*)scratch, (float*)h, (const float*)scale,
+                                              pl.tabf, pl.tabi, n, pl.nth, pl.ns, pl.nimg, tx,
+                                              (float)mult);
+  });
   count_launch();
-  return check_launch(__func__);
+  return check_launch("k_backproject_z");
 }
 
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st, const void* mask) {

@@ -1,0 +1,50 @@
+"""P and P^T run along z in slabs of planes: the sizes where the slab width, the
+lanes' vectors or the row blocks change or have a remainder, against the oracle.
+
+Tolerances: the FP64 projection bit for bit and its transpose to 1e-12; FP32
+5e-7 relative L2, that of the other FP32 projection tests (weights to about two
+roundings, sums of at most 24 terms per eight rows and then N / 8 of those).
+"""
+import numpy as np
+import pytest
+
+import oracle.oracle as o
+from paper_1901_06503_gb300 import build_lib
+from paper_1901_06503_gb300 import ffpat as F
+from paper_1901_06503_gb300.inputs import random_data, random_volume
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_lib.build()
+    F.lib()
+
+
+def rel(a, b):
+    return float(np.linalg.norm((a - b).ravel()) / max(np.linalg.norm(b.ravel()), 1e-300))
+
+
+@pytest.mark.parametrize("n,nth", [(1, 2), (2, 3), (3, 5), (9, 4), (31, 7), (32, 5), (33, 2),
+                                   (63, 3), (65, 8), (96, 3), (97, 2), (129, 5), (160, 3),
+                                   (161, 2), (193, 3), (257, 2), (321, 3), (385, 2)])
+def test_slab_widths_fp32(n, nth):
+    prob = F.problem(n, 1.0, nth, F.FP32)
+    p, g = (a.astype(np.float32) for a in (random_volume(n, 40 + n), random_data(nth, n, 50 + n)))
+    got = F.project(prob, torch.as_tensor(p, device="cuda")).double().cpu().numpy()
+    assert rel(got, o.project(p.astype(np.float64), nth)) < 5e-7
+    got = F.backproject(prob, torch.as_tensor(g, device="cuda")).double().cpu().numpy()
+    assert rel(got, o.backproject(g.astype(np.float64), n)) < 5e-7
+
+
+@pytest.mark.parametrize("n,nth", [(1, 2), (2, 3), (3, 5), (9, 40), (31, 7), (33, 2), (64, 3),
+                                   (65, 33), (97, 2), (129, 5), (257, 2)])
+def test_slab_widths_fp64(n, nth):
+    prob = F.problem(n, 1.0, nth, F.FP64)
+    p, g = random_volume(n, 60 + n), random_data(nth, n, 70 + n)
+    got = F.project(prob, torch.as_tensor(p, device="cuda")).cpu().numpy()
+    assert np.array_equal(got, o.project(p, nth))
+    got = F.backproject(prob, torch.as_tensor(g, device="cuda")).cpu().numpy()
+    assert rel(got, o.backproject(g, n)) < 1e-12
