@@ -264,8 +264,9 @@ int ffpat_profile_read(ffpat_profile *out);
 int64_t ffpat_launch_count(void);
 
 /* Choice of leapfrog kernel (process-wide): 0 = automatic (the TMA-fed kernels
- * when N % 4 == 0 for float or N % 2 == 0 for double and all arrays are
- * 16-byte aligned -- for FP32 and FP32-Kahan the whole time loop in one
+ * where all arrays are 16-byte aligned, on copies with rows padded to 16 bytes
+ * when N % 4 != 0 for float or N % 2 != 0 for double (the differentiated
+ * operator's checkpointed loops excepted) -- for FP32 and FP32-Kahan the whole time loop in one
  * cooperative launch where its work items fit the GPU at once (N <= 128 on
  * GB300) and the stream is not capturing, else two steps per pass for
  * 128 <= N <= 1624 -- else the plain 2.5D kernel), 1 = always the plain

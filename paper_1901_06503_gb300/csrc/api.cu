@@ -81,6 +81,16 @@ int check_launch(const char* what) {
 
 static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Wave-grid rows of a multiple of 16 bytes, the TMA kernels' layout (measured
+// against the plain kernel on the rows as they are: W at 150^3 FP32-Kahan 28.6 ->
+// 13 us a step, 101^3 FP32 10.6 -> 4.1 us); grids of fewer than five points stay
+// as they are.
+static int padded_row(const Plan& pl) {
+  const int q = (int)(16 / pl.esize);
+  return (pl.nw + q - 1) / q * q;
+}
+static bool ragged(const Plan& pl) { return pl.nw >= 5 && padded_row(pl) != pl.nw; }
+
 // Validate the problem and fill the size fields of the plan.
 static int validate(const ffpat_problem* pr, Plan& pl) {
   g_err[0] = 0;
@@ -112,6 +122,11 @@ static int validate(const ffpat_problem* pr, Plan& pl) {
   pl.nw3 = (size_t)pl.nw * pl.nw * pl.nw;
   pl.nd = (size_t)pl.nth * pl.nw * pl.nw;
   pl.esize = pl.prec == FFPAT_FP64 ? 8 : 4;
+  pl.np = pl.n;
+  // rows that are no multiple of 16 bytes are padded on the wave grid, where
+  // they would otherwise rule out the TMA kernels; a requested kernel (any
+  // path but the automatic one) runs on the rows as they are
+  pl.nwp = ragged(pl) && g_stencil_path.load() == 0 ? padded_row(pl) : pl.nw;
   return FFPAT_OK;
 }
 
@@ -130,18 +145,22 @@ static size_t carve(Plan& pl, void* ws) {
     off += up256(bytes);
     return p;
   };
-  const size_t vol = pl.n3 * pl.esize, wvol = pl.nw3 * pl.esize;
+  // (the layout depends on the problem alone, not on the path that runs)
+  const bool apart = pl.pad != 0 || ragged(pl);  // the wave grid has volumes of its own
+  const size_t vol = pl.n3 * pl.esize;
+  const size_t wvol = (size_t)pl.nw * pl.nw * (ragged(pl) ? padded_row(pl) : pl.nw) * pl.esize;
   // the wave input doubles as the z-innermost operand of P, the data scratch as
   // that of P^T (rows padded to 16 bytes)
   const size_t zvol = zvolume_bytes(pl.nw, pl.esize), dat = zdata_bytes(pl.nw, pl.nth, pl.esize);
   pl.kap = take(vol);
-  pl.kapw = pl.pad ? take(wvol) : pl.kap;
+  pl.kapw = apart ? take(wvol) : pl.kap;
   for (int i = 0; i < 6; ++i) pl.s[i] = i < nstate(pl) ? take(wvol) : nullptr;
   pl.x = take(pl.pad ? vol : zvol);
   pl.v = take(vol);
-  pl.xw = pl.pad ? take(zvol) : nullptr;
-  pl.xo = pl.pad ? take(vol) : nullptr;
-  pl.xg = pl.pad ? take(wvol) : nullptr;
+  pl.xw = apart ? take(zvol > wvol ? zvol : wvol) : nullptr;
+  pl.xo = apart ? take(vol) : nullptr;
+  pl.xg = pl.pad ? take(pl.nw3 * pl.esize) : nullptr;
+  if (direct(pl)) pl.kapw = pl.kap;
   pl.r = take(dat);
   pl.r2 = take(dat);
   pl.partials = (double*)take(sizeof(double) * kNumQuant * kReduceBlocks);
@@ -229,7 +248,7 @@ static int setup_speed(Plan& pl, const void* c, cudaStream_t st) {
   pl.cmax = h3[0];
   TRY(time_steps(pl, pl.cmax, &pl.nt, &pl.dt));
   TRY(launch_kappa(wave_plan(pl), c, st));
-  if (pl.pad) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
+  if (!direct(pl)) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
   return FFPAT_OK;
 }
 
@@ -249,11 +268,14 @@ int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_
 // 15.4 / 46.9 / 135), and tie at 144^3, whose 64-wide tiles are a third empty
 constexpr int kTwoStepMinN = 128;
 
+// The kernel path of a time loop: padded rows exist only on the automatic path.
+static int stencil_path(const Plan& pl) { return pl.np != pl.n ? 0 : g_stencil_path.load(); }
+
 // Whether a three-term FP32 time loop takes two steps per pass: the rule of
 // W's own loop (TMA layout, N in the two-step kernel's range, automatic
 // choice from kTwoStepMinN or the two-step path requested)
 bool two_step_three_term(const Plan& pl, bool tma) {
-  const int path = g_stencil_path.load();
+  const int path = stencil_path(pl);
   return pl.prec == FFPAT_FP32 && tma && pl.n <= kTwoStepMaxN &&
          (path == 3 || (path == 0 && pl.n >= kTwoStepMinN));
 }
@@ -292,7 +314,7 @@ static int wave_sequence(const Plan& pl, const void* in, void* out, const void**
                          long long* nlaunch, long long* npairs, cudaStream_t st) {
   const int nt = pl.nt;
   const void* ptrs[10] = {in, out, pl.kap, pl.s[0], pl.s[1], pl.s[2], pl.s[3], pl.s[4], pl.s[5]};
-  const int path = g_stencil_path.load();
+  const int path = stencil_path(pl);
   const bool tma = path != 1 && tma_supported(pl, ptrs, 9);
   if (path >= 2 && !tma)
     return fail(FFPAT_EINVAL, "TMA stencil requested but N = %d or an array alignment rules it out",
@@ -437,7 +459,7 @@ static int run_wave(const Plan& pl, const void* in, void* out, const void** resu
   // grids that fit the GPU's CTA slots run the whole loop in one cooperative
   // launch (no graph: there is one launch to make; a caller that is capturing
   // gets the step-by-step loop)
-  const int path = g_stencil_path.load();
+  const int path = stencil_path(pl);
   const int form = pl.prec == FFPAT_FP32_KAHAN ? 1 : 0;
   if (pl.prec != FFPAT_FP64 && (path == 4 || (path == 0 && cap == cudaStreamCaptureStatusNone))) {
     const void* ptrs[5] = {in, out, pl.kap, pl.s[0], pl.s[1]};
@@ -473,8 +495,8 @@ static int run_wave(const Plan& pl, const void* in, void* out, const void** resu
     std::vector<const void*> key = {in, out, pl.kap, pl.s[0], pl.s[1], pl.s[2], pl.s[3],
                                     pl.s[4], pl.s[5], (const void*)(intptr_t)pl.nt,
                                     (const void*)(intptr_t)pl.prec,
-                                    (const void*)(intptr_t)g_stencil_path.load(),
-                                    (const void*)(intptr_t)pl.n, (const void*)(intptr_t)dev};
+                                    (const void*)(intptr_t)path, (const void*)(intptr_t)pl.n,
+                                    (const void*)(intptr_t)pl.np, (const void*)(intptr_t)dev};
     std::unique_lock<std::mutex> lk(g_graph_mu);
     int hit = -1;
     for (int i = (int)g_graphs.size() - 1; i >= 0; --i)
@@ -534,20 +556,20 @@ static int run_wave(const Plan& pl, const void* in, void* out, const void** resu
 
 
 // W E v: the wave-grid field at T of the box source v, left in a state
-// buffer returned through *pN (pad = 0: W v).
+// buffer returned through *pN (direct: W v).
 static int wave_fwd(const Plan& pl, const void* v, const void** pN, cudaStream_t st) {
-  if (pl.pad == 0) return run_wave(pl, v, nullptr, pN, st);
+  if (direct(pl)) return run_wave(pl, v, nullptr, pN, st);
   TRY(launch_embed(pl, v, pl.xw, st));
   return run_wave(wave_plan(pl), pl.xw, nullptr, pN, st);
 }
 
-// The wave-grid input buffer of wave_back (pl.x without padding).
-static void* wave_in(const Plan& pl) { return pl.pad ? pl.xw : pl.x; }
+// The wave-grid input buffer of wave_back.
+static void* wave_in(const Plan& pl) { return direct(pl) ? pl.x : pl.xw; }
 
 // E^T W x for a wave-grid x (already scaled by kappa: W^T = K^-1 W K), the
-// box result returned through *w (a state buffer, or pl.xo when padded).
+// box result returned through *w (a state buffer, or pl.xo unless direct).
 static int wave_back(const Plan& pl, const void* x, const void** w, cudaStream_t st) {
-  if (pl.pad == 0) return run_wave(pl, x, nullptr, w, st);
+  if (direct(pl)) return run_wave(pl, x, nullptr, w, st);
   const void* r = nullptr;
   TRY(run_wave(wave_plan(pl), x, nullptr, &r, st));
   TRY(launch_restrict(pl, r, pl.xo, st));
@@ -755,7 +777,7 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
   TRY(setup(problem, pl, c, ws, ws_bytes, st));
   if (!in || !out) return fail(FFPAT_EINVAL, "in or out is NULL");
   if (!transpose) {
-    if (pl.pad == 0) {
+    if (direct(pl)) {
       // out may overlap in: then the loop ends in a state buffer and is
       // copied out (a step must not write the array it reads)
       const size_t bytes = pl.n3 * pl.esize;
@@ -769,10 +791,19 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
       }
     } else {
       TRY(launch_embed(pl, in, pl.xw, st));
-      TRY(run_wave(wave_plan(pl), pl.xw, out, nullptr, st));
+      if (pl.nwp == pl.nw) {
+        TRY(run_wave(wave_plan(pl), pl.xw, out, nullptr, st));
+      } else {
+        // padded rows: the field is copied out row by row
+        const void* w = nullptr;
+        TRY(run_wave(wave_plan(pl), pl.xw, nullptr, &w, st));
+        const size_t es = pl.esize;
+        CK(cudaMemcpy2DAsync(out, pl.nw * es, w, pl.nwp * es, pl.nw * es, (size_t)pl.nw * pl.nw,
+                             cudaMemcpyDeviceToDevice, st));
+      }
     }
   } else {
-    TRY(launch_kscale(wave_plan(pl), in, wave_in(pl), true, st));
+    TRY(launch_kmul_rows(wave_plan(pl), in, pl.nw, wave_in(pl), st));
     const void* w = nullptr;
     TRY(wave_back(pl, wave_in(pl), &w, st));
     TRY(launch_kscale(pl, w, out, false, st));
@@ -793,7 +824,7 @@ static int project_alone(const ffpat_problem* problem, const void* in, void* out
   char* mem = nullptr;
   CK(cudaMallocAsync((void**)&mem, tb + zb, st));
   int rc = upload_tables(pl, mem, st);
-  const Plan wp = wave_plan(pl);
+  const Plan wp = dense_rows(wave_plan(pl));
   if (rc == FFPAT_OK)
     rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb)
                    : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb);
@@ -917,7 +948,7 @@ int ffpat_fbp(const ffpat_problem* problem, const void* G, void* out, void* ws, 
   TRY(upload_tables(pl, pl.tab, st));
   const Plan wp = wave_plan(pl);
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(wp, pl.r2, out, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(dense_rows(wp), pl.r2, out, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
   return FFPAT_OK;
 }
 
@@ -929,7 +960,7 @@ static int power_iteration_w(const Plan& pl, int iters, double* est, cudaStream_
   for (int it = 0; it < iters; ++it) {
     const void* w = nullptr;
     TRY(wave_fwd(pl, pl.v, &w, st));
-    TRY(launch_kscale(wave_plan(pl), w, wave_in(pl), true, st));
+    TRY(launch_kmul_rows(wave_plan(pl), w, pl.nwp, wave_in(pl), st));
     TRY(wave_back(pl, wave_in(pl), &w, st));
     TRY(launch_kscale(pl, w, pl.v, false, st));
     TRY(launch_dot(pl, pl.n3, pl.v, pl.v, sq, st));
@@ -976,7 +1007,7 @@ int ffpat_fb_two_step_ex(const ffpat_problem* problem, const void* c, const void
   const Plan wp = wave_plan(pl);
   void* gt = pl.pad ? pl.xg : pl.v;
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(wp, pl.r2, gt, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(dense_rows(wp), pl.r2, gt, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
   int k = 0;
   for (; k < max_iters; ++k) {
     Trace trace_it("FB iteration (Algorithm 9)");

@@ -117,17 +117,40 @@ __global__ void k_kscale(const T* __restrict__ a, T* __restrict__ out, const T* 
     out[i] = mul ? a[i] * kap[i] : a[i] / kap[i];
 }
 
-// to_wave: the wave grid (nw^3) gets the box (n^3) in its central cells and
-// zero elsewhere; else the box gets the central cells of the wave grid
+// Volumes with padded rows (n points in np elements) next to dense ones: a warp
+// a row, so no element needs a division.  kappa = q c^2 (k_kappa's arithmetic)
+// and out = a kap.
 template <typename T>
-__global__ void k_box_copy(const T* __restrict__ src, T* __restrict__ dst, int n, int nw, int pad,
-                           bool to_wave) {
-  const int m = to_wave ? nw : n;
-  const size_t len = (size_t)m * m * m;
+__global__ void __launch_bounds__(256)
+    k_rows(const T* __restrict__ a, int ap, T* __restrict__ out, const T* __restrict__ kap, int n,
+           int np, double q) {
+  const int lane = threadIdx.x & 31;
+  const int rows = n * n, step = gridDim.x * (blockDim.x / 32);
+  for (int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; r < rows; r += step) {
+    const T* ar = a + (size_t)r * ap;
+    const size_t o = (size_t)r * np;
+    for (int x = lane; x < n; x += 32) {
+      if (kap) {
+        out[o + x] = ar[x] * kap[o + x];
+      } else {
+        const double cv = (double)ar[x];
+        out[o + x] = (T)(cv * cv * q);
+      }
+    }
+  }
+}
+
+// to_wave: the wave grid (nw^3 in rows of np) gets the box (n^3) in its central
+// cells and zero elsewhere; else the box gets the central cells of the wave grid
+template <typename T>
+__global__ void k_box_copy(const T* __restrict__ src, T* __restrict__ dst, int n, int nw, int np,
+                           int pad, bool to_wave) {
+  const int mx = to_wave ? np : n, m = to_wave ? nw : n;
+  const size_t len = (size_t)mx * m * m;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % m);
-    const size_t t = i / m;
+    const int x = (int)(i % mx);
+    const size_t t = i / mx;
     const int y = (int)(t % m);
     const int z = (int)(t / m);
     if (to_wave) {
@@ -135,7 +158,7 @@ __global__ void k_box_copy(const T* __restrict__ src, T* __restrict__ dst, int n
       const bool in = bx >= 0 && by >= 0 && bz >= 0 && bx < n && by < n && bz < n;
       dst[i] = in ? src[((size_t)bz * n + by) * n + bx] : T(0);
     } else {
-      dst[i] = src[((size_t)(z + pad) * nw + (y + pad)) * nw + (x + pad)];
+      dst[i] = src[((size_t)(z + pad) * nw + (y + pad)) * np + (x + pad)];
     }
   }
 }
@@ -277,6 +300,28 @@ __global__ void __launch_bounds__(kReduceThreads)
   }
 }
 
+// the same with padded rows: w, kap, x in rows of np elements, g dense
+template <typename T>
+__global__ void __launch_bounds__(kReduceThreads)
+    k_resid_kap_rows(const T* __restrict__ w, const T* __restrict__ g, const T* __restrict__ kap,
+                     T* __restrict__ x, int n, int np, double* __restrict__ partials) {
+  double rr = 0.0;
+  const int lane = threadIdx.x & 31;
+  const int rows = n * n, step = gridDim.x * (blockDim.x / 32);
+  for (int r = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; r < rows; r += step)
+    for (int i = lane; i < n; i += 32) {
+      const size_t o = (size_t)r * np + i;
+      const T d = w[o] - g[(size_t)r * n + i];
+      x[o] = kap[o] * d;
+      rr = fma((double)d, (double)d, rr);
+    }
+  rr = block_sum(rr);
+  if (threadIdx.x == 0) {
+    partials[blockIdx.x] = rr;
+    partials[kReduceBlocks + blockIdx.x] = rr;
+  }
+}
+
 // out = (a - b) / kap   (last step of the transposed recurrence, back from kap-scaled form)
 template <typename T>
 __global__ void k_sub_div(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ kap,
@@ -333,10 +378,30 @@ int launch_speed_stats(const Plan& pl, const void* c, double* out3, cudaStream_t
   return check_launch(__func__);
 }
 
+static int rows_kernel(const Plan& pl, const void* a, int ap, void* out, const void* kap, double q,
+                       cudaStream_t st) {
+  const long long rows = (long long)pl.n * pl.n;
+  const unsigned nb = (unsigned)(rows < 8LL * 16 * kNumSMs ? (rows + 7) / 8 : 16 * kNumSMs);
+  if (pl.prec == FFPAT_FP64)
+    k_rows<double><<<nb, 256, 0, st>>>((const double*)a, ap, (double*)out, (const double*)kap, pl.n,
+                                       pl.np, q);
+  else
+    k_rows<float><<<nb, 256, 0, st>>>((const float*)a, ap, (float*)out, (const float*)kap, pl.n,
+                                      pl.np, q);
+  count_launch();
+  return check_launch(__func__);
+}
+
+int launch_kmul_rows(const Plan& pl, const void* a, int ap, void* out, cudaStream_t st) {
+  if (pl.np == pl.n && ap == pl.n) return launch_kscale(pl, a, out, true, st);
+  return rows_kernel(pl, a, ap, out, pl.kap, 0.0, st);
+}
+
 int launch_kappa(const Plan& pl, const void* c, cudaStream_t st) {
   const unsigned nb = ew_blocks(pl.n3);
   const double r = pl.dt / pl.dx;
   const double q = r * r / 12.0;
+  if (pl.np != pl.n) return rows_kernel(pl, c, pl.n, pl.kap, nullptr, q, st);
   if (pl.prec == FFPAT_FP64)
     k_kappa<double><<<nb, 256, 0, st>>>((const double*)c, (double*)pl.kap, pl.n3, q);
   else
@@ -356,13 +421,13 @@ int launch_kscale(const Plan& pl, const void* a, void* out, bool mul, cudaStream
 }
 
 static int box_copy(const Plan& pl, const void* src, void* dst, bool to_wave, cudaStream_t st) {
-  const unsigned nb = ew_blocks(to_wave ? pl.nw3 : pl.n3);
+  const unsigned nb = ew_blocks(to_wave ? (size_t)pl.nw * pl.nw * pl.nwp : pl.n3);
   if (pl.prec == FFPAT_FP64)
-    k_box_copy<double><<<nb, 256, 0, st>>>((const double*)src, (double*)dst, pl.n, pl.nw, pl.pad,
-                                           to_wave);
+    k_box_copy<double><<<nb, 256, 0, st>>>((const double*)src, (double*)dst, pl.n, pl.nw, pl.nwp,
+                                           pl.pad, to_wave);
   else
-    k_box_copy<float><<<nb, 256, 0, st>>>((const float*)src, (float*)dst, pl.n, pl.nw, pl.pad,
-                                          to_wave);
+    k_box_copy<float><<<nb, 256, 0, st>>>((const float*)src, (float*)dst, pl.n, pl.nw, pl.nwp,
+                                          pl.pad, to_wave);
   count_launch();
   return check_launch(__func__);
 }
@@ -443,12 +508,22 @@ int launch_prox_finish(const Plan& pl, void* h, const void* hn, double* dst, cud
 
 int launch_resid_kap(const Plan& pl, const void* w, const void* g, void* x, double* dst,
                      cudaStream_t st) {
-  if (pl.prec == FFPAT_FP64)
+  if (pl.np != pl.n) {
+    if (pl.prec == FFPAT_FP64)
+      k_resid_kap_rows<double><<<kReduceBlocks, kReduceThreads, 0, st>>>(
+          (const double*)w, (const double*)g, (const double*)pl.kap, (double*)x, pl.n, pl.np,
+          pl.partials);
+    else
+      k_resid_kap_rows<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
+          (const float*)w, (const float*)g, (const float*)pl.kap, (float*)x, pl.n, pl.np,
+          pl.partials);
+  } else if (pl.prec == FFPAT_FP64) {
     k_resid_kap<double><<<kReduceBlocks, kReduceThreads, 0, st>>>(
         (const double*)w, (const double*)g, (const double*)pl.kap, (double*)x, pl.n3, pl.partials);
-  else
+  } else {
     k_resid_kap<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
         (const float*)w, (const float*)g, (const float*)pl.kap, (float*)x, pl.n3, pl.partials);
+  }
   k_finalize<<<1, kReduceThreads, 0, st>>>(pl.partials, 2, dst);
   count_launch(2);
   return check_launch(__func__);

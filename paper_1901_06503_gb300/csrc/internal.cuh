@@ -25,14 +25,16 @@ struct Plan {
   int n = 0, nth = 0, ns = 0, nt = 0, prec = 0, precond = 0;
   int pad = 0, nw = 0;    // cells of padding per side; wave grid points per axis
   int nimg = 0;           // box points per axis in every view (cell size 2 / nimg)
+  int np = 0;             // row pitch of this view's volumes (elements; slices n np apart)
+  int nwp = 0;            // row pitch of the wave grid's volumes: nw, or rounded up to 16 bytes
   double T = 0, cfl = 0, dx = 0, dt = 0, cmax = 0;
   size_t n3 = 0, nd = 0, esize = 0, nw3 = 0;
   // workspace carve (device)
   void* kap = nullptr;    // kappa / 12 on the image box
-  void* kapw = nullptr;   // kappa / 12 on the wave grid (== kap without padding)
+  void* kapw = nullptr;   // kappa / 12 on the wave grid (== kap when direct())
   void* s[6] = {};        // wavefield state (wave grid): three-term p^{n-1}, p^n; increment form p, p', d, e, d', e'
-  void* xw = nullptr;     // wave-grid input of a padded W or W^T
-  void* xo = nullptr;     // image-box result of a padded W^T
+  void* xw = nullptr;     // wave-grid input of W or W^T unless direct()
+  void* xo = nullptr;     // image-box result of W^T unless direct()
   void* xg = nullptr;     // wave-grid scratch (the FBP of Algorithm 9 when padded)
   void* x = nullptr;      // image-domain scratch (adjoint input / gradient)
   void* v = nullptr;      // image-domain scratch (power iteration vector)
@@ -48,13 +50,22 @@ struct Plan {
   const double* dct_mu = nullptr;
   unsigned* sync = nullptr;    // step flags of the resident time loop (kResidentMaxItems)
 };
+// Whether a box volume is a wave-grid volume as it stands (no padding cells, no
+// padded rows), so that W runs on the caller's arrays.
+inline bool direct(const Plan& pl) { return pl.pad == 0 && pl.nwp == pl.nw; }
 // The plan as the wave kernels see it: the wave grid and its kappa.
 inline Plan wave_plan(const Plan& pl) {
   Plan w = pl;
   w.n = pl.nw;
+  w.np = pl.nwp;
   w.n3 = pl.nw3;
   w.kap = pl.kapw;
   return w;
+}
+// The same grid with dense rows (the caller's own arrays).
+inline Plan dense_rows(Plan pl) {
+  pl.np = pl.n;
+  return pl;
 }
 // bytes of the three angle tables (double, float, fixed point) for nth angles
 inline size_t table_bytes(int nth) { return (size_t)nth * 2 * (8 + 4 + 4); }
@@ -196,7 +207,6 @@ int launch_debug_samples(const Plan& pl, int count, const int32_t* jkm, int32_t*
 // fb.cu
 int launch_speed_stats(const Plan& pl, const void* c, double* out3, cudaStream_t st);
 int launch_kappa(const Plan& pl, const void* c, cudaStream_t st);
-// out[i] = a[i] * kap[i] (mul = true) or a[i] / kap[i]
 // prox.cu: prox of the gradient regulariser, (I + a D^T D)^{-1} in -> out
 // through the scratch volumes s0, s1 (in, out != s0, s1; in == out allowed).
 size_t dct_bytes(int n, size_t esize);
@@ -208,10 +218,14 @@ int launch_prox_grad(const Plan& pl, double a, const void* in, void* out, void* 
 int launch_prox_prep(const Plan& pl, const void* h, const void* w, double step, void* x,
                      cudaStream_t st, const double* step_dev = nullptr);
 int launch_prox_finish(const Plan& pl, void* h, const void* hn, double* dst, cudaStream_t st);
-// padding: box (n^3) -> wave grid (zero outside the box), and wave grid -> box
+// box (n^3) -> wave grid (zero outside the box and at the end of padded rows),
+// and wave grid -> box
 int launch_embed(const Plan& pl, const void* box, void* wave, cudaStream_t st);
 int launch_restrict(const Plan& pl, const void* wave, void* box, cudaStream_t st);
+// out[i] = a[i] * kap[i] (mul = true) or a[i] / kap[i] on dense rows
 int launch_kscale(const Plan& pl, const void* a, void* out, bool mul, cudaStream_t st);
+// out = a kap on the wave view `pl`; a has rows of `ap` elements, out of pl.np
+int launch_kmul_rows(const Plan& pl, const void* a, int ap, void* out, cudaStream_t st);
 // out[i] = a[i] * s  (s a device double)
 int launch_scale_dev(const Plan& pl, size_t len, const void* a, void* out, const double* s,
                      cudaStream_t st);
@@ -226,7 +240,7 @@ int launch_fb_update(const Plan& pl, void* h, const void* w, double step, double
                      const void* support = nullptr);
 int launch_inv_sqrt(const double* src, double* dst, cudaStream_t st);
 int launch_sub_div(const Plan& pl, const void* a, const void* b, void* out, cudaStream_t st);
-// x = kap (w - g), dst[0] = dst[1] = sum (w - g)^2
+// x = kap (w - g), dst[0] = dst[1] = sum (w - g)^2; w, x have rows of pl.np, g of pl.n
 int launch_resid_kap(const Plan& pl, const void* w, const void* g, void* x, double* dst,
                      cudaStream_t st);
 int launch_scale_div(const Plan& pl, const void* a, const void* c, double s, void* out,

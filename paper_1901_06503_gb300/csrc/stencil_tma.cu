@@ -301,7 +301,7 @@ __device__ __forceinline__ void issue_round(const Maps& maps, T* pst, T* qst, ui
 template <typename T, int FORM, bool START, int RPT>
 __global__ void __launch_bounds__(NTX* NTY, 2)
     k_step_tma(const __grid_constant__ Maps maps, T* __restrict__ o0, T* __restrict__ o1,
-               T* __restrict__ o2, int n, int zc, int tiles_x, int tiles_y, int nitems) {
+               T* __restrict__ o2, int n, int np, int zc, int tiles_x, int tiles_y, int nitems) {
   using G = Geo<T, RPT>;
   constexpr int NQ = Streams<T, FORM, START>::NQ;
   extern __shared__ unsigned char smem_raw[];
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(NTX* NTY, 2)
   if (*(volatile unsigned*)&g_tma_status != 0u) return;
   __syncthreads();
   unsigned phase = 0;  // one parity bit per barrier slot
-  const size_t plane = (size_t)n * n;
+  const size_t plane = (size_t)n * np;
 
   for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
     const int tix = item % tiles_x;
@@ -375,13 +375,13 @@ __global__ void __launch_bounds__(NTX* NTY, 2)
             const float w = START ? 0.5f : 1.0f;
             const float2 wu = mul2(make_float2(w, w), lds2(Q + qo));
             if (x < n && y < n)
-              *reinterpret_cast<float2*>(o0 + (size_t)z * plane + (size_t)y * n + x) =
+              *reinterpret_cast<float2*>(o0 + (size_t)z * plane + (size_t)y * np + x) =
                   fma2(wu, L, lds2(Q + QS + qo));
             continue;
           }
           const float2 K = lds2(Q + (NQ - 1) * QS + qo);
-          if (x < n && y < n) {  // N is even, so x + 1 < n as well
-            const size_t gi = (size_t)z * plane + (size_t)y * n + x;
+          if (x < n && y < n) {  // np is even: x + 1 is in the row, if only in its padding
+            const size_t gi = (size_t)z * plane + (size_t)y * np + x;
             if constexpr (FORM == 0) {
               if constexpr (START) {
                 *reinterpret_cast<float2*>(o0 + gi) = start_pair(v.c, K, L);
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(NTX* NTY, 2)
             const T c = P0[o];
             const T k = Q[(NQ - 1) * (G::QBYTES / sizeof(T)) + qo];
             if (x < n && y < n) {
-              const size_t gi = (size_t)z * plane + (size_t)y * n + x;
+              const size_t gi = (size_t)z * plane + (size_t)y * np + x;
               if constexpr (START) {
                 o0[gi] = c + T(0.5) * k * L;
                 if (o1) o1[gi] = c;
@@ -683,19 +683,19 @@ struct Step2Item {
   float* o0;
   float* o1;
   float* o2;
-  int n, x0, y0, z0, z1;
+  int n, np, x0, y0, z0, z1;
 };
 
 // a single problem: items are (tile, z-range) in x, y, z order
 struct Step2One {
   const Maps2* maps;
   float *o0, *o1, *o2;
-  int n, zc, tiles_x, tiles_y;
+  int n, np, zc, tiles_x, tiles_y;
   __device__ Step2Item operator()(int item) const {
     const int tix = item % tiles_x;
     const int tiy = (item / tiles_x) % tiles_y;
     const int z0 = (item / (tiles_x * tiles_y)) * zc;
-    return Step2Item{maps, o0, o1, o2, n, tix * TBX, tiy * tb2::TH2, z0, min(n, z0 + zc)};
+    return Step2Item{maps, o0, o1, o2, n, np, tix * TBX, tiy * tb2::TH2, z0, min(n, z0 + zc)};
   }
 };
 
@@ -756,7 +756,7 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
     float* __restrict__ o1 = it.o1;
     float* __restrict__ o2 = it.o2;
     const int n = it.n, x0 = it.x0, y0 = it.y0, z0 = it.z0, z1 = it.z1;
-    const unsigned plane = (unsigned)n * (unsigned)n;
+    const unsigned plane = (unsigned)n * (unsigned)it.np;
     // iteration i computes step A at plane z0 - 2 + i and step B at z0 - 4 + i;
     // round r brings plane z0 - 4 + r of p^n (for r <= M + 3) and of the
     // streams (for 2 <= r <= M + 1)
@@ -810,10 +810,10 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
       float2 a0 = zero, a1 = zero, a2 = zero, a3 = zero;
       float2 uq0 = zero, uq1 = zero, vq0 = zero, vq1 = zero, kq0 = zero, kq1 = zero;
       const int x = x0 + 2 * lane, y = y0 + warp;
-      const bool store = inner && x < n && y < n;  // N % 4 == 0: x + 1 < n as well
+      const bool store = inner && x < n && y < n;  // np % 4 == 0: x + 1 is in the row as well
       // offset of plane z0 - 4 + i (unsigned arithmetic: early values wrap and are
       // unused; N <= kTwoStepMaxN keeps every used offset below 2^32)
-      unsigned gi = (unsigned)z0 * plane + (unsigned)y * (unsigned)n + (unsigned)x - 4u * plane;
+      unsigned gi = (unsigned)z0 * plane + (unsigned)y * (unsigned)it.np + (unsigned)x - 4u * plane;
       for (int ib = 0; ib < M; ib += RING) {
 #pragma unroll
         for (int u = 0; u < RING; ++u) {
@@ -932,15 +932,15 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
 
 __global__ void __launch_bounds__(tb2::NT2, 1)
     k_step2_kahan(const __grid_constant__ Maps2 maps, float* __restrict__ po,
-                  float* __restrict__ dout, float* __restrict__ eout, int n, int zc, int tiles_x,
-                  int tiles_y, int nitems) {
-  step2_body<1>(Step2One{&maps, po, dout, eout, n, zc, tiles_x, tiles_y}, nitems);
+                  float* __restrict__ dout, float* __restrict__ eout, int n, int np, int zc,
+                  int tiles_x, int tiles_y, int nitems) {
+  step2_body<1>(Step2One{&maps, po, dout, eout, n, np, zc, tiles_x, tiles_y}, nitems);
 }
 
 __global__ void __launch_bounds__(tb2::NT2, 1)
     k_step2_f32(const __grid_constant__ Maps2 maps, float* __restrict__ o1,
-                float* __restrict__ o2, int n, int zc, int tiles_x, int tiles_y, int nitems) {
-  step2_body<0>(Step2One{&maps, o1, o2, nullptr, n, zc, tiles_x, tiles_y}, nitems);
+                float* __restrict__ o2, int n, int np, int zc, int tiles_x, int tiles_y, int nitems) {
+  step2_body<0>(Step2One{&maps, o1, o2, nullptr, n, np, zc, tiles_x, tiles_y}, nitems);
 }
 
 // ---- two FP32-Kahan steps per pass for several problems in one launch
@@ -966,7 +966,7 @@ struct Step2Batch {
     while (item >= bp->item_end[r]) ++r;
     const Batch2Req& q = bp->r[r];
     const int local = item - (r ? bp->item_end[r - 1] : 0);
-    return Step2One{&q.maps, q.o0, q.o1, q.o2, q.n, q.zc, q.tiles_x, q.tiles_y}(local);
+    return Step2One{&q.maps, q.o0, q.o1, q.o2, q.n, q.n, q.zc, q.tiles_x, q.tiles_y}(local);
   }
 };
 
@@ -1011,7 +1011,7 @@ struct ResParams {
   float* buf[2];      // step s writes buf[s & 1] ...
   float* out;         // ... except the last step, which writes here when non-null
   unsigned* sync;     // one step flag per work item, zero at launch
-  int n, zc, tiles_x, tiles_y, nt;
+  int n, np, zc, tiles_x, tiles_y, nt;
 };
 
 // Step boundary of the resident loop, point to point: a CTA publishes that
@@ -1072,7 +1072,7 @@ __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uin
                                          unsigned parity, float2 (&sa)[rs::ZM][2],
                                          float2 (&sb)[rs::ZM], float2* __restrict__ es,
                                          float* __restrict__ dst,
-                                         int n, int nz, int z0, int x0, int y0) {
+                                         int n, int np, int nz, int z0, int x0, int y0) {
   using G = rs::G;
   const int tx = threadIdx.x, ty = threadIdx.y;
   bool ok = true;
@@ -1080,10 +1080,12 @@ __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uin
   for (int i = 0; i < 4; ++i)
     if (ok) ok = mbar_wait(&bar[i], parity, kWaitCycles);
   const int xl = 2 * tx, x = x0 + xl;
+  const unsigned plane = (unsigned)(n * np);  // small grids: 32-bit offsets
 #pragma unroll
   for (int rr = 0; rr < 2; ++rr) {
     const int ry = ty + TBY * rr, y = y0 + ry;
     const int o = (ry + 2) * G::BXH + xl + G::XH;
+    const unsigned o0 = (unsigned)z0 * plane + (unsigned)(y * np + x);
     float2 c0 = lds2(pst + o), c1 = lds2(pst + rs::PF + o);
     float2 c2 = lds2(pst + 2 * rs::PF + o), c3 = lds2(pst + 3 * rs::PF + o);
 #pragma unroll
@@ -1124,8 +1126,8 @@ __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uin
           w = START ? start_pair(v.c, K, L) : three_term_pair(v.c, K, L, sa[zi][rr]);
           sa[zi][rr] = v.c;
         }
-        if (x < n && y < n)  // N % 4 == 0, so x + 1 < n as well
-          *reinterpret_cast<float2*>(dst + (size_t)(z0 + zi) * n * n + (size_t)y * n + x) = w;
+        if (x < n && y < n)  // np % 4 == 0: x + 1 is in the row as well
+          *reinterpret_cast<float2*>(dst + (o0 + (unsigned)zi * plane)) = w;
         c0 = c1;
         c1 = c2;
         c2 = c3;
@@ -1194,8 +1196,8 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_wave_resident(const __grid_cons
       tma_load_3d(pst + tid * rs::PF, src, x0 - G::XH, y0 - 2, z0 - 2 + tid, &bar[tid]);
     }
     const unsigned parity = (unsigned)s & 1u;
-    ok = s == 0 ? res_step<FORM, true>(pst, kst, bar, parity, sa, sb, es, dst, n, nz, z0, x0, y0)
-                : res_step<FORM, false>(pst, kst, bar, parity, sa, sb, es, dst, n, nz, z0, x0, y0);
+    ok = s == 0 ? res_step<FORM, true>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz, z0, x0, y0)
+                : res_step<FORM, false>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz, z0, x0, y0);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
@@ -1229,9 +1231,9 @@ std::once_flag g_encode_once;
 
 struct MapKey {
   const void* ptr;
-  int n, esize, bx, by;
+  int n, np, esize, bx, by;
   bool operator==(const MapKey& o) const {
-    return ptr == o.ptr && n == o.n && esize == o.esize && bx == o.bx && by == o.by;
+    return ptr == o.ptr && n == o.n && np == o.np && esize == o.esize && bx == o.bx && by == o.by;
   }
 };
 struct MapKeyHash {
@@ -1241,17 +1243,19 @@ struct MapKeyHash {
   }
 };
 
-int make_map_box(CUtensorMap* m, const void* base, int n, int esize, int bx, int by);
+int make_map_box(CUtensorMap* m, const void* base, int n, int np, int esize, int bx, int by);
 
 // the single-step kernels' boxes: p^n with the two-point halo, or the bare tile
-int make_map(CUtensorMap* m, const void* base, int n, int esize, bool halo, int th = TBY) {
+int make_map(CUtensorMap* m, const void* base, int n, int np, int esize, bool halo, int th = TBY) {
   const int xh = 16 / esize;
-  return make_map_box(m, base, n, esize, halo ? TBX + 2 * xh : TBX, halo ? th + 4 : th);
+  return make_map_box(m, base, n, np, esize, halo ? TBX + 2 * xh : TBX, halo ? th + 4 : th);
 }
 
-int make_map_box(CUtensorMap* m, const void* base, int n, int esize, int bx, int by) {
+// an n^3 volume in rows of np elements: the tensor is n wide, so TMA fills the
+// rows' padding with zeros like everything else outside the grid
+int make_map_box(CUtensorMap* m, const void* base, int n, int np, int esize, int bx, int by) {
   static thread_local std::unordered_map<MapKey, CUtensorMap, MapKeyHash> cache;
-  const MapKey key{base, n, esize, bx, by};
+  const MapKey key{base, n, np, esize, bx, by};
   auto it = cache.find(key);
   if (it != cache.end()) {
     *m = it->second;
@@ -1267,7 +1271,7 @@ int make_map_box(CUtensorMap* m, const void* base, int n, int esize, int bx, int
   });
   if (!g_encode) return FFPAT_ECUDA;
   cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)n};
-  cuuint64_t strides[2] = {(cuuint64_t)n * esize, (cuuint64_t)n * n * esize};
+  cuuint64_t strides[2] = {(cuuint64_t)np * esize, (cuuint64_t)n * np * esize};
   cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = g_encode(
@@ -1395,7 +1399,7 @@ int launch_one(const Plan& pl, const Maps& maps, void* o0, void* o1, void* o2, c
   const int nitems = tiles_x * tiles_y * zchunks;
   const int grid = nitems < slots ? nitems : slots;
   const cudaError_t e =
-      launch_pdl(kern, dim3(grid), dim3(NTX, NTY), smem, st, maps, (T*)o0, (T*)o1, (T*)o2, n, zc,
+      launch_pdl(kern, dim3(grid), dim3(NTX, NTY), smem, st, maps, (T*)o0, (T*)o1, (T*)o2, n, pl.np, zc,
                  tiles_x, tiles_y, nitems);
   count_launch();
   if (e != cudaSuccess) {
@@ -1408,7 +1412,7 @@ int launch_one(const Plan& pl, const Maps& maps, void* o0, void* o1, void* o2, c
 }  // namespace
 
 bool tma_supported(const Plan& pl, const void* const* ptrs, int count) {
-  if (pl.esize == 4 ? (pl.n % 4) : (pl.n % 2)) return false;
+  if (pl.esize == 4 ? (pl.np % 4) : (pl.np % 2)) return false;
   for (int i = 0; i < count; ++i)
     if (ptrs[i] && ((uintptr_t)ptrs[i] & 15)) return false;
   return true;
@@ -1432,11 +1436,11 @@ static int launch_step_tma_r(const Plan& pl, int form, bool start, const void* p
   Maps maps;
   const int es = (int)pl.esize;
   const int th = TBY * RPT;
-  if (make_map(&maps.p, p, pl.n, es, true, th) != FFPAT_OK) return check_launch("tensor map (p)");
+  if (make_map(&maps.p, p, pl.n, pl.np, es, true, th) != FFPAT_OK) return check_launch("tensor map (p)");
   const int nq = form == 2 ? 2 : (start ? 1 : (form == 0 ? 2 : 3));
   for (int i = 0; i < 3; ++i) {
     if (i < nq) {
-      if (make_map(&maps.q[i], q[i], pl.n, es, false, th) != FFPAT_OK)
+      if (make_map(&maps.q[i], q[i], pl.n, pl.np, es, false, th) != FFPAT_OK)
         return check_launch("tensor map (q)");
     } else {
       maps.q[i] = maps.p;
@@ -1483,12 +1487,12 @@ int launch_step_batch(const BatchStep* steps, int count, cudaStream_t st) {
   for (int i = 0; i < count; ++i) {
     const BatchStep& b = steps[i];
     BatchReq& r = bp.r[i];
-    if (make_map(&r.p, b.p, b.n, 4, true, G::TH) != FFPAT_OK ||
-        make_map(&r.q[2], b.kap, b.n, 4, false, G::TH) != FFPAT_OK)
+    if (make_map(&r.p, b.p, b.n, b.n, 4, true, G::TH) != FFPAT_OK ||
+        make_map(&r.q[2], b.kap, b.n, b.n, 4, false, G::TH) != FFPAT_OK)
       return report(FFPAT_ECUDA, "batched step: tensor map");
     if (!b.start) {
-      if (make_map(&r.q[0], b.d, b.n, 4, false, G::TH) != FFPAT_OK ||
-          make_map(&r.q[1], b.e, b.n, 4, false, G::TH) != FFPAT_OK)
+      if (make_map(&r.q[0], b.d, b.n, b.n, 4, false, G::TH) != FFPAT_OK ||
+          make_map(&r.q[1], b.e, b.n, b.n, 4, false, G::TH) != FFPAT_OK)
         return report(FFPAT_ECUDA, "batched step: tensor map");
     } else {
       r.q[0] = r.q[2];
@@ -1557,7 +1561,7 @@ int launch_step2(Kern kern, size_t smem_need, const char* name, const Plan& pl, 
   const int nitems = tiles_x * tiles_y * zchunks;
   const int grid = nitems < slots ? nitems : slots;
   const cudaError_t le = launch_pdl(kern, dim3(grid), dim3(tb2::NT2), smem, st, maps, outs..., n,
-                                    zc, tiles_x, tiles_y, nitems);
+                                    pl.np, zc, tiles_x, tiles_y, nitems);
   count_launch();
   if (le != cudaSuccess) {
     cudaGetLastError();
@@ -1571,10 +1575,10 @@ int launch_step2_kahan(const Plan& pl, const void* p, const void* d, const void*
   if (pl.n > kTwoStepMaxN)
     return report(FFPAT_EINVAL, "two-step pass: N = %d > %d (32-bit offsets)", pl.n, kTwoStepMaxN);
   Maps2 maps;
-  if (make_map_box(&maps.p, p, pl.n, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
-      make_map_box(&maps.q[0], d, pl.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
-      make_map_box(&maps.q[1], e, pl.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
-      make_map_box(&maps.q[2], pl.kap, pl.n, 4, tb2::QW, tb2::QH) != FFPAT_OK)
+  if (make_map_box(&maps.p, p, pl.n, pl.np, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
+      make_map_box(&maps.q[0], d, pl.n, pl.np, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
+      make_map_box(&maps.q[1], e, pl.n, pl.np, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
+      make_map_box(&maps.q[2], pl.kap, pl.n, pl.np, 4, tb2::QW, tb2::QH) != FFPAT_OK)
     return report(FFPAT_ECUDA, "two-step kernel: tensor map");
   return launch_step2(k_step2_kahan, tb2::smem_bytes<1>(), "k_step2_kahan", pl, maps, st,
                       (float*)po, (float*)dout, (float*)eout);
@@ -1585,9 +1589,9 @@ int launch_step2_f32(const Plan& pl, const void* pm, const void* p, void* o1, vo
   if (pl.n > kTwoStepMaxN)
     return report(FFPAT_EINVAL, "two-step pass: N = %d > %d (32-bit offsets)", pl.n, kTwoStepMaxN);
   Maps2 maps;
-  if (make_map_box(&maps.p, p, pl.n, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
-      make_map_box(&maps.q[0], pm, pl.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
-      make_map_box(&maps.q[1], pl.kap, pl.n, 4, tb2::QW, tb2::QH) != FFPAT_OK)
+  if (make_map_box(&maps.p, p, pl.n, pl.np, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
+      make_map_box(&maps.q[0], pm, pl.n, pl.np, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
+      make_map_box(&maps.q[1], pl.kap, pl.n, pl.np, 4, tb2::QW, tb2::QH) != FFPAT_OK)
     return report(FFPAT_ECUDA, "two-step kernel: tensor map");
   maps.q[2] = maps.q[1];
   return launch_step2(k_step2_f32, tb2::smem_bytes<0>(), "k_step2_f32", pl, maps, st,
@@ -1620,10 +1624,10 @@ int launch_step2_batch(const BatchStep2* steps, int count, cudaStream_t st) {
       return report(FFPAT_EINVAL, "batched two-step pass: N = %d > %d (32-bit offsets)", b.n,
                     kTwoStepMaxN);
     Batch2Req& r = bp.r[i];
-    if (make_map_box(&r.maps.p, b.p, b.n, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
-        make_map_box(&r.maps.q[0], b.d, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
-        make_map_box(&r.maps.q[1], b.e, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
-        make_map_box(&r.maps.q[2], b.kap, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK)
+    if (make_map_box(&r.maps.p, b.p, b.n, b.n, 4, tb2::PW, tb2::PH) != FFPAT_OK ||
+        make_map_box(&r.maps.q[0], b.d, b.n, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
+        make_map_box(&r.maps.q[1], b.e, b.n, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK ||
+        make_map_box(&r.maps.q[2], b.kap, b.n, b.n, 4, tb2::QW, tb2::QH) != FFPAT_OK)
       return report(FFPAT_ECUDA, "batched two-step pass: tensor map");
     r.o0 = b.pout;
     r.o1 = b.dout;
@@ -1687,7 +1691,7 @@ int resident_zchunk(int n, int slots, int sms) {
 }  // namespace
 
 int resident_zc(const Plan& pl, int form) {
-  if (pl.esize != 4 || pl.n % 4 != 0 || pl.n < 4 || !pl.sync) return 0;
+  if (pl.esize != 4 || pl.np % 4 != 0 || pl.n < 4 || !pl.sync) return 0;
   int occ = 0;
   const int slots = form == 1 ? resident_slots<1>(&occ) : resident_slots<0>(&occ);
   if (slots <= 0 || occ <= 0) return 0;
@@ -1701,16 +1705,17 @@ int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, vo
   if (zc <= 0) return report(FFPAT_EINVAL, "resident time loop: N = %d does not fit", pl.n);
   static thread_local ResParams rp;
   const int n = pl.n;
-  if (make_map(&rp.pin, in, n, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&rp.pb[0], b0, n, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&rp.pb[1], b1, n, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&rp.kap, pl.kap, n, 4, false, rs::G::TH) != FFPAT_OK)
+  if (make_map(&rp.pin, in, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&rp.pb[0], b0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&rp.pb[1], b1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&rp.kap, pl.kap, n, pl.np, 4, false, rs::G::TH) != FFPAT_OK)
     return report(FFPAT_ECUDA, "resident time loop: tensor map");
   rp.buf[0] = (float*)b0;
   rp.buf[1] = (float*)b1;
   rp.out = (float*)out;
   rp.sync = pl.sync;
   rp.n = n;
+  rp.np = pl.np;
   rp.zc = zc;
   rp.tiles_x = (n + TBX - 1) / TBX;
   rp.tiles_y = (n + rs::G::TH - 1) / rs::G::TH;

@@ -549,7 +549,8 @@ template <int V, int C>
 __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
     k_backproject_z(const float* __restrict__ gt, float* __restrict__ h,
                     const float* __restrict__ scale, const float* __restrict__ tabf,
-                    const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg, int tx,
+                    const int32_t* __restrict__ tabi, int n, int np, int nth, int ns, int nimg,
+                    int tx,
                     float mult) {
   constexpr int RL = ZRow<V, C>::RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -635,7 +636,7 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
       const int x = blockIdx.x * sx + v % sx, y = blockIdx.y * 2 * ty + v / sx;
       const int z = zbase + c * 32 * V + zl;
       if (x >= n || y >= n || z >= n) continue;
-      const size_t o = ((size_t)z * n + y) * n + x;
+      const size_t o = ((size_t)z * n + y) * np + x;
       float out = f * stage[zl * (nv + 1) + v];
       if (scale) out *= scale[o];
       if (mult != 1.0f) out *= mult;
@@ -661,7 +662,7 @@ template <int V>
 __global__ void __launch_bounds__(128)
     k_backproject_z64(const double* __restrict__ gt, double* __restrict__ h,
                       const double* __restrict__ scale, const double* __restrict__ tab, int n,
-                      int nth, int ns, int nimg, int zp, int tb, double mult) {
+                      int np, int nth, int ns, int nimg, int zp, int tb, double mult) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double* W = reinterpret_cast<double*>(smem_raw) + (size_t)warp * kB64Angles * 12;
@@ -751,7 +752,7 @@ __global__ void __launch_bounds__(128)
     const int x = blockIdx.x * side + v % side, y = blockIdx.y * side + v / side;
     const int z = zbase + zl;
     if (x >= n || y >= n || z >= n) continue;
-    const size_t o = ((size_t)z * n + y) * n + x;
+    const size_t o = ((size_t)z * n + y) * np + x;
     double out = (2.0 / nimg) * stage[v * 32 * V + zl];
     if (scale) out *= scale[o];
     if (mult != 1.0) out *= mult;
@@ -894,9 +895,9 @@ int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cuda
                    const void* mask, void* scratch) {
   const int n = pl.n, rl = slab_planes(n, pl.esize), slabs = (n + rl - 1) / rl;
   if (!scratch) return report(FFPAT_EINVAL, "launch_project: no scratch volume");
-  const size_t nn = (size_t)n * n;
+  const size_t so = pl.np, sz = (size_t)n * pl.np;  // p[z][y][x] in rows of np
   if (pl.prec == FFPAT_FP64) {
-    const int rc = launch_zlast<double>(p, scratch, n, n, n, (size_t)n, nn, rl, st);
+    const int rc = launch_zlast<double>(p, scratch, n, n, n, so, sz, rl, st);
     if (rc != FFPAT_OK) return rc;
     const int V = choose_v64(n, 2);
     // slabs of 32 V planes, up to four of them in a CTA (they share the sample
@@ -914,7 +915,7 @@ int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cuda
     count_launch();
     return check_launch("k_project_z64");
   }
-  const int rc = launch_zlast<float>(p, scratch, n, n, n, (size_t)n, nn, rl, st);
+  const int rc = launch_zlast<float>(p, scratch, n, n, n, so, sz, rl, st);
   if (rc != FFPAT_OK) return rc;
   // rays (warps) a CTA: fewer while the grid would not give every SM two CTAs
   int rg = kPWarps;
@@ -946,7 +947,7 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
     auto kern =
         V == 4 ? k_backproject_z64<4> : (V == 2 ? k_backproject_z64<2> : k_backproject_z64<1>);
     kern<<<dim3(tiles, tiles, vs), 32 * tb * tb, list > stage ? list : stage, st>>>(
-        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.nth, pl.ns, pl.nimg,
+        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.np, pl.nth, pl.ns, pl.nimg,
         rl, tb, mult);
     count_launch();
     return check_launch("k_backproject_z64");
@@ -968,7 +969,7 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
     k_backproject_z<V.value, C.value>
         <<<dim3((n + 2 * tx - 1) / (2 * tx), (n + 2 * ty - 1) / (2 * ty), slabs), 32 * tx * ty,
            list > stage ? list : stage, st>>>((const float*)scratch, (float*)h, (const float*)scale,
-                                              pl.tabf, pl.tabi, n, pl.nth, pl.ns, pl.nimg, tx,
+                                              pl.tabf, pl.tabi, n, pl.np, pl.nth, pl.ns, pl.nimg, tx,
                                               (float)mult);
   });
   count_launch();
