@@ -47,7 +47,7 @@
  *   - `ws` is caller-owned device scratch of at least
  *     ffpat_workspace_bytes(problem) bytes, 256-byte aligned; its contents on
  *     entry do not matter.  Two calls that run concurrently need two
- *     workspaces.  For FP32 grids up to 128^3 the wave time loop is one
+ *     workspaces.  For grids up to 128^3 (FP64: 96^3) the wave time loop is one
  *     cooperative launch that occupies every SM while it runs, so such loops
  *     issued on several streams run one after another rather than side by
  *     side (the results do not depend on it).
@@ -266,10 +266,10 @@ int64_t ffpat_launch_count(void);
 /* Choice of leapfrog kernel (process-wide): 0 = automatic (the TMA-fed kernels
  * where all arrays are 16-byte aligned, on copies with rows padded to 16 bytes
  * when N % 4 != 0 for float or N % 2 != 0 for double (the differentiated
- * operator's checkpointed loops excepted) -- for FP32 and FP32-Kahan the whole time loop in one
+ * operator's checkpointed loops excepted) -- the whole time loop in one
  * cooperative launch where its work items fit the GPU at once (N <= 128 on
- * GB300) and the stream is not capturing, else two steps per pass for
- * 128 <= N <= 1624 -- else the plain 2.5D kernel), 1 = always the plain
+ * GB300, FP64 N <= 96) and the stream is not capturing, else two steps per pass
+ * for 128 <= N <= 1624 (FP32, FP32-Kahan) -- else the plain 2.5D kernel), 1 = always the plain
  * kernel, 2 = the single-step TMA kernel, 3 = the two-step TMA kernels for
  * FP32 and FP32-Kahan (N <= 1624; single steps for FP64), 4 = the resident
  * time loop (FP32, FP32-Kahan);

@@ -461,17 +461,20 @@ static int run_wave(const Plan& pl, const void* in, void* out, const void** resu
   // gets the step-by-step loop)
   const int path = stencil_path(pl);
   const int form = pl.prec == FFPAT_FP32_KAHAN ? 1 : 0;
-  if (pl.prec != FFPAT_FP64 && (path == 4 || (path == 0 && cap == cudaStreamCaptureStatusNone))) {
+  const bool f64 = pl.prec == FFPAT_FP64;  // (a requested path 4 is an FP32 one)
+  if ((path == 4 && !f64) || (path == 0 && cap == cudaStreamCaptureStatusNone)) {
     const void* ptrs[5] = {in, out, pl.kap, pl.s[0], pl.s[1]};
-    const bool fits = tma_supported(pl, ptrs, 5) && resident_zc(pl, form) > 0;
+    const bool fits = tma_supported(pl, ptrs, 5) &&
+                      (f64 ? resident64_zc(pl) : resident_zc(pl, form)) > 0;
     if (path == 4 && !fits)
       return fail(FFPAT_EINVAL,
                   "resident time loop requested but N = %d, the precision or an array alignment "
                   "rules it out", pl.n);
     bool refused = false;
-    const int rc = fits ? launch_wave_resident(pl, form, in, out, pl.s[0], pl.s[1], &res, st,
-                                               &refused)
-                        : FFPAT_EINVAL;
+    const int rc = !fits ? FFPAT_EINVAL
+                   : f64 ? launch_wave_resident64(pl, in, out, pl.s[0], pl.s[1], &res, st, &refused)
+                         : launch_wave_resident(pl, form, in, out, pl.s[0], pl.s[1], &res, st,
+                                                &refused);
     // a cooperative launch turned down for lack of room falls back to the
     // step-by-step loop below unless the resident loop was asked for
     if (fits && rc != FFPAT_OK && !(refused && path == 0)) return rc;

@@ -176,6 +176,11 @@ int launch_step2_kahan(const Plan& pl, const void* p, const void* d, const void*
 int resident_zc(const Plan& pl, int form);
 int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, void* b0, void* b1,
                          const void** result, cudaStream_t st, bool* refused = nullptr);
+// The same for FP64 three-term problems (N <= 96 on GB300): bit for bit the
+// single-step TMA loop.
+int resident64_zc(const Plan& pl);
+int launch_wave_resident64(const Plan& pl, const void* in, void* out, void* b0, void* b1,
+                           const void** result, cudaStream_t st, bool* refused);
 // Two FP32 three-term leapfrog steps in one HBM pass (needs N % 4 == 0, 16-byte
 // aligned arrays): reads p^{n-1} (pm) and p^n (p), writes p^{n+1} (o1) and
 // p^{n+2} (o2); o1, o2 alias neither input.  Bit-identical to two single steps.

@@ -406,20 +406,19 @@ __global__ void __launch_bounds__(NTX* NTY, 2)
           for (int h = 0; h < 2; ++h) {
             const int xl = tx + 32 * h;
             const int x = x0 + xl;
+            if (x >= n || y >= n) continue;  // whole warps of FP64 work in ragged tiles
             const int o = (ry + 2) * G::BXH + xl + G::XH;
             const int qo = ry * TBX + xl;
             const T L = lap12_sum(P0, Pm1, Pp1, Pm2, Pp2, o, G::BXH);
             const T c = P0[o];
             const T k = Q[(NQ - 1) * (G::QBYTES / sizeof(T)) + qo];
-            if (x < n && y < n) {
-              const size_t gi = (size_t)z * plane + (size_t)y * np + x;
-              if constexpr (START) {
-                o0[gi] = c + T(0.5) * k * L;
-                if (o1) o1[gi] = c;
-              } else {
-                const T pm = Q[qo];
-                o0[gi] = fma(k, L, fma(2.0, c, -pm));
-              }
+            const size_t gi = (size_t)z * plane + (size_t)y * np + x;
+            if constexpr (START) {
+              o0[gi] = c + T(0.5) * k * L;
+              if (o1) o1[gi] = c;
+            } else {
+              const T pm = Q[qo];
+              o0[gi] = fma(k, L, fma(2.0, c, -pm));
             }
           }
         }
@@ -1214,6 +1213,136 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_wave_resident(const __grid_cons
   }
 }
 
+// ---- the resident loop in FP64 (N <= 96 on GB300).  The same scheme; what
+// bounds it is the FP64 pipe (14 instructions a point at about 1.7 lanes a cycle
+// and SM), so the tiles are small, 32 x 8 columns of at most rd::ZM planes, one
+// point a thread and plane, to spread small grids over all SMs (64 x 16 tiles
+// put 32^3 on 8 of them).  p^{n-1} stays in registers, kap / 12 in the thread's
+// own shared-memory slots, p^n goes through L2.  The arithmetic is lap12_sum's
+// and the single step's, term for term, so the result is theirs bit for bit.
+namespace rd {
+constexpr int ZM = 6;            // planes of one work item at most
+constexpr int TX = 32, TY = 8;   // columns of one work item
+constexpr int PW = TX + 4, PH = TY + 4;
+constexpr int PE = PW * PH;      // one halo plane
+constexpr int NPL = ZM + 4;
+constexpr size_t kSmem =
+    (size_t)NPL * PE * 8 + (size_t)ZM * TX * TY * 8 + NPL * 8 + 1024;
+static_assert(PE * 8 % 128 == 0, "TMA destinations stay 128-byte aligned");
+}  // namespace rd
+
+struct Res64Params {
+  CUtensorMap pin;    // p^0 (halo box)
+  CUtensorMap pb[2];  // the state buffers (halo box)
+  const double* kap;  // kap / 12
+  double* buf[2];     // step s writes buf[s & 1] ...
+  double* out;        // ... except the last step, which writes here when non-null
+  unsigned* sync;
+  int n, np, zc, tiles_x, tiles_y, nt;
+};
+
+template <bool START>
+__device__ __forceinline__ bool res64_step(const double* pst, const double* ks, uint64_t* bar,
+                                           unsigned parity, double (&pm)[rd::ZM],
+                                           double* __restrict__ dst, size_t plane, int nz,
+                                           bool active) {
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (ok) ok = mbar_wait(&bar[i], parity, kWaitCycles);
+  const int o = (threadIdx.y + 2) * rd::PW + threadIdx.x + 2;
+  double c0 = pst[o], c1 = pst[rd::PE + o], c2 = pst[2 * rd::PE + o], c3 = pst[3 * rd::PE + o];
+#pragma unroll
+  for (int zi = 0; zi < rd::ZM; ++zi) {
+    if (zi < nz) {
+      if (ok) ok = mbar_wait(&bar[zi + 4], parity, kWaitCycles);
+      const double* P0 = pst + (zi + 2) * rd::PE;
+      const double c4 = pst[(zi + 4) * rd::PE + o];
+      if (active) {
+        double s1 = P0[o - 1] + P0[o + 1];
+        s1 += P0[o - rd::PW];
+        s1 += P0[o + rd::PW];
+        s1 += c1;
+        s1 += c3;
+        double s2 = fma(90.0, c2, P0[o - 2]);
+        s2 += P0[o + 2];
+        s2 += P0[o - 2 * rd::PW];
+        s2 += P0[o + 2 * rd::PW];
+        s2 += c0;
+        s2 += c4;
+        const double L = fma(16.0, s1, -s2);
+        const double k = ks[zi * rd::TX * rd::TY];
+        dst[zi * plane] = START ? c2 + 0.5 * k * L : fma(k, L, fma(2.0, c2, -pm[zi]));
+        pm[zi] = c2;
+      }
+      c0 = c1;
+      c1 = c2;
+      c2 = c3;
+      c3 = c4;
+    }
+  }
+  return ok;
+}
+
+__global__ void __launch_bounds__(rd::TX* rd::TY, 4)
+    k_wave_resident64(const __grid_constant__ Res64Params rp) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  double* pst = reinterpret_cast<double*>(smem);
+  double* kst = pst + rd::NPL * rd::PE;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(kst + rd::ZM * rd::TX * rd::TY);
+  const int tid = threadIdx.y * rd::TX + threadIdx.x;
+  const int n = rp.n, item = blockIdx.x;
+  const int tix = item % rp.tiles_x, tiy = (item / rp.tiles_x) % rp.tiles_y;
+  const int tz = item / (rp.tiles_x * rp.tiles_y);
+  const int z0 = tz * rp.zc, nz = min(n - z0, rp.zc);
+  const int nzc = (n + rp.zc - 1) / rp.zc;
+  const int zr = rp.zc >= 2 ? 1 : 2;  // z-chunks a two-plane halo reaches
+  const int x0 = tix * rd::TX, y0 = tiy * rd::TY;
+  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+  const bool active = x < n && y < n;
+  const size_t plane = (size_t)n * rp.np;
+  const size_t first = active ? ((size_t)z0 * n + y) * rp.np + x : 0;
+  if (tid == 0) {
+    for (int i = 0; i < rd::NPL; ++i) mbar_init(&bar[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  double* ks = kst + tid;
+  double pm[rd::ZM];
+#pragma unroll
+  for (int zi = 0; zi < rd::ZM; ++zi) {
+    pm[zi] = 0.0;
+    if (active && zi < nz) ks[zi * rd::TX * rd::TY] = rp.kap[first + zi * plane];
+  }
+  __syncthreads();
+  if (*(volatile unsigned*)&g_tma_status != 0u) return;
+  for (int s = 0; s < rp.nt; ++s) {
+    const CUtensorMap* src = s == 0 ? &rp.pin : &rp.pb[(s - 1) & 1];
+    double* dst = ((s == rp.nt - 1 && rp.out) ? rp.out : rp.buf[s & 1]) + first;
+    if (tid < nz + 4) {
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      mbar_expect_tx(&bar[tid], rd::PE * 8);
+      tma_load_3d(pst + tid * rd::PE, src, x0 - 2, y0 - 2, z0 - 2 + tid, &bar[tid]);
+    }
+    const unsigned parity = (unsigned)s & 1u;
+    const bool ok = s == 0
+                        ? res64_step<true>(pst, ks, bar, parity, pm, dst, plane, nz, active)
+                        : res64_step<false>(pst, ks, bar, parity, pm, dst, plane, nz, active);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) {
+        atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
+        for (int i = 0; i < nz + 4; ++i) mbar_wait(&bar[i], parity, 1 << 24);
+      }
+      return;
+    }
+    if (s + 1 < rp.nt && !neighbour_sync(rp.sync, (unsigned)(s + 1), tix, tiy, tz, rp.tiles_x,
+                                         rp.tiles_y, nzc, zr)) {
+      if (tid == 0) atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
+      return;
+    }
+  }
+}
+
 // ------------------------------------------------------------- host side --
 
 // FFPAT_ZCHUNK=<planes> fixes the z-range of one work item of the TMA
@@ -1696,6 +1825,96 @@ int resident_zc(const Plan& pl, int form) {
   const int slots = form == 1 ? resident_slots<1>(&occ) : resident_slots<0>(&occ);
   if (slots <= 0 || occ <= 0) return 0;
   return resident_zchunk(pl.n, slots, slots / occ);
+}
+
+// ---- FP64
+namespace {
+int resident64_slots(int* sms_out) {
+  static int occ = 0, sms = 0;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(k_wave_resident64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)rd::kSmem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_wave_resident64, rd::TX * rd::TY,
+                                                      rd::kSmem) != cudaSuccess)
+      occ = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 0;
+    cudaGetLastError();
+  });
+  *sms_out = sms;
+  return occ * sms;
+}
+}  // namespace
+
+// z-range of the FP64 resident loop's items, 0 where it does not run: all items
+// at once on the GPU; the least planes on the busiest SM (the FP64 pipe is the
+// bound), the longer range on ties (fewer halo planes and flags)
+int resident64_zc(const Plan& pl) {
+  if (pl.esize != 8 || pl.np % 2 != 0 || pl.n < 4 || !pl.sync) return 0;
+  int sms = 0;
+  const int slots = resident64_slots(&sms);
+  if (slots <= 0) return 0;
+  const int n = pl.n, tiles = ((n + rd::TX - 1) / rd::TX) * ((n + rd::TY - 1) / rd::TY);
+  int best = 0;
+  long long best_cost = 0;
+  for (int zc = 1; zc <= rd::ZM; ++zc) {
+    const long long items = (long long)tiles * ((n + zc - 1) / zc);
+    if (items > slots || items > kResidentMaxItems) continue;
+    const long long cost = (items + sms - 1) / sms * zc;
+    if (best == 0 || cost <= best_cost) {
+      best = zc;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+int launch_wave_resident64(const Plan& pl, const void* in, void* out, void* b0, void* b1,
+                           const void** result, cudaStream_t st, bool* refused) {
+  *refused = false;
+  const int zc = resident64_zc(pl), n = pl.n;
+  if (zc <= 0) return report(FFPAT_EINVAL, "FP64 resident time loop: N = %d does not fit", n);
+  static thread_local Res64Params rp;
+  if (make_map_box(&rp.pin, in, n, pl.np, 8, rd::PW, rd::PH) != FFPAT_OK ||
+      make_map_box(&rp.pb[0], b0, n, pl.np, 8, rd::PW, rd::PH) != FFPAT_OK ||
+      make_map_box(&rp.pb[1], b1, n, pl.np, 8, rd::PW, rd::PH) != FFPAT_OK)
+    return report(FFPAT_ECUDA, "FP64 resident time loop: tensor map");
+  rp.kap = (const double*)pl.kap;
+  rp.buf[0] = (double*)b0;
+  rp.buf[1] = (double*)b1;
+  rp.out = (double*)out;
+  rp.sync = pl.sync;
+  rp.n = n;
+  rp.np = pl.np;
+  rp.zc = zc;
+  rp.tiles_x = (n + rd::TX - 1) / rd::TX;
+  rp.tiles_y = (n + rd::TY - 1) / rd::TY;
+  rp.nt = pl.nt;
+  const int items = rp.tiles_x * rp.tiles_y * ((n + zc - 1) / zc);
+  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
+    return check_launch("FP64 resident time loop: flag reset");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(items);
+  cfg.blockDim = dim3(rd::TX, rd::TY);
+  cfg.dynamicSmemBytes = rd::kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_wave_resident64, rp);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (e == cudaErrorCooperativeLaunchTooLarge) *refused = true;  // nothing ran
+    return report(FFPAT_ECUDA, "k_wave_resident64 launch: %s", cudaGetErrorString(e));
+  }
+  count_launch();
+  if (result) *result = out ? out : rp.buf[(pl.nt - 1) & 1];
+  return check_launch("k_wave_resident64");
 }
 
 int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, void* b0, void* b1,
