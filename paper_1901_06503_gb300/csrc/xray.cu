@@ -103,6 +103,15 @@ __device__ __forceinline__ void ray_range(float cs, float sn, int k, int n, int 
   if (mhi < mlo) mhi = mlo;
 }
 
+// Programmatic dependent launch: k_zlast lets its consumer start, and the
+// consumer waits for k_zlast (its writes visible) before it reads the operand.
+__device__ __forceinline__ void launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_operand() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ------------------------------------------------- z-innermost operands --
 // out[slab][o][i][rl] = in[o so + z sz + i], z = slab rl + r: the volume (o = y,
 // i = x) or the data (o = theta, i = xi) with z innermost, in slabs of rl planes
@@ -113,6 +122,7 @@ __global__ void __launch_bounds__(256)
     k_zlast(const T* __restrict__ in, T* __restrict__ out, int nz, int ni, size_t so, size_t sz,
             int rl) {
   __shared__ T t[32][33];
+  launch_dependents();  // the consumer works out its first weights meanwhile
   const size_t o = blockIdx.z;
   const int i0 = blockIdx.x * 32, z0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += 8) {
@@ -252,10 +262,10 @@ __device__ __forceinline__ RowTaps row_taps(int a, int k, long long CS, long lon
   return r;
 }
 
-// P for all planes of a slab at once.  A CTA takes one angle, as many
-// neighbouring rays as it has warps and one slab; a warp owns a ray, a lane V C
-// planes.  Row by row of the major axis, the taps of every ray are worked out
-// into shared memory (kPRows rows at a time) and applied to all planes: two
+// P for all planes of a slab at once.  A CTA takes one angle, rg neighbouring
+// rays and one slab; a warp owns a ray, or every `split`-th block of kPSum rows
+// of it, a lane V C planes.  Row by row of the major axis, the taps of every ray are worked out
+// into shared memory (ch rows at a time) and applied to all planes: two
 // broadcast shared loads, then two to four taps of C vector loads and V C / 2
 // packed FMAs.  The loads hit L1 (neighbouring rays share their cells), whose
 // 128 B a cycle are the bound for long rows, instruction issue for short ones.
@@ -265,7 +275,6 @@ __device__ __forceinline__ RowTaps row_taps(int a, int k, long long CS, long lon
 // flight).  Per standalone call, 384^3 and 180 angles: 13.0 -> 5.2 ms against
 // the plane-by-plane kernel it replaces, 256^3 and 180: 3.7 -> 1.7 ms.
 // Sums: per kPSum rows, then over those.
-constexpr int kPRows = 32;
 constexpr int kPSum = 8;
 constexpr int kPWarps = 16;
 
@@ -285,14 +294,16 @@ template <int V, int C>
 __global__ void __launch_bounds__(kPWarps * 32, 2)
     k_project_z(const float* __restrict__ pt, float* __restrict__ g,
                 const float* __restrict__ sub, const float* __restrict__ mask,
-                const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg) {
+                const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg,
+                int rg, int ch) {
   constexpr int RL = ZRow<V, C>::RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int rg = blockDim.x / 32;
-  float4* w4 = reinterpret_cast<float4*>(smem_raw);            // [kPRows][rg]
-  int* xb = reinterpret_cast<int*>(w4 + (size_t)kPRows * rg);  // [kPRows][rg]: 8 base + count
-  float* stage = reinterpret_cast<float*>(smem_raw);           // [RL][rg + 1], afterwards
+  const int split = blockDim.x / 32 / rg;
+  float4* w4 = reinterpret_cast<float4*>(smem_raw);            // [ch][rg]
+  int* xb = reinterpret_cast<int*>(w4 + (size_t)ch * rg);       // [ch][rg]: 8 base + count
+  float* stage = reinterpret_cast<float*>(smem_raw);           // [split][RL][rg + 1], afterwards
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ray = warp % rg, part = warp / rg;
   const int j = blockIdx.y, k0 = blockIdx.x * rg;
   const int zbase = blockIdx.z * RL;
   const float* __restrict__ pz = pt + (size_t)blockIdx.z * n * n * RL + lane * V;
@@ -303,8 +314,8 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
   const long long sa = (long long)(ymajor ? n : 1) * RL, sb = (long long)(ymajor ? 1 : n) * RL;
   ZAcc<V * C> total;
   total.zero();
-  for (int a0 = 0; a0 < n; a0 += kPRows) {
-    const int rows = min(kPRows, n - a0);
+  for (int a0 = 0; a0 < n; a0 += ch) {
+    const int rows = min(ch, n - a0);
     __syncthreads();
     for (int e = tid; e < rows * rg; e += blockDim.x) {
       const int k = k0 + e % rg;
@@ -313,17 +324,18 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
       w4[e] = make_float4(t.w[0], t.w[1], t.w[2], t.w[3]);
       xb[e] = t.base * 8 + t.count;
     }
+    if (a0 == 0) wait_for_operand();
     __syncthreads();
-    const float* prow = pz + a0 * sa;
 #pragma unroll 1
-    for (int rs = 0; rs < rows; rs += kPSum) {
+    for (int rs = part * kPSum; rs < rows; rs += split * kPSum) {
       ZAcc<V * C> c;
       c.zero();
       const int re = min(rs + kPSum, rows);
+      const float* prow = pz + (a0 + rs) * sa;
 #pragma unroll 1
       for (int r = rs; r < re; ++r, prow += sa) {
-        const int code = xb[r * rg + warp], cnt = code & 7;
-        const float4 w = w4[r * rg + warp];
+        const int code = xb[r * rg + ray], cnt = code & 7;
+        const float4 w = w4[r * rg + ray];
         const float* q = prow + (code >> 3) * sb;
         if (cnt == 3)
           ray_taps<3, V, C>(q, sb, w, c);
@@ -340,14 +352,16 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < V * C; ++i)
-    stage[ZRow<V, C>::plane(lane, i) * (rg + 1) + warp] = total.get(i);
+    stage[(part * RL + ZRow<V, C>::plane(lane, i)) * (rg + 1) + ray] = total.get(i);
   __syncthreads();
   const float scale = 2.0f / (float)nimg;
   for (int e = tid; e < RL * rg; e += blockDim.x) {
     const int r = e % rg, zl = e / rg;
     if (k0 + r >= n || zbase + zl >= n) continue;
     const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
-    float out = scale * stage[zl * (rg + 1) + r];
+    float sum = stage[zl * (rg + 1) + r];
+    for (int q = 1; q < split; ++q) sum += stage[(q * RL + zl) * (rg + 1) + r];
+    float out = scale * sum;
     if (sub) out = out - sub[o];
     if (mask) out = out * mask[o];
     g[o] = out;
@@ -398,6 +412,7 @@ __global__ void __launch_bounds__(384)
   }
   __syncthreads();
   const int lo = s_lo, hi = s_hi;
+  wait_for_operand();
   double acc0[V], acc1[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) acc0[v] = acc1[v] = 0.0;
@@ -596,6 +611,7 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
     for (int d = 0; d < kBDet; ++d)
       if (d >= first) wl[4 * (d - first)] = w[d];
     if (vox == 0) info[al] = (kd + first) * 8 + count;
+    if (ja == 0) wait_for_operand();
     __syncwarp();
     const int jn = min(kBAngles, nth - ja);
     const float* row = gz + (size_t)ja * n * RL;
@@ -706,6 +722,7 @@ __global__ void __launch_bounds__(128)
         info[lane * 4 + v] = kb * 8 + on;
       }
     }
+    if (ja == 0) wait_for_operand();
     __syncwarp();
     const int jn = min(kB64Angles, nth - ja);
     for (int t = 0; t < jn; ++t) {
@@ -859,6 +876,24 @@ static int launch_zlast(const void* in, void* out, int nz, int ni, int no, size_
   return check_launch("k_zlast");
 }
 
+// the consumer of k_zlast's output: may start before k_zlast has finished
+template <typename... KArgs, typename... Args>
+static void launch_after_zlast(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem,
+                               cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);  // errors: check_launch
+  count_launch();
+}
+
 // f(V, C) as compile-time constants for a slab of rl planes
 template <class Fn>
 static void with_slab(int rl, Fn f) {
@@ -908,26 +943,28 @@ int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cuda
     const int zg = (vs + nslab - 1) / nslab;
     while (rg > 4 && (n + rg - 1) / rg * (long long)pl.nth * zg < 2 * kNumSMs) rg -= 4;
     const size_t list = (size_t)kP64Samples * rg * 36, stage = (size_t)nslab * 32 * V * (rg + 1) * 8;
-    auto kern = V == 2 ? k_project_z64<2> : k_project_z64<1>;
-    kern<<<dim3((n + rg - 1) / rg, pl.nth, zg), 32 * nslab * (rg / 2), list > stage ? list : stage,
-           st>>>((const double*)scratch, (double*)g, (const double*)sub, (const double*)mask, pl.tab,
-                 pl.tabf, n, pl.nth, pl.ns, pl.nimg, rl, nslab, rg);
-    count_launch();
+    launch_after_zlast(V == 2 ? k_project_z64<2> : k_project_z64<1>,
+                       dim3((n + rg - 1) / rg, pl.nth, zg), 32 * nslab * (rg / 2),
+                       list > stage ? list : stage, st, (const double*)scratch, (double*)g,
+                       (const double*)sub, (const double*)mask, pl.tab, pl.tabf, n, pl.nth, pl.ns,
+                       pl.nimg, rl, nslab, rg);
     return check_launch("k_project_z64");
   }
   const int rc = launch_zlast<float>(p, scratch, n, n, n, so, sz, rl, st);
   if (rc != FFPAT_OK) return rc;
-  // rays (warps) a CTA: fewer while the grid would not give every SM two CTAs
-  int rg = kPWarps;
-  while (rg > 4 && (n + rg - 1) / rg * (long long)pl.nth * slabs < 2 * kNumSMs) rg -= 4;
-  const size_t list = (size_t)kPRows * rg * 20, stage = (size_t)rl * (rg + 1) * 4;
+  // 16 warps a CTA: one a ray where the rays fill two CTAs on every SM, else
+  // two or four a ray, and longer row blocks between the CTA's barriers (latency
+  // is the bound there: 68^3, 17 angles 25 -> 14 us)
+  const long long rays = (long long)n * pl.nth * slabs, fill = 2LL * kNumSMs * kPWarps;
+  const int split = rays >= fill ? 1 : (2 * rays >= fill ? 2 : 4), rg = kPWarps / split;
+  const int ch = split == 1 ? 32 : 128;
+  const size_t list = (size_t)ch * rg * 20, stage = (size_t)split * rl * (rg + 1) * 4;
   with_slab(rl, [&](auto V, auto C) {
-    k_project_z<V.value, C.value>
-        <<<dim3((n + rg - 1) / rg, pl.nth, slabs), 32 * rg, list > stage ? list : stage, st>>>(
-            (const float*)scratch, (float*)g, (const float*)sub, (const float*)mask, pl.tabi, n,
-            pl.nth, pl.ns, pl.nimg);
+    launch_after_zlast(k_project_z<V.value, C.value>, dim3((n + rg - 1) / rg, pl.nth, slabs),
+                       32 * kPWarps, list > stage ? list : stage, st, (const float*)scratch,
+                       (float*)g, (const float*)sub, (const float*)mask, pl.tabi, n, pl.nth, pl.ns,
+                       pl.nimg, rg, ch);
   });
-  count_launch();
   return check_launch("k_project_z");
 }
 
@@ -944,12 +981,11 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
     if ((long long)((n + 3) / 4) * ((n + 3) / 4) * vs < 2 * kNumSMs) tb = 1;
     const int side = 2 * tb, tiles = (n + side - 1) / side;
     const size_t list = (size_t)tb * tb * kB64WarpBytes, stage = (size_t)side * side * 32 * V * 8;
-    auto kern =
-        V == 4 ? k_backproject_z64<4> : (V == 2 ? k_backproject_z64<2> : k_backproject_z64<1>);
-    kern<<<dim3(tiles, tiles, vs), 32 * tb * tb, list > stage ? list : stage, st>>>(
-        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.np, pl.nth, pl.ns, pl.nimg,
-        rl, tb, mult);
-    count_launch();
+    launch_after_zlast(
+        V == 4 ? k_backproject_z64<4> : (V == 2 ? k_backproject_z64<2> : k_backproject_z64<1>),
+        dim3(tiles, tiles, vs), 32 * tb * tb, list > stage ? list : stage, st,
+        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.np, pl.nth, pl.ns,
+        pl.nimg, rl, tb, mult);
     return check_launch("k_backproject_z64");
   }
   const int rc = launch_zlast<float>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
@@ -966,13 +1002,12 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
   const size_t list = (size_t)tx * ty * kBWarpBytes;
   with_slab(rl, [&](auto V, auto C) {
     const size_t stage = (size_t)32 * V.value * (4 * tx * ty + 1) * 4;
-    k_backproject_z<V.value, C.value>
-        <<<dim3((n + 2 * tx - 1) / (2 * tx), (n + 2 * ty - 1) / (2 * ty), slabs), 32 * tx * ty,
-           list > stage ? list : stage, st>>>((const float*)scratch, (float*)h, (const float*)scale,
-                                              pl.tabf, pl.tabi, n, pl.np, pl.nth, pl.ns, pl.nimg, tx,
-                                              (float)mult);
+    launch_after_zlast(k_backproject_z<V.value, C.value>,
+                       dim3((n + 2 * tx - 1) / (2 * tx), (n + 2 * ty - 1) / (2 * ty), slabs),
+                       32 * tx * ty, list > stage ? list : stage, st, (const float*)scratch,
+                       (float*)h, (const float*)scale, pl.tabf, pl.tabi, n, pl.np, pl.nth, pl.ns,
+                       pl.nimg, tx, (float)mult);
   });
-  count_launch();
   return check_launch("k_backproject_z");
 }
 
