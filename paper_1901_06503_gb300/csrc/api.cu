@@ -213,16 +213,17 @@ void fill_tables_host(int nth, unsigned char* buf) {
   }
 }
 
-static int upload_tables(Plan& pl, void* base, cudaStream_t st) {
+// Queue their upload from `buf`, which the caller keeps until the stream has
+// been synchronised (every entry point does so anyway before it returns, or for
+// the sound speed's maximum).
+static int upload_tables(Plan& pl, void* base, std::vector<unsigned char>& buf, cudaStream_t st) {
   const size_t m = 2 * (size_t)pl.nth;
-  std::vector<unsigned char> buf(table_bytes(pl.nth));
+  buf.resize(table_bytes(pl.nth));
   fill_tables_host(pl.nth, buf.data());
   pl.tab = (double*)base;
   pl.tabf = (float*)((char*)base + 8 * m);
   pl.tabi = (int32_t*)((char*)base + 12 * m);
   CK(cudaMemcpyAsync(base, buf.data(), buf.size(), cudaMemcpyHostToDevice, st));
-  // the host buffer dies at return: make sure the copy has consumed it
-  CK(cudaStreamSynchronize(st));
   return FFPAT_OK;
 }
 
@@ -235,29 +236,34 @@ int time_steps(const Plan& pl, double cmax, int* nt, double* dt) {
   return FFPAT_OK;
 }
 
-// c statistics -> Nt, dt, kappa (one device-to-host read of three doubles).
-// c and kapw live on the wave grid; kap is kapw's restriction to the box.
-static int setup_speed(Plan& pl, const void* c, cudaStream_t st) {
-  if (!c) return fail(FFPAT_EINVAL, "c is NULL");
-  TRY(launch_speed_stats(wave_plan(pl), c, pl.scal, st));
-  double h3[3];
-  CK(cudaMemcpyAsync(h3, pl.scal, sizeof h3, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (h3[2] != 0.0)
-    return fail(FFPAT_EINVAL, "sound speed has %.0f entries that are not finite and > 0", h3[2]);
-  pl.cmax = h3[0];
-  TRY(time_steps(pl, pl.cmax, &pl.nt, &pl.dt));
-  TRY(launch_kappa(wave_plan(pl), c, st));
-  if (!direct(pl)) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
-  return FFPAT_OK;
-}
-
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
           cudaStream_t st) {
   g_err[0] = 0;
   TRY(attach(pr, pl, ws, ws_bytes));
-  TRY(upload_tables(pl, pl.tab, st));
-  TRY(setup_speed(pl, c, st));
+  if (!c) return fail(FFPAT_EINVAL, "c is NULL");
+  // c's maximum and validity -> Nt, dt, kappa: one device-to-host read; the
+  // host works out the angle tables meanwhile
+  TRY(launch_speed_stats(wave_plan(pl), c, st));
+  std::vector<unsigned char> tabs;
+  double rows[2 * kReduceBlocks];
+  const int rc = upload_tables(pl, pl.tab, tabs, st);
+  cudaError_t e = cudaMemcpyAsync(rows, pl.partials, sizeof rows, cudaMemcpyDeviceToHost, st);
+  const cudaError_t es = cudaStreamSynchronize(st);  // `tabs` and `rows` are free after it
+  TRY(rc);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return fail(FFPAT_ECUDA, "sound speed: %s", cudaGetErrorString(e));
+  double cmax = rows[0], bad = 0.0;
+  for (int i = 0; i < kReduceBlocks; ++i) {
+    cmax = fmax(cmax, rows[2 * i]);
+    bad += rows[2 * i + 1];
+  }
+  if (bad != 0.0)
+    return fail(FFPAT_EINVAL, "sound speed has %.0f entries that are not finite and > 0", bad);
+  pl.cmax = cmax;
+  TRY(time_steps(pl, pl.cmax, &pl.nt, &pl.dt));
+  // c and kapw live on the wave grid; kap is kapw's restriction to the box
+  TRY(launch_kappa(wave_plan(pl), c, st));
+  if (!direct(pl)) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
   return FFPAT_OK;
 }
 
@@ -740,11 +746,13 @@ int ffpat_debug_samples(const ffpat_problem* problem, int32_t count, const int32
   cudaStream_t st = (cudaStream_t)stream;
   void* tabs = nullptr;
   CK(cudaMallocAsync(&tabs, table_bytes(pl.nth), st));
-  int rc = upload_tables(pl, tabs, st);
+  std::vector<unsigned char> host;
+  int rc = upload_tables(pl, tabs, host, st);
   if (rc == FFPAT_OK) rc = launch_debug_samples(wave_plan(pl), count, jkm, ij, f, st);
-  CK(cudaFreeAsync(tabs, st));
+  const cudaError_t ef = cudaFreeAsync(tabs, st), es = cudaStreamSynchronize(st);
   TRY(rc);
-  CK(cudaStreamSynchronize(st));
+  CK(ef);
+  CK(es);
   return FFPAT_OK;
 }
 
@@ -826,14 +834,16 @@ static int project_alone(const ffpat_problem* problem, const void* in, void* out
   const size_t zb = transpose ? zdata_bytes(pl.nw, pl.nth, pl.esize) : zvolume_bytes(pl.nw, pl.esize);
   char* mem = nullptr;
   CK(cudaMallocAsync((void**)&mem, tb + zb, st));
-  int rc = upload_tables(pl, mem, st);
+  std::vector<unsigned char> tabs;
+  int rc = upload_tables(pl, mem, tabs, st);
   const Plan wp = dense_rows(wave_plan(pl));
   if (rc == FFPAT_OK)
     rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb)
                    : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb);
-  CK(cudaFreeAsync(mem, st));
+  const cudaError_t ef = cudaFreeAsync(mem, st), es = cudaStreamSynchronize(st);
   TRY(rc);
-  CK(cudaStreamSynchronize(st));
+  CK(ef);
+  CK(es);
   return FFPAT_OK;
 }
 
@@ -948,7 +958,11 @@ int ffpat_fbp(const ffpat_problem* problem, const void* G, void* out, void* ws, 
   g_err[0] = 0;
   TRY(attach(problem, pl, ws, ws_bytes));
   if (!G || !out) return fail(FFPAT_EINVAL, "G or out is NULL");
-  TRY(upload_tables(pl, pl.tab, st));
+  std::vector<unsigned char> tabs;
+  int rc = upload_tables(pl, pl.tab, tabs, st);
+  // (the only synchronisation of this call: the tables' host copy dies here)
+  if (cudaStreamSynchronize(st) != cudaSuccess && rc == FFPAT_OK) rc = check_launch("angle tables");
+  TRY(rc);
   const Plan wp = wave_plan(pl);
   TRY(launch_ramp(wp, G, pl.r2, st));
   TRY(launch_backproject(dense_rows(wp), pl.r2, out, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));

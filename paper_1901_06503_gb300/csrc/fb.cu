@@ -28,21 +28,6 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
-__device__ __forceinline__ double block_max(double v) {
-  __shared__ double sm[32];
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sm[w] = v;
-  __syncthreads();
-  double t = -INFINITY;
-  if (w == 0) {
-    t = lane < (int)(blockDim.x >> 5) ? sm[lane] : -INFINITY;
-    for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_down_sync(0xffffffffu, t, o));
-  }
-  return t;
-}
-
 // sum `nq` rows of kReduceBlocks partials (fixed order) into dst[0..nq)
 __global__ void __launch_bounds__(kReduceThreads)
     k_finalize(const double* __restrict__ partials, int nq, double* __restrict__ dst) {
@@ -54,47 +39,38 @@ __global__ void __launch_bounds__(kReduceThreads)
   }
 }
 
-// max c, -min c, count of invalid entries (not finite or <= 0)
+// per CTA: max c, and whether any entry is not finite and > 0 (as a count).  The
+// loop and the reductions run in the input's own type (a maximum of floats is
+// exact in float, and the count is an integer), so FP32 input stays off the FP64
+// pipe; the host takes the maximum of the CTAs' rows, which spares a launch.
 template <typename T>
 __global__ void __launch_bounds__(kReduceThreads)
-    k_speed_stats(const T* __restrict__ c, size_t len, double* __restrict__ partials) {
-  // the element loop runs in the input's own type (max and min of floats are
-  // exact in float, and the count is an integer): FP32 input stays off the
-  // FP64 pipe; only the per-thread results go through the FP64 block reductions
-  T mxt = T(-INFINITY), mnt = T(INFINITY);
-  unsigned nbad = 0;
+    k_speed_stats(const T* __restrict__ c, size_t len, double* __restrict__ rows) {
+  __shared__ T smx[kReduceThreads / 32];
+  __shared__ unsigned sbad[kReduceThreads / 32];
+  T mx = T(-INFINITY);
+  unsigned bad = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x) {
     const T v = c[i];
-    if (!(v > T(0)) || !isfinite(v)) ++nbad;
-    mxt = fmax(mxt, v);
-    mnt = fmin(mnt, v);
+    if (!(v > T(0)) || !isfinite(v)) ++bad;
+    mx = fmax(mx, v);
   }
-  const double mx = block_max((double)mxt);
-  const double nmn = block_max(-(double)mnt);
-  const double bad = block_sum((double)nbad);
+  bad = __reduce_add_sync(0xffffffffu, bad);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) {
+    smx[threadIdx.x / 32] = mx;
+    sbad[threadIdx.x / 32] = bad;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    partials[blockIdx.x] = mx;
-    partials[kReduceBlocks + blockIdx.x] = nmn;
-    partials[2 * kReduceBlocks + blockIdx.x] = bad;
-  }
-}
-
-__global__ void __launch_bounds__(kReduceThreads)
-    k_speed_final(const double* __restrict__ partials, double* __restrict__ dst) {
-  double mx = -INFINITY, nmn = -INFINITY, bad = 0.0;
-  for (int i = threadIdx.x; i < kReduceBlocks; i += blockDim.x) {
-    mx = fmax(mx, partials[i]);
-    nmn = fmax(nmn, partials[kReduceBlocks + i]);
-    bad += partials[2 * kReduceBlocks + i];
-  }
-  mx = block_max(mx);
-  nmn = block_max(nmn);
-  bad = block_sum(bad);
-  if (threadIdx.x == 0) {
-    dst[0] = mx;
-    dst[1] = -nmn;
-    dst[2] = bad;
+    double nbad = 0.0;
+    for (int w = 0; w < kReduceThreads / 32; ++w) {
+      mx = fmax(mx, smx[w]);
+      nbad += (double)sbad[w];
+    }
+    rows[2 * blockIdx.x] = (double)mx;
+    rows[2 * blockIdx.x + 1] = nbad;
   }
 }
 
@@ -368,13 +344,12 @@ unsigned ew_blocks(size_t len) {
 
 }  // namespace
 
-int launch_speed_stats(const Plan& pl, const void* c, double* out3, cudaStream_t st) {
+int launch_speed_stats(const Plan& pl, const void* c, cudaStream_t st) {
   if (pl.prec == FFPAT_FP64)
     k_speed_stats<double><<<kReduceBlocks, kReduceThreads, 0, st>>>((const double*)c, pl.n3, pl.partials);
   else
     k_speed_stats<float><<<kReduceBlocks, kReduceThreads, 0, st>>>((const float*)c, pl.n3, pl.partials);
-  k_speed_final<<<1, kReduceThreads, 0, st>>>(pl.partials, out3);
-  count_launch(2);
+  count_launch();
   return check_launch(__func__);
 }
 

@@ -210,7 +210,8 @@ int launch_debug_samples(const Plan& pl, int count, const int32_t* jkm, int32_t*
                          cudaStream_t st);
 
 // fb.cu
-int launch_speed_stats(const Plan& pl, const void* c, double* out3, cudaStream_t st);
+// (max c, count of entries not finite and > 0) per CTA into pl.partials: kReduceBlocks pairs
+int launch_speed_stats(const Plan& pl, const void* c, cudaStream_t st);
 int launch_kappa(const Plan& pl, const void* c, cudaStream_t st);
 // prox.cu: prox of the gradient regulariser, (I + a D^T D)^{-1} in -> out
 // through the scratch volumes s0, s1 (in, out != s0, s1; in == out allowed).
