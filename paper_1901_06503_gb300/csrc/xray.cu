@@ -777,41 +777,92 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// Lambda on rows of n detectors.  A CTA computes the taps once (FP64, then
-// rounded to T) and walks rows; each row sits in shared memory between n
-// zeros on either side, so out-of-range neighbours read as zero (the same
-// sums, term for term, as testing the range).
+// Lambda on rows of n detectors.  Only odd taps (and t_0) are nonzero, so the
+// outputs of one parity are a dense Toeplitz product with the inputs of the other:
+// n / 2 multiply-adds an output, bound by the FMA pipe.  A CTA stages `groups`
+// groups of kRRows rows, the rows of a group interleaved; a warp owns 32 M outputs
+// of one parity (lane + 32 m) in one group: per input it reads M taps (the taps
+// by signed odd distance, consecutive lanes consecutive taps) and the input of
+// all eight rows (broadcast) for 8 M multiply-adds.  The same kernel in FP64.
+constexpr int kRRows = 8;
+
 template <typename T>
-__global__ void __launch_bounds__(128)
-    k_ramp(const T* __restrict__ r, T* __restrict__ out, const T* __restrict__ mask, int n,
-           int nimg, int rows) {
-  extern __shared__ unsigned char smem_raw[];
-  T* tap = reinterpret_cast<T*>(smem_raw);  // tap[d] for d < n (odd d nonzero)
-  T* row = tap + n;                         // zeros, the row, zeros: 3n
-  const double dxi = 2.0 / nimg;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double t;
-    if (i == 0)
-      t = 1.0 / (8.0 * dxi);
-    else if (i % 2 == 0)
-      t = 0.0;
-    else
-      t = -1.0 / (2.0 * kPi * kPi * (double)i * (double)i * dxi);
-    tap[i] = (T)t;
-    row[i] = T(0);
-    row[2 * n + i] = T(0);
+__device__ __forceinline__ void ramp_fma(T t, const T* __restrict__ x, T (&acc)[kRRows]) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 a = *reinterpret_cast<const float4*>(x), b = *reinterpret_cast<const float4*>(x + 4);
+    const float2 v[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+                         make_float2(b.z, b.w)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 r = ffma2(t, v[i], make_float2(acc[2 * i], acc[2 * i + 1]));
+      acc[2 * i] = r.x;
+      acc[2 * i + 1] = r.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kRRows; ++i) acc[i] = fma(t, x[i], acc[i]);
   }
-  const T* rc = row + n;
-  for (int rw = blockIdx.x; rw < rows; rw += gridDim.x) {
-    const size_t base = (size_t)rw * n;
-    __syncthreads();  // the previous row is read (and the taps and zeros written)
-    for (int i = threadIdx.x; i < n; i += blockDim.x) row[n + i] = r[base + i];
+}
+
+template <typename T, int M>
+__global__ void __launch_bounds__(512)
+    k_ramp(const T* __restrict__ r, T* __restrict__ out, const T* __restrict__ mask, int n,
+           int nimg, int rows, int groups, int blocks, int jc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* s = reinterpret_cast<T*>(smem_raw);       // [group][j][kRRows], jc inputs at a time
+  T* ts = s + (size_t)groups * jc * kRRows;    // ts[H + u] = t_|2u + 1|, -H <= u < H
+  const int H = n / 2 + 1 + 32 * M * blocks;   // outputs past the row read (unused) taps
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double dxi = 2.0 / nimg;
+  for (int i = tid; i < 2 * H; i += blockDim.x) {
+    const double d = 2.0 * (i - H) + 1.0;
+    ts[i] = (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi));
+  }
+  const int row0 = blockIdx.x * groups * kRRows, live = min(groups * kRRows, rows - row0);
+  // warp -> (group, parity of its outputs, block of 32 M of them)
+  const int blk = blockIdx.y * blocks + warp % blocks, p = (warp / blocks) & 1;
+  const int g = warp / (2 * blocks);
+  const int q0 = blk * 32 * M + lane;  // output k = 2 (q0 + 32 m) + p
+  const T* x = s + ((size_t)g * jc + (1 - p)) * kRRows;  // inputs j = 2 i + 1 - p
+  T acc[M][kRRows];
+#pragma unroll
+  for (int m = 0; m < M; ++m)
+#pragma unroll
+    for (int i = 0; i < kRRows; ++i) acc[m][i] = T(0);
+  for (int j0 = 0; j0 < n; j0 += jc) {
+    const int len = min(jc, n - j0);
     __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      T acc = tap[0] * rc[k];
-      for (int d = 1; d < n; d += 2) acc += tap[d] * (rc[k - d] + rc[k + d]);
-      if (mask) acc = acc * mask[base + k];
-      out[base + k] = acc;
+    for (int q = warp; q < groups * kRRows; q += blockDim.x / 32) {
+      const T* src = r + (size_t)(row0 + q) * n + j0;
+      T* dst = s + (size_t)(q / kRRows) * jc * kRRows + q % kRRows;
+      for (int j = lane; j < len; j += 32) dst[j * kRRows] = q < live ? src[j] : T(0);
+    }
+    __syncthreads();
+    const int nj = (len + p) / 2;
+    // the tap of input i of output q: u = q + p - 1 - i; outputs past the row
+    // (q up to n / 2 + 32 M blocks) stay within H
+    const T* t = ts + H + min(q0, n / 2 + 32 * M * (blocks - 1)) + p - 1 - j0 / 2;
+#pragma unroll 2
+    for (int i = 0; i < nj; ++i) {
+      T w[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) w[m] = t[32 * m - i];
+#pragma unroll
+      for (int m = 0; m < M; ++m) ramp_fma<T>(w[m], x + (size_t)i * 2 * kRRows, acc[m]);
+    }
+  }
+  const T t0 = (T)(1.0 / (8.0 * dxi));
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int k = 2 * (q0 + 32 * m) + p;
+    if (k >= n) continue;
+#pragma unroll
+    for (int i = 0; i < kRRows; ++i) {
+      if (g * kRRows + i >= live) continue;
+      const size_t o = (size_t)(row0 + g * kRRows + i) * n + k;
+      T v = fma(t0, r[o], acc[m][i]);
+      if (mask) v = v * mask[o];
+      out[o] = v;
     }
   }
 }
@@ -1011,32 +1062,52 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
   return check_launch("k_backproject_z");
 }
 
-int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st, const void* mask) {
-  const int rows = pl.nth * pl.n;
-  const size_t smem = 4 * (size_t)pl.n * pl.esize;
-  // eight 128-thread CTAs per SM walk the rows
-  const unsigned grid = (unsigned)(rows < 8 * kNumSMs ? rows : 8 * kNumSMs);
+// The shape of Lambda: blocks of 32 M outputs of one parity, the widest M that
+// leaves the fewest idle lanes; up to four blocks and four groups of rows a CTA
+// (16 warps, two parities); 512 inputs staged at a time (all of them up to 512^3).
+template <typename T, int M>
+static int ramp_launch(const Plan& pl, const void* r, void* out, const void* mask,
+                       cudaStream_t st) {
+  const int n = pl.n, rows = pl.nth * n, h = (n + 1) / 2;
+  const int nb = (h + 32 * M - 1) / (32 * M), blocks = nb < 4 ? nb : 4;
+  int groups = 4;
+  while (groups > 1 && 2 * blocks * groups > 16) groups /= 2;
+  const int jc = n < 512 ? (n + 1) / 2 * 2 : 512, H = n / 2 + 1 + 32 * M * blocks;
+  const size_t smem = ((size_t)groups * jc * kRRows + 2 * (size_t)H) * sizeof(T);
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_ramp<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                200 * 1024);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(k_ramp<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024);
+    attr = cudaFuncSetAttribute(k_ramp<T, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                220 * 1024);
   });
-  if (attr != cudaSuccess || smem > 200 * 1024) {
+  if (attr != cudaSuccess || smem > 220 * 1024) {
     cudaGetLastError();
     return report(FFPAT_ECUDA, "k_ramp: %zu bytes of shared memory refused", smem);
   }
-  if (pl.prec == FFPAT_FP64)
-    k_ramp<double><<<grid, 128, smem, st>>>((const double*)r, (double*)out, (const double*)mask,
-                                            pl.n, pl.nimg, rows);
-  else
-    k_ramp<float><<<grid, 128, smem, st>>>((const float*)r, (float*)out, (const float*)mask, pl.n,
-                                           pl.nimg, rows);
+  const int rg = groups * kRRows;
+  k_ramp<T, M><<<dim3((rows + rg - 1) / rg, (nb + blocks - 1) / blocks), 64 * blocks * groups, smem,
+                 st>>>((const T*)r, (T*)out, (const T*)mask, n, pl.nimg, rows, groups, blocks, jc);
   count_launch();
-  return check_launch(__func__);
+  return check_launch("k_ramp");
+}
+
+int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st, const void* mask) {
+  const int h = (pl.n + 1) / 2;
+  int best = 1, idle = INT_MAX;
+  for (int m = 1; m <= 4; ++m) {
+    const int lanes = (h + 32 * m - 1) / (32 * m) * 32 * m;
+    if (lanes <= idle) {
+      best = m;
+      idle = lanes;
+    }
+  }
+  const bool f64 = pl.prec == FFPAT_FP64;
+  switch (best) {
+    case 1: return f64 ? ramp_launch<double, 1>(pl, r, out, mask, st) : ramp_launch<float, 1>(pl, r, out, mask, st);
+    case 2: return f64 ? ramp_launch<double, 2>(pl, r, out, mask, st) : ramp_launch<float, 2>(pl, r, out, mask, st);
+    case 3: return f64 ? ramp_launch<double, 3>(pl, r, out, mask, st) : ramp_launch<float, 3>(pl, r, out, mask, st);
+    default: return f64 ? ramp_launch<double, 4>(pl, r, out, mask, st) : ramp_launch<float, 4>(pl, r, out, mask, st);
+  }
 }
 
 int launch_debug_samples(const Plan& pl, int count, const int32_t* jkm, int32_t* ij, double* f,

@@ -48,3 +48,16 @@ def test_slab_widths_fp64(n, nth):
     assert np.array_equal(got, o.project(p, nth))
     got = F.backproject(prob, torch.as_tensor(g, device="cuda")).cpu().numpy()
     assert rel(got, o.backproject(g, n)) < 1e-12
+
+
+# Lambda: blocks of 32 M outputs of one parity (M = 1 .. 4), eight rows a group,
+# 512 inputs at a time, outputs over several CTAs beyond 1024 of a parity
+@pytest.mark.parametrize("n,nth", [(1, 3), (2, 1), (3, 5), (63, 1), (65, 2), (66, 3), (127, 1),
+                                   (193, 1), (257, 1), (385, 1), (511, 1), (514, 1), (1030, 1)])
+def test_ramp_shapes(n, nth):
+    rows = random_data(nth, n, 80 + n)
+    for prec, dt, tol in ((F.FP64, np.float64, 1e-12), (F.FP32, np.float32, 5e-7)):
+        prob = F.problem(n, 1.0, nth, prec)
+        r = rows.astype(dt)
+        got = F.ramp(prob, torch.as_tensor(r, device="cuda")).double().cpu().numpy()
+        assert rel(got, o.ramp(r.astype(np.float64))) < tol
