@@ -85,14 +85,14 @@ static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 // against the plain kernel on the rows as they are: W at 150^3 FP32-Kahan 28.6 ->
 // 13 us a step, 101^3 FP32 10.6 -> 4.1 us); grids of fewer than five points stay
 // as they are.
-static int padded_row(const Plan& pl) {
+int padded_row(const Plan& pl) {
   const int q = (int)(16 / pl.esize);
   return (pl.nw + q - 1) / q * q;
 }
 static bool ragged(const Plan& pl) { return pl.nw >= 5 && padded_row(pl) != pl.nw; }
 
 // Validate the problem and fill the size fields of the plan.
-static int validate(const ffpat_problem* pr, Plan& pl) {
+static int validate(const ffpat_problem* pr, Plan& pl, bool any_path = false) {
   g_err[0] = 0;
   if (!pr) return fail(FFPAT_EINVAL, "problem is NULL");
   if (pr->n < 1 || pr->n > 2048) return fail(FFPAT_EINVAL, "n = %d outside [1, 2048]", pr->n);
@@ -125,8 +125,9 @@ static int validate(const ffpat_problem* pr, Plan& pl) {
   pl.np = pl.n;
   // rows that are no multiple of 16 bytes are padded on the wave grid, where
   // they would otherwise rule out the TMA kernels; a requested kernel (any
-  // path but the automatic one) runs on the rows as they are
-  pl.nwp = ragged(pl) && g_stencil_path.load() == 0 ? padded_row(pl) : pl.nw;
+  // path but the automatic one) runs on the rows as they are, unless data in
+  // padded rows outlive the call (any_path: the checkpoints)
+  pl.nwp = ragged(pl) && (any_path || g_stencil_path.load() == 0) ? padded_row(pl) : pl.nw;
   return FFPAT_OK;
 }
 
@@ -176,8 +177,8 @@ static size_t carve(Plan& pl, void* ws) {
   return off;
 }
 
-int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes) {
-  TRY(validate(pr, pl));
+int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path) {
+  TRY(validate(pr, pl, any_path));
   const size_t need = carve(pl, nullptr);
   if (!ws) return fail(FFPAT_EINVAL, "workspace is NULL (%zu bytes needed)", need);
   if (((uintptr_t)ws & 255) != 0) return fail(FFPAT_EINVAL, "workspace not 256-byte aligned");
@@ -237,9 +238,9 @@ int time_steps(const Plan& pl, double cmax, int* nt, double* dt) {
 }
 
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
-          cudaStream_t st) {
+          cudaStream_t st, bool any_path) {
   g_err[0] = 0;
-  TRY(attach(pr, pl, ws, ws_bytes));
+  TRY(attach(pr, pl, ws, ws_bytes, any_path));
   if (!c) return fail(FFPAT_EINVAL, "c is NULL");
   // c's maximum and validity -> Nt, dt, kappa: one device-to-host read; the
   // host works out the angle tables meanwhile
@@ -284,6 +285,13 @@ bool two_step_three_term(const Plan& pl, bool tma) {
   const int path = stencil_path(pl);
   return pl.prec == FFPAT_FP32 && tma && pl.n <= kTwoStepMaxN &&
          (path == 3 || (path == 0 && pl.n >= kTwoStepMinN));
+}
+
+bool resident_segments(const Plan& pl, bool tma, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return pl.prec == FFPAT_FP32 && tma && stencil_path(pl) == 0 &&
+         cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+         segments_resident(pl);
 }
 
 // algorithmic HBM bytes per point of a two-step pass beyond a single step's:

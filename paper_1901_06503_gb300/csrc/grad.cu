@@ -11,6 +11,13 @@
 // and the kappa-derivatives mu^{n+1} L(p^n) (weight 1/2 for the start step)
 // are accumulated; grad_c = 2 acc / c because dkappa/dc = 2 kappa / c and the
 // factors kappa/12 and 12 cancel.  Memory: 2 ceil(Nt/k) + k + 2 volumes.
+//
+// Where the resident time loop runs (FP32, N <= 128), the forward pass is one
+// cooperative launch that stores the checkpoints as it goes, and a segment of
+// the backward pass two: recompute (writing L(p^n) in place of p^n) and
+// transposed steps with the accumulation.  Elsewhere they are loops of launches.
+// FP32 volumes with ragged rows run on padded rows (wave_plan), FP64 ones as
+// they are.
 #include "internal.cuh"
 
 namespace ffpat {
@@ -32,7 +39,9 @@ struct Ckpt {
 int ckpt_layout(const Plan& pl, int nt, int every, void* base, Ckpt* ck) {
   if (pl.pad != 0) return report(FFPAT_EINVAL, "the differentiated operator needs pad = 0");
   if (every < 1 || every > 4096) return report(FFPAT_EINVAL, "checkpoint interval %d", every);
-  ck->vol = up256(pl.n3 * pl.esize);
+  // (FP32 volumes may have padded rows, FP64 ones never: see grad_view)
+  const size_t row = pl.esize == 4 ? padded_row(pl) : pl.n;
+  ck->vol = up256((size_t)pl.n * pl.n * row * pl.esize);
   ck->every = every;
   ck->nseg = (nt + every - 1) / every;
   ck->base = (unsigned char*)base;
@@ -45,9 +54,17 @@ void as_three_term(Plan& pl) {
   if (pl.prec == FFPAT_FP32_KAHAN) pl.prec = FFPAT_FP32;
 }
 
-bool use_tma(const Plan& pl, const Ckpt& ck, const void* a, const void* b) {
-  const void* ptrs[9] = {a, b, pl.kap, pl.s[0], pl.s[1], pl.s[2], pl.s[3], pl.x, ck.base};
-  return tma_supported(pl, ptrs, 9) && (ck.vol % 16) == 0;
+bool use_tma(const Plan& pl, const Ckpt& ck, const void* a) {
+  const void* ptrs[8] = {a, pl.kap, pl.s[0], pl.s[1], pl.s[2], pl.s[3], pl.x, ck.base};
+  return tma_supported(pl, ptrs, 8) && (ck.vol % 16) == 0;
+}
+
+// The view the steps run on: the wave grid with its padded rows in FP32; dense
+// rows in FP64 (whose accumulation kernel is the plain one) and for a checkpoint
+// buffer that TMA cannot address.  The same for the forward and the backward pass.
+Plan grad_view(const Plan& pl, const Ckpt& ck) {
+  const Plan w = wave_plan(pl);
+  return pl.esize == 4 && use_tma(w, ck, nullptr) ? w : pl;
 }
 
 // two steps per pass in the checkpointed loops: W's rule, and checkpoints at
@@ -77,7 +94,7 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
                        void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   Plan pl;
-  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st);
+  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, true);
   if (rc0 != FFPAT_OK) return rc0;
   if (!h || !g || !ckpt) return report(FFPAT_EINVAL, "h, g or ckpt is NULL");
   as_three_term(pl);
@@ -85,25 +102,41 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
   if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
   if (ckpt_bytes < ck.bytes())
     return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
-  const bool tma = use_tma(pl, ck, h, g);
-  const bool two = use_two(pl, ck, tma);
+  const Plan w = grad_view(pl, ck);
+  const void* in = h;
+  if (w.np != w.n) {  // the source in padded rows
+    const int rc = launch_embed(pl, h, pl.xw, st);
+    if (rc != FFPAT_OK) return rc;
+    in = pl.xw;
+  }
+  const bool tma = use_tma(w, ck, in);
+  if (resident_segments(w, tma, st)) {
+    const ResidentSave save{ck.base, ck.vol / 4, every};
+    const void* last = nullptr;
+    bool refused = false;
+    const int rc = launch_wave_resident(w, 0, in, nullptr, pl.s[0], pl.s[1], &last, st, &refused,
+                                        &save);
+    if (rc == FFPAT_OK) return launch_project(w, last, g, nullptr, st, nullptr, pl.x);
+    if (!refused) return rc;  // refused: step by step
+  }
+  const bool two = use_two(w, ck, tma);
   // S[a] = p^m, S[b] = p^{m+1}; a two-step pass writes the other pair
   void* S[4] = {pl.s[0], pl.s[1], pl.s[2], pl.s[3]};
   int a = 0, b = 1;
-  int rc = step3(pl, tma, true, h, nullptr, S[b], S[a], st);  // p^0, p^1
+  int rc = step3(w, tma, true, in, nullptr, S[b], S[a], st);  // p^0, p^1
   if (rc != FFPAT_OK) return rc;
-  const size_t vb = pl.n3 * pl.esize;
+  const size_t vb = (size_t)w.n * w.n * w.np * w.esize;
   if (cudaMemcpyAsync(ck.a(0), S[a], vb, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(ck.b(0), S[b], vb, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return check_launch("checkpoint copy");
   for (int m = 0; m + 1 < pl.nt;) {
     if (two && m + 3 <= pl.nt) {
-      rc = launch_step2_f32(pl, S[a], S[b], S[a ^ 2], S[b ^ 2], st);  // p^{m+2}, p^{m+3}
+      rc = launch_step2_f32(w, S[a], S[b], S[a ^ 2], S[b ^ 2], st);  // p^{m+2}, p^{m+3}
       a ^= 2;
       b ^= 2;
       m += 2;
     } else {
-      rc = step3(pl, tma, false, S[b], S[a], S[a], nullptr, st);  // p^{m+2} over p^m
+      rc = step3(w, tma, false, S[b], S[a], S[a], nullptr, st);  // p^{m+2} over p^m
       const int t = a;
       a = b;
       b = t;
@@ -117,7 +150,7 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
         return check_launch("checkpoint copy");
     }
   }
-  return launch_project(pl, S[b], g, nullptr, st, nullptr, pl.x);
+  return launch_project(w, S[b], g, nullptr, st, nullptr, pl.x);
 }
 
 int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad_g, void* grad_h,
@@ -125,7 +158,7 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
                    size_t ws_bytes, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   Plan pl;
-  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st);
+  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, true);
   if (rc0 != FFPAT_OK) return rc0;
   if (!grad_g || !ckpt) return report(FFPAT_EINVAL, "grad_g or ckpt is NULL");
   as_three_term(pl);
@@ -133,16 +166,25 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
   if (ckpt_bytes < ck.bytes())
     return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
-  const bool tma = use_tma(pl, ck, grad_h, c);
-  const bool two = use_two(pl, ck, tma);
-  const size_t vb = pl.n3 * pl.esize;
+  const Plan w = grad_view(pl, ck);
+  const bool tma = use_tma(w, ck, nullptr);
+  const bool two = use_two(w, ck, tma), resident = resident_segments(w, tma, st);
+  const bool rows = w.np != w.n;
+  const size_t vb = (size_t)w.n * w.n * w.np * w.esize;
   // mu^{Nt} = (kappa / 12) P^T grad_g, mu^{Nt+1} = 0
-  // B[u] = mu^{n+1}, B[v] = mu^{n+2}; a two-step pass writes mu^n, mu^{n-1}
-  // into the other two buffers
+  // B[u] = mu^{n+1}, B[v] = mu^{n+2}; a pass writes into the other two buffers
   void* B[4] = {pl.x, pl.s[0], pl.s[1], pl.s[2]};
-  const bool two_t = two_step_three_term(pl, tma) && pl.s[1] && pl.s[2];
+  const bool two_t = two_step_three_term(w, tma) && pl.s[1] && pl.s[2];
   int u = 0, v = 1;
-  int rc = launch_backproject(pl, grad_g, B[u], pl.kap, st, pl.r);
+  auto others = [&](int* x, int* y) {
+    *x = 0;
+    while (*x == u || *x == v) ++*x;
+    *y = *x + 1;
+    while (*y == u || *y == v) ++*y;
+  };
+  const void* end = nullptr;  // start(mu^1) - mu^2 where a resident segment left it
+  const void* tmp = nullptr;  // start(mu^1) else
+  int rc = launch_backproject(w, grad_g, B[u], w.kap, st, pl.r);
   if (rc != FFPAT_OK) return rc;
   if (cudaMemsetAsync(B[v], 0, vb, st) != cudaSuccess ||
       cudaMemsetAsync(ck.acc(), 0, vb, st) != cudaSuccess)
@@ -150,15 +192,32 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   for (int s = ck.nseg - 1; s >= 0; --s) {
     const int lo = s * every;
     const int hi = (lo + every - 1 < pl.nt - 1) ? lo + every - 1 : pl.nt - 1;
+    if (resident) {
+      // seg(j) holds L(p^{lo+j}); the states pass through the spare volumes
+      const int steps = hi - lo + 1;
+      int x, y;
+      others(&x, &y);
+      rc = launch_segment_recompute(w, ck.a(s), ck.b(s), pl.s[3], ck.seg(every), ck.seg(0),
+                                    ck.vol / 4, steps, st);
+      if (rc == FFPAT_OK)
+        rc = launch_segment_transpose(w, B[u], B[v], B[x], B[y], ck.acc(), ck.seg(0), ck.vol / 4,
+                                      steps, lo == 0, st);
+      if (rc != FFPAT_OK) return rc;
+      const int last = (steps - 1) & 1 ? y : x, prev = (steps - 1) & 1 ? x : y;
+      v = steps > 1 ? prev : u;  // mu^{lo+1}
+      u = last;                  // mu^{lo}
+      if (lo == 0) end = B[u];
+      continue;
+    }
     auto P = [&](int j) -> void* { return j == 0 ? ck.a(s) : (j == 1 ? ck.b(s) : ck.seg(j)); };
     // recompute p^{lo+2} .. p^{hi} from the checkpoint, two steps per pass
     // where allowed
     for (int j = 1; j + 1 <= hi - lo;) {
       if (two && j + 2 <= hi - lo) {
-        rc = launch_step2_f32(pl, P(j - 1), P(j), P(j + 1), P(j + 2), st);
+        rc = launch_step2_f32(w, P(j - 1), P(j), P(j + 1), P(j + 2), st);
         j += 2;
       } else {
-        rc = step3(pl, tma, false, P(j), P(j - 1), P(j + 1), nullptr, st);
+        rc = step3(w, tma, false, P(j), P(j - 1), P(j + 1), nullptr, st);
         j += 1;
       }
       if (rc != FFPAT_OK) return rc;
@@ -168,37 +227,54 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
       if (two_t && n - 1 >= lo && n - 1 >= 1) {
         // mu^n, mu^{n-1} in one pass; the accumulations in the order of
         // the single steps (mu^{n+1} L(p^n), then mu^n L(p^{n-1}))
-        int x = 0;
-        while (x == u || x == v) ++x;
-        int y = x + 1;
-        while (y == u || y == v) ++y;
-        rc = launch_step2_f32(pl, B[v], B[u], B[x], B[y], st);
-        if (rc == FFPAT_OK) rc = launch_lap_accum(pl, ck.acc(), B[u], pn, 1.0, st);
-        if (rc == FFPAT_OK) rc = launch_lap_accum(pl, ck.acc(), B[x], P(n - 1 - lo), 1.0, st);
+        int x, y;
+        others(&x, &y);
+        rc = launch_step2_f32(w, B[v], B[u], B[x], B[y], st);
+        if (rc == FFPAT_OK) rc = launch_lap_accum(w, ck.acc(), B[u], pn, 1.0, st);
+        if (rc == FFPAT_OK) rc = launch_lap_accum(w, ck.acc(), B[x], P(n - 1 - lo), 1.0, st);
         if (rc != FFPAT_OK) return rc;
         u = y;  // mu^{n-1}
         v = x;  // mu^n
         n -= 2;
       } else if (n >= 1) {
-        rc = launch_lap_accum(pl, ck.acc(), B[u], pn, 1.0, st);
-        if (rc == FFPAT_OK) rc = step3(pl, tma, false, B[u], B[v], B[v], nullptr, st);  // mu^n
+        rc = launch_lap_accum(w, ck.acc(), B[u], pn, 1.0, st);
+        if (rc == FFPAT_OK) rc = step3(w, tma, false, B[u], B[v], B[v], nullptr, st);  // mu^n
         if (rc != FFPAT_OK) return rc;
         const int t = u;
         u = v;
         v = t;
         n -= 1;
       } else {
-        rc = launch_lap_accum(pl, ck.acc(), B[u], pn, 0.5, st);
-        void* tmp = ck.seg(0);
-        if (rc == FFPAT_OK) rc = step3(pl, tma, true, B[u], nullptr, tmp, nullptr, st);
-        if (rc == FFPAT_OK && grad_h) rc = launch_sub_div(pl, tmp, B[v], grad_h, st);
+        rc = launch_lap_accum(w, ck.acc(), B[u], pn, 0.5, st);
+        if (rc == FFPAT_OK) rc = step3(w, tma, true, B[u], nullptr, ck.seg(0), nullptr, st);
         if (rc != FFPAT_OK) return rc;
+        tmp = ck.seg(0);
         n -= 1;
       }
     }
   }
-  if (grad_c) return launch_scale_div(pl, ck.acc(), c, 2.0, grad_c, st);
-  return FFPAT_OK;
+  // grad_h = (start(mu^1) - mu^2) / (kappa / 12), grad_c = 2 acc / c, on dense rows
+  if (grad_h && end) {
+    if (rows) rc = launch_restrict(pl, end, pl.xo, st);
+    if (rc == FFPAT_OK) rc = launch_kscale(pl, rows ? pl.xo : end, grad_h, false, st);
+  } else if (grad_h) {
+    const void *ta = tmp, *tb = B[v];
+    if (rows) {
+      rc = launch_restrict(pl, tmp, pl.xo, st);
+      if (rc == FFPAT_OK) rc = launch_restrict(pl, B[v], pl.v, st);
+      ta = pl.xo;
+      tb = pl.v;
+    }
+    if (rc == FFPAT_OK) rc = launch_sub_div(pl, ta, tb, grad_h, st);
+  }
+  if (rc != FFPAT_OK || !grad_c) return rc;
+  const void* acc = ck.acc();
+  if (rows) {
+    rc = launch_restrict(pl, acc, pl.xo, st);
+    if (rc != FFPAT_OK) return rc;
+    acc = pl.xo;
+  }
+  return launch_scale_div(pl, acc, c, 2.0, grad_c, st);
 }
 
 }  // extern "C"

@@ -74,14 +74,20 @@ constexpr int kResidentMaxItems = 1024;  // work items (step flags) of the resid
 constexpr int kScal = 64;
 
 // api.cu helpers shared with the server and the gradient path
+// (any_path: ragged rows are padded whatever the stencil path)
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
-          cudaStream_t st);
+          cudaStream_t st, bool any_path = false);
 // one three-term leapfrog launch (TMA kernel when the layout allows)
 int step3(const Plan& pl, bool tma, bool start, const void* p, const void* qin, void* qout,
           void* copy0, cudaStream_t st);
 // whether a three-term FP32 time loop takes two steps per pass (W's own rule)
 bool two_step_three_term(const Plan& pl, bool tma);
-int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes);
+// whether the differentiated operator's loops run as resident segments
+// (automatic path, not while capturing)
+bool resident_segments(const Plan& pl, bool tma, cudaStream_t st);
+// row pitch the wave grid's volumes may have (whatever the path)
+int padded_row(const Plan& pl);
+int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path = false);
 int time_steps(const Plan& pl, double cmax, int* nt, double* dt);
 void fill_tables_host(int nth, unsigned char* buf);  // table_bytes(nth) bytes
 
@@ -174,8 +180,28 @@ int launch_step2_kahan(const Plan& pl, const void* p, const void* d, const void*
 // (may be null) is set when the cooperative launch was turned down because
 // the grid cannot be co-resident at the moment: nothing ran.
 int resident_zc(const Plan& pl, int form);
+// save (form 0): also the checkpoint pairs (p^m, p^{m+1}), m = i every < nt, at
+// base + 2 i vol and one vol further (vol in floats).
+struct ResidentSave {
+  void* base;
+  size_t vol;
+  int every;
+};
 int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, void* b0, void* b1,
-                         const void** result, cudaStream_t st, bool* refused = nullptr);
+                         const void** result, cudaStream_t st, bool* refused = nullptr,
+                         const ResidentSave* save = nullptr);
+// Checkpoint segments of the differentiated operator in the resident scheme
+// (FP32 three-term, segments_resident() grids).  recompute: from p0 = p^lo, p1 =
+// p^{lo+1}, L(p^{lo+i}) to lp + i lpvol for i < steps.  transpose: `steps` steps
+// of mu from mu1 = mu^{n+1}, mu2 = mu^{n+2}, step s into the buffer s & 1, and
+// acc += mu^{n+1} L(p^n); ends: the last is n = 0 (weight 1/2; it writes
+// start(mu^1) - mu^2).  b0, b1 alias no input.
+bool segments_resident(const Plan& pl);
+int launch_segment_recompute(const Plan& pl, const void* p0, const void* p1, void* b0, void* b1,
+                             void* lp, size_t lpvol, int steps, cudaStream_t st);
+int launch_segment_transpose(const Plan& pl, const void* mu1, const void* mu2, void* b0, void* b1,
+                             void* acc, const void* lp, size_t lpvol, int steps, bool ends,
+                             cudaStream_t st);
 // The same for FP64 three-term problems (N <= 96 on GB300): bit for bit the
 // single-step TMA loop.
 int resident64_zc(const Plan& pl);

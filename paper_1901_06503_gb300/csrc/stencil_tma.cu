@@ -1011,6 +1011,9 @@ struct ResParams {
   float* out;         // ... except the last step, which writes here when non-null
   unsigned* sync;     // one step flag per work item, zero at launch
   int n, np, zc, tiles_x, tiles_y, nt;
+  float* ck;          // checkpoints (SAVE): the pair (p^{m}, p^{m+1}), m = i every, at
+  size_t ckvol;       // ck + 2 i ckvol and one ckvol further
+  int every;
 };
 
 // Step boundary of the resident loop, point to point: a CTA publishes that
@@ -1066,12 +1069,14 @@ __device__ __forceinline__ bool neighbour_sync(unsigned* flags, unsigned s1, int
 // rows and keeps the four column values it already read (z-2 .. z+1) in
 // registers, so each plane costs one new column load (z+2) and the six x/y
 // neighbour loads; the arithmetic is gather_pair's, value for value.
-template <int FORM, bool START>
+template <int FORM, bool START, bool SAVE>
 __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uint64_t* bar,
                                          unsigned parity, float2 (&sa)[rs::ZM][2],
                                          float2 (&sb)[rs::ZM], float2* __restrict__ es,
                                          float* __restrict__ dst,
-                                         int n, int np, int nz, int z0, int x0, int y0) {
+                                         int n, int np, int nz, int z0, int x0, int y0,
+                                         float* sv0 = nullptr, float* sv1 = nullptr,
+                                         float* sv2 = nullptr) {
   using G = rs::G;
   const int tx = threadIdx.x, ty = threadIdx.y;
   bool ok = true;
@@ -1127,6 +1132,14 @@ __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uin
         }
         if (x < n && y < n)  // np % 4 == 0: x + 1 is in the row as well
           *reinterpret_cast<float2*>(dst + (o0 + (unsigned)zi * plane)) = w;
+        if constexpr (SAVE) {
+          if (x < n && y < n) {
+            const unsigned o1 = o0 + (unsigned)zi * plane;
+            if (START) *reinterpret_cast<float2*>(sv0 + o1) = c2;
+            if (sv1) *reinterpret_cast<float2*>(sv1 + o1) = w;
+            if (sv2) *reinterpret_cast<float2*>(sv2 + o1) = w;
+          }
+        }
         c0 = c1;
         c1 = c2;
         c2 = c3;
@@ -1139,7 +1152,7 @@ __device__ __forceinline__ bool res_step(const float* pst, const float* kst, uin
   return ok;
 }
 
-template <int FORM>
+template <int FORM, bool SAVE>
 __global__ void __launch_bounds__(NTX* NTY, 2) k_wave_resident(const __grid_constant__ ResParams rp) {
   using G = rs::G;
   extern __shared__ unsigned char smem_raw[];
@@ -1195,8 +1208,19 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_wave_resident(const __grid_cons
       tma_load_3d(pst + tid * rs::PF, src, x0 - G::XH, y0 - 2, z0 - 2 + tid, &bar[tid]);
     }
     const unsigned parity = (unsigned)s & 1u;
-    ok = s == 0 ? res_step<FORM, true>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz, z0, x0, y0)
-                : res_step<FORM, false>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz, z0, x0, y0);
+    float *sv0 = nullptr, *sv1 = nullptr, *sv2 = nullptr;
+    if constexpr (SAVE) {
+      // p^{s+1} is the second of its pair when s is a checkpoint step, the first
+      // of the next when s + 1 is one
+      if (s == 0) sv0 = rp.ck;
+      if (s % rp.every == 0) sv1 = rp.ck + (size_t)(2 * (s / rp.every) + 1) * rp.ckvol;
+      if ((s + 1) % rp.every == 0 && s + 1 < rp.nt)
+        sv2 = rp.ck + (size_t)(2 * ((s + 1) / rp.every)) * rp.ckvol;
+    }
+    ok = s == 0 ? res_step<FORM, true, SAVE>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz,
+                                             z0, x0, y0, sv0, sv1, sv2)
+                : res_step<FORM, false, SAVE>(pst, kst, bar, parity, sa, sb, es, dst, n, rp.np, nz,
+                                              z0, x0, y0, sv0, sv1, sv2);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
@@ -1210,6 +1234,232 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_wave_resident(const __grid_cons
       if (tid == 0) atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
       return;
     }
+  }
+}
+
+// ---- the differentiated operator's segments in the resident scheme (FP32, the
+// grids of the resident loop).  A backward pass recomputes the states of a
+// checkpoint segment and then runs the transposed steps through it, gathering
+// acc += w mu^{n+1} L(p^n).  Step by step that is three launches of about 8 us
+// a step at small grids; here it is two cooperative launches a segment:
+//   SEG_RECOMPUTE  steps p^lo .. p^hi from the checkpoint pair and writes
+//                  L(p^n), which the step computes anyway, in place of p^n;
+//   SEG_TRANSPOSE  steps mu and adds mu^{n+1} L(p^n) point by point, the sums
+//                  on chip (first row of a thread in registers, second in shared
+//                  memory); at n = 0 it writes start(mu^1) - mu^2.
+// Arithmetic and order are the single steps' (three_term_pair, start_pair, the
+// accumulation form of k_step_tma), so the gradients are theirs bit for bit.
+enum { SEG_RECOMPUTE = 0, SEG_TRANSPOSE = 1 };
+
+struct SegParams {
+  CUtensorMap in0;    // p^lo / mu^{hi+1} (halo boxes)
+  CUtensorMap in1;    // p^{lo+1}
+  CUtensorMap pb[2];  // the buffers
+  CUtensorMap kap;
+  float* buf[2];
+  const float* pm;    // mu^{hi+2}
+  float* acc;
+  float* lp;          // L(p^{lo+i}) at lp + i lpvol
+  size_t lpvol;
+  unsigned* sync;
+  int n, np, zc, tiles_x, tiles_y, steps, ends;  // ends: the last step is n = 0
+};
+
+template <int MODE>
+__device__ __forceinline__ bool seg_step(const float* pst, const float* kst, uint64_t* bar,
+                                         unsigned parity, float2 (&sa)[rs::ZM][2],
+                                         float2 (&sb)[rs::ZM], float2* __restrict__ es,
+                                         float* __restrict__ dst, float* __restrict__ lp, int n,
+                                         int np, int nz, int z0, int x0, int y0, bool end) {
+  using G = rs::G;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int xl = 2 * tx, x = x0 + xl;
+  const unsigned plane = (unsigned)(n * np);
+  const unsigned base = (unsigned)z0 * plane + (unsigned)((y0 + ty) * np + x);
+  const bool in0 = x < n && y0 + ty < n, in1 = x < n && y0 + ty + TBY < n;
+  // L(p^n) of the first row before the planes arrive, of the second as the first is used
+  float2 q[rs::ZM];
+  if constexpr (MODE == SEG_TRANSPOSE) {
+#pragma unroll
+    for (int zi = 0; zi < rs::ZM; ++zi)
+      q[zi] = zi < nz && in0 ? __ldcs(reinterpret_cast<const float2*>(lp + base + (unsigned)zi * plane))
+                             : make_float2(0.f, 0.f);
+  }
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (ok) ok = mbar_wait(&bar[i], parity, kWaitCycles);
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    const int ry = ty + TBY * rr;
+    const int o = (ry + 2) * G::BXH + xl + G::XH;
+    const unsigned o0 = base + (unsigned)(rr * TBY * np);
+    const bool in = rr == 0 ? in0 : in1;
+    float2 c0 = lds2(pst + o), c1 = lds2(pst + rs::PF + o);
+    float2 c2 = lds2(pst + 2 * rs::PF + o), c3 = lds2(pst + 3 * rs::PF + o);
+#pragma unroll
+    for (int zi = 0; zi < rs::ZM; ++zi) {
+      if (zi < nz) {
+        if (rr == 0 && ok) ok = mbar_wait(&bar[zi + 4], parity, kWaitCycles);
+        const float* P0 = pst + (zi + 2) * rs::PF;
+        const float2 c4 = lds2(pst + (zi + 4) * rs::PF + o);
+        const float2 XM = lds2(P0 + o - 2), XP = lds2(P0 + o + 2);
+        Nb2 v;
+        v.c = c2;
+        v.xm1 = make_float2(XM.y, c2.x);
+        v.xp1 = make_float2(c2.y, XP.x);
+        v.xm2 = XM;
+        v.xp2 = XP;
+        v.ym1 = lds2(P0 + o - G::BXH);
+        v.yp1 = lds2(P0 + o + G::BXH);
+        v.ym2 = lds2(P0 + o - 2 * G::BXH);
+        v.yp2 = lds2(P0 + o + 2 * G::BXH);
+        v.zm1 = c1;
+        v.zp1 = c3;
+        v.zm2 = c0;
+        v.zp2 = c4;
+        const float2 L = lap12_pair(v);
+        const float2 K = lds2(kst + zi * rs::QF + ry * TBX + xl);
+        const unsigned oz = o0 + (unsigned)zi * plane;
+        if constexpr (MODE == SEG_RECOMPUTE) {
+          if (in) {
+            *reinterpret_cast<float2*>(lp + oz) = L;
+            if (dst) *reinterpret_cast<float2*>(dst + oz) = three_term_pair(c2, K, L, sa[zi][rr]);
+          }
+        } else {
+          const float wt = end ? 0.5f : 1.0f;
+          float2* ap = es + (zi * TBY + ty) * NTX + tx;
+          const float2 a = fma2(mul2(make_float2(wt, wt), c2), q[zi], rr == 0 ? sb[zi] : *ap);
+          if (rr == 0) {
+            sb[zi] = a;
+            if (in1)
+              q[zi] = __ldcs(reinterpret_cast<const float2*>(lp + oz + (unsigned)(TBY * np)));
+          } else {
+            *ap = a;
+          }
+          if (in)
+            *reinterpret_cast<float2*>(dst + oz) =
+                end ? sub2(start_pair(c2, K, L), sa[zi][rr]) : three_term_pair(c2, K, L, sa[zi][rr]);
+        }
+        sa[zi][rr] = c2;
+        c0 = c1;
+        c1 = c2;
+        c2 = c3;
+        c3 = c4;
+        asm volatile("" ::: "memory");
+      }
+    }
+  }
+  return ok;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_constant__ SegParams sp) {
+  using G = rs::G;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  float* pst = reinterpret_cast<float*>(smem);
+  float* kst = reinterpret_cast<float*>(smem + rs::NPL * G::PBYTES);
+  float2* es = reinterpret_cast<float2*>(smem + rs::NPL * G::PBYTES + rs::ZM * G::QBYTES);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + rs::NPL * G::PBYTES + rs::ZM * G::QBYTES +
+                                              rs::EBYTES);
+  const int tid = threadIdx.y * NTX + threadIdx.x;
+  const int n = sp.n, np = sp.np, item = blockIdx.x;
+  const int tix = item % sp.tiles_x, tiy = (item / sp.tiles_x) % sp.tiles_y;
+  const int tz = item / (sp.tiles_x * sp.tiles_y);
+  const int z0 = tz * sp.zc, nz = min(n - z0, sp.zc);
+  const int nzc = (n + sp.zc - 1) / sp.zc;
+  const int zr = sp.zc >= 2 ? 1 : 2;
+  const int x0 = tix * TBX, y0 = tiy * G::TH;
+  if (tid == 0) {
+    for (int i = 0; i <= rs::NPL; ++i) mbar_init(&bar[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (*(volatile unsigned*)&g_tma_status != 0u) return;
+  if (tid == 0) {
+    mbar_expect_tx(&bar[rs::NPL], (unsigned)(nz * G::QBYTES));
+    for (int zi = 0; zi < nz; ++zi)
+      tma_load_3d(kst + zi * rs::QF, &sp.kap, x0, y0, z0 + zi, &bar[rs::NPL]);
+  }
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 sa[rs::ZM][2], sb[rs::ZM];
+  const unsigned plane = (unsigned)(n * np);
+  const int x = x0 + 2 * (int)threadIdx.x;
+#pragma unroll
+  for (int zi = 0; zi < rs::ZM; ++zi)
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const int y = y0 + (int)threadIdx.y + TBY * rr;
+      const unsigned o = (unsigned)(z0 + zi) * plane + (unsigned)(y * np + x);
+      const bool in = zi < nz && x < n && y < n;
+      float2 a = zero;
+      sa[zi][rr] = zero;
+      if constexpr (MODE == SEG_TRANSPOSE) {
+        if (in) {
+          sa[zi][rr] = *reinterpret_cast<const float2*>(sp.pm + o);
+          a = *reinterpret_cast<const float2*>(sp.acc + o);
+        }
+      }
+      if (rr == 0)
+        sb[zi] = a;
+      else
+        es[(zi * TBY + threadIdx.y) * NTX + threadIdx.x] = a;
+    }
+  bool ok = mbar_wait(&bar[rs::NPL], 0, kWaitCycles);
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) {
+      atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
+      mbar_wait(&bar[rs::NPL], 0, 1 << 24);
+    }
+    return;
+  }
+  for (int s = 0; s < sp.steps; ++s) {
+    // RECOMPUTE: step s works on p^{lo+s}: the pair's volumes, then the buffers
+    // (p^{lo+i} in buffer i & 1); TRANSPOSE: on mu^{hi+1-s}, mu^{hi-s} to s & 1
+    const CUtensorMap* src;
+    float* dst;
+    float* lp;
+    if constexpr (MODE == SEG_RECOMPUTE) {
+      src = s == 0 ? &sp.in0 : (s == 1 ? &sp.in1 : &sp.pb[s & 1]);
+      dst = s >= 1 && s + 1 < sp.steps ? sp.buf[(s + 1) & 1] : nullptr;
+      lp = sp.lp + (size_t)s * sp.lpvol;
+    } else {
+      src = s == 0 ? &sp.in0 : &sp.pb[(s - 1) & 1];
+      dst = sp.buf[s & 1];
+      lp = sp.lp + (size_t)(sp.steps - 1 - s) * sp.lpvol;
+    }
+    if (tid < nz + 4) {
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      mbar_expect_tx(&bar[tid], G::PBYTES);
+      tma_load_3d(pst + tid * rs::PF, src, x0 - G::XH, y0 - 2, z0 - 2 + tid, &bar[tid]);
+    }
+    const unsigned parity = (unsigned)s & 1u;
+    ok = seg_step<MODE>(pst, kst, bar, parity, sa, sb, es, dst, lp, n, np, nz, z0, x0, y0,
+                        sp.ends != 0 && s + 1 == sp.steps);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) {
+        atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
+        for (int i = 0; i < nz + 4; ++i) mbar_wait(&bar[i], parity, 1 << 24);
+      }
+      return;
+    }
+    if (s + 1 < sp.steps && !neighbour_sync(sp.sync, (unsigned)(s + 1), tix, tiy, tz, sp.tiles_x,
+                                            sp.tiles_y, nzc, zr)) {
+      if (tid == 0) atomicCAS(&g_tma_status, 0u, (unsigned)(-FFPAT_ETIMEDOUT));
+      return;
+    }
+  }
+  if constexpr (MODE == SEG_TRANSPOSE) {
+#pragma unroll
+    for (int zi = 0; zi < rs::ZM; ++zi)
+#pragma unroll
+      for (int rr = 0; rr < 2; ++rr) {
+        const int y = y0 + (int)threadIdx.y + TBY * rr;
+        if (zi < nz && x < n && y < n)
+          *reinterpret_cast<float2*>(sp.acc + ((unsigned)(z0 + zi) * plane + (unsigned)(y * np + x))) =
+              rr == 0 ? sb[zi] : es[(zi * TBY + threadIdx.y) * NTX + threadIdx.x];
+      }
   }
 }
 
@@ -1782,7 +2032,7 @@ int resident_slots(int* occ_out) {
   static int occ = 0, sms = 0;
   static std::once_flag once;
   std::call_once(once, [] {
-    auto kern = k_wave_resident<FORM>;
+    auto kern = k_wave_resident<FORM, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs::kSmem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTX * NTY, rs::kSmem) !=
         cudaSuccess)
@@ -1917,8 +2167,57 @@ int launch_wave_resident64(const Plan& pl, const void* in, void* out, void* b0, 
   return check_launch("k_wave_resident64");
 }
 
+// One cooperative launch of a resident kernel over all items; *refused when the
+// grid cannot be co-resident at the moment (nothing ran).
+namespace {
+template <class Params>
+int launch_resident(void (*kern)(Params), const Params& params, const Plan& pl, int items,
+                    cudaStream_t st, bool* refused, const char* name) {
+  if (items > kResidentMaxItems)
+    return report(FFPAT_EINVAL, "resident time loop: %d work items > %d", items, kResidentMaxItems);
+  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
+    return check_launch("resident time loop: flag reset");
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(items);
+  cfg.blockDim = dim3(NTX, NTY);
+  cfg.dynamicSmemBytes = rs::kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, params);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    // the grid could not be made co-resident now (fewer SMs than the
+    // occupancy query promised): nothing ran, the caller may step instead
+    if (refused && e == cudaErrorCooperativeLaunchTooLarge) *refused = true;
+    return report(FFPAT_ECUDA, "%s launch: %s", name, cudaGetErrorString(e));
+  }
+  count_launch();
+  return check_launch(name);
+}
+
+// the shared-memory opt-in of the kernels that take resident_slots' occupancy
+template <class K>
+bool resident_fits(K kern, int slots) {
+  int occ = 0, dev = 0, sms = 0;
+  const bool ok =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs::kSmem) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTX * NTY, rs::kSmem) ==
+          cudaSuccess &&
+      cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+  cudaGetLastError();
+  return ok && occ * sms >= slots;
+}
+}  // namespace
+
 int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, void* b0, void* b1,
-                         const void** result, cudaStream_t st, bool* refused) {
+                         const void** result, cudaStream_t st, bool* refused,
+                         const ResidentSave* save) {
   if (refused) *refused = false;
   const int zc = resident_zc(pl, form);
   if (zc <= 0) return report(FFPAT_EINVAL, "resident time loop: N = %d does not fit", pl.n);
@@ -1939,33 +2238,81 @@ int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, vo
   rp.tiles_x = (n + TBX - 1) / TBX;
   rp.tiles_y = (n + rs::G::TH - 1) / rs::G::TH;
   rp.nt = pl.nt;
+  rp.ck = save ? (float*)save->base : nullptr;
+  rp.ckvol = save ? save->vol : 0;
+  rp.every = save ? save->every : 1;
   const int items = rp.tiles_x * rp.tiles_y * ((n + zc - 1) / zc);
-  if (items > kResidentMaxItems)
-    return report(FFPAT_EINVAL, "resident time loop: %d work items > %d", items, kResidentMaxItems);
-  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
-    return check_launch("resident time loop: barrier reset");
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(items);
-  cfg.blockDim = dim3(NTX, NTY);
-  cfg.dynamicSmemBytes = rs::kSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = form == 1 ? cudaLaunchKernelEx(&cfg, k_wave_resident<1>, rp)
-                                  : cudaLaunchKernelEx(&cfg, k_wave_resident<0>, rp);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    // the grid could not be made co-resident now (fewer SMs than the
-    // occupancy query promised): nothing ran, the caller may step instead
-    if (refused && e == cudaErrorCooperativeLaunchTooLarge) *refused = true;
-    return report(FFPAT_ECUDA, "k_wave_resident launch: %s", cudaGetErrorString(e));
-  }
-  count_launch();
-  if (result) *result = (pl.nt >= 1 && out) ? out : (pl.nt >= 1 ? rp.buf[(pl.nt - 1) & 1] : in);
-  return check_launch("k_wave_resident");
+  const int rc =
+      save ? launch_resident(k_wave_resident<0, true>, rp, pl, items, st, refused, "k_wave_resident")
+           : form == 1
+                 ? launch_resident(k_wave_resident<1, false>, rp, pl, items, st, refused,
+                                   "k_wave_resident")
+                 : launch_resident(k_wave_resident<0, false>, rp, pl, items, st, refused,
+                                   "k_wave_resident");
+  if (rc != FFPAT_OK) return rc;
+  if (result) *result = out ? out : rp.buf[(pl.nt - 1) & 1];
+  return FFPAT_OK;
+}
+
+bool segments_resident(const Plan& pl) {
+  int occ = 0;
+  const int zc = resident_zc(pl, 0), slots = resident_slots<0>(&occ);
+  if (zc <= 0) return false;
+  static bool fits = false;
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    fits = resident_fits(k_wave_resident<0, true>, slots) &&
+           resident_fits(k_seg_resident<SEG_RECOMPUTE>, slots) &&
+           resident_fits(k_seg_resident<SEG_TRANSPOSE>, slots);
+  });
+  return fits;
+}
+
+static int launch_segment(const Plan& pl, int mode, const void* in0, const void* in1, void* b0,
+                          void* b1, const void* pm, void* acc, void* lp, size_t lpvol, int steps,
+                          bool ends, cudaStream_t st) {
+  const int zc = resident_zc(pl, 0), n = pl.n;
+  if (zc <= 0) return report(FFPAT_EINVAL, "resident segment: N = %d does not fit", n);
+  static thread_local SegParams sp;
+  if (make_map(&sp.in0, in0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp.in1, in1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp.pb[0], b0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp.pb[1], b1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp.kap, pl.kap, n, pl.np, 4, false, rs::G::TH) != FFPAT_OK)
+    return report(FFPAT_ECUDA, "resident segment: tensor map");
+  sp.buf[0] = (float*)b0;
+  sp.buf[1] = (float*)b1;
+  sp.pm = (const float*)pm;
+  sp.acc = (float*)acc;
+  sp.lp = (float*)lp;
+  sp.lpvol = lpvol;
+  sp.sync = pl.sync;
+  sp.n = n;
+  sp.np = pl.np;
+  sp.zc = zc;
+  sp.tiles_x = (n + TBX - 1) / TBX;
+  sp.tiles_y = (n + rs::G::TH - 1) / rs::G::TH;
+  sp.steps = steps;
+  sp.ends = ends ? 1 : 0;
+  const int items = sp.tiles_x * sp.tiles_y * ((n + zc - 1) / zc);
+  return mode == SEG_RECOMPUTE
+             ? launch_resident(k_seg_resident<SEG_RECOMPUTE>, sp, pl, items, st, nullptr,
+                               "k_seg_resident")
+             : launch_resident(k_seg_resident<SEG_TRANSPOSE>, sp, pl, items, st, nullptr,
+                               "k_seg_resident");
+}
+
+int launch_segment_recompute(const Plan& pl, const void* p0, const void* p1, void* b0, void* b1,
+                             void* lp, size_t lpvol, int steps, cudaStream_t st) {
+  return launch_segment(pl, SEG_RECOMPUTE, p0, p1, b0, b1, nullptr, nullptr, lp, lpvol, steps,
+                        false, st);
+}
+
+int launch_segment_transpose(const Plan& pl, const void* mu1, const void* mu2, void* b0, void* b1,
+                             void* acc, const void* lp, size_t lpvol, int steps, bool ends,
+                             cudaStream_t st) {
+  return launch_segment(pl, SEG_TRANSPOSE, mu1, mu1, b0, b1, mu2, acc, (void*)lp, lpvol, steps,
+                        ends, st);
 }
 
 int read_device_status(unsigned* out, bool clear) {
