@@ -779,92 +779,109 @@ __global__ void __launch_bounds__(128)
 
 // Lambda on rows of n detectors.  Only odd taps (and t_0) are nonzero, so the
 // outputs of one parity are a dense Toeplitz product with the inputs of the other:
-// n / 2 multiply-adds an output, bound by the FMA pipe.  A CTA stages `groups`
-// groups of kRRows rows, the rows of a group interleaved; a warp owns 32 M outputs
-// of one parity (lane + 32 m) in one group: per input it reads M taps (the taps
-// by signed odd distance, consecutive lanes consecutive taps) and the input of
-// all eight rows (broadcast) for 8 M multiply-adds.  The same kernel in FP64.
-constexpr int kRRows = 8;
+// n / 2 multiply-adds an output, bound by the FMA pipe.  A CTA stages 32 rows with
+// the rows innermost (lane = row); a warp owns kROut outputs of one parity in all
+// 32: per input it loads one value a row and one new tap (broadcast; the other
+// taps slide through registers) for kROut multiply-adds.  The same kernel in FP64.
+// On smooth rows t_0 r_k nearly cancels the nearest taps' sum, so those (|d| <=
+// kRNear) are summed apart, outwards from t_0, and the product holds the others
+// (a tenth of t_0 in all), whose rounding then shows as little.
+// 384^3 and 180 angles: 1.63 -> 0.41 ms against two inputs and a tap loaded for
+// every multiply-add, 256^3 and 180: 0.50 -> 0.125 ms (0.16 with one CTA an SM at
+// 127 registers, 0.17 with eight outputs a warp).
+constexpr int kROut = 16;
+constexpr int kRNear = 3;
+constexpr int kRPitch = 33;  // of a staged input: 32 rows and one word against bank conflicts
 
 template <typename T>
-__device__ __forceinline__ void ramp_fma(T t, const T* __restrict__ x, T (&acc)[kRRows]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4 a = *reinterpret_cast<const float4*>(x), b = *reinterpret_cast<const float4*>(x + 4);
-    const float2 v[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
-                         make_float2(b.z, b.w)};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 r = ffma2(t, v[i], make_float2(acc[2 * i], acc[2 * i + 1]));
-      acc[2 * i] = r.x;
-      acc[2 * i + 1] = r.y;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < kRRows; ++i) acc[i] = fma(t, x[i], acc[i]);
-  }
-}
-
-template <typename T, int M>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
     k_ramp(const T* __restrict__ r, T* __restrict__ out, const T* __restrict__ mask, int n,
-           int nimg, int rows, int groups, int blocks, int jc) {
+           int nimg, int rows, int jc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* s = reinterpret_cast<T*>(smem_raw);       // [group][j][kRRows], jc inputs at a time
-  T* ts = s + (size_t)groups * jc * kRRows;    // ts[H + u] = t_|2u + 1|, -H <= u < H
-  const int H = n / 2 + 1 + 32 * M * blocks;   // outputs past the row read (unused) taps
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x / 32;
+  const int ko = blockIdx.y * warps * kROut;   // first output of the CTA (a multiple of 32)
+  const int nout = warps * kROut;
+  const int H = n / 2 + 2 * kROut + nout / 2;  // taps by u, d = 2 u + 1, -H <= u < H
+  T* s = reinterpret_cast<T*>(smem_raw);       // [max(jc, nout)][kRPitch]
+  T* ts = s + (size_t)max(jc, nout) * kRPitch;
   const double dxi = 2.0 / nimg;
   for (int i = tid; i < 2 * H; i += blockDim.x) {
     const double d = 2.0 * (i - H) + 1.0;
-    ts[i] = (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi));
+    ts[i] = fabs(d) > kRNear ? (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi)) : T(0);
   }
-  const int row0 = blockIdx.x * groups * kRRows, live = min(groups * kRRows, rows - row0);
-  // warp -> (group, parity of its outputs, block of 32 M of them)
-  const int blk = blockIdx.y * blocks + warp % blocks, p = (warp / blocks) & 1;
-  const int g = warp / (2 * blocks);
-  const int q0 = blk * 32 * M + lane;  // output k = 2 (q0 + 32 m) + p
-  const T* x = s + ((size_t)g * jc + (1 - p)) * kRRows;  // inputs j = 2 i + 1 - p
-  T acc[M][kRRows];
+  const int row0 = blockIdx.x * 32, live = min(32, rows - row0);
+  // outputs k = 2 (q0 + m) + p, inputs j = 2 i + 1 - p, tap u = q0 + m + p - 1 - i
+  const int p = warp & 1, q0 = ko / 2 + (warp >> 1) * kROut;
+  T acc[kROut];
 #pragma unroll
-  for (int m = 0; m < M; ++m)
-#pragma unroll
-    for (int i = 0; i < kRRows; ++i) acc[m][i] = T(0);
+  for (int m = 0; m < kROut; ++m) acc[m] = T(0);
   for (int j0 = 0; j0 < n; j0 += jc) {
     const int len = min(jc, n - j0);
     __syncthreads();
-    for (int q = warp; q < groups * kRRows; q += blockDim.x / 32) {
+    for (int q = warp; q < 32; q += warps) {
       const T* src = r + (size_t)(row0 + q) * n + j0;
-      T* dst = s + (size_t)(q / kRRows) * jc * kRRows + q % kRRows;
-      for (int j = lane; j < len; j += 32) dst[j * kRRows] = q < live ? src[j] : T(0);
+      for (int j = lane; j < len; j += 32) s[j * kRPitch + q] = q < live ? src[j] : T(0);
     }
     __syncthreads();
-    const int nj = (len + p) / 2;
-    // the tap of input i of output q: u = q + p - 1 - i; outputs past the row
-    // (q up to n / 2 + 32 M blocks) stay within H
-    const T* t = ts + H + min(q0, n / 2 + 32 * M * (blocks - 1)) + p - 1 - j0 / 2;
-#pragma unroll 2
-    for (int i = 0; i < nj; ++i) {
-      T w[M];
+    const int ni = (len + p) / 2;
+    const T* x = s + (1 - p) * kRPitch + lane;
+    const T* t = ts + H + q0 + p - 1 - j0 / 2;  // t[m - i]: the tap of output m, input i
+    T w[kROut];  // slot (m - i) mod kROut
 #pragma unroll
-      for (int m = 0; m < M; ++m) w[m] = t[32 * m - i];
+    for (int m = 1; m < kROut; ++m) w[m] = t[m];
+    int i = 0;
+    for (; i + kROut <= ni; i += kROut) {
 #pragma unroll
-      for (int m = 0; m < M; ++m) ramp_fma<T>(w[m], x + (size_t)i * 2 * kRRows, acc[m]);
+      for (int e = 0; e < kROut; ++e) {
+        const T v = x[(i + e) * 2 * kRPitch];
+        w[(kROut - e) % kROut] = t[-(i + e)];
+#pragma unroll
+        for (int m = 0; m < kROut; ++m)
+          acc[m] = fma(w[(m - e + kROut) % kROut], v, acc[m]);
+      }
+    }
+    for (; i < ni; ++i) {  // the rest, taps from shared memory
+      const T v = x[i * 2 * kRPitch];
+#pragma unroll
+      for (int m = 0; m < kROut; ++m) acc[m] = fma(t[m - i], v, acc[m]);
     }
   }
+  // the nearest taps, outwards from t_0 (the rows still staged when jc >= n)
   const T t0 = (T)(1.0 / (8.0 * dxi));
+  T tn[(kRNear + 1) / 2];
 #pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const int k = 2 * (q0 + 32 * m) + p;
-    if (k >= n) continue;
+  for (int e = 0; e < (kRNear + 1) / 2; ++e) {
+    const double d = 2.0 * e + 1.0;
+    tn[e] = (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi));
+  }
+  const bool staged = jc >= n;
+  const T* own = r + (size_t)(row0 + min(lane, live - 1)) * n;
+  auto at = [&](int j) -> T {
+    return j < 0 || j >= n ? T(0) : (staged ? s[j * kRPitch + lane] : own[j]);
+  };
 #pragma unroll
-    for (int i = 0; i < kRRows; ++i) {
-      if (g * kRRows + i >= live) continue;
-      const size_t o = (size_t)(row0 + g * kRRows + i) * n + k;
-      T v = fma(t0, r[o], acc[m][i]);
+  for (int m = 0; m < kROut; ++m) {
+    const int k = 2 * (q0 + m) + p;
+    T v = t0 * at(k);
+#pragma unroll
+    for (int e = 0; e < (kRNear + 1) / 2; ++e)
+      v += tn[e] * (at(k - 2 * e - 1) + at(k + 2 * e + 1));
+    acc[m] = v + acc[m];
+  }
+  // through shared memory to the rows
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < kROut; ++m)
+    s[(2 * ((warp >> 1) * kROut + m) + p) * kRPitch + lane] = acc[m];
+  __syncthreads();
+  const int kn = min(nout, n - ko);
+  for (int q = warp; q < live; q += warps)
+    for (int k = lane; k < kn; k += 32) {
+      const size_t o = (size_t)(row0 + q) * n + ko + k;
+      T v = s[k * kRPitch + q];
       if (mask) v = v * mask[o];
       out[o] = v;
     }
-  }
 }
 
 __global__ void k_debug_samples(int count, const int32_t* __restrict__ jkm, int32_t* __restrict__ ij,
@@ -1062,52 +1079,34 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
   return check_launch("k_backproject_z");
 }
 
-// The shape of Lambda: blocks of 32 M outputs of one parity, the widest M that
-// leaves the fewest idle lanes; up to four blocks and four groups of rows a CTA
-// (16 warps, two parities); 512 inputs staged at a time (all of them up to 512^3).
-template <typename T, int M>
+template <typename T>
 static int ramp_launch(const Plan& pl, const void* r, void* out, const void* mask,
                        cudaStream_t st) {
-  const int n = pl.n, rows = pl.nth * n, h = (n + 1) / 2;
-  const int nb = (h + 32 * M - 1) / (32 * M), blocks = nb < 4 ? nb : 4;
-  int groups = 4;
-  while (groups > 1 && 2 * blocks * groups > 16) groups /= 2;
-  const int jc = n < 512 ? (n + 1) / 2 * 2 : 512, H = n / 2 + 1 + 32 * M * blocks;
-  const size_t smem = ((size_t)groups * jc * kRRows + 2 * (size_t)H) * sizeof(T);
+  const int n = pl.n, rows = pl.nth * n;
+  // pairs of warps (both parities of 2 kROut outputs), up to eight a CTA, spread
+  // evenly; 512 inputs staged at a time (all of them up to 512^3)
+  const int pairs = (n + 2 * kROut - 1) / (2 * kROut), gy = (pairs + 7) / 8;
+  const int warps = 2 * ((pairs + gy - 1) / gy), nout = warps * kROut;
+  const int jc = n < 512 ? (n + 1) / 2 * 2 : 512, H = n / 2 + 2 * kROut + nout / 2;
+  const size_t smem = ((size_t)(jc > nout ? jc : nout) * kRPitch + 2 * (size_t)H) * sizeof(T);
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_ramp<T, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                220 * 1024);
+    attr = cudaFuncSetAttribute(k_ramp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
   });
   if (attr != cudaSuccess || smem > 220 * 1024) {
     cudaGetLastError();
     return report(FFPAT_ECUDA, "k_ramp: %zu bytes of shared memory refused", smem);
   }
-  const int rg = groups * kRRows;
-  k_ramp<T, M><<<dim3((rows + rg - 1) / rg, (nb + blocks - 1) / blocks), 64 * blocks * groups, smem,
-                 st>>>((const T*)r, (T*)out, (const T*)mask, n, pl.nimg, rows, groups, blocks, jc);
+  k_ramp<T><<<dim3((rows + 31) / 32, gy), 32 * warps, smem, st>>>(
+      (const T*)r, (T*)out, (const T*)mask, n, pl.nimg, rows, jc);
   count_launch();
   return check_launch("k_ramp");
 }
 
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st, const void* mask) {
-  const int h = (pl.n + 1) / 2;
-  int best = 1, idle = INT_MAX;
-  for (int m = 1; m <= 4; ++m) {
-    const int lanes = (h + 32 * m - 1) / (32 * m) * 32 * m;
-    if (lanes <= idle) {
-      best = m;
-      idle = lanes;
-    }
-  }
-  const bool f64 = pl.prec == FFPAT_FP64;
-  switch (best) {
-    case 1: return f64 ? ramp_launch<double, 1>(pl, r, out, mask, st) : ramp_launch<float, 1>(pl, r, out, mask, st);
-    case 2: return f64 ? ramp_launch<double, 2>(pl, r, out, mask, st) : ramp_launch<float, 2>(pl, r, out, mask, st);
-    case 3: return f64 ? ramp_launch<double, 3>(pl, r, out, mask, st) : ramp_launch<float, 3>(pl, r, out, mask, st);
-    default: return f64 ? ramp_launch<double, 4>(pl, r, out, mask, st) : ramp_launch<float, 4>(pl, r, out, mask, st);
-  }
+  return pl.prec == FFPAT_FP64 ? ramp_launch<double>(pl, r, out, mask, st)
+                               : ramp_launch<float>(pl, r, out, mask, st);
 }
 
 int launch_debug_samples(const Plan& pl, int count, const int32_t* jkm, int32_t* ij, double* f,

@@ -50,8 +50,8 @@ def test_slab_widths_fp64(n, nth):
     assert rel(got, o.backproject(g, n)) < 1e-12
 
 
-# Lambda: blocks of 32 M outputs of one parity (M = 1 .. 4), eight rows a group,
-# 512 inputs at a time, outputs over several CTAs beyond 1024 of a parity
+# Lambda: 32 rows a CTA, 16 outputs of one parity a warp, 512 inputs at a time,
+# outputs over several CTAs beyond 256
 @pytest.mark.parametrize("n,nth", [(1, 3), (2, 1), (3, 5), (63, 1), (65, 2), (66, 3), (127, 1),
                                    (193, 1), (257, 1), (385, 1), (511, 1), (514, 1), (1030, 1)])
 def test_ramp_shapes(n, nth):
