@@ -329,11 +329,20 @@ __global__ void __launch_bounds__(NTX* NTY, 2)
   unsigned phase = 0;  // one parity bit per barrier slot
   const size_t plane = (size_t)n * np;
 
-  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
+  // FP32 (bound by bytes): the persistent grid walks items of zc planes.  FP64
+  // (bound by the FP64 pipe, so equal work matters and halo planes do not): the
+  // planes of all tiles in one line, an equal stretch for every CTA, which may
+  // end one tile and begin the next
+  constexpr bool kEven = sizeof(T) == 8;
+  long long w = kEven ? (long long)blockIdx.x * nitems * n / gridDim.x : blockIdx.x;
+  const long long wend = kEven ? ((long long)blockIdx.x + 1) * nitems * n / gridDim.x : nitems;
+  while (w < wend) {
+    const int item = (int)(kEven ? w / n : w);
     const int tix = item % tiles_x;
     const int tiy = (item / tiles_x) % tiles_y;
-    const int z0 = (item / (tiles_x * tiles_y)) * zc;
-    const int z1 = min(n, z0 + zc);
+    const int z0 = kEven ? (int)(w % n) : (item / (tiles_x * tiles_y)) * zc;
+    const int z1 = kEven ? (int)min((long long)n, z0 + (wend - w)) : min(n, z0 + zc);
+    w += kEven ? z1 - z0 : gridDim.x;
     const int x0 = tix * TBX, y0 = tiy * G::TH;
 
     if (tid == 0)
@@ -1774,9 +1783,11 @@ int launch_one(const Plan& pl, const Maps& maps, void* o0, void* o1, void* o2, c
   const int slots = kNumSMs * occ;
   int zc = choose_zchunk(n, tiles_x * tiles_y, slots);
   if (zchunk_override() > 0) zc = zchunk_override() < n ? zchunk_override() : n;
-  const int zchunks = (n + zc - 1) / zc;
+  const int zchunks = sizeof(T) == 8 ? 1 : (n + zc - 1) / zc;  // FP64: nitems = tiles
   const int nitems = tiles_x * tiles_y * zchunks;
-  const int grid = nitems < slots ? nitems : slots;
+  // FP64: at least four planes a CTA
+  const int work = sizeof(T) == 8 ? (nitems * n + 3) / 4 : nitems;
+  const int grid = work < slots ? work : slots;
   const cudaError_t e =
       launch_pdl(kern, dim3(grid), dim3(NTX, NTY), smem, st, maps, (T*)o0, (T*)o1, (T*)o2, n, pl.np, zc,
                  tiles_x, tiles_y, nitems);
@@ -1797,10 +1808,13 @@ bool tma_supported(const Plan& pl, const void* const* ptrs, int count) {
   return true;
 }
 
-// FFPAT_RPT=<1|2> fixes the rows per thread of the single-step kernel (a
+// FFPAT_RPT=<1|2> fixes the rows per thread of the FP32 single-step kernels (a
 // tuning knob for measurements; 0 or unset = 2: the 64 x 16 tile, measured
-// faster on GB300 at 128^3 - 384^3 in every precision: fewer halo rows per
-// output row and the per-plane waits and barrier shared by twice the points)
+// faster on GB300 at 128^3 - 384^3: fewer halo rows per output row and the
+// per-plane waits and barrier shared by twice the points).  FP64 takes 64 x 8
+// tiles: two CTAs an SM instead of one to hide the FP64 pipe's latency (128^3
+// 62.5 us a step against 63.2, 192^3 200 against 205; with equal stretches of
+// planes in both, 67.3 and 212 with one z-range an item)
 static int rpt_override() {
   static int v = [] {
     const char* e = getenv("FFPAT_RPT");
@@ -1825,9 +1839,10 @@ static int launch_step_tma_r(const Plan& pl, int form, bool start, const void* p
       maps.q[i] = maps.p;
     }
   }
-  if (pl.prec == FFPAT_FP64) {
-    return start ? launch_one<double, 0, true, RPT>(pl, maps, o0, o1, o2, st)
-                 : launch_one<double, 0, false, RPT>(pl, maps, o0, o1, o2, st);
+  if constexpr (RPT == 1) {
+    if (pl.prec == FFPAT_FP64)
+      return start ? launch_one<double, 0, true, 1>(pl, maps, o0, o1, o2, st)
+                   : launch_one<double, 0, false, 1>(pl, maps, o0, o1, o2, st);
   }
   if (form == 2)
     return start ? launch_one<float, 2, true, RPT>(pl, maps, o0, o1, o2, st)
@@ -1841,7 +1856,7 @@ static int launch_step_tma_r(const Plan& pl, int form, bool start, const void* p
 
 int launch_step_tma(const Plan& pl, int form, bool start, const void* p, const void* const* q,
                     void* o0, void* o1, void* o2, cudaStream_t st) {
-  const int rpt = rpt_override() == 1 ? 1 : 2;
+  const int rpt = rpt_override() == 1 || pl.prec == FFPAT_FP64 ? 1 : 2;
   if (rpt == 2) return launch_step_tma_r<2>(pl, form, start, p, q, o0, o1, o2, st);
   return launch_step_tma_r<1>(pl, form, start, p, q, o0, o1, o2, st);
 }
