@@ -961,14 +961,18 @@ struct Batch2Req {
   int n, zc, tiles_x, tiles_y;
 };
 
+// CAP problems at most: the parameter block is copied with every launch, 0.5 KB a
+// problem
+template <int CAP>
 struct Batch2Params {
   int count;
-  int item_end[kMaxBatch];  // exclusive prefix of the problems' item counts
-  Batch2Req r[kMaxBatch];
+  int item_end[CAP];  // exclusive prefix of the problems' item counts
+  Batch2Req r[CAP];
 };
 
+template <int CAP>
 struct Step2Batch {
-  const Batch2Params* bp;
+  const Batch2Params<CAP>* bp;
   __device__ Step2Item operator()(int item) const {
     int r = 0;
     while (item >= bp->item_end[r]) ++r;
@@ -978,9 +982,10 @@ struct Step2Batch {
   }
 };
 
+template <int CAP>
 __global__ void __launch_bounds__(tb2::NT2, 1)
-    k_step2_batch(const __grid_constant__ Batch2Params bp) {
-  step2_body<1>(Step2Batch{&bp}, bp.item_end[bp.count - 1]);
+    k_step2_batch(const __grid_constant__ Batch2Params<CAP> bp) {
+  step2_body<1>(Step2Batch<CAP>{&bp}, bp.item_end[bp.count - 1]);
 }
 
 // ------------------------------------ resident time loop (small grids) --
@@ -1678,7 +1683,7 @@ int make_map_box(CUtensorMap* m, const void* base, int n, int np, int esize, int
 // in grid_dependency_sync before touching global memory).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t st, Args... args) {
+                       cudaStream_t st, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -1992,22 +1997,20 @@ int launch_step2_f32(const Plan& pl, const void* pm, const void* p, void* o1, vo
                       (float*)o1, (float*)o2);
 }
 
-int launch_step2_batch(const BatchStep2* steps, int count, cudaStream_t st) {
-  if (count < 1) return FFPAT_OK;
-  if (count > kMaxBatch)
-    return report(FFPAT_EINVAL, "batched two-step pass: %d requests > %d", count, kMaxBatch);
+template <int CAP>
+static int step2_batch(const BatchStep2* steps, int count, cudaStream_t st) {
   const size_t smem = tb2::smem_bytes<1>() + 1024;
   static cudaError_t attr = cudaErrorUnknown;
   static std::once_flag once;
   std::call_once(once, [&] {
-    attr = cudaFuncSetAttribute(k_step2_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    attr = cudaFuncSetAttribute(k_step2_batch<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
   });
   if (attr != cudaSuccess) {
     cudaGetLastError();
     return report(FFPAT_ECUDA, "k_step2_batch: %zu bytes of shared memory refused", smem);
   }
-  static thread_local Batch2Params bp;
+  static thread_local Batch2Params<CAP> bp;
   const int slots = kNumSMs;  // one CTA per SM
   const int len = batch_zrange(steps, count, tb2::TH2, slots);
   int total = 0;
@@ -2035,9 +2038,23 @@ int launch_step2_batch(const BatchStep2* steps, int count, cudaStream_t st) {
     bp.item_end[i] = total;
   }
   const int grid = total < slots ? total : slots;
-  k_step2_batch<<<grid, tb2::NT2, smem, st>>>(bp);
+  const cudaError_t e =
+      launch_pdl(k_step2_batch<CAP>, dim3(grid), dim3(tb2::NT2), smem, st, bp);
   count_launch();
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return report(FFPAT_ECUDA, "k_step2_batch launch: %s", cudaGetErrorString(e));
+  }
   return check_launch("k_step2_batch");
+}
+
+int launch_step2_batch(const BatchStep2* steps, int count, cudaStream_t st) {
+  if (count < 1) return FFPAT_OK;
+  if (count > kMaxBatchRequests)
+    return report(FFPAT_EINVAL, "batched two-step pass: %d requests > %d", count, kMaxBatchRequests);
+  if (count <= 4) return step2_batch<4>(steps, count, st);
+  if (count <= 10) return step2_batch<10>(steps, count, st);
+  return step2_batch<kMaxBatch>(steps, count, st);
 }
 
 // ---- the resident time loop (host side)
