@@ -232,6 +232,25 @@ __device__ __forceinline__ float2 lap12_pair(const Nb2& v) {
   return fma2(make_float2(16.0f, 16.0f), d1, nd2);
 }
 
+// The same Laplacian, bit for bit, for a thread that walks a z-column: the z-terms
+// from differences it already formed (a difference and its negative round alike:
+// p(z-1) - c is -(c - p(z-1)), the last plane's forward difference), and the
+// x-neighbours one lane at a time, without assembling the misaligned pairs.
+// dz = p(z+1) - p(z) and ez = p(z+2) - p(z) of this plane, dzm = dz of plane z - 1,
+// ezm = ez of plane z - 2.
+__device__ __forceinline__ float2 lap12_walk(float2 c, float2 xm, float2 xp, float2 ym1, float2 yp1,
+                                             float2 ym2, float2 yp2, float2 dz, float2 dzm,
+                                             float2 ez, float2 ezm) {
+  const float t = __fsub_rn(c.y, c.x);
+  float2 d1 = make_float2(__fadd_rn(__fsub_rn(xm.y, c.x), t), __fsub_rn(__fsub_rn(xp.x, c.y), t));
+  d1 = add2(d1, add2(sub2(ym1, c), sub2(yp1, c)));
+  d1 = add2(d1, sub2(dz, dzm));
+  float2 nd2 = add2(sub2(c, xm), sub2(c, xp));
+  nd2 = add2(nd2, add2(sub2(c, ym2), sub2(c, yp2)));
+  nd2 = add2(nd2, sub2(ezm, ez));
+  return fma2(make_float2(16.0f, 16.0f), d1, nd2);
+}
+
 // the neighbourhoods of the points at o and o + 1 (o even), read with eleven
 // 64-bit shared-memory loads
 __device__ __forceinline__ void gather_pair(const float* P0, const float* Pm1, const float* Pp1,
@@ -815,7 +834,8 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
       float2 c0 = lds2(P + 0 * (PB / 4) + o), c1 = lds2(P + 1 * (PB / 4) + o);
       float2 c2 = lds2(P + 2 * (PB / 4) + o), c3 = lds2(P + 3 * (PB / 4) + o);
       const float2 zero = make_float2(0.f, 0.f);
-      float2 a0 = zero, a1 = zero, a2 = zero, a3 = zero;
+      float2 dA = sub2(c2, c1), eA0 = sub2(c2, c0), eA1 = sub2(c3, c1);  // the column's differences
+      float2 a2 = zero, a3 = zero, dB = zero, eB0 = zero, eB1 = zero;
       float2 uq0 = zero, uq1 = zero, vq0 = zero, vq1 = zero, kq0 = zero, kq1 = zero;
       const int x = x0 + 2 * lane, y = y0 + warp;
       const bool store = inner && x < n && y < n;  // np % 4 == 0: x + 1 is in the row as well
@@ -834,22 +854,10 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
             const float* P0 = P + ((u + 2) & 7) * (PB / 4);
             const float* Qz = Q + NQF * ((u + 2) & 7) * (QB / 4);
             const float2 c4 = lds2(P + ((u + 4) & 7) * (PB / 4) + o);
-            Nb2 v;
-            const float2 XM = lds2(P0 + o - 2), XP = lds2(P0 + o + 2);
-            v.c = c2;
-            v.xm1 = make_float2(XM.y, c2.x);
-            v.xp1 = make_float2(c2.y, XP.x);
-            v.xm2 = XM;
-            v.xp2 = XP;
-            v.ym1 = lds2(P0 + o - PW);
-            v.yp1 = lds2(P0 + o + PW);
-            v.ym2 = lds2(P0 + o - 2 * PW);
-            v.yp2 = lds2(P0 + o + 2 * PW);
-            v.zm1 = c1;
-            v.zp1 = c3;
-            v.zm2 = c0;
-            v.zp2 = c4;
-            const float2 L = lap12_pair(v);
+            const float2 dz = sub2(c3, c2), ez = sub2(c4, c2);
+            const float2 L = lap12_walk(c2, lds2(P0 + o - 2), lds2(P0 + o + 2), lds2(P0 + o - PW),
+                                        lds2(P0 + o + PW), lds2(P0 + o - 2 * PW),
+                                        lds2(P0 + o + 2 * PW), dz, dA, ez, eA0);
             const float2 Kv = lds2(Qz + (NQF - 1) * (QB / 4) + qo);
             float2 an, un, vn;  // level n + 1 at the pair; the values step B takes
             if constexpr (FORM == 1) {
@@ -873,24 +881,12 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
               tb2_fail(abort);
             if (active) *reinterpret_cast<float2*>(A + (u & 3) * (AB / 4) + ao) = an;
             // ---- step B: level n + 2 at plane zB = z - 2 (tile rows only)
+            const float2 dzB = sub2(a3, a2), ezB = sub2(an, a2);
             if (inner && i >= 4) {
-              const float* A0 = A + ((u + 2) & 3) * (AB / 4);
-              Nb2 w;
-              const float2 YM = lds2(A0 + ao - 2), YP = lds2(A0 + ao + 2);
-              w.c = a2;
-              w.xm1 = make_float2(YM.y, a2.x);
-              w.xp1 = make_float2(a2.y, YP.x);
-              w.xm2 = YM;
-              w.xp2 = YP;
-              w.ym1 = lds2(A0 + ao - AW);
-              w.yp1 = lds2(A0 + ao + AW);
-              w.ym2 = lds2(A0 + ao - 2 * AW);
-              w.yp2 = lds2(A0 + ao + 2 * AW);
-              w.zm1 = a1;
-              w.zp1 = a3;
-              w.zm2 = a0;
-              w.zp2 = an;
-              const float2 LB = lap12_pair(w);
+              const float* A0 = A + ((u + 2) & 3) * (AB / 4) + ao;
+              const float2 LB =
+                  lap12_walk(a2, lds2(A0 - 2), lds2(A0 + 2), lds2(A0 - AW), lds2(A0 + AW),
+                             lds2(A0 - 2 * AW), lds2(A0 + 2 * AW), dzB, dB, ezB, eB0);
               if constexpr (FORM == 1) {
                 const Kp2 rb = kahan_pair(a2, kq0, LB, uq0, vq0, false);
                 if (store) {
@@ -904,14 +900,16 @@ __device__ __forceinline__ void step2_body(const Items& items, int nitems) {
               }
             }
             gi += plane;
-            c0 = c1;
-            c1 = c2;
             c2 = c3;
             c3 = c4;
-            a0 = a1;
-            a1 = a2;
+            dA = dz;
+            eA0 = eA1;
+            eA1 = ez;
             a2 = a3;
             a3 = an;
+            dB = dzB;
+            eB0 = eB1;
+            eB1 = ezB;
             uq0 = uq1;
             uq1 = un;
             vq0 = vq1;
