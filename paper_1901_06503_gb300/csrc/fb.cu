@@ -28,15 +28,14 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
-// sum `nq` rows of kReduceBlocks partials (fixed order) into dst[0..nq)
+// sum rows of kReduceBlocks partials (fixed order), one a CTA, into dst[row]
 __global__ void __launch_bounds__(kReduceThreads)
-    k_finalize(const double* __restrict__ partials, int nq, double* __restrict__ dst) {
-  for (int q = 0; q < nq; ++q) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < kReduceBlocks; i += blockDim.x) acc += partials[q * kReduceBlocks + i];
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) dst[q] = acc;
-  }
+    k_finalize(const double* __restrict__ partials, double* __restrict__ dst) {
+  const int q = blockIdx.x;
+  double acc = 0.0;
+  for (int i = threadIdx.x; i < kReduceBlocks; i += blockDim.x) acc += partials[q * kReduceBlocks + i];
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) dst[q] = acc;
 }
 
 // per CTA: max c, and whether any entry is not finite and > 0 (as a count).  The
@@ -432,7 +431,7 @@ int launch_dot(const Plan& pl, size_t len, const void* a, const void* b, double*
     k_dots<double><<<kReduceBlocks, kReduceThreads, 0, st>>>((const double*)a, (const double*)b, len, pl.partials);
   else
     k_dots<float><<<kReduceBlocks, kReduceThreads, 0, st>>>((const float*)a, (const float*)b, len, pl.partials);
-  k_finalize<<<1, kReduceThreads, 0, st>>>(pl.partials, 2, result);
+  k_finalize<<<2, kReduceThreads, 0, st>>>(pl.partials, result);
   count_launch(2);
   return check_launch(__func__);
 }
@@ -447,7 +446,7 @@ int launch_fb_update(const Plan& pl, void* h, const void* w, double step, double
     k_fb_update<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
         (float*)h, (const float*)w, (const float*)pl.kap, pl.n3, step, step_dev, lambda,
         (const float*)support, pl.partials);
-  k_finalize<<<1, kReduceThreads, 0, st>>>(pl.partials, 4, dst);
+  k_finalize<<<4, kReduceThreads, 0, st>>>(pl.partials, dst);
   count_launch(2);
   return check_launch(__func__);
 }
@@ -473,7 +472,7 @@ int launch_prox_finish(const Plan& pl, void* h, const void* hn, double* dst, cud
   else
     k_prox_finish<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
         (const float*)h, (const float*)hn, pl.n, q, pl.partials);
-  k_finalize<<<1, kReduceThreads, 0, st>>>(pl.partials, 4, dst);
+  k_finalize<<<4, kReduceThreads, 0, st>>>(pl.partials, dst);
   count_launch(2);
   if (check_launch(__func__) != FFPAT_OK) return FFPAT_ECUDA;
   if (cudaMemcpyAsync(h, hn, pl.n3 * pl.esize, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
@@ -499,7 +498,7 @@ int launch_resid_kap(const Plan& pl, const void* w, const void* g, void* x, doub
     k_resid_kap<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
         (const float*)w, (const float*)g, (const float*)pl.kap, (float*)x, pl.n3, pl.partials);
   }
-  k_finalize<<<1, kReduceThreads, 0, st>>>(pl.partials, 2, dst);
+  k_finalize<<<2, kReduceThreads, 0, st>>>(pl.partials, dst);
   count_launch(2);
   return check_launch(__func__);
 }

@@ -413,6 +413,7 @@ __global__ void __launch_bounds__(384)
   __syncthreads();
   const int lo = s_lo, hi = s_hi;
   wait_for_operand();
+  constexpr int kGroup = V == 1 ? 4 : 1;
   double acc0[V], acc1[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) acc0[v] = acc1[v] = 0.0;
@@ -438,40 +439,47 @@ __global__ void __launch_bounds__(384)
       at[e] = code;
     }
     __syncthreads();
-    auto sample = [&](int e, double (&acc)[V]) {
-      const int code = at[e];
-      if ((code & 15) == 0) return;  // adds an exact zero
-      const double2 wl = wlo[e], wh = whi[e];
-      const double* q = pz + (long long)(code >> 4) * zp;
-      const double* qh = q + (long long)n * zp;
-      double v[4][V];
+    // kGroup samples of both rays at a time: all their loads in flight, then the
+    // sums (each ray's samples in order)
+    for (int m = 0; m < ms; m += kGroup) {
+      double v[kGroup][2][4][V];
+      int code[kGroup][2];
 #pragma unroll
-      for (int i = 0; i < V; ++i) v[0][i] = v[1][i] = v[2][i] = v[3][i] = 0.0;
-      auto load = [&](const double* p, double (&d)[V]) {
-        if constexpr (V == 1) {
-          d[0] = __ldg(p);
-        } else {
-          const double2 t = __ldg(reinterpret_cast<const double2*>(p));
-          d[0] = t.x;
-          d[1] = t.y;
+      for (int q = 0; q < kGroup; ++q)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          code[q][r] = m + q < ms ? at[(m + q) * rg + r0 + r] : 0;
+          const double* p = pz + (long long)(code[q][r] >> 4) * zp;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const double* c = p + (k & 1 ? zp : 0) + (k & 2 ? (long long)n * zp : 0LL);
+            if constexpr (V == 1) {
+              v[q][r][k][0] = code[q][r] & (1 << k) ? __ldg(c) : 0.0;
+            } else {
+              const double2 t = code[q][r] & (1 << k) ? __ldg(reinterpret_cast<const double2*>(c))
+                                                      : make_double2(0.0, 0.0);
+              v[q][r][k][0] = t.x;
+              v[q][r][k][1] = t.y;
+            }
+          }
         }
-      };
-      if (code & 1) load(q, v[0]);
-      if (code & 2) load(q + zp, v[1]);
-      if (code & 4) load(qh, v[2]);
-      if (code & 8) load(qh + zp, v[3]);
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        double b = __dmul_rn(wl.x, v[0][i]);
-        b = __dadd_rn(b, __dmul_rn(wl.y, v[1][i]));
-        b = __dadd_rn(b, __dmul_rn(wh.x, v[2][i]));
-        b = __dadd_rn(b, __dmul_rn(wh.y, v[3][i]));
-        acc[i] = __dadd_rn(acc[i], b);
-      }
-    };
-    for (int m = 0; m < ms; ++m) {
-      sample(m * rg + r0, acc0);
-      sample(m * rg + r0 + 1, acc1);
+      for (int q = 0; q < kGroup; ++q)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if ((code[q][r] & 15) == 0) continue;  // adds an exact zero
+          const int e = (m + q) * rg + r0 + r;
+          const double2 wl = wlo[e], wh = whi[e];
+          double(&acc)[V] = r == 0 ? acc0 : acc1;
+#pragma unroll
+          for (int i = 0; i < V; ++i) {
+            double b = __dmul_rn(wl.x, v[q][r][0][i]);
+            b = __dadd_rn(b, __dmul_rn(wl.y, v[q][r][1][i]));
+            b = __dadd_rn(b, __dmul_rn(wh.x, v[q][r][2][i]));
+            b = __dadd_rn(b, __dmul_rn(wh.y, v[q][r][3][i]));
+            acc[i] = __dadd_rn(acc[i], b);
+          }
+        }
     }
   }
   __syncthreads();
@@ -697,7 +705,7 @@ __global__ void __launch_bounds__(128)
     __syncwarp();
     if (ja + lane < nth) {
       const double cs = tab[ja + lane], sn = tab[nth + ja + lane];
-#pragma unroll 1
+#pragma unroll(V == 1 ? 2 : 1)
       for (int v = 0; v < 4; ++v) {
         const double X = (x0 + (v & 1)) - 0.5 * (n - 1), Y = (y0 + (v >> 1)) - 0.5 * (n - 1);
         const double kk = fma(X, cs, Y * sn) + 0.5 * (n - 1);
@@ -727,29 +735,59 @@ __global__ void __launch_bounds__(128)
     const int jn = min(kB64Angles, nth - ja);
     for (int t = 0; t < jn; ++t) {
       const double* row = gz + (long long)(ja + t) * n * zp;
+      if constexpr (V == 4) {
+        // enough planes a lane to cover the loads' latency
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const int on = info[t * 4 + v];
-        const double* q = row + (long long)(on >> 3) * zp;
+        for (int v = 0; v < 4; ++v) {
+          const int on = info[t * 4 + v];
+          const double* q = row + (long long)(on >> 3) * zp;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          if (on & (1 << i)) {
-            const double w = W[(t * 4 + v) * 3 + i];
-            if constexpr (V == 1) {
-              acc[v][0] = fma(w, __ldg(q + i * zp), acc[v][0]);
-            } else {
+          for (int i = 0; i < 3; ++i)
+            if (on & (1 << i)) {
+              const double w = W[(t * 4 + v) * 3 + i];
               const double2 d = __ldg(reinterpret_cast<const double2*>(q + i * zp));
               acc[v][0] = fma(w, d.x, acc[v][0]);
               acc[v][1] = fma(w, d.y, acc[v][1]);
-              if constexpr (V == 4) {
-                if (hi_ok) {
-                  const double2 e = __ldg(reinterpret_cast<const double2*>(q + i * zp + 2));
-                  acc[v][2] = fma(w, e.x, acc[v][2]);
-                  acc[v][3] = fma(w, e.y, acc[v][3]);
-                }
+              if (hi_ok) {
+                const double2 e = __ldg(reinterpret_cast<const double2*>(q + i * zp + 2));
+                acc[v][2] = fma(w, e.x, acc[v][2]);
+                acc[v][3] = fma(w, e.y, acc[v][3]);
+              }
+            }
+        }
+      } else {
+        // the detectors of NV voxels in flight, then their multiply-adds
+        constexpr int NV = V == 1 ? 4 : 2;
+#pragma unroll
+        for (int v0 = 0; v0 < 4; v0 += NV) {
+          double d[NV][3][V];
+          int on[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            on[v] = info[t * 4 + v0 + v];
+            const double* q = row + (long long)(on[v] >> 3) * zp;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              const bool use = on[v] & (1 << i);
+              if constexpr (V == 1) {
+                d[v][i][0] = use ? __ldg(q + i * zp) : 0.0;
+              } else {
+                const double2 a = use ? __ldg(reinterpret_cast<const double2*>(q + i * zp))
+                                      : make_double2(0.0, 0.0);
+                d[v][i][0] = a.x;
+                d[v][i][1] = a.y;
               }
             }
           }
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+              if (on[v] & (1 << i)) {
+                const double w = W[(t * 4 + v0 + v) * 3 + i];
+#pragma unroll
+                for (int k = 0; k < V; ++k) acc[v0 + v][k] = fma(w, d[v][i][k], acc[v0 + v][k]);
+              }
         }
       }
     }
@@ -979,13 +1017,14 @@ static void with_slab(int rl, Fn f) {
 }
 
 // FP64: planes per lane, of the widths 1, 2 and 4 up to vmax the one of least
-// cost (FP64 instructions, idle lanes included, plus a little per slab); the
-// wider on ties
-static int choose_v64(int n, int vmax) {
+// cost: FP64 instructions, idle lanes included, plus `extra` per slab for what a
+// slab repeats (the weights of P^T: about 60 instructions a voxel and angle
+// against 2.3 V; P's lists serve all slabs of a CTA); the wider on ties
+static int choose_v64(int n, int vmax, float extra) {
   int best = 1;
   float best_cost = 1e30f;
   for (int v = 1; v <= vmax; v *= 2) {
-    const float c = ((float)v + 0.3f) * (float)((n + 32 * v - 1) / (32 * v));
+    const float c = ((float)v + extra) * (float)((n + 32 * v - 1) / (32 * v));
     if (c <= best_cost) {
       best = v;
       best_cost = c;
@@ -1002,7 +1041,7 @@ int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cuda
   if (pl.prec == FFPAT_FP64) {
     const int rc = launch_zlast<double>(p, scratch, n, n, n, so, sz, rl, st);
     if (rc != FFPAT_OK) return rc;
-    const int V = choose_v64(n, 2);
+    const int V = choose_v64(n, 2, 0.2f);
     // slabs of 32 V planes, up to four of them in a CTA (they share the sample
     // lists), two rays a warp and at most 12 warps; fewer rays a CTA while the
     // grid would not give every SM two
@@ -1044,7 +1083,7 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
   if (pl.prec == FFPAT_FP64) {
     const int rc = launch_zlast<double>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
     if (rc != FFPAT_OK) return rc;
-    const int V = choose_v64(n, 4), vs = (n + 32 * V - 1) / (32 * V);
+    const int V = choose_v64(n, 4, 0.8f), vs = (n + 32 * V - 1) / (32 * V);
     int tb = 2;  // tb x tb blocks of 2 x 2 voxels a CTA
     if ((long long)((n + 3) / 4) * ((n + 3) / 4) * vs < 2 * kNumSMs) tb = 1;
     const int side = 2 * tb, tiles = (n + side - 1) / side;
