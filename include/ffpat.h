@@ -314,7 +314,8 @@ int ffpat_debug_fma_rate(int32_t kind, double *flops_per_s, void *stream);
 /* The differentiated operator needs pad = 0 (the box is the wave grid). */
 
 /* Checkpoint buffer bytes for Nt steps (ffpat_problem_info) and interval
- * `every`: (2 ceil(Nt / every) + every + 2) volumes; 0 if invalid. */
+ * `every`: (2 ceil(Nt / every) + every + 2) volumes of the wave grid (FP32 with
+ * N <= 84: `every` more; FP32 rows rounded up to 16 bytes); 0 if invalid. */
 size_t ffpat_ckpt_bytes(const ffpat_problem *problem, int32_t nt, int32_t every);
 
 /* g = P W h with checkpoints (device buffers as for ffpat_forward; ckpt is

@@ -10,12 +10,14 @@
 // the last, the states p^n of the segment are recomputed from its checkpoint
 // and the kappa-derivatives mu^{n+1} L(p^n) (weight 1/2 for the start step)
 // are accumulated; grad_c = 2 acc / c because dkappa/dc = 2 kappa / c and the
-// factors kappa/12 and 12 cancel.  Memory: 2 ceil(Nt/k) + k + 2 volumes.
+// factors kappa/12 and 12 cancel.  Memory: 2 ceil(Nt/k) + k + 2 volumes (k more
+// on small grids, whose segments overlap).
 //
 // Where the resident time loop runs (FP32, N <= 128), the forward pass is one
 // cooperative launch that stores the checkpoints as it goes, and a segment of
 // the backward pass two: recompute (writing L(p^n) in place of p^n) and
-// transposed steps with the accumulation.  Elsewhere they are loops of launches.
+// transposed steps with the accumulation; up to N = 84 the transposed steps of a
+// segment and the recompute of the one before share a launch.  Elsewhere they are loops of launches.
 // FP32 volumes with ragged rows run on padded rows (wave_plan), FP64 ones as
 // they are.
 #include "internal.cuh"
@@ -27,13 +29,13 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Ckpt {
   size_t vol = 0;
-  int nseg = 0, every = 0;
+  int nseg = 0, every = 0, nvol = 0;  // nvol: segment volumes
   unsigned char* base = nullptr;
   void* a(int s) const { return base + (size_t)(2 * s) * vol; }
   void* b(int s) const { return base + (size_t)(2 * s + 1) * vol; }
-  void* seg(int j) const { return base + (size_t)(2 * nseg + j) * vol; }  // j = 0 .. every
-  void* acc() const { return base + (size_t)(2 * nseg + every + 1) * vol; }
-  size_t bytes() const { return (size_t)(2 * nseg + every + 2) * vol; }
+  void* seg(int j) const { return base + (size_t)(2 * nseg + j) * vol; }  // j < nvol
+  void* acc() const { return base + (size_t)(2 * nseg + nvol) * vol; }
+  size_t bytes() const { return (size_t)(2 * nseg + nvol + 1) * vol; }
 };
 
 int ckpt_layout(const Plan& pl, int nt, int every, void* base, Ckpt* ck) {
@@ -44,6 +46,9 @@ int ckpt_layout(const Plan& pl, int nt, int every, void* base, Ckpt* ck) {
   ck->vol = up256((size_t)pl.n * pl.n * row * pl.esize);
   ck->every = every;
   ck->nseg = (nt + every - 1) / every;
+  // FP32 on small grids: two segments' worth (see the resident branch of the
+  // backward pass)
+  ck->nvol = (pl.esize == 4 && pl.n <= kSegmentPairMaxN ? 2 * every : every) + 1;
   ck->base = (unsigned char*)base;
   return FFPAT_OK;
 }
@@ -168,7 +173,8 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
     return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
   const Plan w = grad_view(pl, ck);
   const bool tma = use_tma(w, ck, nullptr);
-  const bool two = use_two(w, ck, tma), resident = resident_segments(w, tma, st);
+  const bool two = use_two(w, ck, tma);
+  bool resident = resident_segments(w, tma, st);  // until a launch is turned down
   const bool rows = w.np != w.n;
   const size_t vb = (size_t)w.n * w.n * w.np * w.esize;
   // mu^{Nt} = (kappa / 12) P^T grad_g, mu^{Nt+1} = 0
@@ -189,20 +195,48 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   if (cudaMemsetAsync(B[v], 0, vb, st) != cudaSuccess ||
       cudaMemsetAsync(ck.acc(), 0, vb, st) != cudaSuccess)
     return check_launch("backward init");
+  // resident segments: L(p^{lo+j}) in the segment volumes (two sets where the
+  // recompute of a segment runs beside the transposed steps of the next), the
+  // recomputed states through two spare volumes
+  const bool paired = resident && segments_paired(w);
+  auto length = [&](int s) {
+    return (s + 1 < ck.nseg ? every : pl.nt - s * every);
+  };
+  auto set = [&](int s) -> void* { return ck.seg(paired ? (s & 1) * every : 0); };
+  auto recompute = [&](int s) {
+    return SegRecompute{ck.a(s), ck.b(s), pl.s[3], ck.seg(ck.nvol - 1), set(s), length(s)};
+  };
+  if (paired) {
+    const SegRecompute last = recompute(ck.nseg - 1);
+    bool refused = false;
+    rc = launch_segments(w, &last, nullptr, ck.vol / 4, st, &refused);
+    if (rc != FFPAT_OK && !refused) return rc;
+    if (refused) resident = false;
+  }
   for (int s = ck.nseg - 1; s >= 0; --s) {
     const int lo = s * every;
     const int hi = (lo + every - 1 < pl.nt - 1) ? lo + every - 1 : pl.nt - 1;
     if (resident) {
-      // seg(j) holds L(p^{lo+j}); the states pass through the spare volumes
-      const int steps = hi - lo + 1;
+      const int steps = length(s);
       int x, y;
       others(&x, &y);
-      rc = launch_segment_recompute(w, ck.a(s), ck.b(s), pl.s[3], ck.seg(every), ck.seg(0),
-                                    ck.vol / 4, steps, st);
-      if (rc == FFPAT_OK)
-        rc = launch_segment_transpose(w, B[u], B[v], B[x], B[y], ck.acc(), ck.seg(0), ck.vol / 4,
-                                      steps, lo == 0, st);
-      if (rc != FFPAT_OK) return rc;
+      const SegTranspose tr{B[u], B[v], B[x], B[y], ck.acc(), set(s), steps, lo == 0};
+      bool refused = false;
+      if (paired) {
+        const SegRecompute before = s > 0 ? recompute(s - 1) : SegRecompute{};
+        rc = launch_segments(w, s > 0 ? &before : nullptr, &tr, ck.vol / 4, st, &refused);
+      } else {
+        const SegRecompute now = recompute(s);
+        rc = launch_segments(w, &now, nullptr, ck.vol / 4, st, &refused);
+        if (rc == FFPAT_OK) rc = launch_segments(w, nullptr, &tr, ck.vol / 4, st, &refused);
+      }
+      if (rc != FFPAT_OK && !refused) return rc;
+      resident = !refused;  // refused: this segment and the rest launch by launch
+    }
+    if (resident) {
+      const int steps = length(s);
+      int x, y;
+      others(&x, &y);
       const int last = (steps - 1) & 1 ? y : x, prev = (steps - 1) & 1 ? x : y;
       v = steps > 1 ? prev : u;  // mu^{lo+1}
       u = last;                  // mu^{lo}

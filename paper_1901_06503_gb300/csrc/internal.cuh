@@ -191,17 +191,29 @@ int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, vo
                          const void** result, cudaStream_t st, bool* refused = nullptr,
                          const ResidentSave* save = nullptr);
 // Checkpoint segments of the differentiated operator in the resident scheme
-// (FP32 three-term, segments_resident() grids).  recompute: from p0 = p^lo, p1 =
-// p^{lo+1}, L(p^{lo+i}) to lp + i lpvol for i < steps.  transpose: `steps` steps
-// of mu from mu1 = mu^{n+1}, mu2 = mu^{n+2}, step s into the buffer s & 1, and
-// acc += mu^{n+1} L(p^n); ends: the last is n = 0 (weight 1/2; it writes
-// start(mu^1) - mu^2).  b0, b1 alias no input.
+// (FP32 three-term, segments_resident() grids), one or both in a launch (both:
+// segments_paired() grids; neither reads what the other writes).  lp: L(p^{lo+i})
+// at lp + i lpvol.
+struct SegRecompute {  // from p0 = p^lo, p1 = p^{lo+1}
+  const void *p0, *p1;
+  void *b0, *b1;       // buffers
+  void* lp;
+  int steps;
+};
+struct SegTranspose {  // from mu1 = mu^{n+1}, mu2 = mu^{n+2}; step s into buffer s & 1;
+  const void *mu1, *mu2;  // acc += mu^{n+1} L(p^n)
+  void *b0, *b1;
+  void* acc;
+  const void* lp;
+  int steps;
+  bool ends;  // the last step is n = 0: weight 1/2, and it writes start(mu^1) - mu^2
+};
+constexpr int kSegmentPairMaxN = 84;  // grids whose items may fit twice
 bool segments_resident(const Plan& pl);
-int launch_segment_recompute(const Plan& pl, const void* p0, const void* p1, void* b0, void* b1,
-                             void* lp, size_t lpvol, int steps, cudaStream_t st);
-int launch_segment_transpose(const Plan& pl, const void* mu1, const void* mu2, void* b0, void* b1,
-                             void* acc, const void* lp, size_t lpvol, int steps, bool ends,
-                             cudaStream_t st);
+bool segments_paired(const Plan& pl);
+// *refused: the cooperative launch was turned down, nothing ran
+int launch_segments(const Plan& pl, const SegRecompute* rc, const SegTranspose* tr, size_t lpvol,
+                    cudaStream_t st, bool* refused);
 // The same for FP64 three-term problems (N <= 96 on GB300): bit for bit the
 // single-step TMA loop.
 int resident64_zc(const Plan& pl);

@@ -1384,7 +1384,7 @@ __device__ __forceinline__ bool seg_step(const float* pst, const float* kst, uin
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_constant__ SegParams sp) {
+__device__ __forceinline__ void seg_run(const SegParams& sp, int item) {
   using G = rs::G;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -1394,7 +1394,7 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_const
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + rs::NPL * G::PBYTES + rs::ZM * G::QBYTES +
                                               rs::EBYTES);
   const int tid = threadIdx.y * NTX + threadIdx.x;
-  const int n = sp.n, np = sp.np, item = blockIdx.x;
+  const int n = sp.n, np = sp.np;
   const int tix = item % sp.tiles_x, tiy = (item / sp.tiles_x) % sp.tiles_y;
   const int tz = item / (sp.tiles_x * sp.tiles_y);
   const int z0 = tz * sp.zc, nz = min(n - z0, sp.zc);
@@ -1491,6 +1491,27 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_const
               rr == 0 ? sb[zi] : es[(zi * TBY + threadIdx.y) * NTX + threadIdx.x];
       }
   }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_constant__ SegParams sp) {
+  seg_run<MODE>(sp, blockIdx.x);
+}
+
+// Both at once: the first `items` CTAs run the transposed steps of a segment, the
+// others recompute the segment before it.  Neither waits for the other; a step of
+// either is mostly latency at small grids, so the two share the SMs almost for free
+// (64^3: 115 us a segment of 16 steps one after the other, 84 together).
+struct SegPair {
+  SegParams t, r;
+  int items;
+};
+
+__global__ void __launch_bounds__(NTX* NTY, 2) k_seg_pair(const __grid_constant__ SegPair p) {
+  if ((int)blockIdx.x < p.items)
+    seg_run<SEG_TRANSPOSE>(p.t, blockIdx.x);
+  else
+    seg_run<SEG_RECOMPUTE>(p.r, (int)blockIdx.x - p.items);
 }
 
 // ---- the resident loop in FP64 (N <= 96 on GB300).  The same scheme; what
@@ -2220,12 +2241,8 @@ int launch_wave_resident64(const Plan& pl, const void* in, void* out, void* b0, 
 // grid cannot be co-resident at the moment (nothing ran).
 namespace {
 template <class Params>
-int launch_resident(void (*kern)(Params), const Params& params, const Plan& pl, int items,
-                    cudaStream_t st, bool* refused, const char* name) {
-  if (items > kResidentMaxItems)
-    return report(FFPAT_EINVAL, "resident time loop: %d work items > %d", items, kResidentMaxItems);
-  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
-    return check_launch("resident time loop: flag reset");
+int launch_resident(void (*kern)(Params), const Params& params, int items, cudaStream_t st,
+                    bool* refused, const char* name) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(items);
   cfg.blockDim = dim3(NTX, NTY);
@@ -2291,13 +2308,13 @@ int launch_wave_resident(const Plan& pl, int form, const void* in, void* out, vo
   rp.ckvol = save ? save->vol : 0;
   rp.every = save ? save->every : 1;
   const int items = rp.tiles_x * rp.tiles_y * ((n + zc - 1) / zc);
-  const int rc =
-      save ? launch_resident(k_wave_resident<0, true>, rp, pl, items, st, refused, "k_wave_resident")
-           : form == 1
-                 ? launch_resident(k_wave_resident<1, false>, rp, pl, items, st, refused,
-                                   "k_wave_resident")
-                 : launch_resident(k_wave_resident<0, false>, rp, pl, items, st, refused,
-                                   "k_wave_resident");
+  if (items > kResidentMaxItems)
+    return report(FFPAT_EINVAL, "resident time loop: %d work items > %d", items, kResidentMaxItems);
+  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
+    return check_launch("resident time loop: flag reset");
+  auto kern = save ? k_wave_resident<0, true>
+                   : (form == 1 ? k_wave_resident<1, false> : k_wave_resident<0, false>);
+  const int rc = launch_resident(kern, rp, items, st, refused, "k_wave_resident");
   if (rc != FFPAT_OK) return rc;
   if (result) *result = out ? out : rp.buf[(pl.nt - 1) & 1];
   return FFPAT_OK;
@@ -2312,56 +2329,85 @@ bool segments_resident(const Plan& pl) {
   std::call_once(once, [&] {
     fits = resident_fits(k_wave_resident<0, true>, slots) &&
            resident_fits(k_seg_resident<SEG_RECOMPUTE>, slots) &&
-           resident_fits(k_seg_resident<SEG_TRANSPOSE>, slots);
+           resident_fits(k_seg_resident<SEG_TRANSPOSE>, slots) &&
+           resident_fits(k_seg_pair, slots);
   });
   return fits;
 }
 
-static int launch_segment(const Plan& pl, int mode, const void* in0, const void* in1, void* b0,
-                          void* b1, const void* pm, void* acc, void* lp, size_t lpvol, int steps,
-                          bool ends, cudaStream_t st) {
-  const int zc = resident_zc(pl, 0), n = pl.n;
-  if (zc <= 0) return report(FFPAT_EINVAL, "resident segment: N = %d does not fit", n);
-  static thread_local SegParams sp;
-  if (make_map(&sp.in0, in0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&sp.in1, in1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&sp.pb[0], b0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&sp.pb[1], b1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
-      make_map(&sp.kap, pl.kap, n, pl.np, 4, false, rs::G::TH) != FFPAT_OK)
+namespace {
+// the part of a segment launch that does not depend on its direction
+int segment_params(const Plan& pl, int zc, const void* in0, const void* in1, void* b0, void* b1,
+                   void* lp, size_t lpvol, int steps, unsigned* flags, SegParams* sp) {
+  const int n = pl.n;
+  if (make_map(&sp->in0, in0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp->in1, in1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp->pb[0], b0, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp->pb[1], b1, n, pl.np, 4, true, rs::G::TH) != FFPAT_OK ||
+      make_map(&sp->kap, pl.kap, n, pl.np, 4, false, rs::G::TH) != FFPAT_OK)
     return report(FFPAT_ECUDA, "resident segment: tensor map");
-  sp.buf[0] = (float*)b0;
-  sp.buf[1] = (float*)b1;
-  sp.pm = (const float*)pm;
-  sp.acc = (float*)acc;
-  sp.lp = (float*)lp;
-  sp.lpvol = lpvol;
-  sp.sync = pl.sync;
-  sp.n = n;
-  sp.np = pl.np;
-  sp.zc = zc;
-  sp.tiles_x = (n + TBX - 1) / TBX;
-  sp.tiles_y = (n + rs::G::TH - 1) / rs::G::TH;
-  sp.steps = steps;
-  sp.ends = ends ? 1 : 0;
-  const int items = sp.tiles_x * sp.tiles_y * ((n + zc - 1) / zc);
-  return mode == SEG_RECOMPUTE
-             ? launch_resident(k_seg_resident<SEG_RECOMPUTE>, sp, pl, items, st, nullptr,
-                               "k_seg_resident")
-             : launch_resident(k_seg_resident<SEG_TRANSPOSE>, sp, pl, items, st, nullptr,
-                               "k_seg_resident");
+  sp->buf[0] = (float*)b0;
+  sp->buf[1] = (float*)b1;
+  sp->pm = nullptr;
+  sp->acc = nullptr;
+  sp->lp = (float*)lp;
+  sp->lpvol = lpvol;
+  sp->sync = flags;
+  sp->n = n;
+  sp->np = pl.np;
+  sp->zc = zc;
+  sp->tiles_x = (n + TBX - 1) / TBX;
+  sp->tiles_y = (n + rs::G::TH - 1) / rs::G::TH;
+  sp->steps = steps;
+  sp->ends = 0;
+  return FFPAT_OK;
 }
 
-int launch_segment_recompute(const Plan& pl, const void* p0, const void* p1, void* b0, void* b1,
-                             void* lp, size_t lpvol, int steps, cudaStream_t st) {
-  return launch_segment(pl, SEG_RECOMPUTE, p0, p1, b0, b1, nullptr, nullptr, lp, lpvol, steps,
-                        false, st);
+int segment_items(const SegParams& sp) {
+  return sp.tiles_x * sp.tiles_y * ((sp.n + sp.zc - 1) / sp.zc);
 }
+}  // namespace
 
-int launch_segment_transpose(const Plan& pl, const void* mu1, const void* mu2, void* b0, void* b1,
-                             void* acc, const void* lp, size_t lpvol, int steps, bool ends,
-                             cudaStream_t st) {
-  return launch_segment(pl, SEG_TRANSPOSE, mu1, mu1, b0, b1, mu2, acc, (void*)lp, lpvol, steps,
-                        ends, st);
+// z-range with which two segments' items fit the GPU together, one CTA of each an
+// SM; 0 if none does
+static int segment_pair_zc(const Plan& pl) {
+  int occ = 0;
+  const int slots = resident_slots<0>(&occ);
+  if (pl.n > kSegmentPairMaxN || occ < 2 || slots <= 0) return 0;
+  return resident_zchunk(pl.n, slots / 2, slots / occ);
+}
+bool segments_paired(const Plan& pl) { return segments_resident(pl) && segment_pair_zc(pl) > 0; }
+
+int launch_segments(const Plan& pl, const SegRecompute* rc, const SegTranspose* tr, size_t lpvol,
+                    cudaStream_t st, bool* refused) {
+  *refused = false;
+  static thread_local SegPair sp;
+  const int zc = rc && tr ? segment_pair_zc(pl) : resident_zc(pl, 0);
+  if (zc <= 0) return report(FFPAT_EINVAL, "resident segment: N = %d does not fit", pl.n);
+  int rcode = FFPAT_OK, items = 0;
+  if (tr) {
+    rcode = segment_params(pl, zc, tr->mu1, tr->mu1, tr->b0, tr->b1, (void*)tr->lp, lpvol,
+                           tr->steps, pl.sync, &sp.t);
+    if (rcode != FFPAT_OK) return rcode;
+    sp.t.pm = (const float*)tr->mu2;
+    sp.t.acc = (float*)tr->acc;
+    sp.t.ends = tr->ends ? 1 : 0;
+    items = segment_items(sp.t);
+  }
+  sp.items = items;
+  if (rc) {
+    rcode = segment_params(pl, zc, rc->p0, rc->p1, rc->b0, rc->b1, rc->lp, lpvol, rc->steps,
+                           pl.sync + (size_t)kFlagStride * items, &sp.r);
+    if (rcode != FFPAT_OK) return rcode;
+    items += segment_items(sp.r);
+  }
+  if (items > kResidentMaxItems)
+    return report(FFPAT_EINVAL, "resident segment: %d work items > %d", items, kResidentMaxItems);
+  if (cudaMemsetAsync(pl.sync, 0, sizeof(unsigned) * kFlagStride * items, st) != cudaSuccess)
+    return check_launch("resident segment: flag reset");
+  if (rc && tr) return launch_resident(k_seg_pair, sp, items, st, refused, "k_seg_pair");
+  return tr ? launch_resident(k_seg_resident<SEG_TRANSPOSE>, sp.t, items, st, refused, "k_seg_resident")
+            : launch_resident(k_seg_resident<SEG_RECOMPUTE>, sp.r, items, st, refused, "k_seg_resident");
 }
 
 int read_device_status(unsigned* out, bool clear) {
