@@ -1501,7 +1501,7 @@ __global__ void __launch_bounds__(NTX* NTY, 2) k_seg_resident(const __grid_const
 // Both at once: the first `items` CTAs run the transposed steps of a segment, the
 // others recompute the segment before it.  Neither waits for the other; a step of
 // either is mostly latency at small grids, so the two share the SMs almost for free
-// (64^3: 115 us a segment of 16 steps one after the other, 84 together).
+// (64^3: 114 us a segment of 16 steps one after the other, 68 together).
 struct SegPair {
   SegParams t, r;
   int items;
