@@ -831,7 +831,9 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
 }
 
 // P or P^T alone: the angle tables and the z-innermost operand in one
-// stream-ordered allocation.
+// stream-ordered allocation, at most about kAloneScratch of it (larger operands go
+// in several passes over z, so that they may fill most of the device).
+constexpr size_t kAloneScratch = (size_t)1 << 30;
 static int project_alone(const ffpat_problem* problem, const void* in, void* out, bool transpose,
                          cudaStream_t st) {
   Plan pl;
@@ -839,15 +841,16 @@ static int project_alone(const ffpat_problem* problem, const void* in, void* out
   TRY(validate(problem, pl));
   if (!in || !out) return fail(FFPAT_EINVAL, transpose ? "g or h is NULL" : "p or g is NULL");
   const size_t tb = up256(table_bytes(pl.nth));
-  const size_t zb = transpose ? zdata_bytes(pl.nw, pl.nth, pl.esize) : zvolume_bytes(pl.nw, pl.esize);
+  const size_t rows = (size_t)pl.nw * (transpose ? pl.nth : pl.nw);
+  const size_t zb = zscratch_bytes(pl.nw, rows, pl.esize, kAloneScratch);
   char* mem = nullptr;
   CK(cudaMallocAsync((void**)&mem, tb + zb, st));
   std::vector<unsigned char> tabs;
   int rc = upload_tables(pl, mem, tabs, st);
   const Plan wp = dense_rows(wave_plan(pl));
   if (rc == FFPAT_OK)
-    rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb)
-                   : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb);
+    rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb, 1.0, kAloneScratch)
+                   : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb, kAloneScratch);
   const cudaError_t ef = cudaFreeAsync(mem, st), es = cudaStreamSynchronize(st);
   TRY(rc);
   CK(ef);

@@ -233,14 +233,19 @@ int launch_wait_timeout(long long cycles, cudaStream_t st);
 // bytes of a volume / of the data (n detectors, nth angles) with z innermost
 size_t zvolume_bytes(int n, size_t esize);
 size_t zdata_bytes(int n, int nth, size_t esize);
+// the same for `rows` rows when at most `limit` bytes are to be used (0: no limit),
+// the planes then going in several passes
+size_t zscratch_bytes(int n, size_t rows, size_t esize, size_t limit);
 // g = mask .* (P p - sub)  (sub, mask nullable)
-// scratch: zvolume_bytes that alias neither p nor g; receives p with z innermost
+// scratch: zvolume_bytes (zscratch_bytes(n, n^2, .) with a limit) that alias neither
+// p nor g; receives p with z innermost
 int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
-                   const void* mask, void* scratch);
+                   const void* mask, void* scratch, size_t limit = 0);
 // h = mult * scale .* P^T g  (scale nullable)
-// scratch: zdata_bytes that alias neither g nor h; receives g with z innermost
+// scratch: zdata_bytes (zscratch_bytes(n, nth n, .) with a limit) that alias neither
+// g nor h; receives g with z innermost
 int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       void* scratch, double mult = 1.0);
+                       void* scratch, double mult = 1.0, size_t limit = 0);
 // out = mask .* (Lambda r)  (mask nullable)
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st,
                 const void* mask = nullptr);

@@ -294,7 +294,7 @@ template <int V, int C>
 __global__ void __launch_bounds__(kPWarps * 32, 2)
     k_project_z(const float* __restrict__ pt, float* __restrict__ g,
                 const float* __restrict__ sub, const float* __restrict__ mask,
-                const int32_t* __restrict__ tabi, int n, int nth, int ns, int nimg,
+                const int32_t* __restrict__ tabi, int n, int nz, int nth, int ns, int nimg,
                 int rg, int ch) {
   constexpr int RL = ZRow<V, C>::RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
   const float scale = 2.0f / (float)nimg;
   for (int e = tid; e < RL * rg; e += blockDim.x) {
     const int r = e % rg, zl = e / rg;
-    if (k0 + r >= n || zbase + zl >= n) continue;
+    if (k0 + r >= n || zbase + zl >= nz) continue;
     const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
     float sum = stage[zl * (rg + 1) + r];
     for (int q = 1; q < split; ++q) sum += stage[(q * RL + zl) * (rg + 1) + r];
@@ -381,8 +381,8 @@ template <int V>
 __global__ void __launch_bounds__(384)
     k_project_z64(const double* __restrict__ pt, double* __restrict__ g,
                   const double* __restrict__ sub, const double* __restrict__ mask,
-                  const double* __restrict__ tab, const float* __restrict__ tabf, int n, int nth,
-                  int ns, int nimg, int zp, int nslab, int rg) {
+                  const double* __restrict__ tab, const float* __restrict__ tabf, int n, int nz,
+                  int nth, int ns, int nimg, int zp, int nslab, int rg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* wlo = reinterpret_cast<double2*>(smem_raw);               // row j0: (x0, x0 + 1)
   double2* whi = wlo + (size_t)kP64Samples * rg;                      // row j0 + 1
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(384)
   __syncthreads();
   for (int e = tid; e < nslab * 32 * V * rg; e += blockDim.x) {
     const int r = e % rg, zl = e / rg;
-    if (k0 + r >= n || zbase + zl >= n) continue;
+    if (k0 + r >= n || zbase + zl >= nz) continue;
     const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
     double out = __dmul_rn(dx, stage[zl * (rg + 1) + r]);
     if (sub) out = out - sub[o];
@@ -572,8 +572,8 @@ template <int V, int C>
 __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
     k_backproject_z(const float* __restrict__ gt, float* __restrict__ h,
                     const float* __restrict__ scale, const float* __restrict__ tabf,
-                    const int32_t* __restrict__ tabi, int n, int np, int nth, int ns, int nimg,
-                    int tx,
+                    const int32_t* __restrict__ tabi, int n, int np, int nz, int nth, int ns,
+                    int nimg, int tx,
                     float mult) {
   constexpr int RL = ZRow<V, C>::RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
       const int v = e % nv, zl = e / nv;
       const int x = blockIdx.x * sx + v % sx, y = blockIdx.y * 2 * ty + v / sx;
       const int z = zbase + c * 32 * V + zl;
-      if (x >= n || y >= n || z >= n) continue;
+      if (x >= n || y >= n || z >= nz) continue;
       const size_t o = ((size_t)z * n + y) * np + x;
       float out = f * stage[zl * (nv + 1) + v];
       if (scale) out *= scale[o];
@@ -686,7 +686,7 @@ template <int V>
 __global__ void __launch_bounds__(128)
     k_backproject_z64(const double* __restrict__ gt, double* __restrict__ h,
                       const double* __restrict__ scale, const double* __restrict__ tab, int n,
-                      int np, int nth, int ns, int nimg, int zp, int tb, double mult) {
+                      int np, int nz, int nth, int ns, int nimg, int zp, int tb, double mult) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double* W = reinterpret_cast<double*>(smem_raw) + (size_t)warp * kB64Angles * 12;
@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(128)
     const int v = e % (side * side), zl = e / (side * side);
     const int x = blockIdx.x * side + v % side, y = blockIdx.y * side + v / side;
     const int z = zbase + zl;
-    if (x >= n || y >= n || z >= n) continue;
+    if (x >= n || y >= n || z >= nz) continue;
     const size_t o = ((size_t)z * n + y) * np + x;
     double out = (2.0 / nimg) * stage[v * 32 * V + zl];
     if (scale) out *= scale[o];
@@ -972,6 +972,27 @@ size_t zdata_bytes(int n, int nth, size_t esize) {
   return (size_t)nth * n * ((n + rl - 1) / rl * rl) * esize;
 }
 
+// The planes a call takes at a time with `limit` bytes of scratch (0: enough for
+// all) for `rows` rows of planes, and the planes of a slab: whole slabs, the
+// narrowest ones where not even one fits (then the limit is exceeded).
+static int planes_at_once(int n, size_t rows, size_t esize, size_t limit, int* rl) {
+  *rl = slab_planes(n, esize);
+  const size_t all = rows * ((n + *rl - 1) / *rl * (size_t)*rl) * esize;
+  if (limit == 0 || all <= limit) return n;
+  if (esize == 4 && rows * *rl * esize > limit) *rl = 32;
+  const size_t unit = esize == 4 ? *rl : 32;
+  size_t units = limit / (rows * unit * esize);
+  if (units < 1) units = 1;
+  const int planes = (int)(units * unit);
+  if (esize == 8) *rl = planes;
+  return planes;
+}
+size_t zscratch_bytes(int n, size_t rows, size_t esize, size_t limit) {
+  int rl;
+  const size_t nz = planes_at_once(n, rows, esize, limit, &rl);
+  return rows * ((nz + rl - 1) / rl * (size_t)rl) * esize;
+}
+
 template <typename T>
 static int launch_zlast(const void* in, void* out, int nz, int ni, int no, size_t so, size_t sz,
                         int rl, cudaStream_t st) {
@@ -1033,35 +1054,38 @@ static int choose_v64(int n, int vmax, float extra) {
   return best;
 }
 
-int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
-                   const void* mask, void* scratch) {
-  const int n = pl.n, rl = slab_planes(n, pl.esize), slabs = (n + rl - 1) / rl;
-  if (!scratch) return report(FFPAT_EINVAL, "launch_project: no scratch volume");
+// planes z0 .. z0 + nz - 1 of P in slabs of rl
+static int project_planes(const Plan& pl, const void* p, void* g, const void* sub, const void* mask,
+                          void* scratch, int z0, int nz, int rl, cudaStream_t st) {
+  const int n = pl.n, slabs = (nz + rl - 1) / rl;
   const size_t so = pl.np, sz = (size_t)n * pl.np;  // p[z][y][x] in rows of np
+  const size_t es = pl.esize, row0 = (size_t)z0 * n;
+  auto at = [&](const void* q) { return q ? (const char*)q + row0 * es : nullptr; };
+  const void* pz = (const char*)p + (size_t)z0 * sz * es;
   if (pl.prec == FFPAT_FP64) {
-    const int rc = launch_zlast<double>(p, scratch, n, n, n, so, sz, rl, st);
+    const int rc = launch_zlast<double>(pz, scratch, nz, n, n, so, sz, rl, st);
     if (rc != FFPAT_OK) return rc;
-    const int V = choose_v64(n, 2, 0.2f);
+    const int V = choose_v64(nz, 2, 0.2f);
     // slabs of 32 V planes, up to four of them in a CTA (they share the sample
     // lists), two rays a warp and at most 12 warps; fewer rays a CTA while the
     // grid would not give every SM two
-    const int vs = (n + 32 * V - 1) / (32 * V), nslab = vs < 4 ? vs : 4;
+    const int vs = (nz + 32 * V - 1) / (32 * V), nslab = vs < 4 ? vs : 4;
     int rg = nslab == 1 ? 16 : (nslab == 2 ? 12 : (nslab == 3 ? 8 : 6));
     const int zg = (vs + nslab - 1) / nslab;
     while (rg > 4 && (n + rg - 1) / rg * (long long)pl.nth * zg < 2 * kNumSMs) rg -= 4;
     const size_t list = (size_t)kP64Samples * rg * 36, stage = (size_t)nslab * 32 * V * (rg + 1) * 8;
     launch_after_zlast(V == 2 ? k_project_z64<2> : k_project_z64<1>,
                        dim3((n + rg - 1) / rg, pl.nth, zg), 32 * nslab * (rg / 2),
-                       list > stage ? list : stage, st, (const double*)scratch, (double*)g,
-                       (const double*)sub, (const double*)mask, pl.tab, pl.tabf, n, pl.nth, pl.ns,
-                       pl.nimg, rl, nslab, rg);
+                       list > stage ? list : stage, st, (const double*)scratch,
+                       (double*)at(g), (const double*)at(sub), (const double*)at(mask), pl.tab,
+                       pl.tabf, n, nz, pl.nth, pl.ns, pl.nimg, rl, nslab, rg);
     return check_launch("k_project_z64");
   }
-  const int rc = launch_zlast<float>(p, scratch, n, n, n, so, sz, rl, st);
+  const int rc = launch_zlast<float>(pz, scratch, nz, n, n, so, sz, rl, st);
   if (rc != FFPAT_OK) return rc;
   // 16 warps a CTA: one a ray where the rays fill two CTAs on every SM, else
   // two or four a ray, and longer row blocks between the CTA's barriers (latency
-  // is the bound there: 68^3, 17 angles 25 -> 14 us)
+  // is the bound there: 68^3, 17 angles 25 -> 12 us)
   const long long rays = (long long)n * pl.nth * slabs, fill = 2LL * kNumSMs * kPWarps;
   const int split = rays >= fill ? 1 : (2 * rays >= fill ? 2 : 4), rg = kPWarps / split;
   const int ch = split == 1 ? 32 : 128;
@@ -1069,21 +1093,37 @@ int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cuda
   with_slab(rl, [&](auto V, auto C) {
     launch_after_zlast(k_project_z<V.value, C.value>, dim3((n + rg - 1) / rg, pl.nth, slabs),
                        32 * kPWarps, list > stage ? list : stage, st, (const float*)scratch,
-                       (float*)g, (const float*)sub, (const float*)mask, pl.tabi, n, pl.nth, pl.ns,
-                       pl.nimg, rg, ch);
+                       (float*)at(g), (const float*)at(sub), (const float*)at(mask), pl.tabi, n, nz,
+                       pl.nth, pl.ns, pl.nimg, rg, ch);
   });
   return check_launch("k_project_z");
 }
 
-int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       void* scratch, double mult) {
-  const int n = pl.n, rl = slab_planes(n, pl.esize), slabs = (n + rl - 1) / rl;
-  if (!scratch) return report(FFPAT_EINVAL, "launch_backproject: no data scratch");
-  const size_t nn = (size_t)n * n;
-  if (pl.prec == FFPAT_FP64) {
-    const int rc = launch_zlast<double>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
+int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
+                   const void* mask, void* scratch, size_t limit) {
+  if (!scratch) return report(FFPAT_EINVAL, "launch_project: no scratch volume");
+  int rl;
+  const int step = planes_at_once(pl.n, (size_t)pl.n * pl.n, pl.esize, limit, &rl);
+  for (int z0 = 0; z0 < pl.n; z0 += step) {
+    const int nz = pl.n - z0 < step ? pl.n - z0 : step;
+    const int rc = project_planes(pl, p, g, sub, mask, scratch, z0, nz, rl, st);
     if (rc != FFPAT_OK) return rc;
-    const int V = choose_v64(n, 4, 0.8f), vs = (n + 32 * V - 1) / (32 * V);
+  }
+  return FFPAT_OK;
+}
+
+// planes z0 .. z0 + nz - 1 of P^T in slabs of rl
+static int backproject_planes(const Plan& pl, const void* g, void* h, const void* scale,
+                              void* scratch, int z0, int nz, int rl, double mult,
+                              cudaStream_t st) {
+  const int n = pl.n, slabs = (nz + rl - 1) / rl;
+  const size_t nn = (size_t)n * n, es = pl.esize, vol0 = (size_t)z0 * n * pl.np;
+  const void* gz = (const char*)g + (size_t)z0 * n * es;
+  auto at = [&](const void* q) { return q ? (const char*)q + vol0 * es : nullptr; };
+  if (pl.prec == FFPAT_FP64) {
+    const int rc = launch_zlast<double>(gz, scratch, nz, n, pl.nth, nn, (size_t)n, rl, st);
+    if (rc != FFPAT_OK) return rc;
+    const int V = choose_v64(nz, 4, 0.8f), vs = (nz + 32 * V - 1) / (32 * V);
     int tb = 2;  // tb x tb blocks of 2 x 2 voxels a CTA
     if ((long long)((n + 3) / 4) * ((n + 3) / 4) * vs < 2 * kNumSMs) tb = 1;
     const int side = 2 * tb, tiles = (n + side - 1) / side;
@@ -1091,11 +1131,11 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
     launch_after_zlast(
         V == 4 ? k_backproject_z64<4> : (V == 2 ? k_backproject_z64<2> : k_backproject_z64<1>),
         dim3(tiles, tiles, vs), 32 * tb * tb, list > stage ? list : stage, st,
-        (const double*)scratch, (double*)h, (const double*)scale, pl.tab, n, pl.np, pl.nth, pl.ns,
-        pl.nimg, rl, tb, mult);
+        (const double*)scratch, (double*)at(h), (const double*)at(scale), pl.tab, n, pl.np, nz,
+        pl.nth, pl.ns, pl.nimg, rl, tb, mult);
     return check_launch("k_backproject_z64");
   }
-  const int rc = launch_zlast<float>(g, scratch, n, n, pl.nth, nn, (size_t)n, rl, st);
+  const int rc = launch_zlast<float>(gz, scratch, nz, n, pl.nth, nn, (size_t)n, rl, st);
   if (rc != FFPAT_OK) return rc;
   // blocks of 2 x 2 voxels a CTA: neighbouring blocks share detectors in L1;
   // fewer while the grid would not give every SM two CTAs
@@ -1112,10 +1152,23 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
     launch_after_zlast(k_backproject_z<V.value, C.value>,
                        dim3((n + 2 * tx - 1) / (2 * tx), (n + 2 * ty - 1) / (2 * ty), slabs),
                        32 * tx * ty, list > stage ? list : stage, st, (const float*)scratch,
-                       (float*)h, (const float*)scale, pl.tabf, pl.tabi, n, pl.np, pl.nth, pl.ns,
-                       pl.nimg, tx, (float)mult);
+                       (float*)at(h), (const float*)at(scale), pl.tabf, pl.tabi, n, pl.np, nz,
+                       pl.nth, pl.ns, pl.nimg, tx, (float)mult);
   });
   return check_launch("k_backproject_z");
+}
+
+int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
+                       void* scratch, double mult, size_t limit) {
+  if (!scratch) return report(FFPAT_EINVAL, "launch_backproject: no data scratch");
+  int rl;
+  const int step = planes_at_once(pl.n, (size_t)pl.nth * pl.n, pl.esize, limit, &rl);
+  for (int z0 = 0; z0 < pl.n; z0 += step) {
+    const int nz = pl.n - z0 < step ? pl.n - z0 : step;
+    const int rc = backproject_planes(pl, g, h, scale, scratch, z0, nz, rl, mult, st);
+    if (rc != FFPAT_OK) return rc;
+  }
+  return FFPAT_OK;
 }
 
 template <typename T>

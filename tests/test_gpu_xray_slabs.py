@@ -61,3 +61,34 @@ def test_ramp_shapes(n, nth):
         r = rows.astype(dt)
         got = F.ramp(prob, torch.as_tensor(r, device="cuda")).double().cpu().numpy()
         assert rel(got, o.ramp(r.astype(np.float64))) < tol
+
+
+# standalone calls take operands beyond 1 GiB in several passes over z: P in two at
+# 656^3 FP32 (384 planes and 272) and 520^3 FP64 (480 and 40), P^T in two or more with
+# that many rows of data.  The planes are independent: with the planes moved by half
+# the grid every result moves with them, out of one pass into another; rays of every
+# pass are checked against the oracle too.
+@pytest.mark.parametrize("n,prec", [(656, F.FP32), (520, F.FP64)])
+def test_passes_over_z(n, prec):
+    dt = torch.float64 if prec == F.FP64 else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    tol = 1e-12 if prec == F.FP64 else 5e-7
+
+    def off(a, b):
+        return float((a.double() - b.double()).norm() / b.double().norm())
+
+    prob = F.problem(n, 1.0, 2, prec)
+    p = torch.randn((n, n, n), generator=gen, device="cuda", dtype=dt)
+    got = F.project(prob, p)
+    assert off(F.project(prob, p.roll(n // 2, 0)).roll(-(n // 2), 1), got) < tol
+    jlk = [(j, z, k) for j in (0, 1) for z in (0, 383, 384, 479, 480, n - 1)
+           for k in range(0, n, 37)]
+    want = o.project_rays(p.double().cpu().numpy(), 2, jlk)
+    have = np.array([got[t].item() for t in jlk])
+    assert rel(have, want) < tol
+    del p, got
+    nth = 2 * n if prec == F.FP32 else 520
+    prob = F.problem(n, 1.0, nth, prec)
+    g = torch.randn((nth, n, n), generator=gen, device="cuda", dtype=dt)
+    got = F.backproject(prob, g)
+    assert off(F.backproject(prob, g.roll(n // 2, 1)).roll(-(n // 2), 0), got) < tol
