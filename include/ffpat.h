@@ -266,7 +266,7 @@ int64_t ffpat_launch_count(void);
 /* Choice of leapfrog kernel (process-wide): 0 = automatic (the TMA-fed kernels
  * where all arrays are 16-byte aligned, on copies with rows padded to 16 bytes
  * when N % 4 != 0 for float or N % 2 != 0 for double (the differentiated
- * operator's checkpointed loops excepted) -- the whole time loop in one
+ * operator's FP64 checkpointed loops excepted) -- the whole time loop in one
  * cooperative launch where its work items fit the GPU at once (N <= 128 on
  * GB300, FP64 N <= 96) and the stream is not capturing, else two steps per pass
  * for 128 <= N <= 1624 (FP32, FP32-Kahan) -- else the plain 2.5D kernel), 1 = always the plain
@@ -388,7 +388,9 @@ int ffpat_server_destroy(ffpat_server *server);
  * library's device code is loaded on a device and held until exit; under
  * CUDA's lazy module loading (the default) that load happens during the first
  * call on each device, which may allocate once; later calls allocate nothing.
- * Problems whose ffpat_workspace_bytes exceeds 32 MiB fail with FFPAT_EINVAL
+ * Problems whose whole workspace of dense volumes and data (that is
+ * ffpat_workspace_bytes without what the kernels' layouts add) exceeds 32 MiB
+ * fail with FFPAT_EINVAL
  * (a wave grid N + 2 pad <= 64 with up to 180 angles fits every precision;
  * without padding that is N <= 64); a device index >= 64 fails with
  * FFPAT_EINVAL.  The first call on a device looks up the array's device

@@ -177,6 +177,59 @@ static size_t carve(Plan& pl, void* ws) {
   return off;
 }
 
+// The part of the workspace that the forward operator uses.
+static size_t carve_forward(Plan& pl, void* ws) {
+  char* b = (char*)ws;
+  size_t off = 0;
+  auto take = [&](size_t bytes) -> void* {
+    void* p = b ? (void*)(b + off) : nullptr;
+    off += up256(bytes);
+    return p;
+  };
+  const bool own = direct(pl);
+  const size_t wvol = (size_t)pl.nw * pl.nw * pl.nwp * pl.esize;
+  const size_t zvol = zvolume_bytes(pl.nw, pl.esize);
+  pl.kap = take(pl.n3 * pl.esize);
+  pl.kapw = own ? pl.kap : take(wvol);
+  for (int i = 0; i < 6; ++i) pl.s[i] = i < nstate(pl) ? take(wvol) : nullptr;
+  pl.x = own ? take(zvol) : nullptr;
+  pl.xw = own ? nullptr : take(zvol > wvol ? zvol : wvol);
+  pl.partials = (double*)take(sizeof(double) * kNumQuant * kReduceBlocks);
+  pl.tab = (double*)take(table_bytes(pl.nth));
+  pl.sync = (unsigned*)take(128 * (size_t)kResidentMaxItems);
+  return off;
+}
+
+// Bytes that a whole workspace of dense, unrounded volumes and data has: the
+// measure by which ffpat_forward_noalloc accepts a problem, whatever the
+// kernels' layouts add to ffpat_workspace_bytes.  What it accepts fits
+// carve_forward with dense rows: the volumes and data left out there are more
+// than the slabs' rounding.
+static size_t dense_workspace(const Plan& pl) {
+  const size_t vol = up256(pl.n3 * pl.esize), wvol = up256(pl.nw3 * pl.esize);
+  size_t b = 3 * vol + nstate(pl) * wvol + 2 * up256(pl.nd * pl.esize);
+  if (pl.pad) b += 3 * wvol + vol;
+  return b + up256(sizeof(double) * kNumQuant * kReduceBlocks) + up256(sizeof(double) * kScal) +
+         up256(sizeof(double) * 8 * kMaxHist) + up256(table_bytes(pl.nth)) +
+         up256(dct_bytes(pl.n, pl.esize)) + up256(128 * (size_t)kResidentMaxItems);
+}
+
+int plan_noalloc(const ffpat_problem* pr, Plan& pl, void* ws, size_t limit) {
+  TRY(validate(pr, pl));
+  const size_t need = dense_workspace(pl);
+  if (need > limit)
+    return fail(FFPAT_EINVAL,
+                "ffpat_forward_noalloc: the problem needs %zu bytes of scratch but the static "
+                "scratch holds %zu (a wave grid N + 2 pad <= 64 with <= 180 angles fits every "
+                "precision)", need, limit);
+  // padded rows where they fit too
+  if (carve_forward(pl, nullptr) > limit) pl.nwp = pl.nw;
+  if (carve_forward(pl, nullptr) > limit)
+    return fail(FFPAT_EINVAL, "ffpat_forward_noalloc: no room for P's operand in the static scratch");
+  if (ws) carve_forward(pl, ws);
+  return FFPAT_OK;
+}
+
 int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path) {
   TRY(validate(pr, pl, any_path));
   const size_t need = carve(pl, nullptr);
@@ -237,10 +290,16 @@ int time_steps(const Plan& pl, double cmax, int* nt, double* dt) {
   return FFPAT_OK;
 }
 
+static int setup_attached(Plan& pl, const void* c, cudaStream_t st);
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
           cudaStream_t st, bool any_path) {
   g_err[0] = 0;
   TRY(attach(pr, pl, ws, ws_bytes, any_path));
+  return setup_attached(pl, c, st);
+}
+
+// the rest of setup() on a carved plan
+static int setup_attached(Plan& pl, const void* c, cudaStream_t st) {
   if (!c) return fail(FFPAT_EINVAL, "c is NULL");
   // c's maximum and validity -> Nt, dt, kappa: one device-to-host read; the
   // host works out the angle tables meanwhile
@@ -594,6 +653,24 @@ static int wave_back(const Plan& pl, const void* x, const void** w, cudaStream_t
   return FFPAT_OK;
 }
 
+static int apply_forward(const Plan& pl, const void* h, void* g, cudaStream_t st) {
+  if (!h || !g) return fail(FFPAT_EINVAL, "h or g is NULL");
+  const void* pN = nullptr;
+  TRY(wave_fwd(pl, h, &pN, st));
+  TRY(launch_project(wave_plan(pl), pN, g, nullptr, st, nullptr, wave_in(pl)));
+  return FFPAT_OK;
+}
+
+int forward_noalloc(const ffpat_problem* pr, const void* c, const void* h, void* g, void* ws,
+                    size_t limit, cudaStream_t st) {
+  Trace trace_("ffpat_forward");
+  Plan pl;
+  g_err[0] = 0;
+  TRY(plan_noalloc(pr, pl, ws, limit));
+  TRY(setup_attached(pl, c, st));
+  return apply_forward(pl, h, g, st);
+}
+
 // h = E^T W^T P^T g  ->  x = K P^T g ; w = E^T W x ; h = w / K
 static int apply_adjoint(const Plan& pl, const void* g, void* h, cudaStream_t st) {
   const Plan wp = wave_plan(pl);
@@ -770,11 +847,7 @@ int ffpat_forward(const ffpat_problem* problem, const void* c, const void* h, vo
   cudaStream_t st = (cudaStream_t)stream;
   Plan pl;
   TRY(setup(problem, pl, c, ws, ws_bytes, st));
-  if (!h || !g) return fail(FFPAT_EINVAL, "h or g is NULL");
-  const void* pN = nullptr;
-  TRY(wave_fwd(pl, h, &pN, st));
-  TRY(launch_project(wave_plan(pl), pN, g, nullptr, st, nullptr, wave_in(pl)));
-  return FFPAT_OK;
+  return apply_forward(pl, h, g, st);
 }
 
 int ffpat_adjoint(const ffpat_problem* problem, const void* c, const void* g, void* h, void* ws,

@@ -88,6 +88,11 @@ bool resident_segments(const Plan& pl, bool tma, cudaStream_t st);
 // row pitch the wave grid's volumes may have (whatever the path)
 int padded_row(const Plan& pl);
 int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path = false);
+// the forward operator in `limit` bytes of scratch at ws (ffpat_forward_noalloc);
+// plan_noalloc alone (ws nullable) says whether the problem is accepted
+int plan_noalloc(const ffpat_problem* pr, Plan& pl, void* ws, size_t limit);
+int forward_noalloc(const ffpat_problem* pr, const void* c, const void* h, void* g, void* ws,
+                    size_t limit, cudaStream_t st);
 int time_steps(const Plan& pl, double cmax, int* nt, double* dt);
 void fill_tables_host(int nth, unsigned char* buf);  // table_bytes(nth) bytes
 

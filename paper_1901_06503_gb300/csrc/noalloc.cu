@@ -16,8 +16,9 @@
 // array is committed when that module is loaded on a device; under CUDA's
 // lazy module loading (the default) that happens during the first call on
 // each device, which may therefore allocate device memory once; later calls
-// allocate nothing.  Problems whose workspace (ffpat_workspace_bytes) is larger
-// are rejected.  The workspace grows with the wave grid N_w = N + 2 pad:
+// allocate nothing.  Problems are measured by a whole workspace of dense volumes
+// and data (ffpat_workspace_bytes without what the kernels' layouts add to it);
+// those beyond the array are rejected.  It grows with the wave grid N_w = N + 2 pad:
 // without padding, N <= 64 with up to 180 angles fits in every precision
 // (N_w <= 64 with up to 180 angles in general).
 //
@@ -75,19 +76,14 @@ int scratch_address(void** out) {
 
 extern "C" int ffpat_forward_noalloc(const ffpat_problem* problem, const void* c, const void* h,
                                      void* g, void* stream) {
-  const size_t need = ffpat_workspace_bytes(problem);
-  if (need == 0) return FFPAT_EINVAL;  // invalid problem; ffpat_last_error() says why
-  if (need > ffpat::kScratchBytes)
-    return ffpat::report(FFPAT_EINVAL,
-                         "ffpat_forward_noalloc: the problem needs %zu bytes of scratch but the "
-                         "static scratch holds %zu (a wave grid N + 2 pad <= 64 with <= 180 "
-                         "angles fits every precision)",
-                         need, ffpat::kScratchBytes);
+  ffpat::Plan probe;
+  const int ok = ffpat::plan_noalloc(problem, probe, nullptr, ffpat::kScratchBytes);
+  if (ok != FFPAT_OK) return ok;  // ffpat_last_error() says why
   void* ws = nullptr;
   const int rc = ffpat::scratch_address(&ws);
   if (rc != FFPAT_OK) return rc;
   // launch the time loop step by step: the library's CUDA-graph replay would
   // create a capture stream and instantiate a graph, which allocate
   ffpat::NoGraphs no_graphs;
-  return ffpat_forward(problem, c, h, g, ws, ffpat::kScratchBytes, stream);
+  return ffpat::forward_noalloc(problem, c, h, g, ws, ffpat::kScratchBytes, (cudaStream_t)stream);
 }

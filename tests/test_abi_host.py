@@ -54,6 +54,19 @@ def test_workspace_grows_with_problem(L):
     assert padded >= big + 4 * (128**3 - 64**3) * 8
 
 
+# the most angles that fit 32 MiB of dense volumes and data, per (precision, n, pad)
+@pytest.mark.parametrize("prec,n,pad,most", [
+    (0, 17, 1, 5627), (0, 34, 4, 1022), (0, 53, 16, 32), (0, 91, 0, 21), (1, 16, 16, 1622),
+    (1, 32, 33, 81), (1, 51, 0, 1410), (1, 71, 0, 571), (2, 3, 33, 558), (2, 20, 0, 10157),
+    (2, 37, 1, 2472), (2, 56, 7, 457), (2, 80, 4, 5)])
+def test_noalloc_accepts_by_the_dense_size(L, prec, n, pad, most):
+    for nth, accepted in ((1, True), (most, True), (most + 1, False)):
+        prob = F.problem(n, 0.2, nth, prec, pad=pad)
+        assert L.ffpat_forward_noalloc(ctypes.byref(prob), None, None, None, None) < 0
+        msg = L.ffpat_last_error()  # accepted ones fail later: no device, or c is NULL
+        assert (b"static scratch" not in msg) == accepted
+
+
 def test_padding_rejected_where_unsupported(L):
     prob = F.problem(16, 1.0, 4, F.FP32_KAHAN, pad=4)
     assert L.ffpat_ckpt_bytes(ctypes.byref(prob), 10, 4) == 0
