@@ -83,7 +83,7 @@ static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Wave-grid rows of a multiple of 16 bytes, the TMA kernels' layout (measured
 // against the plain kernel on the rows as they are: W at 150^3 FP32-Kahan 28.6 ->
-// 13 us a step, 101^3 FP32 10.6 -> 4.1 us); grids of fewer than five points stay
+// 12.1 us a step, 101^3 FP32 10.6 -> 4.1 us); grids of fewer than five points stay
 // as they are.
 int padded_row(const Plan& pl) {
   const int q = (int)(16 / pl.esize);

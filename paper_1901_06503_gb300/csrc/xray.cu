@@ -181,6 +181,13 @@ __device__ __forceinline__ float2 ffma2(float w, float2 x, float2 a) {
   return o;
 }
 
+// What adding t to s0 (the sum: s1) rounded off; 0 where the sum has overflowed,
+// so that it stays infinite.
+__device__ __forceinline__ float rounded_off(float t, float s1, float s0) {
+  const float e = __fsub_rn(t, __fsub_rn(s1, s0));
+  return fabsf(e) < 1e32f ? e : 0.0f;
+}
+
 template <int N>
 struct ZAcc {
   float2 a[N / 2 + 1];  // pairs; the last one's first lane is the odd plane
@@ -193,11 +200,13 @@ struct ZAcc {
     for (int i = 0; i < N / 2; ++i) a[i] = ffma2(w, make_float2(v[2 * i], v[2 * i + 1]), a[i]);
     if constexpr (N % 2) a[N / 2].x = fmaf(w, v[N - 1], a[N / 2].x);
   }
-  __device__ __forceinline__ void add(const ZAcc& o) {
+  // adds o and leaves in o what the additions rounded off
+  __device__ __forceinline__ void add_carry(ZAcc& o) {
 #pragma unroll
     for (int i = 0; i <= N / 2; ++i) {
-      a[i].x += o.a[i].x;
-      a[i].y += o.a[i].y;
+      const float2 s = make_float2(__fadd_rn(a[i].x, o.a[i].x), __fadd_rn(a[i].y, o.a[i].y));
+      o.a[i] = make_float2(rounded_off(o.a[i].x, s.x, a[i].x), rounded_off(o.a[i].y, s.y, a[i].y));
+      a[i] = s;
     }
   }
   __device__ __forceinline__ float get(int i) const { return i & 1 ? a[i / 2].y : a[i / 2].x; }
@@ -274,7 +283,10 @@ __device__ __forceinline__ RowTaps row_taps(int a, int k, long long CS, long lon
 // (192^3, 90 angles: 0.36 ms, against 0.54 with 16 warps and two rows in
 // flight).  Per standalone call, 384^3 and 180 angles: 13.0 -> 5.2 ms against
 // the plane-by-plane kernel it replaces, 256^3 and 180: 3.7 -> 1.7 ms.
-// Sums: per kPSum rows, then over those.
+// Sums: per kPSum rows, then over those; what adding a group rounds off starts
+// the next one, so that the error does not grow with N (a smooth volume, relative:
+// 150^3 8.3e-8 -> 4.7e-8, 256^3 9.6e-8 -> 3.0e-8; 192^3 and 90 angles, standalone
+// call, 541 -> 547 us).
 constexpr int kPSum = 8;
 constexpr int kPWarps = 16;
 
@@ -312,8 +324,9 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
   const bool ymajor = abs(CSi) >= abs(SNi);
   const float inv = 1.0f / (float)(ymajor ? 2 * CS : -2 * SN);
   const long long sa = (long long)(ymajor ? n : 1) * RL, sb = (long long)(ymajor ? 1 : n) * RL;
-  ZAcc<V * C> total;
+  ZAcc<V * C> total, c;
   total.zero();
+  c.zero();
   for (int a0 = 0; a0 < n; a0 += ch) {
     const int rows = min(ch, n - a0);
     __syncthreads();
@@ -328,8 +341,6 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
     __syncthreads();
 #pragma unroll 1
     for (int rs = part * kPSum; rs < rows; rs += split * kPSum) {
-      ZAcc<V * C> c;
-      c.zero();
       const int re = min(rs + kPSum, rows);
       const float* prow = pz + (a0 + rs) * sa;
 #pragma unroll 1
@@ -346,7 +357,7 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
         else if (cnt == 1)
           ray_taps<1, V, C>(q, sb, w, c);
       }
-      total.add(c);
+      total.add_carry(c);
     }
   }
   __syncthreads();
@@ -359,8 +370,12 @@ __global__ void __launch_bounds__(kPWarps * 32, 2)
     const int r = e % rg, zl = e / rg;
     if (k0 + r >= n || zbase + zl >= nz) continue;
     const size_t o = ((size_t)j * n + zbase + zl) * n + k0 + r;
-    float sum = stage[zl * (rg + 1) + r];
-    for (int q = 1; q < split; ++q) sum += stage[(q * RL + zl) * (rg + 1) + r];
+    float sum = stage[zl * (rg + 1) + r], carry = 0.0f;
+    for (int q = 1; q < split; ++q) {
+      const float t = stage[(q * RL + zl) * (rg + 1) + r] + carry, s = __fadd_rn(sum, t);
+      carry = rounded_off(t, s, sum);
+      sum = s;
+    }
     float out = scale * sum;
     if (sub) out = out - sub[o];
     if (mask) out = out * mask[o];

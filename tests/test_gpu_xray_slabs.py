@@ -92,3 +92,23 @@ def test_passes_over_z(n, prec):
     g = torch.randn((nth, n, n), generator=gen, device="cuda", dtype=dt)
     got = F.backproject(prob, g)
     assert off(F.backproject(prob, g.roll(n // 2, 1)).roll(-(n // 2), 0), got) < tol
+
+
+# P of a smooth volume, where the rows' sums all have one sign: the error of a long
+# plain sum would grow with N.  Expected at most 8e-8: the rounded cell size (6e-8
+# where 2 / N is no power of two), the last addition and the product (3.4e-8 each)
+# and the groups of eight rows (24 additions each, N / 8 of them averaged: 2e-8).
+@pytest.mark.parametrize("n,nth", [(32, 4), (64, 3), (100, 4), (150, 4), (256, 2)])
+def test_smooth_sums(n, nth):
+    x = np.linspace(-1, 1, n)
+    p = np.exp(-4 * ((x - 0.1) ** 2 + (x[:, None] + 0.2) ** 2 + x[:, None, None] ** 2))
+    p = p.astype(np.float32)
+    got = F.project(F.problem(n, 1.0, nth, F.FP32), torch.as_tensor(p, device="cuda"))
+    assert rel(got.double().cpu().numpy(), o.project(p.astype(np.float64), nth)) < 8e-8
+
+
+# sums beyond the largest float are infinite, not NaN
+def test_overflow_stays_infinite():
+    p = torch.full((64, 64, 64), 3e38, device="cuda")
+    g = F.project(F.problem(64, 1.0, 4, F.FP32), p)
+    assert not torch.isnan(g).any() and torch.isinf(g[:, :, 32]).all()
