@@ -329,9 +329,9 @@ static int setup_attached(Plan& pl, const void* c, cudaStream_t st) {
 
 // FP32 and FP32-Kahan run two steps per pass (where the resident time loop
 // does not run): measured on GB300 the two-step passes win at every size from
-// 128^3 to 384^3 (FP32-Kahan 15.5 / 47.5 / 133 against 18.1 / 82.5 / 262 us per
-// step at 160^3 / 256^3 / 384^3; FP32 three-term 14.0 / 42.3 / 118 against
-// 15.4 / 46.9 / 135), and tie at 144^3, whose 64-wide tiles are a third empty
+// 128^3 to 384^3 (FP32-Kahan 14.5 / 45.3 / 123 against 17.9 / 82.8 / 262 us per
+// step at 160^3 / 256^3 / 384^3; FP32 three-term 12.9 / 38.8 / 103 against
+// 15.3 / 46.9 / 135), and tie at 144^3, whose 64-wide tiles are a third empty
 constexpr int kTwoStepMinN = 128;
 
 // The kernel path of a time loop: padded rows exist only on the automatic path.
