@@ -848,6 +848,20 @@ constexpr int kROut = 16;
 constexpr int kRNear = 3;
 constexpr int kRPitch = 33;  // of a staged input: 32 rows and one word against bank conflicts
 
+// (Lambda row)_k by the odd taps alone.  The Toeplitz product has zeros for taps
+// among those of its other parity (|d| <= kRNear), which make NaN of an infinite
+// input: an output that is NaN is taken from here, which says whether it is.
+template <typename T>
+__device__ __noinline__ T ramp_direct(const T* __restrict__ row, int k, int n, int nimg) {
+  const double dxi = 2.0 / nimg;
+  T v = (T)(1.0 / (8.0 * dxi)) * row[k];
+  for (int d = 1; d < n && v == v; d += 2) {
+    const T t = (T)(-1.0 / (2.0 * kPi * kPi * (double)d * d * dxi));
+    v += t * ((k >= d ? row[k - d] : T(0)) + (k + d < n ? row[k + d] : T(0)));
+  }
+  return v;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
     k_ramp(const T* __restrict__ r, T* __restrict__ out, const T* __restrict__ mask, int n,
@@ -934,6 +948,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
     for (int k = lane; k < kn; k += 32) {
       const size_t o = (size_t)(row0 + q) * n + ko + k;
       T v = s[k * kRPitch + q];
+      if (v != v) v = ramp_direct(r + (size_t)(row0 + q) * n, ko + k, n, nimg);
       if (mask) v = v * mask[o];
       out[o] = v;
     }
