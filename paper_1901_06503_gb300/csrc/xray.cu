@@ -552,6 +552,29 @@ __device__ __forceinline__ int voxel_sums(long long KK, long long MM, float cs, 
   return KI - 1 + hk;
 }
 
+// The sum of voxel (x, y) over the detectors it sees, one plane (gp: its data,
+// detectors rl apart), in the order of k_backproject_z.  There the four voxels of a
+// block share their detectors, with zero weights, which make NaN of an infinite
+// datum that a voxel does not see: a NaN is taken from here instead.
+__device__ __noinline__ float voxel_alone(const float* __restrict__ gp, int rl, int x, int y,
+                                          const float* __restrict__ tabf,
+                                          const int32_t* __restrict__ tabi, int n, int nth,
+                                          int ns) {
+  const long long X2 = 2 * x - (n - 1), Y2 = 2 * y - (n - 1);
+  const long long ck = (long long)(n - 1) << 30, cm = (long long)(ns - 1) << 30;
+  float acc = 0.0f;
+  for (int j = 0; j < nth; ++j) {
+    const long long CS = tabi[j], SN = tabi[nth + j];
+    float r[3];
+    const int kb = voxel_sums(X2 * CS + Y2 * SN + ck, Y2 * CS - X2 * SN + cm, tabf[j],
+                              tabf[nth + j], ns, r);
+    for (int i = 0; i < 3; ++i)
+      if (r[i] != 0.0f && (unsigned)(kb + i) < (unsigned)n)
+        acc = fmaf(r[i], gp[((size_t)j * n + kb + i) * rl], acc);
+  }
+  return acc;
+}
+
 // P^T for all planes of a slab at once.  A warp owns a block of 2 x 2 voxels
 // and the slab's planes, V C a lane.  Its lanes work out the weights of eight
 // angles at a time (a lane: one voxel and angle) into the warp's part of shared
@@ -662,6 +685,7 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
   const int sx = 2 * tx, nv = 4 * warps;
   const float f = 2.0f / (float)nimg;
   float* stage = reinterpret_cast<float*>(smem_raw);  // [32 V planes][nv + 1]
+  bool nan = false;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     __syncthreads();
@@ -682,8 +706,22 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
       if (scale) out *= scale[o];
       if (mult != 1.0f) out *= mult;
       h[o] = out;
+      nan |= isnan(out);
     }
   }
+  if (nan)  // the elements that this thread wrote
+    for (int e = tid; e < nv * RL; e += blockDim.x) {
+      const int v = e % nv, zl = e / nv;
+      const int x = blockIdx.x * sx + v % sx, y = blockIdx.y * 2 * ty + v / sx;
+      if (x >= n || y >= n || zbase + zl >= nz) continue;
+      const size_t o = ((size_t)(zbase + zl) * n + y) * np + x;
+      if (!isnan(h[o])) continue;
+      float out = f * voxel_alone(gt + (size_t)blockIdx.z * nth * n * RL + zl, RL, x, y, tabf, tabi,
+                                  n, nth, ns);
+      if (scale) out *= scale[o];
+      if (mult != 1.0f) out *= mult;
+      h[o] = out;
+    }
 }
 
 // ------------------------------------------------------------- P^T, FP64 --
