@@ -92,7 +92,7 @@ int padded_row(const Plan& pl) {
 static bool ragged(const Plan& pl) { return pl.nw >= 5 && padded_row(pl) != pl.nw; }
 
 // Validate the problem and fill the size fields of the plan.
-static int validate(const ffpat_problem* pr, Plan& pl, bool any_path = false) {
+static int validate(const ffpat_problem* pr, Plan& pl, Rows rows = Rows::kAuto) {
   g_err[0] = 0;
   if (!pr) return fail(FFPAT_EINVAL, "problem is NULL");
   if (pr->n < 1 || pr->n > 2048) return fail(FFPAT_EINVAL, "n = %d outside [1, 2048]", pr->n);
@@ -125,9 +125,10 @@ static int validate(const ffpat_problem* pr, Plan& pl, bool any_path = false) {
   pl.np = pl.n;
   // rows that are no multiple of 16 bytes are padded on the wave grid, where
   // they would otherwise rule out the TMA kernels; a requested kernel (any
-  // path but the automatic one) runs on the rows as they are, unless data in
-  // padded rows outlive the call (any_path: the checkpoints)
-  pl.nwp = ragged(pl) && (any_path || g_stencil_path.load() == 0) ? padded_row(pl) : pl.nw;
+  // path but the automatic one) runs on the rows as they are, unless the caller
+  // says which (the differentiated operator, whose checkpoints outlive the call)
+  const bool pad = rows == Rows::kPadded || (rows == Rows::kAuto && g_stencil_path.load() == 0);
+  pl.nwp = ragged(pl) && pad ? padded_row(pl) : pl.nw;
   return FFPAT_OK;
 }
 
@@ -137,8 +138,14 @@ static int nstate(const Plan& pl) {
   return pl.prec == FFPAT_FP32_KAHAN ? 6 : (pl.prec == FFPAT_FP32 ? 4 : 2);
 }
 
-// Carve the workspace (ws == nullptr: size only).
-static size_t carve(Plan& pl, void* ws) {
+// Carve the workspace (ws == nullptr: size only), the forward operator's part alone
+// with forward_only.  The z-innermost operands of P and P^T have no volumes of their
+// own: they take what is free around the state volumes (project_scratch,
+// backproject_scratch), which is why the wave input lies before those and the
+// residual behind them.  A grid of at least 32 points thus needs no more than dense
+// volumes and data would (dense_workspace), padded rows excepted; smaller ones have
+// room for a slab of 32 planes in the wave input and in each data array.
+static size_t carve(Plan& pl, void* ws, bool forward_only = false) {
   char* b = (char*)ws;
   size_t off = 0;
   auto take = [&](size_t bytes) -> void* {
@@ -146,65 +153,70 @@ static size_t carve(Plan& pl, void* ws) {
     off += up256(bytes);
     return p;
   };
-  // (the layout depends on the problem alone, not on the path that runs)
-  const bool apart = pl.pad != 0 || ragged(pl);  // the wave grid has volumes of its own
-  const size_t vol = pl.n3 * pl.esize;
-  const size_t wvol = (size_t)pl.nw * pl.nw * (ragged(pl) ? padded_row(pl) : pl.nw) * pl.esize;
-  // the wave input doubles as the z-innermost operand of P, the data scratch as
-  // that of P^T (rows padded to 16 bytes)
-  const size_t zvol = zvolume_bytes(pl.nw, pl.esize), dat = zdata_bytes(pl.nw, pl.nth, pl.esize);
-  pl.kap = take(vol);
-  pl.kapw = apart ? take(wvol) : pl.kap;
-  for (int i = 0; i < 6; ++i) pl.s[i] = i < nstate(pl) ? take(wvol) : nullptr;
-  pl.x = take(pl.pad ? vol : zvol);
-  pl.v = take(vol);
-  pl.xw = apart ? take(zvol > wvol ? zvol : wvol) : nullptr;
-  pl.xo = apart ? take(vol) : nullptr;
-  pl.xg = pl.pad ? take(pl.nw3 * pl.esize) : nullptr;
-  if (direct(pl)) pl.kapw = pl.kap;
-  pl.r = take(dat);
-  pl.r2 = take(dat);
+  // (the layout depends on the problem alone, not on the path that runs; the
+  // allocation-free call has one size and fits its rows to it)
+  const int row = forward_only ? pl.nwp : (ragged(pl) ? padded_row(pl) : pl.nw);
+  const size_t vol = pl.n3 * pl.esize, area = (size_t)pl.nw * pl.nw;
+  const size_t wvol = area * row * pl.esize;
+  const size_t slab = (size_t)(pl.esize == 4 ? kMinPlanes32 : kMinPlanes64) * pl.esize;
+  const size_t zvol = area * slab, zdat = (size_t)pl.nth * pl.nw * slab;
+  const size_t dat = pl.nd * pl.esize > zdat ? pl.nd * pl.esize : zdat;
+  pl.nstate = nstate(pl);
+  pl.svol = up256(wvol);
+  pl.kap = take(pl.pad ? vol : wvol);
+  pl.kapw = pl.pad ? take(wvol) : pl.kap;
+  pl.v = forward_only ? nullptr : take(vol);
+  pl.xg = pl.pad && !forward_only ? take(pl.nw3 * pl.esize) : nullptr;
+  pl.x = pl.pad && !forward_only ? take(vol) : nullptr;
+  pl.xw = take(wvol > zvol ? wvol : zvol);
+  if (!pl.pad) pl.x = pl.xw;
+  for (int i = 0; i < 6; ++i) pl.s[i] = i < pl.nstate ? take(wvol) : nullptr;
+  if (!forward_only) {
+    pl.dvol = up256(dat);
+    pl.r = take(dat);
+    // on ragged grids Lambda's result lies in the state volumes where it and P^T's
+    // operand fit there one after the other: no W runs while it is in use, and it
+    // is more than the rows' padding adds beyond 24 angles
+    const bool in_state = ragged(pl) && pl.nw >= 32 &&
+                          (size_t)pl.nstate * pl.svol >= zscratch_bytes(pl.nw, (size_t)pl.nth * pl.nw,
+                                                                        pl.esize, (size_t)-1);
+    pl.r2 = in_state ? pl.s[0] : take(dat);
+  }
   pl.partials = (double*)take(sizeof(double) * kNumQuant * kReduceBlocks);
-  pl.scal = (double*)take(sizeof(double) * kScal);
-  pl.hist = (double*)take(sizeof(double) * 8 * kMaxHist);
+  if (!forward_only) {
+    pl.scal = (double*)take(sizeof(double) * kScal);
+    pl.hist = (double*)take(sizeof(double) * 8 * kMaxHist);
+  }
   void* tabs = take(table_bytes(pl.nth));
   pl.tab = (double*)tabs;
   pl.tabf = tabs ? (float*)((char*)tabs + 16 * (size_t)pl.nth) : nullptr;
   pl.tabi = tabs ? (int32_t*)((char*)tabs + 24 * (size_t)pl.nth) : nullptr;
-  pl.dct = take(dct_bytes(pl.n, pl.esize));
-  pl.dct_mu = pl.dct ? (const double*)((char*)pl.dct + 2 * (size_t)pl.n * pl.n * pl.esize) : nullptr;
+  if (!forward_only) {
+    pl.dct = take(dct_bytes(pl.n, pl.esize));
+    pl.dct_mu =
+        pl.dct ? (const double*)((char*)pl.dct + 2 * (size_t)pl.n * pl.n * pl.esize) : nullptr;
+  }
   pl.sync = (unsigned*)take(128 * (size_t)kResidentMaxItems);
   return off;
 }
 
-// The part of the workspace that the forward operator uses.
-static size_t carve_forward(Plan& pl, void* ws) {
-  char* b = (char*)ws;
-  size_t off = 0;
-  auto take = [&](size_t bytes) -> void* {
-    void* p = b ? (void*)(b + off) : nullptr;
-    off += up256(bytes);
-    return p;
-  };
-  const bool own = direct(pl);
-  const size_t wvol = (size_t)pl.nw * pl.nw * pl.nwp * pl.esize;
-  const size_t zvol = zvolume_bytes(pl.nw, pl.esize);
-  pl.kap = take(pl.n3 * pl.esize);
-  pl.kapw = own ? pl.kap : take(wvol);
-  for (int i = 0; i < 6; ++i) pl.s[i] = i < nstate(pl) ? take(wvol) : nullptr;
-  pl.x = own ? take(zvol) : nullptr;
-  pl.xw = own ? nullptr : take(zvol > wvol ? zvol : wvol);
-  pl.partials = (double*)take(sizeof(double) * kNumQuant * kReduceBlocks);
-  pl.tab = (double*)take(table_bytes(pl.nth));
-  pl.sync = (unsigned*)take(128 * (size_t)kResidentMaxItems);
-  return off;
+Scratch project_scratch(const Plan& pl, const void* pN) {
+  char *lo = (char*)pl.xw, *hi = (char*)pl.s[0] + pl.nstate * pl.svol, *p = (char*)pN;
+  const size_t before = p - lo, after = hi - (p + pl.svol);
+  return before >= after ? Scratch{lo, before} : Scratch{p + pl.svol, after};
+}
+
+Scratch backproject_scratch(const Plan& pl, const void* g) {
+  char *lo = (char*)pl.s[0], *r = lo + pl.nstate * pl.svol, *hi = r + pl.dvol;
+  if (g == pl.r2 && r2_in_state(pl)) lo += pl.dvol;
+  if (g == pl.r) hi = r;
+  return Scratch{lo, (size_t)(hi - lo)};
 }
 
 // Bytes that a whole workspace of dense, unrounded volumes and data has: the
 // measure by which ffpat_forward_noalloc accepts a problem, whatever the
-// kernels' layouts add to ffpat_workspace_bytes.  What it accepts fits
-// carve_forward with dense rows: the volumes and data left out there are more
-// than the slabs' rounding.
+// kernels' layouts add to ffpat_workspace_bytes.  What it accepts fits the forward
+// operator's part with dense rows.
 static size_t dense_workspace(const Plan& pl) {
   const size_t vol = up256(pl.n3 * pl.esize), wvol = up256(pl.nw3 * pl.esize);
   size_t b = 3 * vol + nstate(pl) * wvol + 2 * up256(pl.nd * pl.esize);
@@ -223,15 +235,15 @@ int plan_noalloc(const ffpat_problem* pr, Plan& pl, void* ws, size_t limit) {
                 "scratch holds %zu (a wave grid N + 2 pad <= 64 with <= 180 angles fits every "
                 "precision)", need, limit);
   // padded rows where they fit too
-  if (carve_forward(pl, nullptr) > limit) pl.nwp = pl.nw;
-  if (carve_forward(pl, nullptr) > limit)
+  if (carve(pl, nullptr, true) > limit) pl.nwp = pl.nw;
+  if (carve(pl, nullptr, true) > limit)
     return fail(FFPAT_EINVAL, "ffpat_forward_noalloc: no room for P's operand in the static scratch");
-  if (ws) carve_forward(pl, ws);
+  if (ws) carve(pl, ws, true);
   return FFPAT_OK;
 }
 
-int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path) {
-  TRY(validate(pr, pl, any_path));
+int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, Rows rows) {
+  TRY(validate(pr, pl, rows));
   const size_t need = carve(pl, nullptr);
   if (!ws) return fail(FFPAT_EINVAL, "workspace is NULL (%zu bytes needed)", need);
   if (((uintptr_t)ws & 255) != 0) return fail(FFPAT_EINVAL, "workspace not 256-byte aligned");
@@ -292,9 +304,9 @@ int time_steps(const Plan& pl, double cmax, int* nt, double* dt) {
 
 static int setup_attached(Plan& pl, const void* c, cudaStream_t st);
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
-          cudaStream_t st, bool any_path) {
+          cudaStream_t st, Rows rows) {
   g_err[0] = 0;
-  TRY(attach(pr, pl, ws, ws_bytes, any_path));
+  TRY(attach(pr, pl, ws, ws_bytes, rows));
   return setup_attached(pl, c, st);
 }
 
@@ -323,7 +335,7 @@ static int setup_attached(Plan& pl, const void* c, cudaStream_t st) {
   TRY(time_steps(pl, pl.cmax, &pl.nt, &pl.dt));
   // c and kapw live on the wave grid; kap is kapw's restriction to the box
   TRY(launch_kappa(wave_plan(pl), c, st));
-  if (!direct(pl)) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
+  if (pl.pad) TRY(launch_restrict(pl, pl.kapw, pl.kap, st));
   return FFPAT_OK;
 }
 
@@ -639,17 +651,14 @@ static int wave_fwd(const Plan& pl, const void* v, const void** pN, cudaStream_t
   return run_wave(wave_plan(pl), pl.xw, nullptr, pN, st);
 }
 
-// The wave-grid input buffer of wave_back.
-static void* wave_in(const Plan& pl) { return direct(pl) ? pl.x : pl.xw; }
-
 // E^T W x for a wave-grid x (already scaled by kappa: W^T = K^-1 W K), the
-// box result returned through *w (a state buffer, or pl.xo unless direct).
+// box result returned through *w: a state buffer, in rows of kap_pitch().
 static int wave_back(const Plan& pl, const void* x, const void** w, cudaStream_t st) {
-  if (direct(pl)) return run_wave(pl, x, nullptr, w, st);
-  const void* r = nullptr;
-  TRY(run_wave(wave_plan(pl), x, nullptr, &r, st));
-  TRY(launch_restrict(pl, r, pl.xo, st));
-  *w = pl.xo;
+  TRY(run_wave(wave_plan(pl), x, nullptr, w, st));
+  if (!pl.pad) return FFPAT_OK;
+  void* box = *w == pl.s[0] ? pl.s[1] : pl.s[0];
+  TRY(launch_restrict(pl, *w, box, st));
+  *w = box;
   return FFPAT_OK;
 }
 
@@ -657,8 +666,7 @@ static int apply_forward(const Plan& pl, const void* h, void* g, cudaStream_t st
   if (!h || !g) return fail(FFPAT_EINVAL, "h or g is NULL");
   const void* pN = nullptr;
   TRY(wave_fwd(pl, h, &pN, st));
-  TRY(launch_project(wave_plan(pl), pN, g, nullptr, st, nullptr, wave_in(pl)));
-  return FFPAT_OK;
+  return launch_project(wave_plan(pl), pN, g, nullptr, st, nullptr, project_scratch(pl, pN));
 }
 
 int forward_noalloc(const ffpat_problem* pr, const void* c, const void* h, void* g, void* ws,
@@ -674,9 +682,9 @@ int forward_noalloc(const ffpat_problem* pr, const void* c, const void* h, void*
 // h = E^T W^T P^T g  ->  x = K P^T g ; w = E^T W x ; h = w / K
 static int apply_adjoint(const Plan& pl, const void* g, void* h, cudaStream_t st) {
   const Plan wp = wave_plan(pl);
-  TRY(launch_backproject(wp, g, wave_in(pl), wp.kap, st, pl.r));
+  TRY(launch_backproject(wp, g, pl.xw, wp.kap, st, backproject_scratch(pl, g)));
   const void* w = nullptr;
-  TRY(wave_back(pl, wave_in(pl), &w, st));
+  TRY(wave_back(pl, pl.xw, &w, st));
   TRY(launch_kscale(pl, w, h, false, st));
   return FFPAT_OK;
 }
@@ -691,16 +699,17 @@ static int data_gradient(const Plan& pl, const void* v, const void* g, const voi
   TRY(wave_fwd(pl, v, &pN, st));
   {
     Trace trace_data("P, residual, Lambda, P^T");
-    TRY(launch_project(wp, pN, pl.r, g, st, mask, wave_in(pl)));
-    const void* lr = pl.r;
+    void* r = residual(pl);
+    TRY(launch_project(wp, pN, r, g, st, mask, project_scratch(pl, pN)));
+    const void* lr = r;
     if (pl.precond == FFPAT_PRECOND_RAMP) {
-      TRY(launch_ramp(wp, pl.r, pl.r2, st, mask));
+      TRY(launch_ramp(wp, r, pl.r2, st, mask));
       lr = pl.r2;
     }
-    if (dots) TRY(launch_dot(pl, pl.nd, lr, pl.r, dots, st));
-    TRY(launch_backproject(wp, lr, wave_in(pl), wp.kap, st, lr == pl.r ? pl.r2 : pl.r));
+    if (dots) TRY(launch_dot(pl, pl.nd, lr, r, dots, st));
+    TRY(launch_backproject(wp, lr, pl.xw, wp.kap, st, backproject_scratch(pl, lr)));
   }
-  TRY(wave_back(pl, wave_in(pl), w, st));
+  TRY(wave_back(pl, pl.xw, w, st));
   return FFPAT_OK;
 }
 
@@ -895,9 +904,9 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
       }
     }
   } else {
-    TRY(launch_kmul_rows(wave_plan(pl), in, pl.nw, wave_in(pl), st));
+    TRY(launch_kmul_rows(wave_plan(pl), in, pl.nw, pl.xw, st));
     const void* w = nullptr;
-    TRY(wave_back(pl, wave_in(pl), &w, st));
+    TRY(wave_back(pl, pl.xw, &w, st));
     TRY(launch_kscale(pl, w, out, false, st));
   }
   return FFPAT_OK;
@@ -915,15 +924,16 @@ static int project_alone(const ffpat_problem* problem, const void* in, void* out
   if (!in || !out) return fail(FFPAT_EINVAL, transpose ? "g or h is NULL" : "p or g is NULL");
   const size_t tb = up256(table_bytes(pl.nth));
   const size_t rows = (size_t)pl.nw * (transpose ? pl.nth : pl.nw);
-  const size_t zb = zscratch_bytes(pl.nw, rows, pl.esize, kAloneScratch);
+  const size_t least = rows * 32 * pl.esize;
+  const size_t zb = zscratch_bytes(pl.nw, rows, pl.esize, least > kAloneScratch ? least : kAloneScratch);
   char* mem = nullptr;
   CK(cudaMallocAsync((void**)&mem, tb + zb, st));
   std::vector<unsigned char> tabs;
   int rc = upload_tables(pl, mem, tabs, st);
   const Plan wp = dense_rows(wave_plan(pl));
   if (rc == FFPAT_OK)
-    rc = transpose ? launch_backproject(wp, in, out, nullptr, st, mem + tb, 1.0, kAloneScratch)
-                   : launch_project(wp, in, out, nullptr, st, nullptr, mem + tb, kAloneScratch);
+    rc = transpose ? launch_backproject(wp, in, out, nullptr, st, Scratch{mem + tb, zb})
+                   : launch_project(wp, in, out, nullptr, st, nullptr, Scratch{mem + tb, zb});
   const cudaError_t ef = cudaFreeAsync(mem, st), es = cudaStreamSynchronize(st);
   TRY(rc);
   CK(ef);
@@ -1049,7 +1059,8 @@ int ffpat_fbp(const ffpat_problem* problem, const void* G, void* out, void* ws, 
   TRY(rc);
   const Plan wp = wave_plan(pl);
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(dense_rows(wp), pl.r2, out, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(dense_rows(wp), pl.r2, out, nullptr, st, backproject_scratch(pl, pl.r2),
+                         2.0 * M_PI / (pl.nth * pl.dx)));
   return FFPAT_OK;
 }
 
@@ -1061,8 +1072,8 @@ static int power_iteration_w(const Plan& pl, int iters, double* est, cudaStream_
   for (int it = 0; it < iters; ++it) {
     const void* w = nullptr;
     TRY(wave_fwd(pl, pl.v, &w, st));
-    TRY(launch_kmul_rows(wave_plan(pl), w, pl.nwp, wave_in(pl), st));
-    TRY(wave_back(pl, wave_in(pl), &w, st));
+    TRY(launch_kmul_rows(wave_plan(pl), w, pl.nwp, pl.xw, st));
+    TRY(wave_back(pl, pl.xw, &w, st));
     TRY(launch_kscale(pl, w, pl.v, false, st));
     TRY(launch_dot(pl, pl.n3, pl.v, pl.v, sq, st));
     TRY(launch_scale_dev(pl, pl.n3, pl.v, pl.v, sq, st));
@@ -1108,15 +1119,16 @@ int ffpat_fb_two_step_ex(const ffpat_problem* problem, const void* c, const void
   const Plan wp = wave_plan(pl);
   void* gt = pl.pad ? pl.xg : pl.v;
   TRY(launch_ramp(wp, G, pl.r2, st));
-  TRY(launch_backproject(dense_rows(wp), pl.r2, gt, nullptr, st, pl.r, 2.0 * M_PI / (pl.nth * pl.dx)));
+  TRY(launch_backproject(dense_rows(wp), pl.r2, gt, nullptr, st, backproject_scratch(pl, pl.r2),
+                         2.0 * M_PI / (pl.nth * pl.dx)));
   int k = 0;
   for (; k < max_iters; ++k) {
     Trace trace_it("FB iteration (Algorithm 9)");
     double* hk = pl.hist + 8 * (size_t)k;
     const void* w = nullptr;
     TRY(wave_fwd(pl, h_inout, &w, st));
-    TRY(launch_resid_kap(wp, w, gt, wave_in(pl), hk, st));
-    TRY(wave_back(pl, wave_in(pl), &w, st));
+    TRY(launch_resid_kap(wp, w, gt, pl.xw, hk, st));
+    TRY(wave_back(pl, pl.xw, &w, st));
     if (regulariser == FFPAT_REG_GRAD2)
       TRY(prox_grad_step(pl, h_inout, w, step, lambda, hk + 2, st));
     else

@@ -84,12 +84,23 @@ __global__ void k_kappa(const T* __restrict__ c, T* __restrict__ kap, size_t len
   }
 }
 
+// Where element i of a dense n^3 volume lies in rows of n + extra elements: w and kap
+// on padded rows are read in place (a copy of either without the padding costs a
+// volume of memory and another pass; the division is hidden behind the loads).
+struct PitchedAt {
+  unsigned n, extra;
+  __device__ __forceinline__ size_t operator()(size_t i) const {
+    if (extra == 0) return i;
+    return i + (i >> 32 ? i / n : (size_t)((unsigned)i / n)) * extra;
+  }
+};
+
 template <typename T>
 __global__ void k_kscale(const T* __restrict__ a, T* __restrict__ out, const T* __restrict__ kap,
-                         size_t len, bool mul) {
+                         size_t len, bool mul, PitchedAt at) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x)
-    out[i] = mul ? a[i] * kap[i] : a[i] / kap[i];
+    out[i] = mul ? a[at(i)] * kap[at(i)] : a[at(i)] / kap[at(i)];
 }
 
 // Volumes with padded rows (n points in np elements) next to dense ones: a warp
@@ -173,7 +184,7 @@ __global__ void __launch_bounds__(kReduceThreads)
 template <typename T>
 __global__ void __launch_bounds__(kReduceThreads)
     k_fb_update(T* __restrict__ h, const T* __restrict__ w, const T* __restrict__ kap, size_t len,
-                double step, const double* __restrict__ step_dev, double lambda,
+                PitchedAt at, double step, const double* __restrict__ step_dev, double lambda,
                 const T* __restrict__ support, double* __restrict__ partials) {
   double l1 = 0.0, hh = 0.0, dd = 0.0, nn = 0.0;
   if (step_dev) step = *step_dev;
@@ -181,7 +192,7 @@ __global__ void __launch_bounds__(kReduceThreads)
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x) {
     const T hv = h[i];
-    const T grad = w[i] / kap[i];
+    const T grad = w[at(i)] / kap[at(i)];
     const T f = (hv - s * grad) - sl;
     T hn = f > T(0) ? f : T(0);
     if (support) hn = hn * support[i];
@@ -208,13 +219,13 @@ __global__ void __launch_bounds__(kReduceThreads)
 // the prox; the same arithmetic as k_fb_update before its shrinkage)
 template <typename T>
 __global__ void k_prox_prep(const T* __restrict__ h, const T* __restrict__ w,
-                            const T* __restrict__ kap, T* __restrict__ x, size_t len, double step,
-                            const double* __restrict__ step_dev) {
+                            const T* __restrict__ kap, T* __restrict__ x, size_t len, PitchedAt at,
+                            double step, const double* __restrict__ step_dev) {
   if (step_dev) step = *step_dev;
   const T s = (T)step;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x)
-    x[i] = h[i] - s * (w[i] / kap[i]);
+    x[i] = h[i] - s * (w[at(i)] / kap[at(i)]);
 }
 
 // part 2, after the prox wrote hn: the FP64 partials of R(h) = 1/2 <D h, D h>
@@ -300,19 +311,19 @@ __global__ void __launch_bounds__(kReduceThreads)
 // out = (a - b) / kap   (last step of the transposed recurrence, back from kap-scaled form)
 template <typename T>
 __global__ void k_sub_div(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ kap,
-                          T* __restrict__ out, size_t len) {
+                          T* __restrict__ out, size_t len, PitchedAt at) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x)
-    out[i] = (a[i] - b[i]) / kap[i];
+    out[i] = (a[at(i)] - b[at(i)]) / kap[at(i)];
 }
 
 // out = s * a / c
 template <typename T>
 __global__ void k_scale_div(const T* __restrict__ a, const T* __restrict__ c, T s,
-                            T* __restrict__ out, size_t len) {
+                            T* __restrict__ out, size_t len, PitchedAt at) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < len;
        i += (size_t)gridDim.x * blockDim.x)
-    out[i] = s * a[i] / c[i];
+    out[i] = s * a[at(i)] / c[i];
 }
 
 // counter-based pseudo-random start vector (splitmix64 + Box-Muller)
@@ -339,6 +350,10 @@ unsigned ew_blocks(size_t len) {
   size_t b = (len + 255) / 256;
   const size_t cap = 16 * kNumSMs;
   return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
+}
+
+PitchedAt pitched(const Plan& pl) {
+  return PitchedAt{(unsigned)pl.n, (unsigned)(kap_pitch(pl) - pl.n)};
 }
 
 }  // namespace
@@ -387,9 +402,11 @@ int launch_kappa(const Plan& pl, const void* c, cudaStream_t st) {
 int launch_kscale(const Plan& pl, const void* a, void* out, bool mul, cudaStream_t st) {
   const unsigned nb = ew_blocks(pl.n3);
   if (pl.prec == FFPAT_FP64)
-    k_kscale<double><<<nb, 256, 0, st>>>((const double*)a, (double*)out, (const double*)pl.kap, pl.n3, mul);
+    k_kscale<double><<<nb, 256, 0, st>>>((const double*)a, (double*)out, (const double*)pl.kap, pl.n3, mul,
+                                         pitched(pl));
   else
-    k_kscale<float><<<nb, 256, 0, st>>>((const float*)a, (float*)out, (const float*)pl.kap, pl.n3, mul);
+    k_kscale<float><<<nb, 256, 0, st>>>((const float*)a, (float*)out, (const float*)pl.kap, pl.n3, mul,
+                                        pitched(pl));
   count_launch();
   return check_launch(__func__);
 }
@@ -440,11 +457,11 @@ int launch_fb_update(const Plan& pl, void* h, const void* w, double step, double
                      double* dst, cudaStream_t st, const double* step_dev, const void* support) {
   if (pl.prec == FFPAT_FP64)
     k_fb_update<double><<<kReduceBlocks, kReduceThreads, 0, st>>>(
-        (double*)h, (const double*)w, (const double*)pl.kap, pl.n3, step, step_dev, lambda,
-        (const double*)support, pl.partials);
+        (double*)h, (const double*)w, (const double*)pl.kap, pl.n3, pitched(pl), step, step_dev,
+        lambda, (const double*)support, pl.partials);
   else
     k_fb_update<float><<<kReduceBlocks, kReduceThreads, 0, st>>>(
-        (float*)h, (const float*)w, (const float*)pl.kap, pl.n3, step, step_dev, lambda,
+        (float*)h, (const float*)w, (const float*)pl.kap, pl.n3, pitched(pl), step, step_dev, lambda,
         (const float*)support, pl.partials);
   k_finalize<<<4, kReduceThreads, 0, st>>>(pl.partials, dst);
   count_launch(2);
@@ -456,10 +473,11 @@ int launch_prox_prep(const Plan& pl, const void* h, const void* w, double step, 
   const unsigned nb = ew_blocks(pl.n3);
   if (pl.prec == FFPAT_FP64)
     k_prox_prep<double><<<nb, 256, 0, st>>>((const double*)h, (const double*)w,
-                                            (const double*)pl.kap, (double*)x, pl.n3, step, step_dev);
+                                            (const double*)pl.kap, (double*)x, pl.n3, pitched(pl),
+                                            step, step_dev);
   else
     k_prox_prep<float><<<nb, 256, 0, st>>>((const float*)h, (const float*)w, (const float*)pl.kap,
-                                           (float*)x, pl.n3, step, step_dev);
+                                           (float*)x, pl.n3, pitched(pl), step, step_dev);
   count_launch();
   return check_launch(__func__);
 }
@@ -507,10 +525,10 @@ int launch_sub_div(const Plan& pl, const void* a, const void* b, void* out, cuda
   const unsigned nb = ew_blocks(pl.n3);
   if (pl.prec == FFPAT_FP64)
     k_sub_div<double><<<nb, 256, 0, st>>>((const double*)a, (const double*)b,
-                                          (const double*)pl.kap, (double*)out, pl.n3);
+                                          (const double*)pl.kap, (double*)out, pl.n3, pitched(pl));
   else
     k_sub_div<float><<<nb, 256, 0, st>>>((const float*)a, (const float*)b, (const float*)pl.kap,
-                                         (float*)out, pl.n3);
+                                         (float*)out, pl.n3, pitched(pl));
   count_launch();
   return check_launch(__func__);
 }
@@ -520,10 +538,10 @@ int launch_scale_div(const Plan& pl, const void* a, const void* c, double s, voi
   const unsigned nb = ew_blocks(pl.n3);
   if (pl.prec == FFPAT_FP64)
     k_scale_div<double><<<nb, 256, 0, st>>>((const double*)a, (const double*)c, s, (double*)out,
-                                            pl.n3);
+                                            pl.n3, pitched(pl));
   else
     k_scale_div<float><<<nb, 256, 0, st>>>((const float*)a, (const float*)c, (float)s,
-                                           (float*)out, pl.n3);
+                                           (float*)out, pl.n3, pitched(pl));
   count_launch();
   return check_launch(__func__);
 }

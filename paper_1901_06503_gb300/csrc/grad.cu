@@ -64,12 +64,12 @@ bool use_tma(const Plan& pl, const Ckpt& ck, const void* a) {
   return tma_supported(pl, ptrs, 8) && (ck.vol % 16) == 0;
 }
 
-// The view the steps run on: the wave grid with its padded rows in FP32; dense
-// rows in FP64 (whose accumulation kernel is the plain one) and for a checkpoint
-// buffer that TMA cannot address.  The same for the forward and the backward pass.
-Plan grad_view(const Plan& pl, const Ckpt& ck) {
-  const Plan w = wave_plan(pl);
-  return pl.esize == 4 && use_tma(w, ck, nullptr) ? w : pl;
+// The rows the steps run on: padded in FP32; dense in FP64 (whose accumulation
+// kernel is the plain one) and for a checkpoint buffer that TMA cannot address.  The
+// same for the forward and the backward pass.
+Rows grad_rows(const ffpat_problem* pr, const void* ckpt) {
+  const bool tma = pr && pr->precision != FFPAT_FP64 && ((uintptr_t)ckpt & 15) == 0;
+  return tma ? Rows::kPadded : Rows::kDense;
 }
 
 // two steps per pass in the checkpointed loops: W's rule, and checkpoints at
@@ -99,7 +99,7 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
                        void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   Plan pl;
-  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, true);
+  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, grad_rows(problem, ckpt));
   if (rc0 != FFPAT_OK) return rc0;
   if (!h || !g || !ckpt) return report(FFPAT_EINVAL, "h, g or ckpt is NULL");
   as_three_term(pl);
@@ -107,7 +107,7 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
   if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
   if (ckpt_bytes < ck.bytes())
     return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
-  const Plan w = grad_view(pl, ck);
+  const Plan w = wave_plan(pl);
   const void* in = h;
   if (w.np != w.n) {  // the source in padded rows
     const int rc = launch_embed(pl, h, pl.xw, st);
@@ -121,7 +121,8 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
     bool refused = false;
     const int rc = launch_wave_resident(w, 0, in, nullptr, pl.s[0], pl.s[1], &last, st, &refused,
                                         &save);
-    if (rc == FFPAT_OK) return launch_project(w, last, g, nullptr, st, nullptr, pl.x);
+    if (rc == FFPAT_OK)
+      return launch_project(w, last, g, nullptr, st, nullptr, project_scratch(pl, last));
     if (!refused) return rc;  // refused: step by step
   }
   const bool two = use_two(w, ck, tma);
@@ -155,7 +156,7 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
         return check_launch("checkpoint copy");
     }
   }
-  return launch_project(w, S[b], g, nullptr, st, nullptr, pl.x);
+  return launch_project(w, S[b], g, nullptr, st, nullptr, project_scratch(pl, S[b]));
 }
 
 int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad_g, void* grad_h,
@@ -163,7 +164,7 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
                    size_t ws_bytes, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   Plan pl;
-  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, true);
+  const int rc0 = setup(problem, pl, c, ws, ws_bytes, st, grad_rows(problem, ckpt));
   if (rc0 != FFPAT_OK) return rc0;
   if (!grad_g || !ckpt) return report(FFPAT_EINVAL, "grad_g or ckpt is NULL");
   as_three_term(pl);
@@ -171,11 +172,10 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
   if (ckpt_bytes < ck.bytes())
     return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
-  const Plan w = grad_view(pl, ck);
+  const Plan w = wave_plan(pl);
   const bool tma = use_tma(w, ck, nullptr);
   const bool two = use_two(w, ck, tma);
   bool resident = resident_segments(w, tma, st);  // until a launch is turned down
-  const bool rows = w.np != w.n;
   const size_t vb = (size_t)w.n * w.n * w.np * w.esize;
   // mu^{Nt} = (kappa / 12) P^T grad_g, mu^{Nt+1} = 0
   // B[u] = mu^{n+1}, B[v] = mu^{n+2}; a pass writes into the other two buffers
@@ -190,7 +190,7 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   };
   const void* end = nullptr;  // start(mu^1) - mu^2 where a resident segment left it
   const void* tmp = nullptr;  // start(mu^1) else
-  int rc = launch_backproject(w, grad_g, B[u], w.kap, st, pl.r);
+  int rc = launch_backproject(w, grad_g, B[u], w.kap, st, backproject_scratch(pl, grad_g));
   if (rc != FFPAT_OK) return rc;
   if (cudaMemsetAsync(B[v], 0, vb, st) != cudaSuccess ||
       cudaMemsetAsync(ck.acc(), 0, vb, st) != cudaSuccess)
@@ -288,27 +288,11 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
     }
   }
   // grad_h = (start(mu^1) - mu^2) / (kappa / 12), grad_c = 2 acc / c, on dense rows
-  if (grad_h && end) {
-    if (rows) rc = launch_restrict(pl, end, pl.xo, st);
-    if (rc == FFPAT_OK) rc = launch_kscale(pl, rows ? pl.xo : end, grad_h, false, st);
-  } else if (grad_h) {
-    const void *ta = tmp, *tb = B[v];
-    if (rows) {
-      rc = launch_restrict(pl, tmp, pl.xo, st);
-      if (rc == FFPAT_OK) rc = launch_restrict(pl, B[v], pl.v, st);
-      ta = pl.xo;
-      tb = pl.v;
-    }
-    if (rc == FFPAT_OK) rc = launch_sub_div(pl, ta, tb, grad_h, st);
-  }
+  if (grad_h)
+    rc = end ? launch_kscale(pl, end, grad_h, false, st)
+             : launch_sub_div(pl, tmp, B[v], grad_h, st);
   if (rc != FFPAT_OK || !grad_c) return rc;
-  const void* acc = ck.acc();
-  if (rows) {
-    rc = launch_restrict(pl, acc, pl.xo, st);
-    if (rc != FFPAT_OK) return rc;
-    acc = pl.xo;
-  }
-  return launch_scale_div(pl, acc, c, 2.0, grad_c, st);
+  return launch_scale_div(pl, ck.acc(), c, 2.0, grad_c, st);
 }
 
 }  // extern "C"

@@ -29,17 +29,19 @@ struct Plan {
   int nwp = 0;            // row pitch of the wave grid's volumes: nw, or rounded up to 16 bytes
   double T = 0, cfl = 0, dx = 0, dt = 0, cmax = 0;
   size_t n3 = 0, nd = 0, esize = 0, nw3 = 0;
+  int nstate = 0;         // state volumes in the workspace,
+  size_t svol = 0;        // bytes from one to the next,
+  size_t dvol = 0;        // and of a data array there
   // workspace carve (device)
-  void* kap = nullptr;    // kappa / 12 on the image box
-  void* kapw = nullptr;   // kappa / 12 on the wave grid (== kap when direct())
+  void* kap = nullptr;    // kappa / 12 on the image box, rows of kap_pitch()
+  void* kapw = nullptr;   // kappa / 12 on the wave grid (== kap without padding cells)
   void* s[6] = {};        // wavefield state (wave grid): three-term p^{n-1}, p^n; increment form p, p', d, e, d', e'
-  void* xw = nullptr;     // wave-grid input of W or W^T unless direct()
-  void* xo = nullptr;     // image-box result of W^T unless direct()
+  void* xw = nullptr;     // wave-grid input of W or W^T (== x without padding cells); s[0] follows it
   void* xg = nullptr;     // wave-grid scratch (the FBP of Algorithm 9 when padded)
   void* x = nullptr;      // image-domain scratch (adjoint input / gradient)
   void* v = nullptr;      // image-domain scratch (power iteration vector)
-  void* r = nullptr;      // data-domain scratch (residual)
-  void* r2 = nullptr;     // data-domain scratch (Lambda residual)
+  void* r = nullptr;      // data-domain scratch; follows the last state volume
+  void* r2 = nullptr;     // data-domain scratch, P^T's input; may lie in the state volumes
   double* partials = nullptr;  // kNumQuant * kReduceBlocks doubles
   double* scal = nullptr;      // small device scalars
   double* hist = nullptr;      // per-iteration FB statistics (8 doubles / iteration, up to kMaxHist)
@@ -62,6 +64,9 @@ inline Plan wave_plan(const Plan& pl) {
   w.kap = pl.kapw;
   return w;
 }
+// Row pitch of kap, and of what wave_back() returns: the wave grid's without
+// padding cells.
+inline int kap_pitch(const Plan& pl) { return pl.pad ? pl.np : pl.nwp; }
 // The same grid with dense rows (the caller's own arrays).
 inline Plan dense_rows(Plan pl) {
   pl.np = pl.n;
@@ -74,9 +79,25 @@ constexpr int kResidentMaxItems = 1024;  // work items (step flags) of the resid
 constexpr int kScal = 64;
 
 // api.cu helpers shared with the server and the gradient path
-// (any_path: ragged rows are padded whatever the stencil path)
+// ragged rows: padded on the automatic stencil path, on any, or on none
+enum class Rows { kAuto, kPadded, kDense };
 int setup(const ffpat_problem* pr, Plan& pl, const void* c, void* ws, size_t ws_bytes,
-          cudaStream_t st, bool any_path = false);
+          cudaStream_t st, Rows rows = Rows::kAuto);
+// Where P and P^T put their operand with z innermost: the volumes of the
+// workspace that are free at that time.  P: the larger run beside the field pN (a
+// state volume) among the wave input and the state volumes; P^T: the state volumes
+// and r, less g where g lies in them.
+struct Scratch {
+  void* p;
+  size_t bytes;
+};
+inline bool r2_in_state(const Plan& pl) { return pl.r2 == pl.s[0]; }
+// where P leaves the residual of a data gradient (r2 leaves r to P^T)
+inline void* residual(const Plan& pl) {
+  return pl.precond == FFPAT_PRECOND_RAMP || r2_in_state(pl) ? pl.r : pl.r2;
+}
+Scratch project_scratch(const Plan& pl, const void* pN);
+Scratch backproject_scratch(const Plan& pl, const void* g);
 // one three-term leapfrog launch (TMA kernel when the layout allows)
 int step3(const Plan& pl, bool tma, bool start, const void* p, const void* qin, void* qout,
           void* copy0, cudaStream_t st);
@@ -87,7 +108,7 @@ bool two_step_three_term(const Plan& pl, bool tma);
 bool resident_segments(const Plan& pl, bool tma, cudaStream_t st);
 // row pitch the wave grid's volumes may have (whatever the path)
 int padded_row(const Plan& pl);
-int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, bool any_path = false);
+int attach(const ffpat_problem* pr, Plan& pl, void* ws, size_t ws_bytes, Rows rows = Rows::kAuto);
 // the forward operator in `limit` bytes of scratch at ws (ffpat_forward_noalloc);
 // plan_noalloc alone (ws nullable) says whether the problem is accepted
 int plan_noalloc(const ffpat_problem* pr, Plan& pl, void* ws, size_t limit);
@@ -235,22 +256,19 @@ int read_device_status(unsigned* out, bool clear);
 int launch_wait_timeout(long long cycles, cudaStream_t st);
 
 // xray.cu
-// bytes of a volume / of the data (n detectors, nth angles) with z innermost
-size_t zvolume_bytes(int n, size_t esize);
-size_t zdata_bytes(int n, int nth, size_t esize);
-// the same for `rows` rows when at most `limit` bytes are to be used (0: no limit),
-// the planes then going in several passes
+// bytes of `rows` rows of n planes with z innermost (P: n^2 rows, P^T: nth n) when
+// at most `limit` are to be used, the planes then going in several passes
 size_t zscratch_bytes(int n, size_t rows, size_t esize, size_t limit);
+constexpr int kMinPlanes32 = 32, kMinPlanes64 = 2;  // planes of a pass at least
 // g = mask .* (P p - sub)  (sub, mask nullable)
-// scratch: zvolume_bytes (zscratch_bytes(n, n^2, .) with a limit) that alias neither
-// p nor g; receives p with z innermost
+// scratch: at least the planes of one pass; aliases neither p nor g; receives p with
+// z innermost
 int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
-                   const void* mask, void* scratch, size_t limit = 0);
+                   const void* mask, Scratch scratch);
 // h = mult * scale .* P^T g  (scale nullable)
-// scratch: zdata_bytes (zscratch_bytes(n, nth n, .) with a limit) that alias neither
-// g nor h; receives g with z innermost
+// scratch: the same for g; aliases neither g nor h
 int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       void* scratch, double mult = 1.0, size_t limit = 0);
+                       Scratch scratch, double mult = 1.0);
 // out = mask .* (Lambda r)  (mask nullable)
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st,
                 const void* mask = nullptr);
@@ -276,7 +294,9 @@ int launch_prox_finish(const Plan& pl, void* h, const void* hn, double* dst, cud
 // and wave grid -> box
 int launch_embed(const Plan& pl, const void* box, void* wave, cudaStream_t st);
 int launch_restrict(const Plan& pl, const void* wave, void* box, cudaStream_t st);
-// out[i] = a[i] * kap[i] (mul = true) or a[i] / kap[i] on dense rows
+// The launches below that take w, kap, a or b beside dense volumes read those four
+// in rows of kap_pitch().
+// out[i] = a[i] * kap[i] (mul = true) or a[i] / kap[i]
 int launch_kscale(const Plan& pl, const void* a, void* out, bool mul, cudaStream_t st);
 // out = a kap on the wave view `pl`; a has rows of `ap` elements, out of pl.np
 int launch_kmul_rows(const Plan& pl, const void* a, int ap, void* out, cudaStream_t st);

@@ -217,15 +217,18 @@ int after_wave(ffpat_server* S, Req& r) {
   const Plan& pl = r.pl;
   const bool power = r.it < r.power_iters;
   if (r.phase == kFwd) {
-    if (launch_project(pl, r.cur, pl.r, power ? nullptr : r.g_d, st, nullptr, pl.x) != FFPAT_OK)
+    void* res = residual(pl);
+    if (launch_project(pl, r.cur, res, power ? nullptr : r.g_d, st, nullptr,
+                       project_scratch(pl, r.cur)) != FFPAT_OK)
       return FFPAT_ECUDA;
-    const void* lr = pl.r;
+    const void* lr = res;
     if (pl.precond == FFPAT_PRECOND_RAMP) {
-      if (launch_ramp(pl, pl.r, pl.r2, st) != FFPAT_OK) return FFPAT_ECUDA;
+      if (launch_ramp(pl, res, pl.r2, st) != FFPAT_OK) return FFPAT_ECUDA;
       lr = pl.r2;
     }
-    if (!power && launch_dot(pl, pl.nd, lr, pl.r, pl.hist, st) != FFPAT_OK) return FFPAT_ECUDA;
-    if (launch_backproject(pl, lr, pl.x, pl.kap, st, lr == pl.r ? pl.r2 : pl.r) != FFPAT_OK) return FFPAT_ECUDA;
+    if (!power && launch_dot(pl, pl.nd, lr, res, pl.hist, st) != FFPAT_OK) return FFPAT_ECUDA;
+    if (launch_backproject(pl, lr, pl.x, pl.kap, st, backproject_scratch(pl, lr)) != FFPAT_OK)
+      return FFPAT_ECUDA;
     r.phase = kAdj;
     r.wstep = 0;
     r.w_in = (const float*)pl.x;

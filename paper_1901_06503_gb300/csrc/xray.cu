@@ -1021,19 +1021,24 @@ __global__ void k_debug_samples(int count, const int32_t* __restrict__ jkm, int3
 
 }  // namespace
 
-// Planes in a slab of a z-innermost operand.  FP64: all of them in one slab,
-// rounded up to 16 bytes.  FP32: 32 V C for one of the instantiated (V, C), the
-// one of least time for n planes, slabs x the measured cost of a slab (P + P^T
-// at 128^3, 192^3 and 384^3 with every width, in units of the 64-plane slab):
-// wider slabs share the weights and addresses among more planes, until the last
-// one is mostly idle lanes.
-static int slab_planes(int n, size_t esize) {
-  if (esize == 8) return (n + 1) / 2 * 2;
+// Planes in a slab of a z-innermost operand, `most` of them at most (or as few as a
+// slab can have).  FP64: all of them in one slab, rounded up to 16 bytes.  FP32: 32 V
+// C for one of the instantiated (V, C), the one of least time for n planes, slabs x
+// the measured cost of a slab (P + P^T at 128^3, 192^3 and 384^3 with every width, in
+// units of the 64-plane slab): wider slabs share the weights and addresses among more
+// planes, until the last one is mostly idle lanes.
+static int slab_planes(int n, size_t esize, size_t most) {
+  if (esize == 8) {
+    const int all = (n + 1) / 2 * 2;
+    if ((size_t)all <= most) return all;
+    return most >= 32 ? (int)(most / 32 * 32) : (most >= 2 ? (int)(most / 2 * 2) : kMinPlanes64);
+  }
   static const int rl[] = {32, 64, 96, 128, 160, 192, 256, 320, 384};
   static const float cost[] = {0.85f, 1.0f, 1.14f, 1.25f, 1.4f, 1.5f, 1.85f, 2.3f, 2.7f};
-  int best = 0;
+  int best = kMinPlanes32;
   float best_cost = 1e30f;
   for (int i = 0; i < 9; ++i) {
+    if ((size_t)rl[i] > most) break;
     const float c = cost[i] * (float)((n + rl[i] - 1) / rl[i]);
     if (c < best_cost) {
       best = rl[i];
@@ -1043,29 +1048,14 @@ static int slab_planes(int n, size_t esize) {
   return best;
 }
 
-size_t zvolume_bytes(int n, size_t esize) {
-  const size_t rl = slab_planes(n, esize);
-  return (size_t)n * n * ((n + rl - 1) / rl * rl) * esize;
-}
-size_t zdata_bytes(int n, int nth, size_t esize) {
-  const size_t rl = slab_planes(n, esize);
-  return (size_t)nth * n * ((n + rl - 1) / rl * rl) * esize;
-}
-
-// The planes a call takes at a time with `limit` bytes of scratch (0: enough for
-// all) for `rows` rows of planes, and the planes of a slab: whole slabs, the
-// narrowest ones where not even one fits (then the limit is exceeded).
+// The planes a call takes at a time with `limit` bytes of scratch for `rows` rows of
+// planes, and the planes of a slab: whole slabs, the widest choice that fits (the
+// narrowest where not even one fits; then the limit is exceeded).
 static int planes_at_once(int n, size_t rows, size_t esize, size_t limit, int* rl) {
-  *rl = slab_planes(n, esize);
-  const size_t all = rows * ((n + *rl - 1) / *rl * (size_t)*rl) * esize;
-  if (limit == 0 || all <= limit) return n;
-  if (esize == 4 && rows * *rl * esize > limit) *rl = 32;
-  const size_t unit = esize == 4 ? *rl : 32;
-  size_t units = limit / (rows * unit * esize);
-  if (units < 1) units = 1;
-  const int planes = (int)(units * unit);
-  if (esize == 8) *rl = planes;
-  return planes;
+  const size_t most = limit / (rows * esize);
+  *rl = slab_planes(n, esize, most);
+  const size_t slabs = (n + *rl - 1) / *rl, fit = most / *rl;
+  return slabs <= fit ? n : *rl * (int)(fit < 1 ? 1 : fit);
 }
 size_t zscratch_bytes(int n, size_t rows, size_t esize, size_t limit) {
   int rl;
@@ -1180,13 +1170,15 @@ static int project_planes(const Plan& pl, const void* p, void* g, const void* su
 }
 
 int launch_project(const Plan& pl, const void* p, void* g, const void* sub, cudaStream_t st,
-                   const void* mask, void* scratch, size_t limit) {
-  if (!scratch) return report(FFPAT_EINVAL, "launch_project: no scratch volume");
+                   const void* mask, Scratch scratch) {
+  const size_t rows = (size_t)pl.n * pl.n;
+  if (!scratch.p || zscratch_bytes(pl.n, rows, pl.esize, scratch.bytes) > scratch.bytes)
+    return report(FFPAT_EINVAL, "launch_project: %zu bytes of scratch", scratch.bytes);
   int rl;
-  const int step = planes_at_once(pl.n, (size_t)pl.n * pl.n, pl.esize, limit, &rl);
+  const int step = planes_at_once(pl.n, rows, pl.esize, scratch.bytes, &rl);
   for (int z0 = 0; z0 < pl.n; z0 += step) {
     const int nz = pl.n - z0 < step ? pl.n - z0 : step;
-    const int rc = project_planes(pl, p, g, sub, mask, scratch, z0, nz, rl, st);
+    const int rc = project_planes(pl, p, g, sub, mask, scratch.p, z0, nz, rl, st);
     if (rc != FFPAT_OK) return rc;
   }
   return FFPAT_OK;
@@ -1239,13 +1231,15 @@ static int backproject_planes(const Plan& pl, const void* g, void* h, const void
 }
 
 int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale, cudaStream_t st,
-                       void* scratch, double mult, size_t limit) {
-  if (!scratch) return report(FFPAT_EINVAL, "launch_backproject: no data scratch");
+                       Scratch scratch, double mult) {
+  const size_t rows = (size_t)pl.nth * pl.n;
+  if (!scratch.p || zscratch_bytes(pl.n, rows, pl.esize, scratch.bytes) > scratch.bytes)
+    return report(FFPAT_EINVAL, "launch_backproject: %zu bytes of scratch", scratch.bytes);
   int rl;
-  const int step = planes_at_once(pl.n, (size_t)pl.nth * pl.n, pl.esize, limit, &rl);
+  const int step = planes_at_once(pl.n, rows, pl.esize, scratch.bytes, &rl);
   for (int z0 = 0; z0 < pl.n; z0 += step) {
     const int nz = pl.n - z0 < step ? pl.n - z0 : step;
-    const int rc = backproject_planes(pl, g, h, scale, scratch, z0, nz, rl, mult, st);
+    const int rc = backproject_planes(pl, g, h, scale, scratch.p, z0, nz, rl, mult, st);
     if (rc != FFPAT_OK) return rc;
   }
   return FFPAT_OK;
