@@ -595,10 +595,15 @@ __device__ __noinline__ float voxel_alone(const float* __restrict__ gp, int rl, 
 // A batch of eight angles is spread over all directions: data that change sign
 // slowly with the angle (filtered ones) then keep the partial sums, and with them
 // the rounding of the long sum, small (256^3, 180 angles of filtered data, error
-// against 64 bits 3.1 - 3.6e-7 -> 2.9e-7; at no cost in time).
+// against 64 bits 3.1 - 3.6e-7 -> 2.9e-7).  The list holds addresses: stepping a
+// pointer through the spread rows took 2 % more (fbp at 192^3 / 90 angles 231 -> 222
+// us, 256^3 / 180 779 -> 758 us, 384^3 / 180 2.56 -> 2.51 ms).
 constexpr int kBDet = 5;
 constexpr int kBTileX = 4, kBTileY = 2;  // blocks of a CTA (8 x 4 voxels), one a warp
-constexpr size_t kBWarpBytes = kBAngles * (kBDet * 16 + 4);
+// the detectors of a block and angle: address of the first one's planes, and count
+// (one 16-byte shared load; as two loads 256^3 took 3 % more)
+using BDetectors = ulonglong2;
+constexpr size_t kBWarpBytes = kBAngles * (kBDet * 16 + sizeof(BDetectors));
 
 template <int T, int V, int C>
 __device__ __forceinline__ void block_taps(const float* q, const float4* w,
@@ -627,12 +632,12 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x / 32;
   float4* W = reinterpret_cast<float4*>(smem_raw) + (size_t)warp * kBAngles * kBDet;
-  int* info = reinterpret_cast<int*>(smem_raw + (size_t)warps * kBAngles * kBDet * 16) +
-              warp * kBAngles;
+  BDetectors* list =
+      reinterpret_cast<BDetectors*>(smem_raw + (size_t)warps * kBAngles * kBDet * 16) +
+      warp * kBAngles;
   const int ty = warps / tx;  // tx x ty blocks in this CTA
   const int x0 = 2 * (blockIdx.x * tx + warp % tx), y0 = 2 * (blockIdx.y * ty + warp / tx);
   const int zbase = blockIdx.z * RL;
-  const float* __restrict__ gz = gt + (size_t)blockIdx.z * nth * n * RL + lane * V;
   const long long ck = (long long)(n - 1) << 30, cm = (long long)(ns - 1) << 30;
   // this lane's voxel and angle in the weight pass
   const int vox = lane & 3, al = lane >> 2;
@@ -668,15 +673,17 @@ __global__ void __launch_bounds__(kBTileX* kBTileY * 32, V* C > 8 ? 2 : 3)
 #pragma unroll
     for (int d = 0; d < kBDet; ++d)
       if (d >= first) wl[4 * (d - first)] = w[d];
-    if (vox == 0) info[al] = (kd + first) * 8 + count;
+    if (vox == 0)
+      list[al] = make_ulonglong2(
+          (unsigned long long)(gt + ((size_t)blockIdx.z * nth * n + (long long)(j * n + kd + first)) * RL),
+          ja + al * nb < nth ? count : 0);
     if (ja == 0) wait_for_operand();
     __syncwarp();
-    const int jn = min(kBAngles, (nth - ja + nb - 1) / nb);
-    const float* row = gz + (size_t)ja * n * RL;
 #pragma unroll 1
-    for (int t = 0; t < jn; ++t, row += (size_t)nb * n * RL) {
-      const int code = info[t], cnt = code & 7;
-      const float* q = row + (long long)(code >> 3) * RL;
+    for (int t = 0; t < kBAngles; ++t) {
+      const BDetectors det = list[t];
+      const unsigned cnt = (unsigned)det.y;
+      const float* q = reinterpret_cast<const float*>(det.x) + lane * V;
       const float4* u = W + t * kBDet;
       if (cnt == 4)
         block_taps<4, V, C>(q, u, acc);
