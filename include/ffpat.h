@@ -314,12 +314,14 @@ int ffpat_debug_fma_rate(int32_t kind, double *flops_per_s, void *stream);
 /* The differentiated operator needs pad = 0 (the box is the wave grid). */
 
 /* Checkpoint buffer bytes for Nt steps (ffpat_problem_info) and interval
- * `every`: (2 ceil(Nt / every) + every + 2) volumes of the wave grid (FP32 with
- * N <= 84: `every` more; FP32 rows rounded up to 16 bytes); 0 if invalid. */
+ * `every`: (2 ceil(Nt / every) + every + 2) volumes of the wave grid (FP32 rows
+ * rounded up to 16 bytes), and with FP32, N <= 84 and Nt > every at most `every`
+ * more, with which the backward pass overlaps its segments; 0 if invalid. */
 size_t ffpat_ckpt_bytes(const ffpat_problem *problem, int32_t nt, int32_t every);
 
 /* g = P W h with checkpoints (device buffers as for ffpat_forward; ckpt is
- * caller-owned device memory of ffpat_ckpt_bytes bytes, 256-byte aligned). */
+ * caller-owned device memory of ffpat_ckpt_bytes bytes, 256-byte aligned; without
+ * the volumes for the overlap it is accepted too). */
 int ffpat_forward_ckpt(const ffpat_problem *problem, const void *c, const void *h, void *g,
                        int32_t every, void *ckpt, size_t ckpt_bytes, void *ws, size_t ws_bytes,
                        void *stream);

@@ -10,8 +10,8 @@
 // the last, the states p^n of the segment are recomputed from its checkpoint
 // and the kappa-derivatives mu^{n+1} L(p^n) (weight 1/2 for the start step)
 // are accumulated; grad_c = 2 acc / c because dkappa/dc = 2 kappa / c and the
-// factors kappa/12 and 12 cancel.  Memory: 2 ceil(Nt/k) + k + 2 volumes (k more
-// on small grids, whose segments overlap).
+// factors kappa/12 and 12 cancel.  Memory: 2 ceil(Nt/k) + k + 2 volumes (on small
+// grids up to k more, with which the segments overlap).
 //
 // Where the resident time loop runs (FP32, N <= 128), the forward pass is one
 // cooperative launch that stores the checkpoints as it goes, and a segment of
@@ -30,6 +30,7 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct Ckpt {
   size_t vol = 0;
   int nseg = 0, every = 0, nvol = 0;  // nvol: segment volumes
+  bool paired = false;                // room for two segments' volumes
   unsigned char* base = nullptr;
   void* a(int s) const { return base + (size_t)(2 * s) * vol; }
   void* b(int s) const { return base + (size_t)(2 * s + 1) * vol; }
@@ -38,7 +39,8 @@ struct Ckpt {
   size_t bytes() const { return (size_t)(2 * nseg + nvol + 1) * vol; }
 };
 
-int ckpt_layout(const Plan& pl, int nt, int every, void* base, Ckpt* ck) {
+// (have: bytes at base)
+int ckpt_layout(const Plan& pl, int nt, int every, void* base, size_t have, Ckpt* ck) {
   if (pl.pad != 0) return report(FFPAT_EINVAL, "the differentiated operator needs pad = 0");
   if (every < 1 || every > 4096) return report(FFPAT_EINVAL, "checkpoint interval %d", every);
   // (FP32 volumes may have padded rows, FP64 ones never: see grad_view)
@@ -46,10 +48,18 @@ int ckpt_layout(const Plan& pl, int nt, int every, void* base, Ckpt* ck) {
   ck->vol = up256((size_t)pl.n * pl.n * row * pl.esize);
   ck->every = every;
   ck->nseg = (nt + every - 1) / every;
-  // FP32 on small grids: two segments' worth (see the resident branch of the
-  // backward pass)
-  ck->nvol = (pl.esize == 4 && pl.n <= kSegmentPairMaxN ? 2 * every : every) + 1;
+  ck->nvol = every + 1;
   ck->base = (unsigned char*)base;
+  // FP32 on small grids: room for two segments at a time, where there are two and
+  // the buffer holds them (see the resident branch of the backward pass)
+  if (pl.esize == 4 && pl.n <= kSegmentPairMaxN && ck->nseg >= 2) {
+    Ckpt two = *ck;
+    two.nvol += ck->nseg > 2 ? every : nt - every;  // the odd segments' volumes
+    two.paired = true;
+    if (two.bytes() <= have) *ck = two;
+  }
+  if (ck->bytes() > have)
+    return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", have, ck->bytes());
   return FFPAT_OK;
 }
 
@@ -90,7 +100,7 @@ size_t ffpat_ckpt_bytes(const ffpat_problem* problem, int32_t nt, int32_t every)
   if (ffpat_workspace_bytes(problem) == 0 || nt < 1) return 0;
   if (attach(problem, pl, (void*)256, ffpat_workspace_bytes(problem)) != FFPAT_OK) return 0;
   Ckpt ck;
-  if (ckpt_layout(pl, nt, every, nullptr, &ck) != FFPAT_OK) return 0;
+  if (ckpt_layout(pl, nt, every, nullptr, (size_t)-1, &ck) != FFPAT_OK) return 0;
   return ck.bytes();
 }
 
@@ -104,9 +114,8 @@ int ffpat_forward_ckpt(const ffpat_problem* problem, const void* c, const void* 
   if (!h || !g || !ckpt) return report(FFPAT_EINVAL, "h, g or ckpt is NULL");
   as_three_term(pl);
   Ckpt ck;
-  if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
-  if (ckpt_bytes < ck.bytes())
-    return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
+  const int rc1 = ckpt_layout(pl, pl.nt, every, ckpt, ckpt_bytes, &ck);
+  if (rc1 != FFPAT_OK) return rc1;
   const Plan w = wave_plan(pl);
   const void* in = h;
   if (w.np != w.n) {  // the source in padded rows
@@ -169,9 +178,8 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   if (!grad_g || !ckpt) return report(FFPAT_EINVAL, "grad_g or ckpt is NULL");
   as_three_term(pl);
   Ckpt ck;
-  if (ckpt_layout(pl, pl.nt, every, ckpt, &ck) != FFPAT_OK) return FFPAT_EINVAL;
-  if (ckpt_bytes < ck.bytes())
-    return report(FFPAT_ENOMEM, "checkpoint buffer %zu < %zu bytes", ckpt_bytes, ck.bytes());
+  const int rc1 = ckpt_layout(pl, pl.nt, every, ckpt, ckpt_bytes, &ck);
+  if (rc1 != FFPAT_OK) return rc1;
   const Plan w = wave_plan(pl);
   const bool tma = use_tma(w, ck, nullptr);
   const bool two = use_two(w, ck, tma);
@@ -198,7 +206,7 @@ int ffpat_backward(const ffpat_problem* problem, const void* c, const void* grad
   // resident segments: L(p^{lo+j}) in the segment volumes (two sets where the
   // recompute of a segment runs beside the transposed steps of the next), the
   // recomputed states through two spare volumes
-  const bool paired = resident && segments_paired(w);
+  const bool paired = resident && ck.paired && segments_paired(w);
   auto length = [&](int s) {
     return (s + 1 < ck.nseg ? every : pl.nt - s * every);
   };
