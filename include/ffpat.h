@@ -156,14 +156,21 @@ int ffpat_adjoint(const ffpat_problem *problem, const void *c, const void *g, vo
 int ffpat_wave(const ffpat_problem *problem, const void *c, const void *in, void *out,
                int32_t transpose, void *ws, size_t ws_bytes, void *stream);
 
-/* g = P p (eq. (4)) on the data grid; p: Nw^3, g: n_angles Nw^2.  No workspace. */
+/* g = P p (eq. (4)) on the data grid; p: Nw^3, g: n_angles Nw^2.  No workspace: a
+ * copy of the operand with z innermost is allocated in stream order for the
+ * duration of the call, at most 1 GiB (or 32 planes of it, where that is more:
+ * Nw > 2896 in FP32), and less, down to 32 planes (FP64: 2), where that much is not
+ * to be had.  Synchronises the stream.  g may not overlap p. */
 int ffpat_project(const ffpat_problem *problem, const void *p, void *g, void *stream);
 
-/* h = P^T g, the exact transpose of ffpat_project (backprojection X^* of Sec. 3.1). */
+/* h = P^T g, the exact transpose of ffpat_project (backprojection X^* of Sec. 3.1).
+ * Allocates for g and synchronises as ffpat_project does for p (32 planes are more
+ * than 1 GiB from n_angles Nw = 2^23 on in FP32).  h may not overlap g. */
 int ffpat_backproject(const ffpat_problem *problem, const void *g, void *h, void *stream);
 
 /* out = Lambda r along every detector row (Sec. 3.1): linear convolution with
- * t_0 = 1/(8 dxi), t_d = -1/(2 pi^2 d^2 dxi) for odd d, 0 for even d != 0. */
+ * t_0 = 1/(8 dxi), t_d = -1/(2 pi^2 d^2 dxi) for odd d, 0 for even d != 0.
+ * out may not overlap r (FFPAT_EINVAL if it is r). */
 int ffpat_ramp(const ffpat_problem *problem, const void *r, void *out, void *stream);
 
 /* out = prox of the gradient regulariser, (I + a D^T D)^{-1} f with

@@ -914,7 +914,8 @@ int ffpat_wave(const ffpat_problem* problem, const void* c, const void* in, void
 
 // P or P^T alone: the angle tables and the z-innermost operand in one
 // stream-ordered allocation, at most about kAloneScratch of it (larger operands go
-// in several passes over z, so that they may fill most of the device).
+// in several passes over z, so that they may fill most of the device) and less where
+// that much is not to be had, down to the planes of one pass.
 constexpr size_t kAloneScratch = (size_t)1 << 30;
 static int project_alone(const ffpat_problem* problem, const void* in, void* out, bool transpose,
                          cudaStream_t st) {
@@ -924,10 +925,19 @@ static int project_alone(const ffpat_problem* problem, const void* in, void* out
   if (!in || !out) return fail(FFPAT_EINVAL, transpose ? "g or h is NULL" : "p or g is NULL");
   const size_t tb = up256(table_bytes(pl.nth));
   const size_t rows = (size_t)pl.nw * (transpose ? pl.nth : pl.nw);
-  const size_t least = rows * 32 * pl.esize;
-  const size_t zb = zscratch_bytes(pl.nw, rows, pl.esize, least > kAloneScratch ? least : kAloneScratch);
+  const size_t wide = rows * 32 * pl.esize, least = zscratch_bytes(pl.nw, rows, pl.esize, 0);
+  size_t zb = zscratch_bytes(pl.nw, rows, pl.esize, wide > kAloneScratch ? wide : kAloneScratch);
   char* mem = nullptr;
-  CK(cudaMallocAsync((void**)&mem, tb + zb, st));
+  cudaError_t em;
+  while ((em = cudaMallocAsync((void**)&mem, tb + zb, st)) == cudaErrorMemoryAllocation &&
+         zb > least) {
+    cudaGetLastError();
+    zb = zscratch_bytes(pl.nw, rows, pl.esize, zb / 2);
+  }
+  if (em != cudaSuccess) {
+    cudaGetLastError();
+    return fail(FFPAT_ECUDA, "%zu bytes for the operand: %s", tb + zb, cudaGetErrorString(em));
+  }
   std::vector<unsigned char> tabs;
   int rc = upload_tables(pl, mem, tabs, st);
   const Plan wp = dense_rows(wave_plan(pl));
