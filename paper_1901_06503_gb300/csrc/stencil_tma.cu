@@ -1647,8 +1647,10 @@ __global__ void __launch_bounds__(rd::TX* rd::TY, 4)
 
 // ------------------------------------------------------------- host side --
 
-// FFPAT_ZCHUNK=<planes> fixes the z-range of one work item of the TMA
-// stencil kernels (a tuning knob for measurements; 0 or unset = automatic)
+// FFPAT_ZCHUNK=<planes> fixes the z-range of one work item of the FP32 step
+// kernels and, where that fits, of the FP32 resident loop (a tuning knob for
+// measurements; 0 or unset = automatic).  FP64 steps take equal stretches of planes
+// instead, and the FP64 resident loop its own z-range.
 int zchunk_override() {
   static int v = [] {
     const char* e = getenv("FFPAT_ZCHUNK");

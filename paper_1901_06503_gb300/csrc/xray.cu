@@ -28,9 +28,9 @@
 // frame, i.e. at most 3 x 3 candidates; each contributes hat(dx) hat(dy) times
 // its row value, which is exactly the bilinear weight P gives that voxel.
 //
-// Lambda: one CTA per detector row, the row staged in shared memory, the odd
-// taps t_d = -1/(2 pi^2 d^2 dxi) and t_0 = 1/(8 dxi) applied as a linear
-// (non-circular) convolution.
+// Lambda: the linear (non-circular) convolution of a detector row with the odd
+// taps t_d = -1/(2 pi^2 d^2 dxi) and t_0 = 1/(8 dxi), as a Toeplitz product: a CTA
+// stages 32 rows, 512 inputs at a time, for up to 256 of their outputs.
 #include <limits.h>
 #include <math.h>
 #include <stdlib.h>
@@ -182,7 +182,8 @@ __device__ __forceinline__ float2 ffma2(float w, float2 x, float2 a) {
 }
 
 // What adding t to s0 (the sum: s1) rounded off; 0 where the sum has overflowed,
-// so that it stays infinite.
+// so that it stays infinite.  Exact where |s0| >= |t|, as it is once a sum of one
+// sign has two groups; where t is the larger, s1 - s0 is rounded itself.
 __device__ __forceinline__ float rounded_off(float t, float s1, float s0) {
   const float e = __fsub_rn(t, __fsub_rn(s1, s0));
   return fabsf(e) < 1e32f ? e : 0.0f;
@@ -285,7 +286,8 @@ __device__ __forceinline__ RowTaps row_taps(int a, int k, long long CS, long lon
 // flight).  Per standalone call, 384^3 and 180 angles: 13.0 -> 5.2 ms against
 // the plane-by-plane kernel it replaces, 256^3 and 180: 3.7 -> 1.7 ms.
 // Sums: per kPSum rows, then over those; what adding a group rounds off starts
-// the next one, so that the error does not grow with N (a smooth volume, relative:
+// the next one, so that the error of a sum of one sign, where the groups' total is
+// the large term, does not grow with N (a smooth volume, relative:
 // 150^3 8.3e-8 -> 4.7e-8, 256^3 9.6e-8 -> 3.0e-8; 192^3 and 90 angles, standalone
 // call, 541 -> 547 us).
 constexpr int kPSum = 8;
@@ -585,7 +587,7 @@ __device__ __noinline__ float voxel_alone(const float* __restrict__ gp, int rl, 
 // angles at a time (a lane: one voxel and angle) into the warp's part of shared
 // memory; then, angle by angle, the (at most five) detectors any of the four
 // voxels sees are loaded once and applied to all four: C vector loads and 2 V C
-// packed FMAs per detector (57 % of the issue slots and 52 % of L1's throughput in
+// packed FMAs per detector (58 % of the issue slots and 57 % of L1's throughput in
 // use at 192^3 and 90 angles, waits for loads the first stall; a voxel alone
 // would load three detectors for as many multiply-adds each).  kk of the block
 // spans |cos| + |sin| =: s <= sqrt 2 and a voxel's detectors lie within s of its
@@ -597,7 +599,7 @@ __device__ __noinline__ float voxel_alone(const float* __restrict__ gp, int rl, 
 // the rounding of the long sum, small (256^3, 180 angles of filtered data, error
 // against 64 bits 3.1 - 3.6e-7 -> 2.9e-7).  The list holds addresses: stepping a
 // pointer through the spread rows took 2 % more (fbp at 192^3 / 90 angles 231 -> 222
-// us, 256^3 / 180 779 -> 758 us, 384^3 / 180 2.56 -> 2.51 ms).
+// us, 256^3 / 180 779 -> 757 us, 384^3 / 180 2.56 -> 2.49 ms).
 constexpr int kBDet = 5;
 constexpr int kBTileX = 4, kBTileY = 2;  // blocks of a CTA (8 x 4 voxels), one a warp
 // the detectors of a block and angle: address of the first one's planes, and count
@@ -896,8 +898,8 @@ __global__ void __launch_bounds__(128)
 // On smooth rows t_0 r_k nearly cancels the nearest taps' sum, so those (|d| <=
 // kRNear) are summed apart, outwards from t_0, and the product holds the others
 // (a tenth of t_0 in all), whose rounding then shows as little.
-// 384^3 and 180 angles: 1.63 -> 0.41 ms against two inputs and a tap loaded for
-// every multiply-add, 256^3 and 180: 0.50 -> 0.125 ms (0.16 with one CTA an SM at
+// 384^3 and 180 angles: 1.63 -> 0.40 ms against two inputs and a tap loaded for
+// every multiply-add, 256^3 and 180: 0.50 -> 0.122 ms (0.16 with one CTA an SM at
 // 127 registers, 0.17 with eight outputs a warp).
 constexpr int kROut = 16;
 constexpr int kRNear = 3;
