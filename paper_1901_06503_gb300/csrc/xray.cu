@@ -896,17 +896,20 @@ __global__ void __launch_bounds__(128)
 // 32: per input it loads one value a row and one new tap (broadcast; the other
 // taps slide through registers) for kROut multiply-adds.  The same kernel in FP64.
 // On smooth rows t_0 r_k nearly cancels the nearest taps' sum, so those (|d| <=
-// kRNear) are summed apart, outwards from t_0, and the product holds the others
-// (a tenth of t_0 in all), whose rounding then shows as little.
+// NEAR) are summed apart, outwards from t_0, the two large products without rounding
+// them, and the Toeplitz product holds the others (a tenth of t_0 in all with NEAR =
+// 3), whose rounding then shows as little.  NEAR is 7 beyond 448 points, where more
+// of the others are added (FP32).  Error on smooth rows over that of the sum outwards
+// pair by pair: 0.57 at 64, 0.81 at 256, 0.79 at 384, 0.87 at 512, 0.99 at 1024
+// points (with rounded products and NEAR = 3 throughout 1.03 - 1.5 from 512 on).
 // 384^3 and 180 angles: 1.63 -> 0.40 ms against two inputs and a tap loaded for
 // every multiply-add, 256^3 and 180: 0.50 -> 0.122 ms (0.16 with one CTA an SM at
 // 127 registers, 0.17 with eight outputs a warp).
 constexpr int kROut = 16;
-constexpr int kRNear = 3;
 constexpr int kRPitch = 33;  // of a staged input: 32 rows and one word against bank conflicts
 
 // (Lambda row)_k by the odd taps alone.  The Toeplitz product has zeros for taps
-// among those of its other parity (|d| <= kRNear), which make NaN of an infinite
+// among those of its other parity (|d| <= NEAR), which make NaN of an infinite
 // input: an output that is NaN is taken from here, which says whether it is.
 template <typename T>
 __device__ __noinline__ T ramp_direct(const T* __restrict__ row, int k, int n, int nimg) {
@@ -919,7 +922,14 @@ __device__ __noinline__ T ramp_direct(const T* __restrict__ row, int k, int n, i
   return v;
 }
 
-template <typename T>
+// rows of staged inputs: all of them and what the last outputs' nearest taps reach,
+// or a piece of jc, or the outputs of a CTA
+__host__ __device__ inline int ramp_rows(int n, int jc, int nout, int ctas, int near) {
+  const int reach = jc >= n ? ctas * nout : nout;
+  return (jc > reach ? jc : reach) + 2 * near;
+}
+
+template <typename T, int NEAR>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
     k_ramp(const T* __restrict__ r, T* __restrict__ out, const T* __restrict__ mask, int n,
            int nimg, int rows, int jc) {
@@ -928,13 +938,18 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
   const int ko = blockIdx.y * warps * kROut;   // first output of the CTA (a multiple of 32)
   const int nout = warps * kROut;
   const int H = n / 2 + 2 * kROut + nout / 2;  // taps by u, d = 2 u + 1, -H <= u < H
-  T* s = reinterpret_cast<T*>(smem_raw);       // [max(jc, nout)][kRPitch]
-  T* ts = s + (size_t)max(jc, nout) * kRPitch;
+  // staged inputs [ramp_rows][kRPitch], NEAR rows of room before the first
+  const int srows = ramp_rows(n, jc, nout, gridDim.y, NEAR);
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* ts = s + (size_t)srows * kRPitch;
   const double dxi = 2.0 / nimg;
   for (int i = tid; i < 2 * H; i += blockDim.x) {
     const double d = 2.0 * (i - H) + 1.0;
-    ts[i] = fabs(d) > kRNear ? (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi)) : T(0);
+    ts[i] = fabs(d) > NEAR ? (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi)) : T(0);
   }
+  if (jc >= n)  // zeros around the rows for the nearest taps
+    for (int i = tid; i < (srows - n) * 32; i += blockDim.x)
+      s[(i / 32 < NEAR ? i / 32 : n + i / 32) * kRPitch + i % 32] = T(0);
   const int row0 = blockIdx.x * 32, live = min(32, rows - row0);
   // outputs k = 2 (q0 + m) + p, inputs j = 2 i + 1 - p, tap u = q0 + m + p - 1 - i
   const int p = warp & 1, q0 = ko / 2 + (warp >> 1) * kROut;
@@ -946,11 +961,11 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
     __syncthreads();
     for (int q = warp; q < 32; q += warps) {
       const T* src = r + (size_t)(row0 + q) * n + j0;
-      for (int j = lane; j < len; j += 32) s[j * kRPitch + q] = q < live ? src[j] : T(0);
+      for (int j = lane; j < len; j += 32) s[(NEAR + j) * kRPitch + q] = q < live ? src[j] : T(0);
     }
     __syncthreads();
     const int ni = (len + p) / 2;
-    const T* x = s + (1 - p) * kRPitch + lane;
+    const T* x = s + (NEAR + 1 - p) * kRPitch + lane;
     const T* t = ts + H + q0 + p - 1 - j0 / 2;  // t[m - i]: the tap of output m, input i
     T w[kROut];  // slot (m - i) mod kROut
 #pragma unroll
@@ -972,26 +987,42 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1)
       for (int m = 0; m < kROut; ++m) acc[m] = fma(t[m - i], v, acc[m]);
     }
   }
-  // the nearest taps, outwards from t_0 (the rows still staged when jc >= n)
+  // the nearest taps, outwards from t_0, on the rows as staged or, where that was in
+  // several pieces, on the inputs around the CTA's outputs staged again
+  const T* near = s + (NEAR - (jc < n ? ko : 0)) * kRPitch + lane;  // input j at j kRPitch
+  if (jc < n) {
+    __syncthreads();
+    for (int q = warp; q < 32; q += warps) {
+      const T* src = r + (size_t)(row0 + q) * n;
+      for (int j = lane; j < nout + 2 * NEAR; j += 32) {
+        const int from = ko - NEAR + j;
+        s[j * kRPitch + q] = q < live && (unsigned)from < (unsigned)n ? src[from] : T(0);
+      }
+    }
+    __syncthreads();
+  }
   const T t0 = (T)(1.0 / (8.0 * dxi));
-  T tn[(kRNear + 1) / 2];
+  T tn[(NEAR + 1) / 2];
 #pragma unroll
-  for (int e = 0; e < (kRNear + 1) / 2; ++e) {
+  for (int e = 0; e < (NEAR + 1) / 2; ++e) {
     const double d = 2.0 * e + 1.0;
     tn[e] = (T)(-1.0 / (2.0 * kPi * kPi * d * d * dxi));
   }
-  const bool staged = jc >= n;
-  const T* own = r + (size_t)(row0 + min(lane, live - 1)) * n;
-  auto at = [&](int j) -> T {
-    return j < 0 || j >= n ? T(0) : (staged ? s[j * kRPitch + lane] : own[j]);
-  };
+  auto at = [&](int j) -> T { return near[j * kRPitch]; };
 #pragma unroll
   for (int m = 0; m < kROut; ++m) {
     const int k = 2 * (q0 + m) + p;
-    T v = t0 * at(k);
+    const T pair = at(k - 1) + at(k + 1);
+    T v;
+    if constexpr (sizeof(T) == 4) {  // t_0 r_k + t_1 pair, neither product rounded
+      const T prod = tn[0] * pair;
+      v = fma(t0, at(k), prod) + fma(tn[0], pair, -prod);
+    } else {
+      v = fma(tn[0], pair, t0 * at(k));
+    }
 #pragma unroll
-    for (int e = 0; e < (kRNear + 1) / 2; ++e)
-      v += tn[e] * (at(k - 2 * e - 1) + at(k + 2 * e + 1));
+    for (int e = 1; e < (NEAR + 1) / 2; ++e)
+      v = fma(tn[e], at(k - 2 * e - 1) + at(k + 2 * e + 1), v);
     acc[m] = v + acc[m];
   }
   // through shared memory to the rows
@@ -1254,7 +1285,7 @@ int launch_backproject(const Plan& pl, const void* g, void* h, const void* scale
   return FFPAT_OK;
 }
 
-template <typename T>
+template <typename T, int NEAR>
 static int ramp_launch(const Plan& pl, const void* r, void* out, const void* mask,
                        cudaStream_t st) {
   const int n = pl.n, rows = pl.nth * n;
@@ -1263,25 +1294,28 @@ static int ramp_launch(const Plan& pl, const void* r, void* out, const void* mas
   const int pairs = (n + 2 * kROut - 1) / (2 * kROut), gy = (pairs + 7) / 8;
   const int warps = 2 * ((pairs + gy - 1) / gy), nout = warps * kROut;
   const int jc = n < 512 ? (n + 1) / 2 * 2 : 512, H = n / 2 + 2 * kROut + nout / 2;
-  const size_t smem = ((size_t)(jc > nout ? jc : nout) * kRPitch + 2 * (size_t)H) * sizeof(T);
+  const size_t smem =
+      ((size_t)ramp_rows(n, jc, nout, gy, NEAR) * kRPitch + 2 * (size_t)H) * sizeof(T);
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(k_ramp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    attr = cudaFuncSetAttribute(k_ramp<T, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                220 * 1024);
   });
   if (attr != cudaSuccess || smem > 220 * 1024) {
     cudaGetLastError();
     return report(FFPAT_ECUDA, "k_ramp: %zu bytes of shared memory refused", smem);
   }
-  k_ramp<T><<<dim3((rows + 31) / 32, gy), 32 * warps, smem, st>>>(
+  k_ramp<T, NEAR><<<dim3((rows + 31) / 32, gy), 32 * warps, smem, st>>>(
       (const T*)r, (T*)out, (const T*)mask, n, pl.nimg, rows, jc);
   count_launch();
   return check_launch("k_ramp");
 }
 
 int launch_ramp(const Plan& pl, const void* r, void* out, cudaStream_t st, const void* mask) {
-  return pl.prec == FFPAT_FP64 ? ramp_launch<double>(pl, r, out, mask, st)
-                               : ramp_launch<float>(pl, r, out, mask, st);
+  return pl.prec == FFPAT_FP64 ? ramp_launch<double, 3>(pl, r, out, mask, st)
+         : pl.n <= 448         ? ramp_launch<float, 3>(pl, r, out, mask, st)
+                               : ramp_launch<float, 7>(pl, r, out, mask, st);
 }
 
 int launch_debug_samples(const Plan& pl, int count, const int32_t* jkm, int32_t* ij, double* f,
