@@ -397,9 +397,9 @@ int ffpat_server_destroy(ffpat_server *server);
  * library's device code is loaded on a device and held until exit; under
  * CUDA's lazy module loading (the default) that load happens during the first
  * call on each device, which may allocate once; later calls allocate nothing.
- * Problems whose whole workspace of dense volumes and data (that is
- * ffpat_workspace_bytes without what the kernels' layouts add) exceeds 32 MiB
- * fail with FFPAT_EINVAL
+ * Problems whose whole workspace of dense volumes and data (about
+ * ffpat_workspace_bytes, whatever the kernels' layouts add or share) exceeds 32
+ * MiB fail with FFPAT_EINVAL
  * (a wave grid N + 2 pad <= 64 with up to 180 angles fits every precision;
  * without padding that is N <= 64); a device index >= 64 fails with
  * FFPAT_EINVAL.  The first call on a device looks up the array's device

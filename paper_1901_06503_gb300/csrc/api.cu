@@ -215,7 +215,7 @@ Scratch backproject_scratch(const Plan& pl, const void* g) {
 
 // Bytes that a whole workspace of dense, unrounded volumes and data has: the
 // measure by which ffpat_forward_noalloc accepts a problem, whatever the
-// kernels' layouts add to ffpat_workspace_bytes.  What it accepts fits the forward
+// kernels' layouts add or share.  What it accepts fits the forward
 // operator's part with dense rows.
 static size_t dense_workspace(const Plan& pl) {
   const size_t vol = up256(pl.n3 * pl.esize), wvol = up256(pl.nw3 * pl.esize);

@@ -17,7 +17,7 @@
 // lazy module loading (the default) that happens during the first call on
 // each device, which may therefore allocate device memory once; later calls
 // allocate nothing.  Problems are measured by a whole workspace of dense volumes
-// and data (ffpat_workspace_bytes without what the kernels' layouts add to it);
+// and data (about ffpat_workspace_bytes, whatever the kernels' layouts add or share);
 // those beyond the array are rejected.  It grows with the wave grid N_w = N + 2 pad:
 // without padding, N <= 64 with up to 180 angles fits in every precision
 // (N_w <= 64 with up to 180 angles in general).
